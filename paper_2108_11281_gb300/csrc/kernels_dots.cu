@@ -1,0 +1,717 @@
+// Column dot products and multi-AXPY of the batched Krylov solvers, and the per-column
+// algebra of the fixed-length FGMRES (Saad, Alg. 9.6, with an unnormalised basis).
+//
+// Vector blocks are [row][k] with the k columns (independent systems) innermost.  A thread
+// owns one 16-byte pack of consecutive columns (VEC columns; 1 where k or a pointer does
+// not allow it) and walks the rows of its block's contiguous chunk, so every load is
+// coalesced and a column's sum stays in one lane until the end of the chunk.
+//
+// FP64 additions run at 1.7 per clock and SM on this GPU (0.53 T/s), FP32 ones at 128: the
+// sums over lanes and blocks of FP32 data are kept as float pairs (a hi + lo sum by the
+// two-sum of Knuth, TAOCP 4.2.2; 48 significant bits, far below the rounding of the FP32
+// lane sums they add up) and become FP64 once per column.  Sums of FP64 data stay FP64.
+#include <algorithm>
+#include <initializer_list>
+#include <mutex>
+#include <type_traits>
+
+#include "mlmc_internal.cuh"
+
+namespace mlmc {
+
+namespace {
+
+constexpr int DT = 512;            // threads per block
+constexpr int DOT_PARTS = 152;     // row chunks of a dot product: one block per SM (FP64 data: two)
+constexpr int AXPY_PARTS = 304;    // row chunks of a multi-AXPY: two blocks per SM
+constexpr int DOT_MAXV = 8;        // basis vectors per pass over w
+constexpr int RT = 512;            // threads of a reduction block
+
+template <class T, int VEC> struct alignas(sizeof(T) * VEC) DPack { T v[VEC]; };
+
+// Scalars of a column (real: 1, complex: 2) and their running sums over lanes and blocks.
+struct FF { float h, l; };
+template <class T> struct lane_of;
+template <> struct lane_of<float> { typedef float S; typedef FF A; static constexpr int C = 1; };
+template <> struct lane_of<double> { typedef double S; typedef double A; static constexpr int C = 1; };
+template <> struct lane_of<cfloat> { typedef float S; typedef FF A; static constexpr int C = 2; };
+template <> struct lane_of<cdouble> { typedef double S; typedef double A; static constexpr int C = 2; };
+template <class T> struct acc_of { typedef double type; };
+template <> struct acc_of<cdouble> { typedef cdouble type; };
+template <> struct acc_of<cfloat> { typedef cdouble type; };
+
+__device__ __forceinline__ void acc_zero(FF &a) { a.h = a.l = 0.f; }
+__device__ __forceinline__ void acc_zero(double &a) { a = 0.0; }
+// a += x: the rounding error of each addition goes into the low part
+__device__ __forceinline__ void acc_add(FF &a, float x) {
+  const float s = a.h + x, t = s - a.h;
+  a.l += (a.h - (s - t)) + (x - t);
+  a.h = s;
+}
+__device__ __forceinline__ void acc_add(FF &a, FF b) {
+  acc_add(a, b.h);
+  a.l += b.l;
+}
+__device__ __forceinline__ void acc_add(double &a, double x) { a += x; }
+__device__ __forceinline__ double acc_value(FF a) { return (double)a.h + (double)a.l; }
+__device__ __forceinline__ double acc_value(double a) { return a; }
+
+// a += conj(x) * y on scalars
+__device__ __forceinline__ void dot_fma(float a[1], float x, float y) { a[0] += x * y; }
+__device__ __forceinline__ void dot_fma(double a[1], double x, double y) { a[0] += x * y; }
+__device__ __forceinline__ void dot_fma(float a[2], cfloat x, cfloat y) {
+  a[0] += x.re * y.re + x.im * y.im;
+  a[1] += x.re * y.im - x.im * y.re;
+}
+__device__ __forceinline__ void dot_fma(double a[2], cdouble x, cdouble y) {
+  a[0] += x.re * y.re + x.im * y.im;
+  a[1] += x.re * y.im - x.im * y.re;
+}
+
+template <class T> struct VecList { const T *v[DOT_MAXV]; };
+
+__device__ __forceinline__ void chunk_of(size_t rows, size_t &r0, size_t &r1) {
+  const size_t chunk = (rows + gridDim.x - 1) / gridDim.x;
+  r0 = min((size_t)blockIdx.x * chunk, rows);
+  r1 = min(r0 + chunk, rows);
+}
+
+// Sums `val` (one scalar set per thread: NC scalars of columns cv * VEC ...) over the
+// block's slots in fixed order into out[e], e < E = k * C scalars of one output row.
+// red: DT * NC lane values, red2: DT sums.  Ends with the block synchronised.
+template <class T, int NC>
+__device__ void block_sum(const typename lane_of<T>::S *val, typename lane_of<T>::S *red, typename lane_of<T>::A *red2,
+                          int E, int slots, bool live, typename lane_of<T>::A *out) {
+  typedef typename lane_of<T>::A A;
+  const int tid = threadIdx.x;
+#pragma unroll
+  for (int u = 0; u < NC; ++u) red[tid * NC + u] = live ? val[u] : 0;
+  __syncthreads();
+  // scalar e of the row sits at red[slot * E + e]; G threads share its slots
+  const int G = E < DT ? DT / E : 1;
+  for (int e0 = 0; e0 < E; e0 += DT) {
+    const int e = e0 + tid % min(E, DT), g = tid / min(E, DT);
+    A a;
+    acc_zero(a);
+    if (g < G && e < E)
+      for (int s = g; s < slots; s += G) acc_add(a, red[s * E + e]);
+    if (G > 1) {
+      red2[tid] = a;
+      __syncthreads();
+      if (g == 0) {
+        for (int q = 1; q < G; ++q) acc_add(a, red2[q * E + e]);
+        out[e] = a;
+      }
+    } else if (g == 0 && e < E) {
+      out[e] = a;
+    }
+  }
+  __syncthreads();
+}
+
+}  // namespace
+
+// ------------------------------------------------------------------ dot products
+// partial[part][row0 + r][c] = sum over the chunk's rows of conj(V_r[row][c]) w[row][c], r < NV,
+// then (EXTRA & 2) v0.v0 and (EXTRA & 1) w.w in the following rows: quantities of the same
+// read of the data that would otherwise need passes of their own.
+// HBM-bound on large blocks: 16 warps per SM with about eight 16-byte loads in flight per
+// thread; one block per SM, so only 152 partial sums per column are left to add.  Four FP32
+// vectors of 1024^2 x 64 with the reduction: 209 us, 6.41 TB/s (250 us with 608 blocks of 256
+// threads, 8-byte loads and FP64 block sums); 16384 x 128, L2-resident: 12.4 us (22.6).
+template <class T, int VEC, int NV, int EXTRA>
+__global__ void __launch_bounds__(DT, 1) k_dots(VecList<T> V, const T *__restrict__ w, size_t rows, int k,
+                                                typename lane_of<T>::A *__restrict__ partial, int row0, int nrows) {
+  typedef typename lane_of<T>::S S;
+  typedef typename lane_of<T>::A A;
+  typedef DPack<T, VEC> P;
+  constexpr int C = lane_of<T>::C, NC = VEC * C;
+  constexpr int R = NV + (EXTRA & 1) + (EXTRA >> 1);
+  constexpr int U = NV <= 1 ? 4 : NV <= 3 ? 2 : 1;
+  __shared__ __align__(16) S red[DT * NC];
+  __shared__ A red2[DT];
+  const int kv = k / VEC, slots = DT / kv;
+  const int cv = threadIdx.x % kv, slot = threadIdx.x / kv;
+  const bool live = slot < slots;
+  size_t r0, r1;
+  chunk_of(rows, r0, r1);
+  S acc[R][NC];
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+#pragma unroll
+    for (int u = 0; u < NC; ++u) acc[r][u] = 0;
+  const P *W = (const P *)w;
+  auto step = [&](const P &wv, const P *x) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+#pragma unroll
+      for (int u = 0; u < VEC; ++u) dot_fma(&acc[v][u * C], x[v].v[u], wv.v[u]);
+    if (EXTRA & 2)
+#pragma unroll
+      for (int u = 0; u < VEC; ++u) dot_fma(&acc[NV][u * C], x[0].v[u], x[0].v[u]);
+    if (EXTRA & 1)
+#pragma unroll
+      for (int u = 0; u < VEC; ++u) dot_fma(&acc[NV + (EXTRA >> 1)][u * C], wv.v[u], wv.v[u]);
+  };
+  if (live) {
+    size_t r = r0 + slot;
+    for (; r + (size_t)(U - 1) * slots < r1; r += (size_t)U * slots) {
+      P wv[U], x[U][NV];
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const size_t o = (r + (size_t)q * slots) * kv + cv;
+        wv[q] = W[o];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) x[q][v] = ((const P *)V.v[v])[o];
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q) step(wv[q], x[q]);
+    }
+    for (; r < r1; r += slots) {
+      P wv, x[NV];
+      const size_t o = r * kv + cv;
+      wv = W[o];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) x[v] = ((const P *)V.v[v])[o];
+      step(wv, x);
+    }
+  }
+  const int E = k * C;
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    block_sum<T, NC>(acc[r], red, red2, E, slots, live,
+                     partial + ((size_t)blockIdx.x * nrows + row0 + r) * E);
+}
+
+// out[e] = sum over parts of partial[part][e], e < nrows * k scalars, in fixed order: one
+// block per 32 consecutive scalars (coalesced), 16 warps each taking every 16th part.
+template <class A>
+__global__ void __launch_bounds__(RT) k_dots_reduce(const A *__restrict__ partial, int nparts, int entries,
+                                                    double *__restrict__ out) {
+  __shared__ A red[RT / 32][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + lane;
+  A a;
+  acc_zero(a);
+  if (e < entries) {
+#pragma unroll 4
+    for (int p = warp; p < nparts; p += RT / 32) acc_add(a, partial[(size_t)p * entries + e]);
+  }
+  red[warp][lane] = a;
+  __syncthreads();
+  if (warp == 0 && e < entries) {
+    for (int q = 1; q < RT / 32; ++q) acc_add(a, red[q][lane]);
+    out[e] = acc_value(a);
+  }
+}
+
+int multidot_parts(DType t, size_t rows, int k) {
+  // enough row chunks to give every thread a few rows, at most one block per SM; FP64 data two,
+  // so that a lane adds up half as many products
+  const size_t per = std::max<size_t>(1, (size_t)DT * 8 / std::max(k, 1));
+  const size_t most = dtype_size(dtype_lower(t)) == dtype_size(t) ? DOT_PARTS : 2 * DOT_PARTS;
+  return (int)std::min<size_t>(most, std::max<size_t>(1, (rows + per - 1) / per));
+}
+
+namespace {
+
+// VEC columns per 16-byte pack where every row and every pointer allows it.
+template <class T>
+bool packs_ok(int k, std::initializer_list<const void *> ptrs) {
+  constexpr int VW = 16 / (int)sizeof(T);
+  if (VW == 1) return true;
+  if (k % VW) return false;
+  for (const void *p : ptrs)
+    if ((uintptr_t)p & 15) return false;
+  return true;
+}
+
+template <class T, int VEC, int EXTRA>
+void dots_go(const VecList<T> &V, int nv, const T *w, size_t rows, int k, void *partial, int nparts, int row0,
+             int nrows, cudaStream_t s) {
+  typedef typename lane_of<T>::A A;
+  auto go = [&](auto n) {
+    constexpr int NV = decltype(n)::value;
+    if constexpr (NV == 1 || EXTRA < 2)           // v0.v0 is asked for with the first vector alone
+      k_dots<T, VEC, NV, EXTRA><<<nparts, DT, 0, s>>>(V, w, rows, k, (A *)partial, row0, nrows);
+    else
+      throw cuda_error{cudaErrorInvalidValue, "multidot: v0.v0 needs a single vector"};
+  };
+  switch (nv) {
+    case 1: go(std::integral_constant<int, 1>()); break;
+    case 2: go(std::integral_constant<int, 2>()); break;
+    case 3: go(std::integral_constant<int, 3>()); break;
+    case 4: go(std::integral_constant<int, 4>()); break;
+    case 5: go(std::integral_constant<int, 5>()); break;
+    case 6: go(std::integral_constant<int, 6>()); break;
+    case 7: go(std::integral_constant<int, 7>()); break;
+    default: go(std::integral_constant<int, 8>()); break;
+  }
+  MLMC_LAUNCH_CHECK("k_dots");
+}
+
+// Partial sums of w against nvec basis vectors (v0, then V + i * vstride elements), then
+// (extra & 2) v0.v0 and (extra & 1) w.w; returns the number of passes (launches).
+template <class T>
+int dots_partial(const void *v0, const void *V, size_t vstride, int nvec, const void *w, size_t rows, int k,
+                 void *partial, int nparts, int extra, cudaStream_t s) {
+  constexpr int VW = 16 / (int)sizeof(T);
+  const bool packed = VW > 1 && packs_ok<T>(k, {v0, V, w}) && vstride % VW == 0;
+  if ((packed ? k / VW : k) > DT) throw cuda_error{cudaErrorInvalidValue, "multidot: more column groups than threads"};
+  const int nrows = nvec + (extra & 1) + (extra >> 1);
+  int passes = 0;
+  for (int i0 = 0; i0 < nvec; i0 += DOT_MAXV) {
+    VecList<T> L;
+    const int nv = std::min(nvec - i0, DOT_MAXV);
+    for (int i = 0; i < DOT_MAXV; ++i) {
+      const int id = i0 + std::min(i, nv - 1);
+      L.v[i] = id == 0 ? (const T *)v0 : (const T *)V + (size_t)id * vstride;
+    }
+    // the extra rows ride on the last pass (w.w) or need v0 in it (v0.v0: nvec = 1)
+    const int ex = i0 + nv < nvec ? 0 : extra;
+    auto go = [&](auto vec) {
+      constexpr int VEC = decltype(vec)::value;
+      if (ex == 0) dots_go<T, VEC, 0>(L, nv, (const T *)w, rows, k, partial, nparts, i0, nrows, s);
+      else if (ex == 1) dots_go<T, VEC, 1>(L, nv, (const T *)w, rows, k, partial, nparts, i0, nrows, s);
+      else if (ex == 2) dots_go<T, VEC, 2>(L, nv, (const T *)w, rows, k, partial, nparts, i0, nrows, s);
+      else dots_go<T, VEC, 3>(L, nv, (const T *)w, rows, k, partial, nparts, i0, nrows, s);
+    };
+    if (packed) go(std::integral_constant<int, VW>());
+    else go(std::integral_constant<int, 1>());
+    ++passes;
+  }
+  return passes;
+}
+
+}  // namespace
+
+void launch_multidot(DType t, const void *V, size_t vstride, int nvec, const void *w, size_t rows, int k,
+                     void *partials, int nparts, void *out, cudaStream_t s) {
+  MLMC_DISPATCH(t, T, {
+    typedef typename lane_of<T>::A A;
+    dots_partial<T>(V, V, vstride, nvec, w, rows, k, partials, nparts, 0, s);
+    const int entries = nvec * k * lane_of<T>::C;
+    k_dots_reduce<A><<<(entries + 31) / 32, RT, 0, s>>>((const A *)partials, nparts, entries, (double *)out);
+    MLMC_LAUNCH_CHECK("k_dots_reduce");
+  });
+}
+
+// ------------------------------------------------------------------ multi-AXPY
+// w[r][c] = (INIT ? 0 : w[r][c]) + sign * sum_v V_v[r][c] * h[v * hstride + c] over one pass of
+// nv <= AXPY_GROUP vectors; the coefficients, rounded to the storage precision, sit in shared
+// memory.  norm (optional): per block and column the sum of |w_new|^2 over its rows, for the
+// Arnoldi step, summed per thread in row order (float pairs every 16 rows) and over the
+// block's slots in fixed order; INIT updates (the solution) need none.
+// HBM-bound on large blocks ((nv + 2) passes, nv + 1 with INIT): four FP32 vectors on
+// 1024^2 x 64 take 261 us, 6.18 TB/s (268 us before); on 2.4 MB blocks of 48 columns, whose
+// column groups do not divide 256 threads, 3.7 us (10.3: the norms were summed serially).
+template <class T, class H, int VEC, bool INIT>
+__global__ void __launch_bounds__(DT, 2) k_axpy(T *__restrict__ w, VecList<T> V, int nv, const H *__restrict__ h,
+                                                int hstride, double sign, size_t rows, int k,
+                                                typename lane_of<T>::A *__restrict__ norm) {
+  typedef typename lane_of<T>::S S;
+  typedef typename lane_of<T>::A A;
+  typedef DPack<T, VEC> P;
+  extern __shared__ __align__(16) unsigned char axpy_smem[];
+  __shared__ __align__(16) S red[DT * VEC];
+  __shared__ A red2[DT];
+  T *hs = (T *)axpy_smem;
+  for (int e = threadIdx.x; e < nv * k; e += DT) {
+    const int v = e / k, c = e - v * k;
+    hs[e] = cvt<T, H>(rmul((typename real_of<H>::type)sign, h[(size_t)v * hstride + c]));
+  }
+  __syncthreads();
+  const int kv = k / VEC, slots = DT / kv;
+  const int cv = threadIdx.x % kv, slot = threadIdx.x / kv;
+  const bool live = slot < slots;
+  size_t r0, r1;
+  chunk_of(rows, r0, r1);
+  P *W = (P *)w;
+  const P *Hp = (const P *)hs + cv;
+  S sq[VEC];
+  A tot[VEC];
+#pragma unroll
+  for (int u = 0; u < VEC; ++u) {
+    sq[u] = 0;
+    acc_zero(tot[u]);
+  }
+  if (live) {
+    int n = 0;
+    constexpr int U = 2;
+    size_t r = r0 + slot;
+    for (; r < r1; r += (size_t)U * slots) {
+      P a[U];
+      size_t o[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        o[q] = min(r + (size_t)q * slots, r1 - 1) * kv + cv;   // past the end: a row of the chunk, not stored
+        if (INIT) {
+#pragma unroll
+          for (int u = 0; u < VEC; ++u) a[q].v[u] = zero<T>();
+        } else {
+          a[q] = W[o[q]];
+        }
+      }
+#pragma unroll 2
+      for (int v = 0; v < nv; ++v) {
+        const P hh = Hp[v * kv];
+        P x[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) x[q] = ((const P *)V.v[v])[o[q]];
+#pragma unroll
+        for (int q = 0; q < U; ++q)
+#pragma unroll
+          for (int u = 0; u < VEC; ++u) a[q].v[u] = a[q].v[u] + x[q].v[u] * hh.v[u];
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+        if (r + (size_t)q * slots < r1) {
+          W[o[q]] = a[q];
+          if (!INIT)
+#pragma unroll
+            for (int u = 0; u < VEC; ++u) sq[u] += abs2(a[q].v[u]);
+        }
+      if (!INIT && sizeof(S) == 4 && (++n & 7) == 0) {
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) {
+          acc_add(tot[u], sq[u]);
+          sq[u] = 0;
+        }
+      }
+    }
+  }
+  if (!INIT && norm) {
+    S v[VEC];
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) {
+      acc_add(tot[u], sq[u]);
+      if constexpr (sizeof(S) == 4) v[u] = tot[u].h + tot[u].l;   // one rounding to the lane precision
+      else v[u] = tot[u];
+    }
+    // |w|^2 is real for complex data too: one scalar per column
+    block_sum<typename real_of<T>::type, VEC>(v, red, red2, k, slots, live, norm + (size_t)blockIdx.x * k);
+  }
+}
+
+static const int AXPY_SMEM = 32 * 1024;
+
+int multiaxpy_norm_parts(size_t rows, int k) {
+  const size_t per = std::max<size_t>(1, (size_t)DT * 4 / std::max(k, 1));
+  return (int)std::min<size_t>(AXPY_PARTS, std::max<size_t>(1, (rows + per - 1) / per));
+}
+
+namespace {
+
+template <class T, class H>
+int axpy_all(void *w, const void *v0, const void *V, size_t vstride, int nvec, const void *h, double sign, size_t rows,
+             int k, bool init, void *norm, cudaStream_t s) {
+  constexpr int VW = 16 / (int)sizeof(T);
+  typedef typename lane_of<T>::A A;
+  const bool packed = VW > 1 && packs_ok<T>(k, {w, v0, V}) && vstride % VW == 0;
+  if ((packed ? k / VW : k) > DT) throw cuda_error{cudaErrorInvalidValue, "multiaxpy: more column groups than threads"};
+  int group = std::min(DOT_MAXV, AXPY_SMEM / (k * (int)sizeof(T)));
+  if (group < 1) group = 1;
+  const int parts = multiaxpy_norm_parts(rows, k);
+  int passes = 0;
+  for (int i0 = 0; i0 < nvec; i0 += group) {
+    VecList<T> L;
+    const int nv = std::min(nvec - i0, group);
+    for (int i = 0; i < DOT_MAXV; ++i) {
+      const int id = i0 + std::min(i, nv - 1);
+      L.v[i] = id == 0 ? (const T *)v0 : (const T *)V + (size_t)id * vstride;
+    }
+    const bool first = init && i0 == 0, last = i0 + nv >= nvec;
+    const size_t smem = (size_t)nv * k * sizeof(T);
+    auto go = [&](auto vec, auto ini) {
+      k_axpy<T, H, decltype(vec)::value, decltype(ini)::value><<<parts, DT, smem, s>>>(
+          (T *)w, L, nv, (const H *)h + (size_t)i0 * k, k, sign, rows, k, last ? (A *)norm : nullptr);
+    };
+    if (packed && first) go(std::integral_constant<int, VW>(), std::true_type());
+    else if (packed) go(std::integral_constant<int, VW>(), std::false_type());
+    else if (first) go(std::integral_constant<int, 1>(), std::true_type());
+    else go(std::integral_constant<int, 1>(), std::false_type());
+    MLMC_LAUNCH_CHECK("k_axpy");
+    ++passes;
+  }
+  return passes;
+}
+
+}  // namespace
+
+void launch_multiaxpy(DType t, void *w, const void *V, size_t vstride, int nvec, const void *h, double sign,
+                      size_t rows, int k, bool init, cudaStream_t s) {
+  if (nvec <= 0) return;
+  MLMC_DISPATCH(t, T, axpy_all<T, typename acc_of<T>::type>(w, V, V, vstride, nvec, h, sign, rows, k, init, nullptr, s));
+}
+
+// ------------------------------------------------------------------ fixed-length FGMRES, per column
+// The solver keeps its basis unnormalised: u_0 = b, A z_j = sum_{i <= j} c_ij u_i + u_{j+1} with
+// c_ij = d_ij / n_i, d_ij = u_i^* A z_j, n_i = |u_i|^2.  k_fgmres_mid turns step j's partial dot
+// products into the coefficients -c_ij of the multi-AXPY; k_fgmres_tail does the last step's
+// and then solves min || s_0 e_1 - G y ||, G_ij = d_ij / s_i (i <= j), G_{j+1,j} = s_{j+1}, with
+// s_i = sqrt(n_i), by Givens rotations; x = sum_j y_j z_j.  The norm of the last residual
+// vector u_m is needed only inside G, so it is taken as n_m = |w|^2 - sum_i |d_i|^2 / n_i
+// (w = A z_{m-1}) and u_m is never formed: a relative error eps in the dot products enters
+// R_mm^2 as eps |w|^2, the size of the other entries' errors.
+// Columns whose right-hand side is zero or not finite, and columns that break down (a zero
+// new vector or a zero pivot), stop there: their later y are zero.
+// Both kernels give a block a few columns and let all its threads add the parts (latency-
+// bound); a tile is 8 (FP32 data) or 4 scalars wide, since the FP64 additions of one block's
+// share would otherwise take longer than its loads.  Per step they stand in place of two
+// reductions of one warp per output (4.7 us each, strided loads), a cleared counter and a
+// per-column Givens kernel (4.7 us, 9 us complex; a 4-byte memset node costs 4 us and the
+// kernel after it 5 us of gap in a replayed graph): k_fgmres_mid takes 3.4 us.
+namespace {
+
+template <class T> struct fg {
+  typedef typename lane_of<T>::A A;
+  typedef typename acc_of<T>::type H;
+  static constexpr int C = lane_of<T>::C;
+  static constexpr int ET = sizeof(A) == 8 && sizeof(typename lane_of<T>::S) == 4 ? 8 : 4;   // scalars per tile
+  static constexpr int CB = ET / C;                                                          // columns per tile
+  static constexpr int SL = RT / ET;                                                         // part slices
+  static constexpr int MAXROWS = 34;                                                         // 32 steps, v0.v0, w.w
+};
+
+// sums[r * ET + e] (r < nrows, e < ET) = scalar e0 + e of output row r summed over the parts in
+// fixed order; parts are nrows * E scalars apart, rows E.  red: TR * RT sums.
+constexpr int TR = 8;              // rows whose loads are in flight together
+template <class T>
+__device__ void tile_sum(const typename lane_of<T>::A *__restrict__ partial, int nparts, int nrows, int E, int e0,
+                         typename lane_of<T>::A *red, double *sums) {
+  typedef typename lane_of<T>::A A;
+  constexpr int ET = fg<T>::ET, SL = fg<T>::SL;
+  const int e = threadIdx.x % ET, sl = threadIdx.x / ET;
+  const size_t stride = (size_t)nrows * E;
+  for (int r0 = 0; r0 < nrows; r0 += TR) {
+    const int nr = min(nrows - r0, TR);
+    A a[TR];
+#pragma unroll
+    for (int r = 0; r < TR; ++r) acc_zero(a[r]);
+    if (e0 + e < E) {
+      const A *src = partial + (size_t)r0 * E + e0 + e;
+#pragma unroll 2
+      for (int p = sl; p < nparts; p += SL) {
+        A v[TR];
+#pragma unroll
+        for (int r = 0; r < TR; ++r)
+          if (r < nr) v[r] = src[p * stride + (size_t)r * E];
+#pragma unroll
+        for (int r = 0; r < TR; ++r)
+          if (r < nr) acc_add(a[r], v[r]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < TR; ++r)
+      if (r < nr) red[(r * SL + sl) * ET + e] = a[r];
+    __syncthreads();
+    // eight threads per sum take the slices q, q + 8, ...; then one adds the eight
+    for (int t = threadIdx.x; t < nr * ET * 8; t += RT) {
+      const int q = t & 7, re = t >> 3, r = re / ET, ee = re % ET;
+      A v = red[(r * SL + q) * ET + ee];
+      for (int s2 = q + 8; s2 < SL; s2 += 8) acc_add(v, red[(r * SL + s2) * ET + ee]);
+      red[(r * SL + q) * ET + ee] = v;
+    }
+    __syncthreads();
+    for (int re = threadIdx.x; re < nr * ET; re += RT) {
+      const int r = re / ET, ee = re % ET;
+      A v = red[(r * SL) * ET + ee];
+      for (int q = 1; q < 8; ++q) acc_add(v, red[(r * SL + q) * ET + ee]);
+      sums[(r0 + r) * ET + ee] = acc_value(v);
+    }
+    __syncthreads();
+  }
+}
+
+__device__ __forceinline__ double usable(double n) { return n > 0.0 && isfinite(n) ? n : 1.0; }
+
+__device__ __forceinline__ double at(const double *s, int c, double) { return s[c]; }
+__device__ __forceinline__ cdouble at(const double *s, int c, cdouble) { return {s[2 * c], s[2 * c + 1]}; }
+__device__ __forceinline__ double shfl(double v, int l) { return __shfl_sync(0xffffffffu, v, l); }
+__device__ __forceinline__ cdouble shfl(cdouble v, int l) { return {shfl(v.re, l), shfl(v.im, l)}; }
+
+}  // namespace
+
+// The tile's sums for step j: dots (rows d_0 .. d_j, then v0.v0 when j = 0, then extra rows)
+// into sums, and n_j into n2[j] (global) and nj[c] (shared).
+template <class T>
+__device__ void fgmres_sums(const typename lane_of<T>::A *partial, int nparts, int nrows,
+                            const typename lane_of<T>::A *norm, int norm_parts, int j, int k, int c0, double *n2,
+                            typename lane_of<T>::A *red, double *sums, double *nsum, double *nj) {
+  constexpr int C = fg<T>::C, ET = fg<T>::ET, CB = fg<T>::CB;
+  typedef typename real_of<T>::type R;
+  // a real tile of ET scalars covers this tile's CB columns (complex: also the next tile's)
+  if (j > 0) tile_sum<R>(norm, norm_parts, 1, k, c0, red, nsum);
+  tile_sum<T>(partial, nparts, nrows, k * C, c0 * C, red, sums);
+  if (threadIdx.x < CB) {
+    const int c = threadIdx.x;
+    const double n = j > 0 ? nsum[c] : sums[ET + c * C];
+    nj[c] = n;
+    if (c0 + c < k) n2[(size_t)j * k + c0 + c] = n;
+  }
+  __syncthreads();
+}
+
+// D[(j * (m + 1) + i) * k + c] = d_ij, coef[i * k + c] = -d_ij / n_i for the multi-AXPY of step j.
+template <class T>
+__global__ void __launch_bounds__(RT) k_fgmres_mid(const typename lane_of<T>::A *__restrict__ partial, int nparts,
+                                                   int nrows, const typename lane_of<T>::A *__restrict__ norm,
+                                                   int norm_parts, int j, int m, int k, double *__restrict__ n2,
+                                                   typename acc_of<T>::type *__restrict__ D, T *__restrict__ coef) {
+  typedef typename acc_of<T>::type H;
+  constexpr int ET = fg<T>::ET, CB = fg<T>::CB;
+  __shared__ typename lane_of<T>::A red[TR * RT];
+  __shared__ double sums[fg<T>::MAXROWS * ET], nsum[8], nj[8];
+  const int c0 = blockIdx.x * CB;
+  fgmres_sums<T>(partial, nparts, nrows, norm, norm_parts, j, k, c0, n2, red, sums, nsum, nj);
+  for (int t = threadIdx.x; t < (j + 1) * CB; t += RT) {
+    const int i = t / CB, c = t - i * CB;
+    if (c0 + c >= k) continue;
+    const double n = usable(i == j ? nj[c] : n2[(size_t)i * k + c0 + c]);
+    const H d = at(sums + i * ET, c, H());
+    D[((size_t)j * (m + 1) + i) * k + c0 + c] = d;
+    coef[(size_t)i * k + c0 + c] = cvt<T, H>(rmul(-1.0 / n, d));
+  }
+}
+
+// The last step, j = its - 1, and the least-squares problem: y[i * k + c], i < its.
+// One warp per column; lane q keeps column q of G.
+template <class T>
+__global__ void __launch_bounds__(RT) k_fgmres_tail(const typename lane_of<T>::A *__restrict__ partial, int nparts,
+                                                    int nrows, const typename lane_of<T>::A *__restrict__ norm,
+                                                    int norm_parts, int its, int m, int k, double *__restrict__ n2,
+                                                    const typename acc_of<T>::type *__restrict__ D,
+                                                    T *__restrict__ y) {
+  typedef typename acc_of<T>::type H;
+  constexpr int ET = fg<T>::ET, CB = fg<T>::CB, C = fg<T>::C;
+  __shared__ typename lane_of<T>::A red[TR * RT];
+  __shared__ double sums[fg<T>::MAXROWS * ET], nsum[8], nj[8];
+  __shared__ double sn[CB][33], is[CB][33];
+  extern __shared__ __align__(16) unsigned char tail_smem[];
+  const int c0 = blockIdx.x * CB, j = its - 1;
+  fgmres_sums<T>(partial, nparts, nrows, norm, norm_parts, j, k, c0, n2, red, sums, nsum, nj);
+  const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (c >= CB || c0 + c >= k) return;
+  H *G = (H *)tail_smem + (size_t)c * (its + 1) * its;      // G[i * its + q]
+  const size_t cg = c0 + c;
+  // norms s_i = sqrt(n_i): zero for a vanished vector, whose 1 / s_i is 1
+  for (int i = lane; i <= its; i += 32) {
+    double n;
+    if (i == its) {
+      n = sums[(nrows - 1) * ET + c * C];                   // |w|^2
+      for (int l = 0; l < its; ++l) {
+        const H d = at(sums + l * ET, c, H());
+        n -= abs2(d) / usable(l == j ? nj[c] : n2[(size_t)l * k + cg]);
+      }
+    } else {
+      n = i == j ? nj[c] : n2[(size_t)i * k + cg];
+    }
+    const double inv = rsqrt(usable(n));
+    is[c][i] = inv;
+    sn[c][i] = n > 0.0 && isfinite(n) ? n * inv : 0.0;
+  }
+  __syncwarp();
+  if (lane < its) {
+    for (int i = 0; i <= lane; ++i) {
+      const H d = lane == j ? at(sums + i * ET, c, H()) : D[((size_t)lane * (m + 1) + i) * k + cg];
+      G[i * its + lane] = rmul(is[c][i], d);
+    }
+    G[(lane + 1) * its + lane] = make<H>(sn[c][lane + 1], 0.0);
+  }
+  __syncwarp();
+  H g = make<H>(sn[c][0], 0.0), gi = zero<H>();             // lane i keeps entry i of the rotated right-hand side
+  double inv = 0.0;                                         // and 1 / R_ii
+  bool active = sn[c][0] > 0.0;
+  int J = 0;
+  for (int i = 0; i < its && active; ++i) {
+    const H a = G[i * its + i];
+    const double b = sn[c][i + 1], r2 = abs2(a) + b * b;
+    if (!(r2 > 0.0)) break;
+    const double ir = rsqrt(r2);
+    const H cc = rmul(ir, a);
+    const double ss = b * ir;
+    if (lane > i && lane < its) {
+      const H u = G[i * its + lane], v = G[(i + 1) * its + lane];
+      G[i * its + lane] = conj(cc) * u + rmul(ss, v);
+      G[(i + 1) * its + lane] = cc * v - rmul(ss, u);
+    }
+    if (lane == i) {
+      gi = conj(cc) * g;
+      inv = ir;
+    }
+    g = rmul(-ss, g);
+    J = i + 1;
+    active = b > 0.0;
+    __syncwarp();
+  }
+  for (int l = J - 1; l >= 0; --l) {
+    H yl = rmul(inv, gi);
+    yl = shfl(yl, l);
+    if (lane < l) gi = gi - G[lane * its + l] * yl;
+    if (lane == l) gi = yl;
+  }
+  if (lane < its) y[(size_t)lane * k + cg] = cvt<T, H>(lane < J ? gi : zero<H>());
+}
+
+// Step j's partial dots of w against u_0 = b, u_1 .. u_j (V + i * vstride), with b.b on the first
+// step and w.w on the last.
+int launch_fgmres_dots(DType t, const void *b, const void *V, size_t vstride, int j, int its, const void *w, size_t rows,
+                       int k, void *partials, cudaStream_t s) {
+  const int extra = (j == 0 ? 2 : 0) | (j == its - 1 ? 1 : 0);
+  int passes = 0;
+  MLMC_DISPATCH(t, T, passes = dots_partial<T>(b, V, vstride, j + 1, w, rows, k, partials, multidot_parts(t, rows, k),
+                                               extra, s));
+  return passes;
+}
+
+void launch_fgmres_mid(DType t, const void *partials, const void *norm, int j, int m, size_t rows, int k, double *n2,
+                       void *D, void *coef, cudaStream_t s) {
+  const int nparts = multidot_parts(t, rows, k), nnorm = multiaxpy_norm_parts(rows, k);
+  MLMC_DISPATCH(t, T, {
+    typedef typename lane_of<T>::A A;
+    typedef typename acc_of<T>::type H;
+    k_fgmres_mid<T><<<(k + fg<T>::CB - 1) / fg<T>::CB, RT, 0, s>>>((const A *)partials, nparts, j + 1 + (j == 0),
+                                                                  (const A *)norm, nnorm, j, m, k, n2, (H *)D,
+                                                                  (T *)coef);
+  });
+  MLMC_LAUNCH_CHECK("k_fgmres_mid");
+}
+
+void launch_fgmres_tail(DType t, const void *partials, const void *norm, int its, int m, size_t rows, int k,
+                        double *n2, const void *D, void *y, cudaStream_t s) {
+  const int nparts = multidot_parts(t, rows, k), nnorm = multiaxpy_norm_parts(rows, k);
+  MLMC_DISPATCH(t, T, {
+    typedef typename lane_of<T>::A A;
+    typedef typename acc_of<T>::type H;
+    auto bytes = [](int n) { return (size_t)fg<T>::CB * (n + 1) * n * sizeof(H); };
+    int dev = 0;
+    MLMC_CUDA(cudaGetDevice(&dev));
+    // the longest solve (32 steps) sets the limit once per device: every later value is smaller
+    static std::once_flag once[64];
+    std::call_once(once[dev & 63], [&] {
+      check_cuda(cudaFuncSetAttribute(k_fgmres_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(32)),
+                 "cudaFuncSetAttribute(k_fgmres_tail)");
+    });
+    k_fgmres_tail<T><<<(k + fg<T>::CB - 1) / fg<T>::CB, RT, bytes(its), s>>>(
+        (const A *)partials, nparts, its + 1 + (its == 1), (const A *)norm, nnorm, its, m, k, n2, (const H *)D, (T *)y);
+  });
+  MLMC_LAUNCH_CHECK("k_fgmres_tail");
+}
+
+// w += sum_v u_v coef[v][c] (u_0 = b, then V + v * vstride), with the partial column norms of the result
+int launch_fgmres_axpy(DType t, void *w, const void *b, const void *V, size_t vstride, int nvec, const void *coef,
+                       size_t rows, int k, void *norm, cudaStream_t s) {
+  int passes = 0;
+  MLMC_DISPATCH(t, T, passes = (axpy_all<T, T>(w, b, V, vstride, nvec, coef, 1.0, rows, k, false, norm, s)));
+  return passes;
+}
+
+// x = sum_v Z_v y[v][c]
+int launch_fgmres_update(DType t, void *x, const void *Z, size_t vstride, int nvec, const void *y, size_t rows, int k,
+                         cudaStream_t s) {
+  int passes = 0;
+  MLMC_DISPATCH(t, T, passes = (axpy_all<T, T>(x, Z, Z, vstride, nvec, y, 1.0, rows, k, true, nullptr, s)));
+  return passes;
+}
+
+}  // namespace mlmc

@@ -1,8 +1,7 @@
-// Per-column kernels of the batched flexible GMRES (Saad, Alg. 9.6): every
+// Per-column kernels of the restarted flexible GMRES (Saad, Alg. 9.6): every
 // column of a vector block is an independent system, and its small Hessenberg
 // least-squares problem (Givens rotations, triangular solve) is handled by one
-// thread in FP64, as are the coefficient rescalings of the fixed-length FGMRES that
-// keeps its basis unnormalised.  Also: sample combination and accumulation (Secs. 2-3), the
+// thread in FP64.  Also: sample combination and accumulation (Secs. 2-3), the
 // fine-operator builders (Examples 5.1 and 5.3) and a dense scatter of the
 // coarsest operator.
 #include "mlmc_internal.cuh"
@@ -21,11 +20,11 @@ template <> __device__ inline cdouble hdiv<cdouble>(cdouble a, cdouble b) {
 }
 template <class H> __device__ inline H hreal(double v) { return make<H>(v, 0.0); }
 
-// sc (optional): norms s_i of the unnormalised basis vectors of the fixed-length
-// variant (see k_multidot_reduce); s_0 = |b|.
+// active[c]: 1 while column c is iterated, 0 when it is done, -1 when its residual norm is not
+// finite.
 template <class H>
 __global__ void k_arnoldi_init(H *g, double *bnorm, double *invnrm, int *active, int *jdone, int k,
-                               double tol, int first, int *nactive, double *sc) {
+                               double tol, int first) {
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= k) return;
   const double g0 = creal_(g[c]);
@@ -35,77 +34,51 @@ __global__ void k_arnoldi_init(H *g, double *bnorm, double *invnrm, int *active,
   g[c] = hreal<H>(beta);
   jdone[c] = 0;
   int a = finite && beta > 0.0 && beta > tol * bnorm[c];
-  active[c] = a;
+  active[c] = finite ? a : -1;
   invnrm[c] = a ? 1.0 / beta : 0.0;
-  if (sc) sc[c] = beta > 0.0 ? beta : 1.0;
-  if (a) atomicAdd(nactive, 1);
-  else if (!finite) atomicAdd(nactive, NONFINITE_COLUMN);    // a residual that is NaN or infinite
-}
-
-// y_i /= s_i for the computed rows: x = sum_i z_i y_i with z_i built from u_i.
-template <class H>
-__global__ void k_lazy_y(H *y, const double *sc, const int *jdone, int m, int k) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= m * k) return;
-  const int i = t / k, c = t - (t / k) * k;
-  if (i < jdone[c]) y[t] = y[t] * hreal<H>(1.0 / sc[t]);
 }
 
 // Hessenberg column j of column c lives at H[(j*(m+1) + i)*k + c], i = 0..j+1.
-// On entry H[j][j+1] holds |w|^2 from a column dot.
-// sc (optional, the unnormalised variant): the new basis vector keeps its norm,
-// s_{j+1} = |u_{j+1}|, and the Hessenberg entry is |u_{j+1}| / s_j.
+// On entry H[j][j+1] holds |w|^2 from a column dot.  One thread per column in blocks of one
+// warp: FP64 runs at two operations per clock and SM, so the columns are spread over SMs, and
+// the square roots and quotients of a step are two reciprocal square roots.
 template <class H>
 __global__ void k_arnoldi_step(H *Hm, H *cs, H *sn, H *g, int j, int m, int k, int *active, int *jdone,
-                               const double *bnorm, double tol, double *invnrm, double *resid, int *nactive,
-                               int fixed, double *sc) {
+                               const double *bnorm, double tol, double *invnrm, double *resid) {
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= k) return;
   H *h = Hm + (size_t)j * (m + 1) * k + c;
-  if (!active[c]) {
+  if (active[c] <= 0) {
     invnrm[c] = 0.0;
-    if (sc) sc[(size_t)(j + 1) * k + c] = 1.0;   // its vectors are zero: any finite scale
     return;
   }
-  double nrm = sqrt(fmax(creal_(h[(size_t)(j + 1) * k]), 0.0));
-  invnrm[c] = nrm > 0.0 ? 1.0 / nrm : 0.0;
-  if (sc) {
-    sc[(size_t)(j + 1) * k + c] = nrm > 0.0 ? nrm : 1.0;
-    nrm = nrm / sc[(size_t)j * k + c];
-  }
-  h[(size_t)(j + 1) * k] = hreal<H>(nrm);
+  const double n2 = creal_(h[(size_t)(j + 1) * k]);
+  const double inv = n2 > 0.0 ? rsqrt(n2) : 0.0;
+  const double nrm = n2 > 0.0 ? n2 * inv : 0.0;
+  invnrm[c] = inv;
+  H a = h[0];
   for (int i = 0; i < j; ++i) {
-    H a = h[(size_t)i * k], b = h[(size_t)(i + 1) * k];
-    H ci = cs[(size_t)i * k + c], si = sn[(size_t)i * k + c];
+    const H b = h[(size_t)(i + 1) * k];
+    const H ci = cs[(size_t)i * k + c], si = sn[(size_t)i * k + c];
     h[(size_t)i * k] = conj(ci) * a + conj(si) * b;
-    h[(size_t)(i + 1) * k] = -(si * a) + ci * b;
+    a = -(si * a) + ci * b;
   }
-  H a = h[(size_t)j * k], b = h[(size_t)(j + 1) * k];
-  double den = sqrt(cabs_(a) * cabs_(a) + cabs_(b) * cabs_(b));
-  H cj, sj;
-  if (den > 0.0) {
-    cj = hdiv(a, hreal<H>(den));
-    sj = hdiv(b, hreal<H>(den));
-  } else {
-    cj = hreal<H>(1.0);
-    sj = hreal<H>(0.0);
-  }
+  const double r2 = abs2(a) + (n2 > 0.0 ? n2 : 0.0);
+  const double ir = r2 > 0.0 ? rsqrt(r2) : 0.0;
+  const H cj = r2 > 0.0 ? rmul(ir, a) : hreal<H>(1.0), sj = hreal<H>(nrm * ir);
   cs[(size_t)j * k + c] = cj;
   sn[(size_t)j * k + c] = sj;
-  h[(size_t)j * k] = hreal<H>(den);
+  h[(size_t)j * k] = hreal<H>(r2 * ir);
   h[(size_t)(j + 1) * k] = hreal<H>(0.0);
-  H gj = g[(size_t)j * k + c];
-  g[(size_t)(j + 1) * k + c] = -(sj * gj);
+  const H gj = g[(size_t)j * k + c], gn = -(sj * gj);
+  g[(size_t)(j + 1) * k + c] = gn;
   g[(size_t)j * k + c] = conj(cj) * gj;
   jdone[c] = j + 1;
-  double r = cabs_(g[(size_t)(j + 1) * k + c]);
+  const double r = cabs_(gn);
   resid[c] = r;
-  bool still = fixed ? (nrm > 0.0 && den > 0.0) : (r > tol * bnorm[c] && den > 0.0 && nrm > 0.0);
-  if (!still) {
+  if (!(r > tol * bnorm[c] && r2 > 0.0 && n2 > 0.0)) {
     active[c] = 0;
     invnrm[c] = 0.0;
-  } else {
-    atomicAdd(nactive, 1);
   }
 }
 
@@ -133,37 +106,27 @@ __global__ void k_add_acc(H *dst, const H *src, int count) {
 }
 
 void launch_arnoldi_init(int hc, void *g, double *bnorm, double *invnrm, int *active, int *jdone, int k,
-                         double tol, int first, int *nactive, cudaStream_t s, double *sc) {
-  unsigned gr = (k + 63) / 64;
-  if (hc) k_arnoldi_init<cdouble><<<gr, 64, 0, s>>>((cdouble *)g, bnorm, invnrm, active, jdone, k, tol, first, nactive,
-                                                     sc);
-  else k_arnoldi_init<double><<<gr, 64, 0, s>>>((double *)g, bnorm, invnrm, active, jdone, k, tol, first, nactive, sc);
+                         double tol, int first, cudaStream_t s) {
+  unsigned gr = (k + 31) / 32;
+  if (hc) k_arnoldi_init<cdouble><<<gr, 32, 0, s>>>((cdouble *)g, bnorm, invnrm, active, jdone, k, tol, first);
+  else k_arnoldi_init<double><<<gr, 32, 0, s>>>((double *)g, bnorm, invnrm, active, jdone, k, tol, first);
   MLMC_LAUNCH_CHECK("k_arnoldi_init");
 }
 
-
-void launch_lazy_y(int hc, void *y, const double *sc, const int *jdone, int m, int k, cudaStream_t s) {
-  unsigned gr = (m * k + 127) / 128;
-  if (hc) k_lazy_y<cdouble><<<gr, 128, 0, s>>>((cdouble *)y, sc, jdone, m, k);
-  else k_lazy_y<double><<<gr, 128, 0, s>>>((double *)y, sc, jdone, m, k);
-  MLMC_LAUNCH_CHECK("k_lazy_y");
-}
-
 void launch_arnoldi_step(int hc, void *H, void *cs, void *sn, void *g, int j, int m, int k, int *active,
-                         int *jdone, const double *bnorm, double tol, double *invnrm, double *resid,
-                         int *nactive, int fixed, cudaStream_t s, double *sc) {
-  unsigned gr = (k + 63) / 64;
-  if (hc) k_arnoldi_step<cdouble><<<gr, 64, 0, s>>>((cdouble *)H, (cdouble *)cs, (cdouble *)sn, (cdouble *)g, j, m, k,
-                                                     active, jdone, bnorm, tol, invnrm, resid, nactive, fixed, sc);
-  else k_arnoldi_step<double><<<gr, 64, 0, s>>>((double *)H, (double *)cs, (double *)sn, (double *)g, j, m, k,
-                                                 active, jdone, bnorm, tol, invnrm, resid, nactive, fixed, sc);
+                         int *jdone, const double *bnorm, double tol, double *invnrm, double *resid, cudaStream_t s) {
+  unsigned gr = (k + 31) / 32;
+  if (hc) k_arnoldi_step<cdouble><<<gr, 32, 0, s>>>((cdouble *)H, (cdouble *)cs, (cdouble *)sn, (cdouble *)g, j, m, k,
+                                                     active, jdone, bnorm, tol, invnrm, resid);
+  else k_arnoldi_step<double><<<gr, 32, 0, s>>>((double *)H, (double *)cs, (double *)sn, (double *)g, j, m, k,
+                                                 active, jdone, bnorm, tol, invnrm, resid);
   MLMC_LAUNCH_CHECK("k_arnoldi_step");
 }
 
 void launch_trisolve(int hc, const void *H, const void *g, void *y, const int *jdone, int m, int k, cudaStream_t s) {
-  unsigned gr = (k + 63) / 64;
-  if (hc) k_trisolve<cdouble><<<gr, 64, 0, s>>>((const cdouble *)H, (const cdouble *)g, (cdouble *)y, jdone, m, k);
-  else k_trisolve<double><<<gr, 64, 0, s>>>((const double *)H, (const double *)g, (double *)y, jdone, m, k);
+  unsigned gr = (k + 31) / 32;
+  if (hc) k_trisolve<cdouble><<<gr, 32, 0, s>>>((const cdouble *)H, (const cdouble *)g, (cdouble *)y, jdone, m, k);
+  else k_trisolve<double><<<gr, 32, 0, s>>>((const double *)H, (const double *)g, (double *)y, jdone, m, k);
   MLMC_LAUNCH_CHECK("k_trisolve");
 }
 

@@ -89,9 +89,10 @@ struct Krylov {
   int hc = 0;               // complex Hessenberg data
   size_t n = 0;
   int k = 0, m = 0;
-  DevBuf V, Z, partials, H, cs, sn, g, y, h2, bnorm, invnrm, resid, active, jdone, nactive;
-  DevBuf sc, hco;           // fixed-length variant: basis-vector norms, Gram-Schmidt coefficients
-  int h_nactive = 0;         // host copy of the active-column count (pageable: the copy waits for it)
+  DevBuf V, Z, partials, H, y;
+  DevBuf cs, sn, g, h2, bnorm, invnrm, resid, active, jdone;   // restarted solves
+  std::vector<int> h_active;                                   // host copy of `active`
+  DevBuf norm, n2, coef;    // fixed-length solves: partial norms, basis norms, multi-AXPY coefficients
 };
 
 struct CycleBufs {
@@ -209,7 +210,9 @@ ProlongView pview(const H_t &h, int l, int lo) {
   return v;
 }
 
-void alloc_krylov(H_t &h, Krylov &K, DType t, size_t n, int k, int m) {
+// Restarted solves keep V_0 .. V_m; fixed-length ones use the right-hand side as u_0 and keep
+// u_1 .. u_m (the last slot holds A z of the last step).
+void alloc_krylov(H_t &h, Krylov &K, DType t, size_t n, int k, int m, bool fixed) {
   K.t = t;
   K.hc = dtype_complex(t);
   K.n = n;
@@ -217,30 +220,46 @@ void alloc_krylov(H_t &h, Krylov &K, DType t, size_t n, int k, int m) {
   K.m = m;
   size_t blk = n * (size_t)k * dtype_size(t);
   size_t as = acc_size(h);
-  K.V.alloc(blk * (m + 1));
+  K.V.alloc(blk * (fixed ? m : m + 1));
   K.Z.alloc(blk * m);
-  // multi-dot partials of up to m + 1 vectors, or the multi-AXPY's fused column norms
-  K.partials.alloc(std::max((size_t)multidot_parts(n, k) * (m + 1), (size_t)multiaxpy_norm_parts(n, k)) * k * as);
+  // a solve may be narrower than k; the part counts fall with the width, their products with it grow
+  size_t dots = 0, norms = 0;
+  for (int kk = 1; kk <= k; ++kk) {
+    dots = std::max(dots, (size_t)multidot_parts(t, n, kk) * kk);
+    norms = std::max(norms, (size_t)multiaxpy_norm_parts(n, kk) * kk);
+  }
+  K.partials.alloc(dots * (m + 2) * as);
   K.H.alloc((size_t)m * (m + 1) * k * as);
+  K.y.alloc((size_t)m * k * as);
+  if (fixed) {
+    K.norm.alloc(norms * as);
+    K.n2.alloc((size_t)m * k * sizeof(double));
+    K.coef.alloc((size_t)m * k * dtype_size(t));
+    return;
+  }
   K.cs.alloc((size_t)m * k * as);
   K.sn.alloc((size_t)m * k * as);
   K.g.alloc((size_t)(m + 1) * k * as);
-  K.y.alloc((size_t)m * k * as);
   K.h2.alloc((size_t)(m + 1) * k * as);
   K.bnorm.alloc(k * sizeof(double));
   K.invnrm.alloc(k * sizeof(double));
   K.resid.alloc(k * sizeof(double));
   K.active.alloc(k * sizeof(int));
   K.jdone.alloc(k * sizeof(int));
-  K.nactive.alloc(sizeof(int));
-  K.sc.alloc((size_t)(m + 1) * k * sizeof(double));
-  K.hco.alloc((size_t)(m + 1) * k * as);
+  K.h_active.resize(k);
 }
 
-int read_nactive(H_t &h, Krylov &K) {
-  check_cuda(cudaMemcpyAsync(&K.h_nactive, K.nactive.p, sizeof(int), cudaMemcpyDeviceToHost, h.stream), "D2H nactive");
+// Number of columns still iterated, or -1 when a column's residual is not finite.
+int read_nactive(H_t &h, Krylov &K, int k) {
+  check_cuda(cudaMemcpyAsync(K.h_active.data(), K.active.p, k * sizeof(int), cudaMemcpyDeviceToHost, h.stream),
+             "D2H active");
   check_cuda(cudaStreamSynchronize(h.stream), "sync");
-  return K.h_nactive;
+  int n = 0;
+  for (int c = 0; c < k; ++c) {
+    if (K.h_active[c] < 0) return -1;
+    n += K.h_active[c];
+  }
+  return n;
 }
 
 // Number of (site, coupled site) pairs of a nearest-neighbour stencil on an
@@ -321,119 +340,102 @@ void dense_apply(H_t &h, int lo, const void *b, void *x, int k) {
   h.cost += (double)C.n * C.n * k;
 }
 
-void multidot(H_t &h, Krylov &K, const void *V, int nvec, const void *w, int k, void *out,
-              const double *lazy_sc = nullptr, void *lazy_coef = nullptr, int lazy_j = 0) {
-  launch_multidot(K.t, V, K.n * (size_t)k, nvec, w, K.n, k, K.partials.p, multidot_parts(K.n, k), out,
-                  K.hc ? C64 : F64, h.stream, lazy_sc, lazy_coef, lazy_j);
+void multidot(H_t &h, Krylov &K, const void *V, int nvec, const void *w, int k, void *out) {
+  launch_multidot(K.t, V, K.n * (size_t)k, nvec, w, K.n, k, K.partials.p, multidot_parts(K.t, K.n, k), out, h.stream);
   h.launches += 2;
 }
 
 using Precond = std::function<void(const void *, void *)>;
 
-// Batched flexible GMRES(m) (Saad, Alg. 9.6) on level l with element type K.t.
-// fixed_its > 0: exactly that many steps from x0 = 0, no host synchronisation
-// (K-cycle coarse correction).  Otherwise restarts from the true residual
-// until every column meets ||b - A x|| <= tol ||b|| or max_iter is reached.
-// Returns the number of iterations.
-int fgmres(H_t &h, Krylov &K, int l, int lo, const void *b, void *x, int k, double tol, int fixed_its,
-           int maxit, const Precond &M, bool reorth, bool *converged) {
+// `its` steps of flexible GMRES from x = 0 (the inner solve and the K-cycle's coarse
+// correction), on level l with element type K.t, without host synchronisation.  The basis stays
+// unnormalised (kernels_dots.cu); u_0 is b itself, which M must not write.  Per step: the
+// operator, the dots, their per-column algebra and the multi-AXPY; the last step forms no new
+// basis vector and the solution is written without being cleared first.
+void fgmres_fixed(H_t &h, Krylov &K, int l, int lo, const void *b, void *x, int k, int its, const Precond &M) {
+  const size_t es = dtype_size(K.t), blk = K.n * (size_t)k;
+  auto Uj = [&](int j) { return (char *)K.V.p + (size_t)(j - 1) * blk * es; };   // j >= 1
+  auto Zj = [&](int j) { return (char *)K.Z.p + (size_t)j * blk * es; };
+  const void *U = Uj(0);                       // u_i = U + i blocks for i >= 1; never read at 0
+  cudaStream_t s = h.stream;
+  for (int j = 0; j < its; ++j) {
+    M(j == 0 ? b : Uj(j), Zj(j));
+    void *w = Uj(j + 1);
+    apply_op(h, l, lo, Zj(j), w, k);
+    h.launches += launch_fgmres_dots(K.t, b, U, blk, j, its, w, K.n, k, K.partials.p, s);
+    if (j == its - 1) break;
+    launch_fgmres_mid(K.t, K.partials.p, K.norm.p, j, K.m, K.n, k, K.n2.as<double>(), K.H.p, K.coef.p, s);
+    h.launches += 1 + launch_fgmres_axpy(K.t, w, b, U, blk, j + 1, K.coef.p, K.n, k, K.norm.p, s);
+  }
+  launch_fgmres_tail(K.t, K.partials.p, K.norm.p, its, K.m, K.n, k, K.n2.as<double>(), K.H.p, K.y.p, s);
+  h.launches += 1 + launch_fgmres_update(K.t, x, K.Z.p, blk, its, K.y.p, K.n, k, s);
+}
+
+// Batched flexible GMRES(m) (Saad, Alg. 9.6) on level l with element type K.t: restarts
+// from the true residual until every column meets ||b - A x|| <= tol ||b|| or max_iter is
+// reached.  Returns the number of iterations.
+int fgmres(H_t &h, Krylov &K, int l, int lo, const void *b, void *x, int k, double tol, int maxit, const Precond &M,
+           bool reorth, bool *converged) {
   const size_t es = dtype_size(K.t), as = acc_size(h);
   const size_t blk = K.n * (size_t)k;
   const int m = K.m;
   auto Vj = [&](int j) { return (char *)K.V.p + (size_t)j * blk * es; };
   auto Zj = [&](int j) { return (char *)K.Z.p + (size_t)j * blk * es; };
   auto Hcol = [&](int j) { return (char *)K.H.p + (size_t)j * (m + 1) * k * as; };
-  const bool fixed = fixed_its > 0;
-  // fixed length (inner solves, K-cycle): the basis vectors stay unnormalised (no
-  // scaling pass over each new vector; see k_multidot_reduce)
-  const bool lazy = fixed && !reorth;
-  double *sc = lazy ? K.sc.as<double>() : nullptr;
   cudaStream_t s = h.stream;
 
-  check_cuda(cudaMemcpyAsync(Vj(0), b, blk * es, cudaMemcpyDeviceToDevice, s), "copy b");
-  multidot(h, K, Vj(0), 1, Vj(0), k, K.g.p);
-  check_cuda(cudaMemsetAsync(K.nactive.p, 0, sizeof(int), s), "memset");
+  multidot(h, K, b, 1, b, k, K.g.p);
   launch_arnoldi_init(K.hc, K.g.p, K.bnorm.as<double>(), K.invnrm.as<double>(), K.active.as<int>(),
-                      K.jdone.as<int>(), k, fixed ? 0.0 : tol, 1, K.nactive.as<int>(), s, sc);
+                      K.jdone.as<int>(), k, tol, 1, s);
   h.launches++;
-  check_cuda(cudaMemsetAsync(x, 0, blk * es, s), "memset x");
   if (converged) *converged = true;
-  if (!fixed) {
-    const int na = read_nactive(h, K);
-    if (na >= NONFINITE_COLUMN) {            // b is not finite: no iteration can help
-      if (converged) *converged = false;
-      return 0;
-    }
-    if (na == 0) return 0;
+  int na = read_nactive(h, K, k);
+  if (na <= 0) {
+    check_cuda(cudaMemsetAsync(x, 0, blk * es, s), "memset x");
+    if (na < 0 && converged) *converged = false;   // b is not finite: no iteration can help
+    return 0;
   }
   int its = 0;
+  const void *r = b;                               // the residual that this cycle starts from
   for (;;) {
-    if (!lazy) {
-      launch_scale_cols(K.t, Vj(0), Vj(0), K.invnrm.p, 0, K.n, k, s);
-      h.launches++;
-    }
+    launch_scale_cols(K.t, Vj(0), r, K.invnrm.p, 0, K.n, k, s);
+    h.launches++;
+    const bool x_zero = its == 0;
     int jlast = 0;
     for (int j = 0; j < m; ++j) {
       M(Vj(j), Zj(j));
       apply_op(h, l, lo, Zj(j), Vj(j + 1), k);
-      // unnormalised basis: the reduction also forms the Hessenberg entries and the
-      // multi-AXPY's coefficients (see k_multidot_reduce)
-      multidot(h, K, K.V.p, j + 1, Vj(j + 1), k, Hcol(j), lazy ? sc : nullptr, lazy ? K.hco.p : nullptr, j);
-      // fixed length: the multi-AXPY also sums |u_{j+1}|^2 per column (no separate norm pass)
-      const int nparts = launch_multiaxpy(K.t, Vj(j + 1), K.V.p, blk, j + 1, lazy ? K.hco.p : Hcol(j),
-                                          K.hc ? C64 : F64, k, -1.0, K.n, k, s, lazy ? K.partials.p : nullptr);
+      multidot(h, K, K.V.p, j + 1, Vj(j + 1), k, Hcol(j));
+      launch_multiaxpy(K.t, Vj(j + 1), K.V.p, blk, j + 1, Hcol(j), -1.0, K.n, k, false, s);
       h.launches++;
       if (reorth) {
         multidot(h, K, K.V.p, j + 1, Vj(j + 1), k, K.h2.p);
-        launch_multiaxpy(K.t, Vj(j + 1), K.V.p, blk, j + 1, K.h2.p, K.hc ? C64 : F64, k, -1.0, K.n, k, s);
+        launch_multiaxpy(K.t, Vj(j + 1), K.V.p, blk, j + 1, K.h2.p, -1.0, K.n, k, false, s);
         launch_add_acc(K.hc, Hcol(j), K.h2.p, (j + 1) * k, s);
         h.launches += 2;
       }
-      if (lazy) {
-        launch_column_reduce(K.hc ? C64 : F64, K.partials.p, nparts, k, (char *)Hcol(j) + (size_t)(j + 1) * k * as, s);
-        h.launches++;
-      } else {
-        multidot(h, K, Vj(j + 1), 1, Vj(j + 1), k, (char *)Hcol(j) + (size_t)(j + 1) * k * as);
-      }
-      check_cuda(cudaMemsetAsync(K.nactive.p, 0, sizeof(int), s), "memset");
+      multidot(h, K, Vj(j + 1), 1, Vj(j + 1), k, (char *)Hcol(j) + (size_t)(j + 1) * k * as);
       launch_arnoldi_step(K.hc, K.H.p, K.cs.p, K.sn.p, K.g.p, j, m, k, K.active.as<int>(), K.jdone.as<int>(),
-                          K.bnorm.as<double>(), tol, K.invnrm.as<double>(), K.resid.as<double>(),
-                          K.nactive.as<int>(), fixed ? 1 : 0, s, sc);
-      h.launches++;
-      if (!lazy) {
-        launch_scale_cols(K.t, Vj(j + 1), Vj(j + 1), K.invnrm.p, 0, K.n, k, s);
-        h.launches++;
-      }
+                          K.bnorm.as<double>(), tol, K.invnrm.as<double>(), K.resid.as<double>(), s);
+      launch_scale_cols(K.t, Vj(j + 1), Vj(j + 1), K.invnrm.p, 0, K.n, k, s);
+      h.launches += 2;
       ++its;
       jlast = j + 1;
-      if (fixed) {
-        if (its >= fixed_its) break;
-        continue;
-      }
-      if (read_nactive(h, K) == 0 || its >= maxit) break;
+      if (read_nactive(h, K, k) == 0 || its >= maxit) break;
     }
     launch_trisolve(K.hc, K.H.p, K.g.p, K.y.p, K.jdone.as<int>(), m, k, s);
-    if (lazy) {
-      launch_lazy_y(K.hc, K.y.p, sc, K.jdone.as<int>(), m, k, s);
-      h.launches++;
-    }
-    launch_multiaxpy(K.t, x, K.Z.p, blk, jlast, K.y.p, K.hc ? C64 : F64, k, 1.0, K.n, k, s);
+    launch_multiaxpy(K.t, x, K.Z.p, blk, jlast, K.y.p, 1.0, K.n, k, x_zero, s);
     h.launches += 2;
-    if (fixed) return its;
     // FP64 true residual: restart, or stop when every column meets tol
     residual_op(h, l, lo, x, b, Vj(0), k);
+    r = Vj(0);
     multidot(h, K, Vj(0), 1, Vj(0), k, K.g.p);
-    check_cuda(cudaMemsetAsync(K.nactive.p, 0, sizeof(int), s), "memset");
     launch_arnoldi_init(K.hc, K.g.p, K.bnorm.as<double>(), K.invnrm.as<double>(), K.active.as<int>(),
-                        K.jdone.as<int>(), k, tol, 0, K.nactive.as<int>(), s);
+                        K.jdone.as<int>(), k, tol, 0, s);
     h.launches++;
-    const int na = read_nactive(h, K);
-    if (na >= NONFINITE_COLUMN) {            // the iterate went NaN / infinite: stop, not converged
-      if (converged) *converged = false;
-      return its;
-    }
+    na = read_nactive(h, K, k);
     if (na == 0) return its;
-    if (its >= maxit) {
+    if (na < 0 || its >= maxit) {            // na < 0: the iterate went NaN / infinite
       if (converged) *converged = false;
       return its;
     }
@@ -489,7 +491,7 @@ void cycle(H_t &h, int lo, int l, const void *b, void *x, int k) {
     cycle(h, lo, l + 1, cn.b.p, cn.x.p, k);
   } else {
     Precond M = [&h, lo, l, k](const void *v, void *z) { cycle(h, lo, l + 1, v, z, k); };
-    fgmres(h, *cn.kcyc, l + 1, lo, cn.b.p, cn.x.p, k, 0.0, h.prm.kcycle_its, h.prm.kcycle_its, M, false, nullptr);
+    fgmres_fixed(h, *cn.kcyc, l + 1, lo, cn.b.p, cn.x.p, k, h.prm.kcycle_its, M);
   }
   // the post-smoothing starts with colour 1 and does not read x there, so colour 1 needs no
   // prolongation, unless the fine-level hooks (learned correction, capture) read all of x
@@ -563,7 +565,7 @@ Precond outer_precond(H_t &h, int l, int k) {
   auto inner = [&h, l, k, lo, nin](const void *b, void *x) {
     if (nin > 0) {
       Precond M = [&h, l, k, lo](const void *v, void *z) { cycle(h, lo, l, v, z, k); };
-      fgmres(h, *h.inner[lo][l], l, lo, b, x, k, 0.0, nin, nin, M, false, nullptr);
+      fgmres_fixed(h, *h.inner[lo][l], l, lo, b, x, k, nin, M);
     } else {
       cycle(h, lo, l, b, x, k);
     }
@@ -618,12 +620,12 @@ int solve_level(H_t &h, int l, const void *b, void *x, int k, double tol, bool *
     coarse_solve(h, b, x, k);
     return 0;
   }
-  int its = fgmres(h, *h.outer[l], l, 0, b, x, k, tol, 0, h.prm.max_iter, outer_precond(h, l, k),
+  int its = fgmres(h, *h.outer[l], l, 0, b, x, k, tol, h.prm.max_iter, outer_precond(h, l, k),
                    h.prm.reorth != 0, conv);
   if (conv && !*conv && h.net_on) {
     // the plain smoother is the fallback: repeat the solve without the network
     h.net_on = 0;
-    its += fgmres(h, *h.outer[l], l, 0, b, x, k, tol, 0, h.prm.max_iter, outer_precond(h, l, k),
+    its += fgmres(h, *h.outer[l], l, 0, b, x, k, tol, h.prm.max_iter, outer_precond(h, l, k),
                   h.prm.reorth != 0, conv);
     h.net_on = 1;
     h.net_fallbacks++;
@@ -786,8 +788,8 @@ double net_loss_grad(H_t &h, const void *r, int k, bool grad, bool read_loss) {
   Krylov &K = *h.outer[0];
   const size_t as = acc_size(h);
   char *nr2 = h.lcol.as<char>(), *nt2 = nr2 + (size_t)k * as;
-  launch_multidot(h.t32, r, cnt, 1, r, F.n, k, K.partials.p, multidot_parts(F.n, k), nr2, C64, s);
-  launch_multidot(h.t32, Tt, cnt, 1, Tt, F.n, k, K.partials.p, multidot_parts(F.n, k), nt2, C64, s);
+  launch_multidot(h.t32, r, cnt, 1, r, F.n, k, K.partials.p, multidot_parts(h.t32, F.n, k), nr2, s);
+  launch_multidot(h.t32, Tt, cnt, 1, Tt, F.n, k, K.partials.p, multidot_parts(h.t32, F.n, k), nt2, s);
   h.launches += 6;
   double loss = 0.0;
   if (read_loss) {
@@ -1245,7 +1247,7 @@ void setup(H_t &h, const mlmc_operator_desc *op, const mlmc_hierarchy_params *p,
       if (l + 1 < h.L) cb.r.alloc(bytes);
       if (p->cycle == MLMC_CYCLE_K && l >= 1 && l + 1 < h.L) {
         cb.kcyc.reset(new Krylov());
-        alloc_krylov(h, *cb.kcyc, t, h.lv[l].n, kc, p->kcycle_its);
+        alloc_krylov(h, *cb.kcyc, t, h.lv[l].n, kc, p->kcycle_its, true);
       }
     }
   }
@@ -1259,19 +1261,21 @@ void setup(H_t &h, const mlmc_operator_desc *op, const mlmc_hierarchy_params *p,
     h.ys[l].alloc(h.lv[l].n * (size_t)width(l) * es);
     if (l + 1 < h.L) {
       h.outer[l].reset(new Krylov());
-      alloc_krylov(h, *h.outer[l], h.t64, h.lv[l].n, width(l), p->fgmres_restart);
+      alloc_krylov(h, *h.outer[l], h.t64, h.lv[l].n, width(l), p->fgmres_restart, false);
       if (p->inner_its > 0) {
         int lo = mixed ? 1 : 0;
         h.inner[lo].resize(h.L);
         h.inner[lo][l].reset(new Krylov());
-        alloc_krylov(h, *h.inner[lo][l], lo ? h.t32 : h.t64, h.lv[l].n, width(l), p->inner_its);
+        alloc_krylov(h, *h.inner[lo][l], lo ? h.t32 : h.t64, h.lv[l].n, width(l), p->inner_its, true);
       }
     }
   }
   (void)k;
   h.dots.alloc(2 * (size_t)h.kbig * 16);
   if (mixed) h.coarse_r.alloc(h.lv[h.L - 1].n * (size_t)std::max(h.kbig, h.wl[h.L - 1]) * dtype_size(h.t64));
-  h.dots_part.alloc((size_t)multidot_parts(h.lv[0].n, h.kbig) * h.kbig * 16);   // sample-dot partial sums
+  size_t dots = 0;                       // sample-dot partial sums of any width on any level
+  for (int kk = 1; kk <= h.kbig; ++kk) dots = std::max(dots, (size_t)multidot_parts(h.t64, h.lv[0].n, kk) * kk);
+  h.dots_part.alloc(dots * 16);
   h.samples.alloc((size_t)h.kbig * 16);
   h.acc.alloc(4 * sizeof(double));
   h.err.alloc(sizeof(int));
@@ -1357,8 +1361,8 @@ int sample_block(H_t &h, int l, int noise, uint64_t seed, uint64_t first, int k,
   int its = solve_level(h, l, h.xs[l].p, h.ys[l].p, k, tol, &c1);
   char *dxy = h.dots.as<char>(), *dzw = dxy + (size_t)k * 16;
   auto coldot = [&](int lev, const void *a, const void *b, void *out) {
-    launch_multidot(h.t64, a, h.lv[lev].n * (size_t)k, 1, b, h.lv[lev].n, k,
-                    h.dots_part.p, multidot_parts(h.lv[lev].n, k), out, h.complex_op ? C64 : F64, s);
+    launch_multidot(h.t64, a, h.lv[lev].n * (size_t)k, 1, b, h.lv[lev].n, k, h.dots_part.p,
+                    multidot_parts(h.t64, h.lv[lev].n, k), out, s);
     h.launches += 2;
   };
   coldot(l, h.xs[l].p, h.ys[l].p, dxy);
@@ -1610,10 +1614,10 @@ int mlmc_column_dots(int complex_data, const void *x, const void *y, int n, int 
     cudaStream_t s = (cudaStream_t)stream;
     g_alloc_stream = s;
     DType t = complex_data ? C64 : F64;
-    int parts = multidot_parts((size_t)n, k);
+    int parts = multidot_parts(t, (size_t)n, k);
     DevBuf part;
     part.alloc((size_t)parts * k * (complex_data ? 16 : 8));
-    launch_multidot(t, x, (size_t)n * k, 1, y, (size_t)n, k, part.p, parts, out, t, s);
+    launch_multidot(t, x, (size_t)n * k, 1, y, (size_t)n, k, part.p, parts, out, s);
     check_cuda(cudaStreamSynchronize(s), "sync");
   });
 }
@@ -1932,7 +1936,7 @@ int mlmc_profile_kernel(mlmc_hierarchy *h, int which, int level, int k, int reps
       Vb.alloc((size_t)nvec * Lv.n * k * es);
       for (int v = 0; v < nvec; ++v)
         launch_noise(H.complex_op, 2 + v, 0, 0, Lv.n, k, t, Vb.as<char>() + (size_t)v * Lv.n * k * es, H.stream);
-      part.alloc((size_t)multidot_parts(Lv.n, k) * nvec * k * 16);
+      part.alloc((size_t)multidot_parts(t, Lv.n, k) * nvec * k * 16);
       outb.alloc((size_t)nvec * k * 16);
       launch_fill_zero(F64, outb.p, (size_t)nvec * k * (H.complex_op ? 2 : 1), H.stream);
     }
@@ -1940,13 +1944,12 @@ int mlmc_profile_kernel(mlmc_hierarchy *h, int which, int level, int k, int reps
       if (which == 2) {
         launch_rbgs_sweep(view(H, l, lo), y, x, k, 0, 0, H.stream);
       } else if (which == 3) {
-        launch_multidot(t, Vb.p, Lv.n * (size_t)k, nvec, x, Lv.n, k, part.p, multidot_parts(Lv.n, k), outb.p,
-                        H.complex_op ? C64 : F64, H.stream);
+        launch_multidot(t, Vb.p, Lv.n * (size_t)k, nvec, x, Lv.n, k, part.p, multidot_parts(t, Lv.n, k), outb.p,
+                        H.stream);
       } else if (which == 5) {
         dense_apply(H, lo, x, y, k);
       } else if (which == 4) {
-        launch_multiaxpy(t, y, Vb.p, Lv.n * (size_t)k, nvec, outb.p, H.complex_op ? C64 : F64, k, -1e-30, Lv.n, k,
-                         H.stream);
+        launch_multiaxpy(t, y, Vb.p, Lv.n * (size_t)k, nvec, outb.p, -1e-30, Lv.n, k, false, H.stream);
       } else if (which == 8) {
         net_forward(H, x, k);
       } else if (which == 9) {

@@ -167,23 +167,33 @@ void launch_sub(DType t, void *out, const void *a, const void *b, size_t count, 
 // y[i][c] = alpha[c] * x[i][c] (+ y if accumulate)
 void launch_scale_cols(DType t, void *y, const void *x, const void *alpha, int alpha_is_inverse_norm,
                        size_t rows, int k, cudaStream_t s);
-// partial[b][v][c] of sum_i conj(V_v[i][c]) * w[i][c], v < nvec; then out[v][c] (fixed order)
-// lazy_sc (optional): the unnormalised-basis epilogue of k_multidot_reduce (out = d / (s_i s_j),
-// lazy_coef = d / s_i^2 with s from lazy_sc, column lazy_j the new one)
+// out[v][c] = sum_i conj(V_v[i][c]) * w[i][c], v < nvec, FP64 (complex FP64), fixed order
+// (kernels_dots.cu).  partials: nparts * nvec * k FP64 (complex FP64) entries, nparts =
+// multidot_parts(t, rows, k) <= 608.
 void launch_multidot(DType t, const void *V, size_t vstride, int nvec, const void *w, size_t rows,
-                     int k, void *partials, int nparts, void *out, DType out_t, cudaStream_t s,
-                     const double *lazy_sc = nullptr, void *lazy_coef = nullptr, int lazy_j = 0);
-// w[i][c] -= sum_v V_v[i][c] * h[v][c]  (h in out precision), optional column mask
-// norm_part (optional): per-block column sums of |w_new|^2 in the FP64 accumulation
-// type (multiaxpy_norm_parts(rows, k) x k entries at most); returns the block count
-// to pass to launch_column_reduce.
-int launch_multiaxpy(DType t, void *w, const void *V, size_t vstride, int nvec, const void *h,
-                     DType h_t, size_t hstride, double sign, size_t rows, int k, cudaStream_t s,
-                     void *norm_part = nullptr);
+                     int k, void *partials, int nparts, void *out, cudaStream_t s);
+int multidot_parts(DType t, size_t rows, int k);
+// w[i][c] = (init ? 0 : w[i][c]) + sign * sum_v V_v[i][c] * h[v][c], h FP64 (complex FP64)
+void launch_multiaxpy(DType t, void *w, const void *V, size_t vstride, int nvec, const void *h, double sign,
+                      size_t rows, int k, bool init, cudaStream_t s);
+
+// The fixed-length FGMRES with an unnormalised basis u_0 = b, u_1, ... (V + i * vstride); each
+// returns its number of launches where that depends on the length.
+// Step j: partial dots of w = A z_j, then the multi-AXPY's coefficients (mid), the multi-AXPY
+// itself with the partial norms of u_{j+1} = w; on the last step the solution's weights (tail)
+// instead.  partials: multidot_parts * (its + 2) * k, norm: multiaxpy_norm_parts * k FP64
+// (complex FP64) entries; n2: its * k; D: its * (m + 1) * k; coef, y: its * k of type t.
+int launch_fgmres_dots(DType t, const void *b, const void *V, size_t vstride, int j, int its, const void *w, size_t rows,
+                       int k, void *partials, cudaStream_t s);
+void launch_fgmres_mid(DType t, const void *partials, const void *norm, int j, int m, size_t rows, int k, double *n2,
+                       void *D, void *coef, cudaStream_t s);
+void launch_fgmres_tail(DType t, const void *partials, const void *norm, int its, int m, size_t rows, int k,
+                        double *n2, const void *D, void *y, cudaStream_t s);
+int launch_fgmres_axpy(DType t, void *w, const void *b, const void *V, size_t vstride, int nvec, const void *coef,
+                       size_t rows, int k, void *norm, cudaStream_t s);
+int launch_fgmres_update(DType t, void *x, const void *Z, size_t vstride, int nvec, const void *y, size_t rows, int k,
+                         cudaStream_t s);
 int multiaxpy_norm_parts(size_t rows, int k);
-// out[c] = sum_p partial[p][c] (fixed order), FP64 or complex FP64
-void launch_column_reduce(DType out_t, const void *partial, int nparts, int k, void *out, cudaStream_t s);
-int multidot_parts(size_t rows, int k);
 
 }  // namespace mlmc
 
@@ -252,21 +262,13 @@ void launch_dense_apply_tc(DType t, const void *Ainv, const void *B, void *Y, in
 }  // namespace mlmc
 
 namespace mlmc {
-// per-column Krylov kernels (kernels_krylov.cu).  `hc` = 1 for complex Hessenberg data.
-// g0[c] holds |r|^2 on entry (from a column dot); sets beta, active, invnrm.
-// sc (optional): per-column norms of the unnormalised basis vectors of the
-// fixed-length FGMRES (s_0 = |b| here; s_{j+1} set by the step)
-// Added to the active-column count by launch_arnoldi_init for every column whose
-// residual norm is not finite (such a column can never converge).
-constexpr int NONFINITE_COLUMN = 1 << 20;
+// per-column Krylov kernels of the restarted FGMRES (kernels_krylov.cu).  `hc` = 1 for complex
+// Hessenberg data.  g0[c] holds |r|^2 on entry (from a column dot); sets beta, invnrm and
+// active (1 / 0; -1 where the residual norm is not finite: such a column can never converge).
 void launch_arnoldi_init(int hc, void *g, double *bnorm, double *invnrm, int *active, int *jdone,
-                         int k, double tol, int first, int *nactive, cudaStream_t s, double *sc = nullptr);
-// unnormalised basis: Gram-Schmidt coefficients d_i / s_i^2 into coef, Hessenberg
-// entries d_i / (s_i s_j) in place; and y_i /= s_i before the solution update
-void launch_lazy_y(int hc, void *y, const double *sc, const int *jdone, int m, int k, cudaStream_t s);
+                         int k, double tol, int first, cudaStream_t s);
 void launch_arnoldi_step(int hc, void *H, void *cs, void *sn, void *g, int j, int m, int k, int *active,
-                         int *jdone, const double *bnorm, double tol, double *invnrm, double *resid,
-                         int *nactive, int fixed, cudaStream_t s, double *sc = nullptr);
+                         int *jdone, const double *bnorm, double tol, double *invnrm, double *resid, cudaStream_t s);
 void launch_trisolve(int hc, const void *H, const void *g, void *y, const int *jdone, int m, int k,
                      cudaStream_t s);
 void launch_add_acc(int hc, void *dst, const void *src, int count, cudaStream_t s);

@@ -110,7 +110,8 @@ extern "C" int mlmc_column_dots_noalloc(int complex_data, const void *x, const v
   void *scratch = nullptr;
   int st = scratch_address(&scratch);
   if (st != MLMC_OK) return st;
-  const int parts = mlmc::multidot_parts((size_t)n, k);   // at most 608
+  const mlmc::DType t = complex_data ? mlmc::C64 : mlmc::F64;
+  const int parts = mlmc::multidot_parts(t, (size_t)n, k);   // at most 304
   if ((size_t)parts * k * 16 > kScratchBytes) {
     g_err = "scratch too small";
     return MLMC_ERR_INVALID_ARG;
@@ -118,8 +119,7 @@ extern "C" int mlmc_column_dots_noalloc(int complex_data, const void *x, const v
   // The partial sums are written in full by the first kernel before the second
   // reads them, so nothing in the array needs clearing between calls.
   try {
-    mlmc::DType t = complex_data ? mlmc::C64 : mlmc::F64;
-    mlmc::launch_multidot(t, x, (size_t)n * k, 1, y, (size_t)n, k, scratch, parts, out, t, (cudaStream_t)stream);
+    mlmc::launch_multidot(t, x, (size_t)n * k, 1, y, (size_t)n, k, scratch, parts, out, (cudaStream_t)stream);
     mlmc::check_cuda(cudaStreamSynchronize((cudaStream_t)stream), "sync");
   } catch (const mlmc::cuda_error &e) {
     g_err = std::string(e.where) + ": " + cudaGetErrorString(e.code);
