@@ -9,6 +9,8 @@
 // channel a holds dof a for real ones.  Weights are FP32 [c_out][c_in][3][3];
 // tap (ty, tx) reads the site (i + tx - 1, j + ty - 1), periodic or zero
 // outside a Dirichlet lattice.
+#include <type_traits>
+
 #include "mlmc_internal.cuh"
 
 namespace mlmc {
@@ -59,179 +61,304 @@ __global__ void k_add_from_channels(T *x, const float *a, int nsite, int d, int 
   }
 }
 
-// ------------------------------------------------------------------ convolution forward
-// out[s][co][c] = act(sum_{tap, ci} W[co][ci][tap] in[tap_site(s)][ci][c]); one thread per (site, column).
-template <int CI, int CO, bool RELU>
-__global__ void __launch_bounds__(256) k_conv_fwd(const float *__restrict__ in, const float *__restrict__ W,
-                                                  float *__restrict__ out, int nx, int ny, int k, int periodic) {
-  // weights transposed to [tap][ci][co] so that 4 outputs take one 16-byte shared load
-  __shared__ __align__(16) float Ws[9 * CI * CO];
-  for (int i = threadIdx.x; i < CO * CI * 9; i += blockDim.x) {
-    int co = i / (CI * 9), ci = (i / 9) % CI, tap = i % 9;
-    Ws[(tap * CI + ci) * CO + co] = W[i];
-  }
-  __syncthreads();
-  const unsigned total = (unsigned)nx * ny * k;
-  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-    const int s = (int)(t / (unsigned)k);
-    const int c = (int)(t - (unsigned)s * k);
-    const int i = s % nx, j = s / nx;
-    float acc[CO];
-#pragma unroll
-    for (int co = 0; co < CO; ++co) acc[co] = 0.f;
-#pragma unroll 1
-    for (int tap = 0; tap < 9; ++tap) {
-      int nb = tap_site(i, j, tap % 3, tap / 3, nx, ny, periodic);
-      if (nb < 0) continue;
-      const float *src = in + (size_t)nb * CI * k + c;
-#pragma unroll
-      for (int ci = 0; ci < CI; ++ci) {
-        float v = src[(size_t)ci * k];
-        const float *w = Ws + (tap * CI + ci) * CO;
-        if constexpr (CO % 4 == 0) {
-#pragma unroll
-          for (int co = 0; co < CO; co += 4) {
-            float4 w4 = *reinterpret_cast<const float4 *>(w + co);
-            acc[co] = fmaf(w4.x, v, acc[co]);
-            acc[co + 1] = fmaf(w4.y, v, acc[co + 1]);
-            acc[co + 2] = fmaf(w4.z, v, acc[co + 2]);
-            acc[co + 3] = fmaf(w4.w, v, acc[co + 3]);
-          }
-        } else {
-#pragma unroll
-          for (int co = 0; co < CO; ++co) acc[co] = fmaf(w[co], v, acc[co]);
-        }
-      }
-    }
-    float *dst = out + (size_t)s * CO * k + c;
-#pragma unroll
-    for (int co = 0; co < CO; ++co) dst[(size_t)co * k] = RELU ? fmaxf(acc[co], 0.f) : acc[co];
-  }
+// ------------------------------------------------------------------ convolutions
+// out[s][co][c] = epi(sum_{tap, ci} W[co][ci][tap] in[tap_site(s)][ci][c]).  A thread computes
+// PX = 8 consecutive sites of a lattice row for one column and at most 8 output channels: a (row,
+// channel) of its inputs is ten loads for three taps, and a 16-byte shared load of weights
+// (four clocks of the load unit) serves 32 multiply-adds.  Bound by FP32 arithmetic: the 256^2 x
+// 32 network (c0 = 4) takes 14.5 GFLOP, 185 us at the measured 39.2 T FMA/s; 345 us here, 586
+// with one site per thread (five load instructions per 16 multiply-adds), 445 with predicates
+// and 64-bit address arithmetic on every load, 378 without the packed multiply-adds.  KC is the
+// block width where it is one of the usual powers of two, known at compile time so that the
+// loads' offsets are immediates (0: any width): the sites between the halo columns are
+// contiguous, and only the two halo columns take a wrap or a Dirichlet zero.
+// The gradient with respect to the input is the same sum with mirrored taps and exchanged
+// channels (mirror = 1, W [CIN][COUT][9]):
+// gin[s][ci] = sum_{tap, co} W[co][ci][tap] gout[s - (tap offset)][co].
+// A layer may read the complex block itself (XIN: two channels per 8-byte load) and write its
+// result there, so that inference needs no layout passes.
+// a0 += x0 * v, a1 += x1 * v as one packed instruction (each half rounds as fmaf does): half the
+// issue slots of two multiply-adds
+__device__ __forceinline__ void fma_pair(float &a0, float &a1, float x0, float x1, float v) {
+  const float2 r = __ffma2_rn(make_float2(x0, x1), make_float2(v, v), make_float2(a0, a1));
+  a0 = r.x;
+  a1 = r.y;
 }
 
-// ------------------------------------------------------------------ backward: data
-// gin[s][ci][c] = mask(s, ci, c) * sum_{tap, co} W[co][ci][tap] gout[s'][co][c], where s' is the
-// site whose tap `tap` reads s (s' = s shifted by the opposite offset).  mask = (act[s][ci][c] > 0)
-// when `act` is given (ReLU of the layer that produced the input), else 1.
-template <int CI, int CO>
-__global__ void __launch_bounds__(256) k_conv_bwd_data(const float *__restrict__ gout, const float *__restrict__ W,
-                                                       const float *__restrict__ act, float *__restrict__ gin, int nx,
-                                                       int ny, int k, int periodic) {
-  // weights transposed to [tap][co][ci]: 4 inputs take one 16-byte shared load
-  __shared__ __align__(16) float Ws[9 * CO * CI];
-  for (int i = threadIdx.x; i < CO * CI * 9; i += blockDim.x) {
-    int co = i / (CI * 9), ci = (i / 9) % CI, tap = i % 9;
-    Ws[(tap * CO + co) * CI + ci] = W[i];
+enum { EPI_NONE = 0, EPI_RELU = 1, EPI_MASK = 2, EPI_STORE_COMPLEX = 3, EPI_ADD_COMPLEX = 4, EPI_ADD = 5 };
+
+template <int CIN, int COUT, int EPI, bool XIN, int KC>
+__global__ void __launch_bounds__(128, 4) k_conv(const float *__restrict__ in, const float *__restrict__ W, int mirror,
+                                                 const float *__restrict__ act, float *__restrict__ out, int nx, int ny,
+                                                 int kk, int periodic) {
+  constexpr int PX = 8, CS = XIN ? 2 : 1;                      // sites per thread, channels per load
+  constexpr int CB = COUT < 8 ? COUT : 8, HALVES = COUT / CB;  // output channels per thread
+  const int k = KC ? KC : kk;
+  __shared__ __align__(16) float Ws[9 * CIN * COUT];           // [ty][ci][tx][co]
+  for (int e = threadIdx.x; e < 9 * CIN * COUT; e += blockDim.x) {
+    const int co = e % COUT, tx = e / COUT % 3, ci = e / (COUT * 3) % CIN, ty = e / (COUT * 3 * CIN);
+    const int tap = ty * 3 + tx;
+    Ws[e] = mirror ? W[(ci * COUT + co) * 9 + 8 - tap] : W[(co * CIN + ci) * 9 + tap];
   }
   __syncthreads();
-  const unsigned total = (unsigned)nx * ny * k;
+  const unsigned groups = (nx + PX - 1) / PX, total = groups * ny * k * HALVES;
   for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-    const int s = (int)(t / (unsigned)k);
-    const int c = (int)(t - (unsigned)s * k);
-    const int i = s % nx, j = s / nx;
-    float acc[CI];
+    unsigned q = t / (unsigned)k;
+    const int c = (int)(t - q * (unsigned)k);
+    // neighbouring groups of k threads take the output halves of the same sites (inputs from L1)
+    const int cb = (int)(q % HALVES) * CB;
+    q /= HALVES;
+    const int j = (int)(q / groups);
+    // the last group of a row whose length PX does not divide is moved back, and leaves the
+    // sites before `first` to the group before it
+    const int first = (int)(q - (unsigned)j * groups) * PX;
+    const int i0 = max(0, min(first, nx - PX));
+    const int n = min(PX, nx);                                 // nx < PX: one short group
+    const int il = i0 > 0 ? i0 - 1 : nx - 1, ir = i0 + n < nx ? i0 + n : 0;
+    const bool onl = i0 > 0 || periodic, onr = i0 + n < nx || periodic;
+    float acc[PX][CB];
 #pragma unroll
-    for (int ci = 0; ci < CI; ++ci) acc[ci] = 0.f;
-#pragma unroll 1
-    for (int tap = 0; tap < 9; ++tap) {
-      // s' with tap_site(s', tap) = s: offset (1 - tx, 1 - ty) from s
-      int nb = tap_site(i, j, 2 - tap % 3, 2 - tap / 3, nx, ny, periodic);
-      if (nb < 0) continue;
-      const float *src = gout + (size_t)nb * CO * k + c;
+    for (int p = 0; p < PX; ++p)
 #pragma unroll
-      for (int co = 0; co < CO; ++co) {
-        float g = src[(size_t)co * k];
-        const float *w = Ws + (tap * CO + co) * CI;
-        if constexpr (CI % 4 == 0) {
+      for (int co = 0; co < CB; ++co) acc[p][co] = 0.f;
+    auto taps = [&](const float *w, const float *v) {
 #pragma unroll
-          for (int ci = 0; ci < CI; ci += 4) {
-            float4 w4 = *reinterpret_cast<const float4 *>(w + ci);
-            acc[ci] = fmaf(w4.x, g, acc[ci]);
-            acc[ci + 1] = fmaf(w4.y, g, acc[ci + 1]);
-            acc[ci + 2] = fmaf(w4.z, g, acc[ci + 2]);
-            acc[ci + 3] = fmaf(w4.w, g, acc[ci + 3]);
+      for (int tx = 0; tx < 3; ++tx) {
+        float wv[CB];
+        if constexpr (CB % 4 == 0) {
+#pragma unroll
+          for (int co = 0; co < CB; co += 4) {
+            const float4 w4 = *reinterpret_cast<const float4 *>(w + tx * COUT + co);
+            wv[co] = w4.x; wv[co + 1] = w4.y; wv[co + 2] = w4.z; wv[co + 3] = w4.w;
           }
+#pragma unroll
+          for (int p = 0; p < PX; ++p)
+#pragma unroll
+            for (int co = 0; co < CB; co += 2) fma_pair(acc[p][co], acc[p][co + 1], wv[co], wv[co + 1], v[p + tx]);
         } else {
 #pragma unroll
-          for (int ci = 0; ci < CI; ++ci) acc[ci] = fmaf(w[ci], g, acc[ci]);
+          for (int co = 0; co < CB; ++co) wv[co] = w[tx * COUT + co];
+#pragma unroll
+          for (int p = 0; p < PX; ++p)
+#pragma unroll
+            for (int co = 0; co < CB; ++co) acc[p][co] = fmaf(wv[co], v[p + tx], acc[p][co]);
         }
       }
-    }
-    float *dst = gin + (size_t)s * CI * k + c;
+    };
+#pragma unroll 1
+    for (int ty = 0; ty < 3; ++ty) {
+      int jj = j + ty - 1;
+      if (periodic) jj = jj < 0 ? jj + ny : jj >= ny ? jj - ny : jj;
+      if (jj < 0 || jj >= ny) continue;
+      const size_t row = (size_t)jj * nx;
+      const float *mid = in + (row + i0) * CIN * k + CS * c;
+      const float *left = in + (row + il) * CIN * k + CS * c, *right = in + (row + ir) * CIN * k + CS * c;
+      const float *w = Ws + ty * CIN * 3 * COUT + cb;
+#pragma unroll 2
+      for (int ci = 0; ci < CIN; ci += CS) {
+        float v[CS][PX + 2];
+        auto load = [&](int u, const float *src, bool ok) {
+          if constexpr (XIN) {
+            const float2 x = ok ? *reinterpret_cast<const float2 *>(src) : make_float2(0.f, 0.f);
+            v[0][u] = x.x;
+            v[1][u] = x.y;
+          } else {
+            v[0][u] = ok ? *src : 0.f;
+          }
+        };
+        load(0, left, onl);
+        if (n == PX) {
 #pragma unroll
-    for (int ci = 0; ci < CI; ++ci) {
-      float m = act ? (act[(size_t)s * CI * k + (size_t)ci * k + c] > 0.f ? 1.f : 0.f) : 1.f;
-      dst[(size_t)ci * k] = acc[ci] * m;
+          for (int u = 0; u < PX; ++u) load(u + 1, mid + u * CIN * k, true);
+          load(PX + 1, right, onr);
+        } else {
+          // a lattice narrower than the group: its right halo comes after n sites
+#pragma unroll
+          for (int u = 0; u <= PX; ++u)
+            load(u + 1, u < n ? mid + u * CIN * k : right, u < n || (u == n && onr));
+        }
+#pragma unroll
+        for (int z = 0; z < CS; ++z) taps(w + (ci + z) * 3 * COUT, v[z]);
+        left += CS * k;
+        mid += CS * k;
+        right += CS * k;
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < PX; ++p) {
+      if (p >= n) break;
+      if (i0 + p < first) continue;
+      const size_t o = (((size_t)j * nx + i0 + p) * COUT + cb) * k;
+      if constexpr (EPI == EPI_STORE_COMPLEX || EPI == EPI_ADD_COMPLEX) {
+#pragma unroll
+        for (int co = 0; co + 1 < CB; co += 2) {
+          float2 *dst = reinterpret_cast<float2 *>(out + o + (size_t)co * k) + c;
+          float2 v = make_float2(acc[p][co], acc[p][co + 1]);
+          if (EPI == EPI_ADD_COMPLEX) {
+            const float2 x = *dst;
+            v.x += x.x;
+            v.y += x.y;
+          }
+          *dst = v;
+        }
+      } else {
+#pragma unroll
+        for (int co = 0; co < CB; ++co) {
+          float *dst = out + o + (size_t)co * k + c;
+          float v = acc[p][co];
+          if (EPI == EPI_RELU) v = fmaxf(v, 0.f);
+          if (EPI == EPI_MASK) v = act[o + (size_t)co * k + c] > 0.f ? v : v * 0.f;
+          if (EPI == EPI_ADD) v += *dst;
+          *dst = v;
+        }
+      }
     }
   }
 }
 
 // ------------------------------------------------------------------ backward: weights
-// partial[block][co][ci][tap] = sum over the block's (site, column) pairs of
-// gout[s][co][c] * in[tap_site(s)][ci][c].  Pairs are staged through shared
-// memory in tiles; each thread owns a fixed set of weight entries, so the
-// per-block sums are deterministic.  Then k_weight_reduce adds the blocks in order.
-template <int CI, int CO>
-__global__ void __launch_bounds__(256) k_conv_bwd_weight(const float *__restrict__ in, const float *__restrict__ gout,
-                                                         float *__restrict__ partial, int nx, int ny, int k,
-                                                         int periodic) {
-  constexpr int NW = CO * CI * 9;
-  constexpr int TP = 32;                       // pairs per tile
-  constexpr int PER = (NW + 255) / 256;        // weight entries per thread
-  __shared__ float g_t[TP][CO];
-  __shared__ float x_t[TP][9][CI];
-  float acc[PER];
+// partial[part][co][ci][tap] = sum over the part's (site, column) pairs of
+// gout[s][co][c] * in[tap_site(s)][ci][c].  Lanes are columns (several lattice rows when k < 32);
+// a warp keeps one input channel's nine taps times COG output channels in registers (72 sums)
+// and walks lattice rows with a 3 x 3 window, so a site costs COG + 3 coalesced loads for
+// 9 COG multiply-adds; the warps of a block walk the same sites for the other channels and
+// share the loads in L1.  The loads run ahead of the products (the window by two sites, the
+// gradients by one: more spills).  16 -> 16 channels on 128^2 x 32 (2.4 GFLOP, 31 us at the
+// measured rate): about 120 us against 1151 us with the pairs staged through shared memory and
+// two shared loads per multiply-add.  The lanes meet once at the end (fixed shuffle tree), the
+// parts in k_weight_reduce.
+constexpr int WG_THREADS = 512, WG_SEG = 16, WG_BLOCKS = 152;
+
+template <int CI, int CO> struct wg {
+  static constexpr int COG = CO < 8 ? CO : 8;
+  static constexpr int COMBOS = CI * (CO / COG);                     // (input channel, output group) pairs
+  static constexpr int CPB = COMBOS < 16 ? COMBOS : 16;              // of one block's 16 warps
+  static constexpr int SLICES = 16 / CPB, GY = COMBOS / CPB;
+  static constexpr int PARTS = WG_BLOCKS / GY * SLICES;
+};
+
+template <int CI, int CO, int KC>
+__global__ void __launch_bounds__(WG_THREADS, 1) k_conv_bwd_weight(const float *__restrict__ in,
+                                                                   const float *__restrict__ gout,
+                                                                   float *__restrict__ partial, int nx, int ny, int kk,
+                                                                   int periodic) {
+  typedef wg<CI, CO> G;
+  constexpr int COG = G::COG;
+  const int k = KC ? KC : kk;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int combo = blockIdx.y * G::CPB + warp % G::CPB, ci = combo % CI, co0 = combo / CI * COG;
+  const int part = blockIdx.x * G::SLICES + warp / G::CPB;
+  const int rpu = k >= 32 ? 1 : 32 / k;                       // lattice rows per unit
+  const int chunks = (k + 31) / 32, segs = (nx + WG_SEG - 1) / WG_SEG;
+  const int units = (ny + rpu - 1) / rpu * chunks * segs;
+  float acc[COG][9];
 #pragma unroll
-  for (int q = 0; q < PER; ++q) acc[q] = 0.f;
-  const unsigned total = (unsigned)nx * ny * k;
-  const unsigned per_block = (total + gridDim.x - 1) / gridDim.x;
-  const unsigned p0 = blockIdx.x * per_block;
-  const unsigned p1 = p0 + per_block < total ? p0 + per_block : total;
-  for (unsigned base = p0; base < p1; base += TP) {
-    // stage TP pairs
-    for (int e = threadIdx.x; e < TP * (CO + 9 * CI); e += blockDim.x) {
-      int p = e / (CO + 9 * CI), r = e % (CO + 9 * CI);
-      unsigned t = base + p;
-      float v = 0.f;
-      if (t < p1) {
-        int s = (int)(t / (unsigned)k), c = (int)(t - (unsigned)s * k);
-        if (r < CO) {
-          v = gout[(size_t)s * CO * k + (size_t)r * k + c];
+  for (int q = 0; q < COG; ++q)
+#pragma unroll
+    for (int p = 0; p < 9; ++p) acc[q][p] = 0.f;
+  const float *X = in + (size_t)ci * k, *Gp = gout + (size_t)co0 * k;
+  for (int u = part; u < units; u += G::PARTS) {
+    const int seg = u % segs, v = u / segs;
+    const int c = k >= 32 ? v % chunks * 32 + lane : lane % k;
+    const int j = k >= 32 ? v / chunks : v * rpu + lane / k;
+    const bool live = c < k && j < ny && (k >= 32 || lane / k < rpu);
+    const int i0 = seg * WG_SEG, i1 = min(i0 + WG_SEG, nx);
+    // the window's rows: which exist (an idle lane has none) and where they start
+    const float *row[3];
+    bool on[3];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      int jj = j + r - 1;
+      if (periodic) jj = jj < 0 ? jj + ny : jj >= ny ? jj - ny : jj;
+      on[r] = live && jj >= 0 && jj < ny;
+      row[r] = X + (on[r] ? (size_t)jj * nx * CI * k + c : 0);
+    }
+    const float *g = Gp + (live ? ((size_t)j * nx + i0) * CO * k + c : 0);
+    auto column = [&](int i, float w[3]) {                   // window column i, -1 <= i <= nx + 1
+      const bool in_row = (unsigned)i < (unsigned)nx;
+      const int ii = in_row ? i : i < 0 ? i + nx : i - nx;
+      const bool ok = in_row || periodic;
+      const size_t o = (size_t)(unsigned)ii * (unsigned)(CI * k);
+#pragma unroll
+      for (int r = 0; r < 3; ++r) w[r] = ok && on[r] && ii < nx ? row[r][o] : 0.f;
+    };
+    auto grads = [&](float w[COG], bool ok) {                // the next site's gradients
+#pragma unroll
+      for (int q = 0; q < COG; ++q) w[q] = live && ok ? g[q * k] : 0.f;
+      g += CO * k;
+    };
+    float a[3], b[3], d[3], e[3], g0[COG];
+    column(i0 - 1, a);
+    column(i0, b);
+    column(i0 + 1, d);
+    column(min(i0 + 2, nx + 1), e);
+    grads(g0, true);
+#pragma unroll 4
+    for (int i = i0; i < i1; ++i) {
+      float en[3], gn[COG];
+      column(min(i + 3, nx + 1), en);                        // used two sites on, if at all
+      grads(gn, i + 1 < i1);
+      auto taps3 = [&](int r, int tx, float x) {
+        if constexpr (COG % 2 == 0) {
+#pragma unroll
+          for (int q = 0; q < COG; q += 2)
+            fma_pair(acc[q][r * 3 + tx], acc[q + 1][r * 3 + tx], g0[q], g0[q + 1], x);
         } else {
-          int q = r - CO, tap = q / CI, ci = q % CI;
-          int nb = tap_site(s % nx, s / nx, tap % 3, tap / 3, nx, ny, periodic);
-          v = nb < 0 ? 0.f : in[(size_t)nb * CI * k + (size_t)ci * k + c];
+#pragma unroll
+          for (int q = 0; q < COG; ++q) acc[q][r * 3 + tx] = fmaf(g0[q], x, acc[q][r * 3 + tx]);
         }
-      }
-      if (r < CO) g_t[p][r] = v;
-      else x_t[p][(r - CO) / CI][(r - CO) % CI] = v;
-    }
-    __syncthreads();
+      };
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-      int w = threadIdx.x + q * 256;
-      if (w < NW) {
-        int co = w / (CI * 9), ci = (w / 9) % CI, tap = w % 9;
-        float a = acc[q];
-        for (int p = 0; p < TP; ++p) a = fmaf(g_t[p][co], x_t[p][tap][ci], a);
-        acc[q] = a;
+      for (int r = 0; r < 3; ++r) {
+        taps3(r, 0, a[r]);
+        taps3(r, 1, b[r]);
+        taps3(r, 2, d[r]);
       }
-    }
-    __syncthreads();
-  }
 #pragma unroll
-  for (int q = 0; q < PER; ++q) {
-    int w = threadIdx.x + q * 256;
-    if (w < NW) partial[(size_t)blockIdx.x * NW + w] = acc[q];
+      for (int r = 0; r < 3; ++r) {
+        a[r] = b[r];
+        b[r] = d[r];
+        d[r] = e[r];
+        e[r] = en[r];
+      }
+#pragma unroll
+      for (int q = 0; q < COG; ++q) g0[q] = gn[q];
+    }
   }
+  float *dst = partial + (size_t)part * CO * CI * 9;
+#pragma unroll
+  for (int q = 0; q < COG; ++q)
+#pragma unroll
+    for (int p = 0; p < 9; ++p) {
+      float v = acc[q][p];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == (q * 9 + p) % 32) dst[((size_t)(co0 + q) * CI + ci) * 9 + p] = v;
+    }
 }
 
-__global__ void k_weight_reduce(const float *partial, int nblocks, int nw, float *grad, float scale) {
-  int w = blockIdx.x * blockDim.x + threadIdx.x;
-  if (w >= nw) return;
-  double s = 0.0;
-  for (int b = 0; b < nblocks; ++b) s += (double)partial[(size_t)b * nw + w];
-  grad[w] = (float)(s * scale);
+// grad[w] = scale * sum over parts of partial[part][w]: a block takes 32 weights (coalesced),
+// its eight warps every eighth part as float pairs (hi + lo, two-sum), added in warp order.
+__global__ void __launch_bounds__(256) k_weight_reduce(const float *partial, int nparts, int nw, float *grad,
+                                                       float scale) {
+  __shared__ float2 red[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = blockIdx.x * 32 + lane;
+  float h = 0.f, l = 0.f;
+  if (w < nw) {
+#pragma unroll 4
+    for (int b = warp; b < nparts; b += 8) {
+      const float x = partial[(size_t)b * nw + w], s = h + x, t = s - h;
+      l += (h - (s - t)) + (x - t);
+      h = s;
+    }
+  }
+  red[warp][lane] = make_float2(h, l);
+  __syncthreads();
+  if (warp == 0 && w < nw) {
+    double s = 0.0;
+    for (int q = 0; q < 8; ++q) s += (double)red[q][lane].x + (double)red[q][lane].y;
+    grad[w] = (float)(s * scale);
+  }
 }
 
 // ------------------------------------------------------------------ Adam
@@ -264,58 +391,95 @@ void launch_add_from_channels(DType t, void *x, const float *a, int nsite, int d
   MLMC_LAUNCH_CHECK("k_add_from_channels");
 }
 
-#define MLMC_CONV_SHAPES(X) X(1, 16) X(2, 16) X(4, 16) X(16, 16) X(16, 1) X(16, 2) X(16, 4)
-
-void launch_conv_fwd(int ci, int co, bool relu, const float *in, const float *W, float *out, int nx, int ny, int k,
-                     int periodic, cudaStream_t s) {
-  unsigned g = cgrid((unsigned)nx * ny * k);
-#define MLMC_FWD(A, B)                                                                                        \
-  if (ci == A && co == B) {                                                                                   \
-    if (relu) k_conv_fwd<A, B, true><<<g, 256, 0, s>>>(in, W, out, nx, ny, k, periodic);                      \
-    else k_conv_fwd<A, B, false><<<g, 256, 0, s>>>(in, W, out, nx, ny, k, periodic);                          \
-    MLMC_LAUNCH_CHECK("k_conv_fwd");                                                                          \
-    return;                                                                                                   \
+// The usual block widths are compile-time constants of the kernels, any other is not.
+template <class F>
+static void by_width(int k, F f) {
+  switch (k) {
+    case 16: f(std::integral_constant<int, 16>()); break;
+    case 32: f(std::integral_constant<int, 32>()); break;
+    case 64: f(std::integral_constant<int, 64>()); break;
+    default: f(std::integral_constant<int, 0>()); break;
   }
-  MLMC_CONV_SHAPES(MLMC_FWD)
+}
+
+template <int CIN, int COUT, int EPI, bool XIN>
+static void conv_go(const float *in, const float *W, int mirror, const float *act, float *out, int nx, int ny, int k,
+                    int periodic, cudaStream_t s) {
+  const size_t threads = (size_t)((nx + 7) / 8) * ny * k * (COUT > 8 ? COUT / 8 : 1);
+  by_width(k, [&](auto kc) {
+    k_conv<CIN, COUT, EPI, XIN, decltype(kc)::value><<<resident_grid((threads + 127) / 128, 4), 128, 0, s>>>(
+        in, W, mirror, act, out, nx, ny, k, periodic);
+  });
+  MLMC_LAUNCH_CHECK("k_conv");
+}
+
+// Layers are c0 -> 16, 16 -> 16 (both with a ReLU) and 16 -> c0, c0 = 1, 2 or 4.
+void launch_conv_fwd(int ci, int co, const float *in, const float *W, float *out, int nx, int ny, int k, int periodic,
+                     cudaStream_t s) {
+#define MLMC_FWD(A, B, E) \
+  if (ci == A && co == B) return conv_go<A, B, E, false>(in, W, 0, nullptr, out, nx, ny, k, periodic, s);
+  MLMC_FWD(1, 16, EPI_RELU) MLMC_FWD(2, 16, EPI_RELU) MLMC_FWD(4, 16, EPI_RELU) MLMC_FWD(16, 16, EPI_RELU)
+  MLMC_FWD(16, 1, EPI_NONE) MLMC_FWD(16, 2, EPI_NONE) MLMC_FWD(16, 4, EPI_NONE)
 #undef MLMC_FWD
   throw cuda_error{cudaErrorInvalidValue, "conv: unsupported channel counts"};
 }
 
+void launch_conv_first(DType t, int ci, const void *x, const float *W, float *out, int nx, int ny, int k, int periodic,
+                       cudaStream_t s) {
+  const float *in = (const float *)x;
+  if (t == C32 && ci == 2) conv_go<2, 16, EPI_RELU, true>(in, W, 0, nullptr, out, nx, ny, k, periodic, s);
+  else if (t == C32 && ci == 4) conv_go<4, 16, EPI_RELU, true>(in, W, 0, nullptr, out, nx, ny, k, periodic, s);
+  else if (t == F32) launch_conv_fwd(ci, 16, in, W, out, nx, ny, k, periodic, s);
+  else throw cuda_error{cudaErrorInvalidValue, "conv: unsupported block"};
+}
+
+void launch_conv_last(DType t, int co, const float *in, const float *W, void *x, bool add, int nx, int ny, int k,
+                      int periodic, cudaStream_t s) {
+  float *out = (float *)x;
+#define MLMC_LAST(TT, B, ADD, E) \
+  if (t == TT && co == B && add == ADD) return conv_go<16, B, E, false>(in, W, 0, nullptr, out, nx, ny, k, periodic, s);
+  MLMC_LAST(C32, 4, true, EPI_ADD_COMPLEX) MLMC_LAST(C32, 4, false, EPI_STORE_COMPLEX)
+  MLMC_LAST(C32, 2, true, EPI_ADD_COMPLEX) MLMC_LAST(C32, 2, false, EPI_STORE_COMPLEX)
+  MLMC_LAST(F32, 1, true, EPI_ADD) MLMC_LAST(F32, 1, false, EPI_NONE)
+#undef MLMC_LAST
+  throw cuda_error{cudaErrorInvalidValue, "conv: unsupported block"};
+}
+
+// gradient wrt the input of a layer 16 -> co, masked by act > 0
 void launch_conv_bwd_data(int ci, int co, const float *gout, const float *W, const float *act, float *gin, int nx,
                           int ny, int k, int periodic, cudaStream_t s) {
-  unsigned g = cgrid((unsigned)nx * ny * k);
-#define MLMC_BWD(A, B)                                                                                        \
-  if (ci == A && co == B) {                                                                                   \
-    k_conv_bwd_data<A, B><<<g, 256, 0, s>>>(gout, W, act, gin, nx, ny, k, periodic);                          \
-    MLMC_LAUNCH_CHECK("k_conv_bwd_data");                                                                     \
-    return;                                                                                                   \
-  }
-  MLMC_CONV_SHAPES(MLMC_BWD)
+#define MLMC_BWD(B) \
+  if (ci == 16 && co == B) return conv_go<B, 16, EPI_MASK, false>(gout, W, 1, act, gin, nx, ny, k, periodic, s);
+  MLMC_BWD(1) MLMC_BWD(2) MLMC_BWD(4) MLMC_BWD(16)
 #undef MLMC_BWD
   throw cuda_error{cudaErrorInvalidValue, "conv: unsupported channel counts"};
 }
 
-int conv_weight_blocks() { return 152 * 2; }
+size_t conv_weight_scratch() {
+  // floats of partial sums of the widest layer in either family of kernels
+  return (size_t)304 * 16 * 16 * 9;
+}
 
 void launch_conv_bwd_weight(int ci, int co, const float *in, const float *gout, float *partial, float *grad,
                             float scale, int nx, int ny, int k, int periodic, cudaStream_t s) {
-  int nb = conv_weight_blocks();
-  int nw = ci * co * 9;
 #define MLMC_BWW(A, B)                                                                                        \
   if (ci == A && co == B) {                                                                                   \
-    k_conv_bwd_weight<A, B><<<nb, 256, 0, s>>>(in, gout, partial, nx, ny, k, periodic);                       \
+    static_assert((size_t)wg<A, B>::PARTS * A * B * 9 <= (size_t)304 * 16 * 16 * 9, "partial sums");          \
+    by_width(k, [&](auto kc) {                                                                                \
+      k_conv_bwd_weight<A, B, decltype(kc)::value>                                                            \
+          <<<dim3(WG_BLOCKS / wg<A, B>::GY, wg<A, B>::GY), WG_THREADS, 0, s>>>(in, gout, partial, nx, ny, k, periodic); \
+    });                                                                                                       \
     MLMC_LAUNCH_CHECK("k_conv_bwd_weight");                                                                   \
-    k_weight_reduce<<<(nw + 127) / 128, 128, 0, s>>>(partial, nb, nw, grad, scale);                           \
-    MLMC_LAUNCH_CHECK("k_weight_reduce");                                                                     \
+    launch_weight_reduce(partial, wg<A, B>::PARTS, A * B * 9, grad, scale, s);                                \
     return;                                                                                                   \
   }
-  MLMC_CONV_SHAPES(MLMC_BWW)
+  MLMC_BWW(1, 16) MLMC_BWW(2, 16) MLMC_BWW(4, 16) MLMC_BWW(16, 16) MLMC_BWW(16, 1) MLMC_BWW(16, 2) MLMC_BWW(16, 4)
 #undef MLMC_BWW
   throw cuda_error{cudaErrorInvalidValue, "conv: unsupported channel counts"};
 }
 
-void launch_weight_reduce(const float *partial, int nblocks, int nw, float *grad, float scale, cudaStream_t s) {
-  k_weight_reduce<<<(nw + 127) / 128, 128, 0, s>>>(partial, nblocks, nw, grad, scale);
+void launch_weight_reduce(const float *partial, int nparts, int nw, float *grad, float scale, cudaStream_t s) {
+  k_weight_reduce<<<(nw + 31) / 32, 256, 0, s>>>(partial, nparts, nw, grad, scale);
   MLMC_LAUNCH_CHECK("k_weight_reduce");
 }
 

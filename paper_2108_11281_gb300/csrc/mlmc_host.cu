@@ -655,7 +655,7 @@ void net_alloc(H_t &h) {
     h.netG.alloc(h.net_nw * sizeof(float));
     h.netM.alloc(h.net_nw * sizeof(float));
     h.netV.alloc(h.net_nw * sizeof(float));
-    h.netPart.alloc((size_t)conv_weight_blocks() * NET_CH * NET_CH * 9 * sizeof(float));
+    h.netPart.alloc(conv_weight_scratch() * sizeof(float));
     h.lcol.alloc(2 * (size_t)h.kmax * 16);
     h.lalpha.alloc((size_t)h.kmax * sizeof(double));
   }
@@ -690,7 +690,7 @@ void conv_forward(H_t &h, int ci, int co, bool relu, const float *in, const floa
   if (conv_on_tc(h, F.nx, k, ci, co))
     launch_conv_tc(in, W, nullptr, out, F.nx, F.ny, k, ci, co, per, 0, relu ? 1 : 0, h.err.as<int>(), h.stream);
   else
-    launch_conv_fwd(ci, co, relu, in, W, out, F.nx, F.ny, k, per, h.stream);
+    launch_conv_fwd(ci, co, in, W, out, F.nx, F.ny, k, per, h.stream);
   h.launches++;
 }
 
@@ -719,15 +719,35 @@ void conv_backward_weight(H_t &h, int ci, int co, const float *in, const float *
   h.launches += 2;
 }
 
-// act3 = net(r) in channel layout; act0..act2 keep the activations
-void net_forward(H_t &h, const void *r, int k) {
+// The hidden activations act1, act2 of net(r); keep_input: act0 holds r in channel layout (the
+// weight gradients and the tensor-core first layer read it there)
+void net_hidden(H_t &h, const void *r, int k, bool keep_input) {
   const Level &F = h.lv[0];
-  cudaStream_t s = h.stream;
-  launch_to_channels(h.t32, r, h.act0.as<float>(), (int)F.nsite, F.d, k, s);
-  h.launches++;
-  conv_forward(h, h.net_c0, NET_CH, true, h.act0.as<float>(), netW1(h), h.act1.as<float>(), k);
+  if (keep_input || conv_on_tc(h, F.nx, k, h.net_c0, NET_CH)) {
+    launch_to_channels(h.t32, r, h.act0.as<float>(), (int)F.nsite, F.d, k, h.stream);
+    h.launches++;
+    conv_forward(h, h.net_c0, NET_CH, true, h.act0.as<float>(), netW1(h), h.act1.as<float>(), k);
+  } else {
+    launch_conv_first(h.t32, h.net_c0, r, netW1(h), h.act1.as<float>(), F.nx, F.ny, k, h.periodic || h.complex_op,
+                      h.stream);
+    h.launches++;
+  }
   conv_forward(h, NET_CH, NET_CH, true, h.act1.as<float>(), netW2(h), h.act2.as<float>(), k);
-  conv_forward(h, NET_CH, h.net_c0, false, h.act2.as<float>(), netW3(h), h.act3.as<float>(), k);
+}
+
+// e = net(r), or e += net(r)
+void net_forward(H_t &h, const void *r, void *e, bool add, int k, bool keep_input = false) {
+  const Level &F = h.lv[0];
+  net_hidden(h, r, k, keep_input);
+  if (conv_on_tc(h, F.nx, k, NET_CH, h.net_c0)) {
+    conv_forward(h, NET_CH, h.net_c0, false, h.act2.as<float>(), netW3(h), h.act3.as<float>(), k);
+    if (!add) launch_fill_zero(h.t32, e, F.n * (size_t)k, h.stream);
+    launch_add_from_channels(h.t32, e, h.act3.as<float>(), (int)F.nsite, F.d, k, h.stream);
+  } else {
+    launch_conv_last(h.t32, h.net_c0, h.act2.as<float>(), netW3(h), e, add, F.nx, F.ny, k, h.periodic || h.complex_op,
+                     h.stream);
+  }
+  h.launches++;
 }
 
 // MLMC_CONV_AUTO: time the network on a fine-level block of the sample width with the
@@ -750,7 +770,7 @@ void tune_conv(H_t &h) {
     h.conv_auto_tc = 0;
     return;
   }
-  void *x = h.cyc[1][0].b.p;
+  void *x = h.cyc[1][0].b.p, *e = h.cyc[1][0].x.p;
   launch_noise(h.complex_op, 9, 0, 0, F.n, k, h.t32, x, h.stream);
   cudaEvent_t e0, e1;
   check_cuda(cudaEventCreate(&e0), "event");
@@ -758,9 +778,9 @@ void tune_conv(H_t &h) {
   float ms[2] = {0.f, 0.f};
   for (int tc = 0; tc < 2; ++tc) {
     h.conv_auto_tc = tc;
-    net_forward(h, x, k);
+    net_forward(h, x, e, false, k);
     check_cuda(cudaEventRecord(e0, h.stream), "record");
-    for (int r = 0; r < 3; ++r) net_forward(h, x, k);
+    for (int r = 0; r < 3; ++r) net_forward(h, x, e, false, k);
     check_cuda(cudaEventRecord(e1, h.stream), "record");
     check_cuda(cudaEventSynchronize(e1), "sync");
     check_cuda(cudaEventElapsedTime(&ms[tc], e0, e1), "elapsed");
@@ -781,16 +801,14 @@ double net_loss_grad(H_t &h, const void *r, int k, bool grad, bool read_loss) {
   cudaStream_t s = h.stream;
   size_t cnt = F.n * (size_t)k;
   void *E = h.cyc[1][0].x.p, *Tt = h.cyc[1][0].b.p;
-  net_forward(h, r, k);
-  launch_fill_zero(h.t32, E, cnt, s);
-  launch_add_from_channels(h.t32, E, h.act3.as<float>(), (int)F.nsite, F.d, k, s);
+  net_forward(h, r, E, false, k, true);
   residual_op(h, 0, 1, E, r, Tt, k);                             // t = r - A e
   Krylov &K = *h.outer[0];
   const size_t as = acc_size(h);
   char *nr2 = h.lcol.as<char>(), *nt2 = nr2 + (size_t)k * as;
   launch_multidot(h.t32, r, cnt, 1, r, F.n, k, K.partials.p, multidot_parts(h.t32, F.n, k), nr2, s);
   launch_multidot(h.t32, Tt, cnt, 1, Tt, F.n, k, K.partials.p, multidot_parts(h.t32, F.n, k), nt2, s);
-  h.launches += 6;
+  h.launches += 4;
   double loss = 0.0;
   if (read_loss) {
     std::vector<char> buf(2 * (size_t)k * as);
@@ -834,9 +852,7 @@ void fine_hooks(H_t &h, void *x, const void *b, int k) {
     const Level &F = h.lv[0];
     void *r = h.cyc[1][0].r.p;
     residual_op(h, 0, 1, x, b, r, k);
-    net_forward(h, r, k);
-    launch_add_from_channels(h.t32, x, h.act3.as<float>(), (int)F.nsite, F.d, k, h.stream);
-    h.launches++;
+    net_forward(h, r, x, true, k);
   }
 }
 
@@ -1951,7 +1967,7 @@ int mlmc_profile_kernel(mlmc_hierarchy *h, int which, int level, int k, int reps
       } else if (which == 4) {
         launch_multiaxpy(t, y, Vb.p, Lv.n * (size_t)k, nvec, outb.p, -1e-30, Lv.n, k, false, H.stream);
       } else if (which == 8) {
-        net_forward(H, x, k);
+        net_forward(H, x, y, false, k);
       } else if (which == 9) {
         launch_residual_restrict(view(H, l, lo), pview(H, l, lo), y, x, H.cyc[lo][l + 1].b.p, k, 0, H.stream);
       } else if (which == 6) {
@@ -2101,10 +2117,7 @@ int mlmc_learned_apply(mlmc_hierarchy *h, const void *r, void *e, int k) {
     if (h->prm.precision != MLMC_PREC_MIXED_FP32) fail(MLMC_ERR_UNSUPPORTED, "the learned correction runs in the mixed form");
     if (!r || !e || k < 1 || k > h->kmax) fail(MLMC_ERR_INVALID_ARG, "bad block");
     net_alloc(*h);
-    const Level &F = h->lv[0];
-    net_forward(*h, r, k);
-    launch_fill_zero(h->t32, e, F.n * (size_t)k, h->stream);
-    launch_add_from_channels(h->t32, e, h->act3.as<float>(), (int)F.nsite, F.d, k, h->stream);
+    net_forward(*h, r, e, false, k);
     check_cuda(cudaStreamSynchronize(h->stream), "sync");
   });
 }

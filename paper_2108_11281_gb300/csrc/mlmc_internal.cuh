@@ -287,11 +287,18 @@ namespace mlmc {
 // learned correction (kernels_learned.cu)
 void launch_to_channels(DType t, const void *x, float *a, int nsite, int d, int k, cudaStream_t s);
 void launch_add_from_channels(DType t, void *x, const float *a, int nsite, int d, int k, cudaStream_t s);
-void launch_conv_fwd(int ci, int co, bool relu, const float *in, const float *W, float *out, int nx, int ny, int k,
+void launch_conv_fwd(int ci, int co, const float *in, const float *W, float *out, int nx, int ny, int k,
                      int periodic, cudaStream_t s);
 void launch_conv_bwd_data(int ci, int co, const float *gout, const float *W, const float *act, float *gin, int nx,
                           int ny, int k, int periodic, cudaStream_t s);
-int conv_weight_blocks();
+// the first and last layer reading and writing the vector block itself (real, or complex
+// interleaved): out = relu(W x); x = W in, or x += W in
+void launch_conv_first(DType t, int ci, const void *x, const float *W, float *out, int nx, int ny, int k, int periodic,
+                       cudaStream_t s);
+void launch_conv_last(DType t, int co, const float *in, const float *W, void *x, bool add, int nx, int ny, int k,
+                      int periodic, cudaStream_t s);
+// floats of scratch for the weight gradients' partial sums
+size_t conv_weight_scratch();
 void launch_conv_bwd_weight(int ci, int co, const float *in, const float *gout, float *partial, float *grad,
                             float scale, int nx, int ny, int k, int periodic, cudaStream_t s);
 // tensor-core convolutions (kernels_conv_tc.cu): forward (mirror = 0; W [cout][cin][9]) or
