@@ -3,7 +3,9 @@
 // Gauss-Jordan inverse and trace of the coarsest operator, and the dense
 // coarsest-level apply used inside every multigrid cycle.
 #include <algorithm>
+#include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "mlmc.h"
 #include "mlmc_internal.cuh"
@@ -648,10 +650,75 @@ void launch_trace(DType t, const void *A, int n, void *out, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------------ dense coarsest apply
-// Y[i][c] = sum_j Ainv[i][j] B[j][c].  64 x 32 output tiles, 128 threads with
-// a 4 x 4 register tile each, j in steps of 16 through shared memory; the j
-// range is split over `splits` blocks (grid.z) writing partial tiles that a
-// second kernel adds in split order.
+// Y[i][c] = sum_j Ainv[i][j] B[j][c].
+//
+// FP64 data, and FP32 data with small n: the outputs are dealt out over all SMs.  A warp holds
+// 32 items (R rows x one column each, items in (row group, column) order, so a ragged k wastes
+// no lanes), the eight warps of a block take an eighth of the j range each and meet in shared
+// memory in order.  FP64 issues one warp instruction per 16 clocks and SM, so its loads need no
+// shared-memory tiling; what counts is that every SM has the same share: 256 x 256 x 64
+// columns, 4.2 M FMA = 6.7 us at the measured rate, took 45 us on the 32 blocks of the tiled
+// kernel below and takes 10.9 us (576 x 576 x 21: 61.5 -> 15.5 us).  With FP32 and n < 512 the
+// chain of dependent loads counts, an eighth as long (128 complex x 32: 14 -> 4 us).
+template <class T, int R>
+__global__ void __launch_bounds__(256) k_dense_spread(const T *__restrict__ A, const T *__restrict__ B,
+                                                      T *__restrict__ Y, int n, int k, int chunk, int vec) {
+  constexpr int VJ = 16 / (int)sizeof(T);                  // entries of a row per 16-byte load
+  __shared__ T red[8][R][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned t = blockIdx.x * 32u + lane;
+  const int rg = (int)(t / (unsigned)k), c = (int)(t - (unsigned)rg * k), row0 = rg * R;
+  const int j0 = min(n, warp * chunk), j1 = min(n, j0 + chunk);
+  T acc[R];
+  const T *a[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    acc[r] = zero<T>();
+    a[r] = A + (size_t)min(row0 + r, n - 1) * n;           // rows past the end repeat the last, unused
+  }
+  const T *b = B + c;
+  int j = j0;
+  if (vec) {
+#pragma unroll 4
+    for (; j + VJ <= j1; j += VJ) {
+      T av[R][VJ], bv[VJ];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const uint4 w = *reinterpret_cast<const uint4 *>(a[r] + j);
+        memcpy(av[r], &w, 16);
+      }
+#pragma unroll
+      for (int q = 0; q < VJ; ++q) bv[q] = b[(size_t)(j + q) * k];
+#pragma unroll
+      for (int q = 0; q < VJ; ++q)
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = acc[r] + av[r][q] * bv[q];
+    }
+  }
+#pragma unroll 4
+  for (; j < j1; ++j) {
+    const T bv = b[(size_t)j * k];
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = acc[r] + a[r][j] * bv;
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) red[warp][r][lane] = acc[r];
+  __syncthreads();
+  for (int e = threadIdx.x; e < R * 32; e += 256) {
+    const int r = e >> 5, l = e & 31;
+    T s = red[0][r][l];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s = s + red[w][r][l];
+    const unsigned tt = blockIdx.x * 32u + l;
+    const int i = (int)(tt / (unsigned)k) * R + r;
+    if (i < n) Y[(size_t)i * k + tt % (unsigned)k] = s;
+  }
+}
+
+// FP32 data with n >= 512 where the tensor-core kernel is not asked for: 64 x 32 output tiles,
+// 128 threads with a 4 x 4 register tile each, j in steps of 16 through shared memory; the j
+// range is split over `splits` blocks (grid.z) writing partial tiles that a second kernel adds
+// in split order.
 constexpr int DA_BM = 64, DA_BN = 32, DA_BK = 16;
 
 template <class T>
@@ -703,7 +770,7 @@ __global__ void __launch_bounds__(128) k_dense_apply(const T *__restrict__ A, co
     }
 }
 
-// Narrow blocks (k <= 8, e.g. the test vectors of the setup's bootstrap cycles): one warp
+// Up to three columns: one warp
 // per row of Ainv, the lanes take j = lane, lane + 32, ... for all k columns, then a
 // fixed shuffle tree per column (deterministic).  Reads Ainv once; no padded columns.
 template <class T>
@@ -768,22 +835,47 @@ int dense_apply_splits(int n, int k) {
 }
 
 void launch_dense_apply(DType t, const void *Ainv, const void *B, void *Y, int n, int k, void *part, cudaStream_t s) {
-  if (k <= 8) {
+  // one warp per row on up to three columns: with fewer columns than that the rows of the
+  // matrix, not the columns, have to be read by consecutive lanes
+  if (k < 4) {
     const unsigned g = resident_grid(((size_t)n * 32 + 255) / 256, 8);
-    MLMC_DISPATCH(t, T, {
-      if (k <= 4)
-        k_dense_apply_narrow<T, 4><<<g, 256, 0, s>>>((const T *)Ainv, (const T *)B, (T *)Y, n, k);
-      else
-        k_dense_apply_narrow<T, 8><<<g, 256, 0, s>>>((const T *)Ainv, (const T *)B, (T *)Y, n, k);
-    });
+    MLMC_DISPATCH(t, T, k_dense_apply_narrow<T, 4><<<g, 256, 0, s>>>((const T *)Ainv, (const T *)B, (T *)Y, n, k));
     MLMC_LAUNCH_CHECK("k_dense_apply_narrow");
+    return;
+  }
+  const bool fp64 = t == F64 || t == C64;
+  if (fp64 || n * (t == C32 ? 2 : 1) < 512) {
+    // rows per thread: the fewest (blocks on the busiest SM) x rows; more rows where that is
+    // equal, since B is read once per row group
+    int R = 4;
+    size_t best = ~(size_t)0;
+    for (int r : {4, 2, 1}) {
+      const size_t blocks = ((size_t)((n + r - 1) / r) * k + 31) / 32, cost = (blocks + 151) / 152 * r;
+      if (cost < best) {
+        best = cost;
+        R = r;
+      }
+    }
+    const unsigned g = (unsigned)(((size_t)((n + R - 1) / R) * k + 31) / 32);
+    MLMC_DISPATCH(t, T, {
+      constexpr int VJ = 16 / (int)sizeof(T);
+      const int chunk = ((n + 7) / 8 + VJ - 1) / VJ * VJ, vec = n % VJ == 0 && ((uintptr_t)Ainv & 15) == 0;
+      auto go = [&](auto r) {
+        k_dense_spread<T, decltype(r)::value><<<g, 256, 0, s>>>((const T *)Ainv, (const T *)B, (T *)Y, n, k, chunk, vec);
+      };
+      if (R == 4) go(std::integral_constant<int, 4>());
+      else if (R == 2) go(std::integral_constant<int, 2>());
+      else go(std::integral_constant<int, 1>());
+    });
+    MLMC_LAUNCH_CHECK("k_dense_spread");
     return;
   }
   int splits = part ? dense_apply_splits(n, k) : 1;
   int jchunk = (n + splits - 1) / splits;
   jchunk = (jchunk + DA_BK - 1) / DA_BK * DA_BK;
   dim3 g((k + DA_BN - 1) / DA_BN, (n + DA_BM - 1) / DA_BM, splits);
-  MLMC_DISPATCH(t, T, {
+  auto go = [&](auto tag) {
+    typedef decltype(tag) T;
     if (splits == 1) {
       k_dense_apply<T><<<g, 128, 0, s>>>((const T *)Ainv, (const T *)B, (T *)Y, n, k, jchunk);
     } else {
@@ -791,7 +883,9 @@ void launch_dense_apply(DType t, const void *Ainv, const void *B, void *Y, int n
       size_t cnt = (size_t)n * k;
       k_dense_sum<T><<<grid_for(cnt, 256), 256, 0, s>>>((const T *)part, splits, cnt, (T *)Y);
     }
-  });
+  };
+  if (t == F32) go(float());
+  else go(cfloat());
   MLMC_LAUNCH_CHECK("k_dense_apply");
 }
 

@@ -1233,13 +1233,12 @@ void setup(H_t &h, const mlmc_operator_desc *op, const mlmc_hierarchy_params *p,
       }
     } else {
       Lv.Ainv64.alloc(Lv.n * Lv.n * es);
-      size_t most = 0;     // the split count depends on the column count of a call
-      for (int kk = 1; kk <= std::max(h.kbig, p->n_tv); ++kk)
-        most = std::max(most, (size_t)dense_apply_splits((int)Lv.n, kk) * kk);
-      size_t part_bytes = most * Lv.n * es;
+      // partial products of the FP32 cycle's apply; their number depends on the column count of a call
+      size_t part_bytes = 0;
       if (mixed)
         for (int kk = 1; kk <= std::max(h.kbig, p->n_tv); ++kk)
-          part_bytes = std::max(part_bytes, dense_apply_tc_part_bytes(dtype_lower(h.t64), (int)Lv.n, kk));
+          part_bytes = std::max({part_bytes, (size_t)dense_apply_splits((int)Lv.n, kk) * kk * Lv.n * es32,
+                                 dense_apply_tc_part_bytes(dtype_lower(h.t64), (int)Lv.n, kk)});
       Lv.dense_part.alloc(part_bytes);
       if (mixed) Lv.Ainv32.alloc(Lv.n * Lv.n * es32);
     }
