@@ -60,12 +60,12 @@ __device__ __forceinline__ double acc_value(double a) { return a; }
 __device__ __forceinline__ void dot_fma(float a[1], float x, float y) { a[0] += x * y; }
 __device__ __forceinline__ void dot_fma(double a[1], double x, double y) { a[0] += x * y; }
 __device__ __forceinline__ void dot_fma(float a[2], cfloat x, cfloat y) {
-  a[0] += x.re * y.re + x.im * y.im;
-  a[1] += x.re * y.im - x.im * y.re;
+  a[0] = fma(x.im, y.im, fma(x.re, y.re, a[0]));
+  a[1] = fma(-x.im, y.re, fma(x.re, y.im, a[1]));
 }
 __device__ __forceinline__ void dot_fma(double a[2], cdouble x, cdouble y) {
-  a[0] += x.re * y.re + x.im * y.im;
-  a[1] += x.re * y.im - x.im * y.re;
+  a[0] = fma(x.im, y.im, fma(x.re, y.re, a[0]));
+  a[1] = fma(-x.im, y.re, fma(x.re, y.im, a[1]));
 }
 
 template <class T> struct VecList { const T *v[DOT_MAXV]; };
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(DT, 2) k_axpy(T *__restrict__ w, VecList<T> V,
 #pragma unroll
         for (int q = 0; q < U; ++q)
 #pragma unroll
-          for (int u = 0; u < VEC; ++u) a[q].v[u] = a[q].v[u] + x[q].v[u] * hh.v[u];
+          for (int u = 0; u < VEC; ++u) a[q].v[u] = madd(a[q].v[u], x[q].v[u], hh.v[u]);
       }
 #pragma unroll
       for (int q = 0; q < U; ++q)

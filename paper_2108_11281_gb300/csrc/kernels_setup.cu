@@ -190,8 +190,8 @@ __global__ void k_galerkin(const T *coef, const T *P, T *cc, int nx, int ny, int
         for (int a = 0; a < d; ++a) {
           T left = conj(PI[(size_t)(loc * d + a) * dc + p]);
           T inner = zero<T>();
-          for (int b = 0; b < d; ++b) inner = inner + B[a * d + b] * PJ[(size_t)(locj * d + b) * dc + q];
-          acc = acc + left * inner;
+          for (int b = 0; b < d; ++b) inner = madd(inner, B[a * d + b], PJ[(size_t)(locj * d + b) * dc + q]);
+          acc = madd(acc, left, inner);
         }
       }
     }
@@ -692,14 +692,14 @@ __global__ void __launch_bounds__(256) k_dense_spread(const T *__restrict__ A, c
 #pragma unroll
       for (int q = 0; q < VJ; ++q)
 #pragma unroll
-        for (int r = 0; r < R; ++r) acc[r] = acc[r] + av[r][q] * bv[q];
+        for (int r = 0; r < R; ++r) acc[r] = madd(acc[r], av[r][q], bv[q]);
     }
   }
 #pragma unroll 4
   for (; j < j1; ++j) {
     const T bv = b[(size_t)j * k];
 #pragma unroll
-    for (int r = 0; r < R; ++r) acc[r] = acc[r] + a[r][j] * bv;
+    for (int r = 0; r < R; ++r) acc[r] = madd(acc[r], a[r][j], bv);
   }
 #pragma unroll
   for (int r = 0; r < R; ++r) red[warp][r][lane] = acc[r];
@@ -756,7 +756,7 @@ __global__ void __launch_bounds__(128) k_dense_apply(const T *__restrict__ A, co
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = acc[a][b] + av[a] * bv[b];
+        for (int b = 0; b < 4; ++b) acc[a][b] = madd(acc[a][b], av[a], bv[b]);
     }
     __syncthreads();
   }
@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(256) k_dense_apply_narrow(const T *__restrict_
       const T *Bj = B + (size_t)j * k;
 #pragma unroll
       for (int c = 0; c < KN; ++c)
-        if (c < k) acc[c] = acc[c] + a * Bj[c];
+        if (c < k) acc[c] = madd(acc[c], a, Bj[c]);
     }
 #pragma unroll
     for (int c = 0; c < KN; ++c) {

@@ -71,7 +71,7 @@ __device__ __forceinline__ void stencil_body(const T *__restrict__ coef, const T
 #pragma unroll
         for (int q = 0; q < D; ++q)
 #pragma unroll
-          for (int u = 0; u < VEC; ++u) acc[r][u] = acc[r][u] + row[q] * xq[q].v[u];
+          for (int u = 0; u < VEC; ++u) acc[r][u] = madd(acc[r][u], row[q], xq[q].v[u]);
       }
     }
     size_t o = (size_t)s * D * kv + c;
@@ -173,14 +173,14 @@ __global__ void __launch_bounds__(256) k_stencil_rows(const T *__restrict__ coef
     if constexpr (CV == 1) {
       const T *xs = x + (size_t)nb[dir] * D * k + c;
 #pragma unroll
-      for (int q = 0; q < D; ++q) acc[0] = acc[0] + row[q] * xs[(size_t)q * k];
+      for (int q = 0; q < D; ++q) acc[0] = madd(acc[0], row[q], xs[(size_t)q * k]);
     } else {
       const V *xs = reinterpret_cast<const V *>(x + (size_t)nb[dir] * D * k + c);
 #pragma unroll
       for (int q = 0; q < D; ++q) {
         const V xv = xs[(size_t)q * kv];
 #pragma unroll
-        for (int u = 0; u < CV; ++u) acc[u] = acc[u] + row[q] * xv.v[u];
+        for (int u = 0; u < CV; ++u) acc[u] = madd(acc[u], row[q], xv.v[u]);
       }
     }
   }
@@ -546,7 +546,7 @@ __device__ __forceinline__ void rbgs_half_body(const T *__restrict__ coef, const
 #pragma unroll
           for (int q = 0; q < D; ++q)
 #pragma unroll
-            for (int u = 0; u < VEC; ++u) res[r][u] = res[r][u] - row[q] * xq[q].v[u];
+            for (int u = 0; u < VEC; ++u) res[r][u] = msub(res[r][u], row[q], xq[q].v[u]);
         }
       }
     }
@@ -562,7 +562,7 @@ __device__ __forceinline__ void rbgs_half_body(const T *__restrict__ coef, const
 #pragma unroll
       for (int q = 0; q < D; ++q)
 #pragma unroll
-        for (int u = 0; u < VEC; ++u) out.v[u] = out.v[u] + row[q] * res[q][u];
+        for (int u = 0; u < VEC; ++u) out.v[u] = madd(out.v[u], row[q], res[q][u]);
       X[o + (size_t)r * kv] = out;
     }
   }
@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(256) k_rbgs_half_rows(const T *__restrict__ co
         for (int q = 0; q < D; ++q) {
           const V xv = xs[(size_t)q * kv];
 #pragma unroll
-          for (int u = 0; u < CV; ++u) acc[u] = acc[u] - row[q] * xv.v[u];
+          for (int u = 0; u < CV; ++u) acc[u] = msub(acc[u], row[q], xv.v[u]);
         }
       }
     }
@@ -663,7 +663,7 @@ __global__ void __launch_bounds__(256) k_rbgs_half_rows(const T *__restrict__ co
 #pragma unroll
     for (int q = 0; q < D; ++q)
 #pragma unroll
-      for (int u = 0; u < CV; ++u) out.v[u] = out.v[u] + di[q] * res[q][cl * CV + u];
+      for (int u = 0; u < CV; ++u) out.v[u] = madd(out.v[u], di[q], res[q][cl * CV + u]);
     *reinterpret_cast<V *>(x + ((size_t)s * D + r) * k + c) = out;
   }
 }

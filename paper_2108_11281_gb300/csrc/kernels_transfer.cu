@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(128) k_restrict(const T *__restrict__ P, const
           for (int q = 0; q < QG; ++q) {
             T pq = conj(Pr[q]);
 #pragma unroll
-            for (int u = 0; u < VEC; ++u) acc[q][u] = acc[q][u] + pq * xv[b8].v[u];
+            for (int u = 0; u < VEC; ++u) acc[q][u] = madd(acc[q][u], pq, xv[b8].v[u]);
           }
         }
       }
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(256) k_restrict_split(const T *__restrict__ P,
       for (int q = 0; q < QG; ++q) {
         const T pq = conj(Pr[q]);
 #pragma unroll
-        for (int u = 0; u < VEC; ++u) acc[q][u] = acc[q][u] + pq * xv.v[u];
+        for (int u = 0; u < VEC; ++u) acc[q][u] = madd(acc[q][u], pq, xv.v[u]);
       }
     }
   }
@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(256) k_prolong_add(const T *__restrict__ P, co
       for (int q = 0; q < DC; ++q) {
         T pq = Pr[q];
 #pragma unroll
-        for (int u = 0; u < VEC; ++u) xv.v[u] = xv.v[u] + pq * e[q].v[u];
+        for (int u = 0; u < VEC; ++u) xv.v[u] = madd(xv.v[u], pq, e[q].v[u]);
       }
       X[o] = xv;
     }
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(KC * RR_SLOTS, 256 / (KC * RR_SLOTS) * 4) k_re
           for (int q = 0; q < D; ++q) {
             const T w = Bd[a * D + q];
 #pragma unroll
-            for (int u = 0; u < VEC; ++u) r[a][u] = r[a][u] - w * xq[q].v[u];
+            for (int u = 0; u < VEC; ++u) r[a][u] = msub(r[a][u], w, xq[q].v[u]);
           }
       }
 #pragma unroll
@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(KC * RR_SLOTS, 256 / (KC * RR_SLOTS) * 4) k_re
         for (int q = 0; q < DC; ++q) {
           const T pq = conj(Pr[q]);
 #pragma unroll
-          for (int u = 0; u < VEC; ++u) acc[q][u] = acc[q][u] + pq * r[a][u];
+          for (int u = 0; u < VEC; ++u) acc[q][u] = madd(acc[q][u], pq, r[a][u]);
         }
       }
     }
@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(128) k_laplace_residual_restrict(const T *__re
       for (int q = 0; q < DC; ++q) {
         const T pq = Pr[q];
 #pragma unroll
-        for (int u = 0; u < VEC; ++u) acc[q][u] = acc[q][u] + pq * r[u];
+        for (int u = 0; u < VEC; ++u) acc[q][u] = madd(acc[q][u], pq, r[u]);
       }
     }
 #pragma unroll
