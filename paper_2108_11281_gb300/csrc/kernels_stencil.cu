@@ -284,8 +284,7 @@ __device__ __forceinline__ void laplace_nbr_sum(const Pack<T, VEC> *__restrict__
 // y = diag x - (sum of the in-grid neighbours) (mode 0) or r = b - that (mode 1),
 // VEC columns per thread with 16-byte loads; grid.y = lattice row, so the +-y
 // neighbours of a block are the rows just touched by the blocks before it (L2
-// hits).  Per element: three additions and one fused multiply-add (FP64 lanes
-// are the limit of the FP64 form on GB300).
+// hits).  FP32; FP64 data take k_laplace_march.
 template <class T, int VEC>
 __device__ __forceinline__ void laplace_body(const T *__restrict__ x, const T *__restrict__ b, T *__restrict__ y,
                                              int nx, int ny, int kv, T diag, int periodic, int mode, int j, int t) {
@@ -310,9 +309,7 @@ __device__ __forceinline__ void laplace_body(const T *__restrict__ x, const T *_
   ((V *)y)[(size_t)s * kv + c] = out;
 }
 
-// Resident grid striding over the units (row j, chunk of 256 threads of the row) in row
-// order: the FP64 apply is bound by the FP64 pipe, which a grid of one block per unit
-// leaves idle between blocks.
+// Resident grid striding over the units (row j, chunk of 256 threads of the row) in row order.
 template <class T, int VEC>
 __global__ void __launch_bounds__(256) k_laplace(const T *__restrict__ x, const T *__restrict__ b, T *__restrict__ y,
                                                  int nx, int ny, int kv, T diag, int periodic, int mode, int bpr) {
@@ -370,79 +367,145 @@ static int laplace_vec(int k) {
   return k % v == 0 ? v : 1;
 }
 
-// One damped-Jacobi sweep of the setup filter for Example 5.1 in one pass:
-// out = x - omega D^-1 (A x) with A x = diag x - (sum of the in-grid neighbours), written
-// as (1 - omega) x + (omega / diag) (sum of the neighbours): one multiply, one FMA and
-// the three additions of the sum per element (out must not alias x).
-template <class T, int VEC>
-__device__ __forceinline__ void laplace_jacobi_body(const T *__restrict__ x, T *__restrict__ out, int nx, int ny,
-                                                    int kv, T keep, T scale, int periodic, int j, int t) {
-  typedef Pack<T, VEC> V;
-  if (t >= nx * kv) return;
-  const int i = t / kv, c = t - (t / kv) * kv;
-  const V *X = (const V *)x;
-  const int s = j * nx + i;
-  const Nbrs n = laplace_nbrs(i, j, nx, ny, periodic);
-  const V xc = X[(size_t)s * kv + c];
-  T sum[VEC];
-  laplace_nbr_sum<T, VEC>(X, n, kv, c, sum);
-  V o;
+// ------------------------------------------------------------------ Example 5.1 in FP64
+// Bound by the FP64 pipe (1.7 - 2 operations per clock and SM).  The neighbour sum of site
+// (i, j) is u(i, j) + u(i - 1, j - 1) with u(i, j) = x(i + 1, j) + x(i, j + 1): each u serves two
+// sites, so a site costs about two additions and one multiply-add instead of three and one.
+// A thread holds a strip of MP lattice columns (one 16-byte pack of right-hand sides) and walks
+// up JB rows, keeping the last row's u; a site's x is loaded about 1.5 times instead of five.
+// The additions are issued as multiply-adds by 1 (same result; 0.63 against 0.53 T/s).
+// 1024^2 x 64: 402 us (3.3 operations per site: 350 us at the measured rate), 531 us with the
+// neighbour sum per site.
+enum { LAP_APPLY = 0, LAP_RESIDUAL = 1, LAP_JACOBI = 2 };
+constexpr int MP = 4;
+
+template <int VEC, int MODE>
+__global__ void __launch_bounds__(128) k_laplace_march(const double *__restrict__ x, const double *__restrict__ b,
+                                                       double *__restrict__ y, int nx, int ny, int kv, double diag,
+                                                       double scale, double one, int periodic, int JB) {
+  typedef Pack<double, VEC> V;
+  const unsigned strips = (nx + MP - 1) / MP, segs = (ny + JB - 1) / JB;
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= strips * segs * (unsigned)kv) return;
+  const unsigned q = t / (unsigned)kv;
+  const int c = (int)(t - q * (unsigned)kv);
+  const int i0 = (int)(q % strips) * MP, j0 = (int)(q / strips) * JB, j1 = min(ny, j0 + JB);
+  // lattice columns i0 - 1 .. i0 + MP: offsets into a row; a column outside a Dirichlet lattice, or
+  // more than one past the end, reads as zero
+  int col[MP + 2];
+  unsigned on = 0;
 #pragma unroll
-  for (int u = 0; u < VEC; ++u) o.v[u] = keep * xc.v[u] + scale * sum[u];
-  ((V *)out)[(size_t)s * kv + c] = o;
-}
-
-template <class T, int VEC>
-__global__ void __launch_bounds__(256) k_laplace_jacobi(const T *__restrict__ x, T *__restrict__ out, int nx, int ny,
-                                                        int kv, T keep, T scale, int periodic, int bpr) {
-  const int units = bpr * ny;
-  for (int u = blockIdx.x; u < units; u += gridDim.x) {
-    const int j = u / bpr;
-    laplace_jacobi_body<T, VEC>(x, out, nx, ny, kv, keep, scale, periodic, j, (u - j * bpr) * 256 + threadIdx.x);
+  for (int u = 0; u < MP + 2; ++u) {
+    int i = i0 + u - 1;
+    bool ok = i >= 0 && i < nx;
+    if (!ok && periodic && i <= nx) {
+      i = i < 0 ? nx - 1 : 0;
+      ok = true;
+    }
+    on |= (unsigned)ok << u;
+    col[u] = (ok ? i : 0) * kv + c;
   }
-}
-
-void launch_laplace_jacobi(const StencilView &A, const void *x, void *out, int k, double omega, cudaStream_t s) {
-  if (!A.const_laplace) throw cuda_error{cudaErrorInvalidValue, "laplace_jacobi: constant-coefficient Laplacian only"};
-  auto go = [&](auto tag, auto vtag) {
-    typedef decltype(tag) T;
-    constexpr int VEC = decltype(vtag)::value;
-    const int kv = k / VEC;
-    const T keep = (T)(1.0 - omega), scale = (T)(omega / A.diag);
-    const int bpr = (A.nx * kv + 255) / 256;
-    static const int occ = blocks_per_sm(k_laplace_jacobi<T, VEC>, 256, 0);
-    k_laplace_jacobi<T, VEC><<<resident_grid((size_t)bpr * A.ny, occ), 256, 0, s>>>(
-        (const T *)x, (T *)out, A.nx, A.ny, kv, keep, scale, A.periodic, bpr);
+  const V *X = (const V *)x;
+  auto load = [&](int j, V v[MP + 2]) {
+    bool ok = j >= 0 && j < ny;
+    if (!ok && periodic) {
+      j = j < 0 ? ny - 1 : 0;
+      ok = true;
+    }
+    const V *row = X + (size_t)(ok ? j : 0) * nx * kv;
+#pragma unroll
+    for (int u = 0; u < MP + 2; ++u) {
+      if (ok && (on >> u & 1)) {
+        v[u] = row[col[u]];
+      } else {
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) v[u].v[e] = 0.0;
+      }
+    }
   };
-  if (A.t == F64) {
-    if (laplace_vec<double>(k) == 2) go(double(), std::integral_constant<int, 2>());
-    else go(double(), std::integral_constant<int, 1>());
-  } else if (A.t == F32) {
-    if (laplace_vec<float>(k) == 4) go(float(), std::integral_constant<int, 4>());
-    else go(float(), std::integral_constant<int, 1>());
-  } else {
-    throw cuda_error{cudaErrorInvalidValue, "constant-coefficient Laplacian is real"};
+  V cur[MP + 2], nxt[MP + 2], up[MP];
+  load(j0 - 1, nxt);
+  load(j0, cur);
+#pragma unroll
+  for (int m = 0; m < MP; ++m)
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) up[m].v[e] = fma(nxt[m + 1].v[e], one, cur[m].v[e]);
+#pragma unroll 2
+  for (int j = j0; j < j1; ++j) {
+    load(j + 1, nxt);
+    V u[MP + 1];                              // u(i0 - 1 + m, j)
+#pragma unroll
+    for (int m = 0; m <= MP; ++m)
+#pragma unroll
+      for (int e = 0; e < VEC; ++e) u[m].v[e] = fma(cur[m + 1].v[e], one, nxt[m].v[e]);
+    const size_t row = (size_t)j * nx * kv;
+#pragma unroll
+    for (int p = 0; p < MP; ++p) {
+      if (i0 + p < nx) {
+        V out;
+        if (MODE == LAP_RESIDUAL) out = ((const V *)b)[row + col[p + 1]];
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) {
+          const double sum = fma(u[p + 1].v[e], one, up[p].v[e]), xc = cur[p + 1].v[e];
+          if (MODE == LAP_APPLY) out.v[e] = fma(diag, xc, -sum);
+          if (MODE == LAP_RESIDUAL) out.v[e] = fma(-diag, xc, fma(sum, one, out.v[e]));
+          if (MODE == LAP_JACOBI) out.v[e] = fma(scale, sum, diag * xc);
+        }
+        ((V *)y)[row + col[p + 1]] = out;
+      }
+    }
+#pragma unroll
+    for (int m = 0; m < MP; ++m) up[m] = u[m];
+#pragma unroll
+    for (int m = 0; m < MP + 2; ++m) cur[m] = nxt[m];
   }
-  MLMC_LAUNCH_CHECK("k_laplace_jacobi");
+}
+
+template <int MODE>
+static void laplace_march(const StencilView &A, const void *x, const void *b, void *y, int k, double diag, double scale,
+                          cudaStream_t s) {
+  const int vec = k % 2 == 0 ? 2 : 1, kv = k / vec;
+  const size_t strips = (A.nx + MP - 1) / MP;
+  // long walks recompute least (one u per strip column and walk); shorter ones where the grid
+  // would not fill the SMs
+  int JB = 64;
+  while (JB > 2 && strips * ((A.ny + JB - 1) / JB) * kv < (size_t)152 * 512) JB /= 2;
+  const size_t threads = strips * ((A.ny + JB - 1) / JB) * kv;
+  const unsigned g = (unsigned)((threads + 127) / 128);
+  if (vec == 2)
+    k_laplace_march<2, MODE><<<g, 128, 0, s>>>((const double *)x, (const double *)b, (double *)y, A.nx, A.ny, kv, diag,
+                                               scale, 1.0, A.periodic, JB);
+  else
+    k_laplace_march<1, MODE><<<g, 128, 0, s>>>((const double *)x, (const double *)b, (double *)y, A.nx, A.ny, kv, diag,
+                                               scale, 1.0, A.periodic, JB);
+}
+
+// One damped-Jacobi sweep of the setup filter for Example 5.1 in one pass (out must not alias x):
+// x - omega D^-1 (A x) with A x = diag x - (sum of the in-grid neighbours), written as
+// (1 - omega) x + (omega / diag) (sum of the neighbours).
+void launch_laplace_jacobi(const StencilView &A, const void *x, void *out, int k, double omega, cudaStream_t s) {
+  if (!A.const_laplace || A.t != F64)
+    throw cuda_error{cudaErrorInvalidValue, "laplace_jacobi: constant-coefficient Laplacian in FP64 only"};
+  laplace_march<LAP_JACOBI>(A, x, nullptr, out, k, 1.0 - omega, omega / A.diag, s);
+  MLMC_LAUNCH_CHECK("k_laplace_march");
 }
 
 static void launch_laplace(const StencilView &A, const void *x, const void *b, void *y, int k, int mode,
                            cudaStream_t s) {
-  auto go = [&](auto tag, auto vtag) {
-    typedef decltype(tag) T;
-    constexpr int VEC = decltype(vtag)::value;
-    int kv = k / VEC;
-    const int bpr = (A.nx * kv + 255) / 256;
-    static const int occ = blocks_per_sm(k_laplace<T, VEC>, 256, 0);
-    k_laplace<T, VEC><<<resident_grid((size_t)bpr * A.ny, occ), 256, 0, s>>>(
-        (const T *)x, (const T *)b, (T *)y, A.nx, A.ny, kv, (T)A.diag, A.periodic, mode, bpr);
-  };
   if (A.t == F64) {
-    if (laplace_vec<double>(k) == 2) go(double(), std::integral_constant<int, 2>());
-    else go(double(), std::integral_constant<int, 1>());
+    if (mode) laplace_march<LAP_RESIDUAL>(A, x, b, y, k, A.diag, 0.0, s);
+    else laplace_march<LAP_APPLY>(A, x, b, y, k, A.diag, 0.0, s);
   } else if (A.t == F32) {
-    if (laplace_vec<float>(k) == 4) go(float(), std::integral_constant<int, 4>());
-    else go(float(), std::integral_constant<int, 1>());
+    auto go = [&](auto vtag) {
+      constexpr int VEC = decltype(vtag)::value;
+      int kv = k / VEC;
+      const int bpr = (A.nx * kv + 255) / 256;
+      static const int occ = blocks_per_sm(k_laplace<float, VEC>, 256, 0);
+      k_laplace<float, VEC><<<resident_grid((size_t)bpr * A.ny, occ), 256, 0, s>>>(
+          (const float *)x, (const float *)b, (float *)y, A.nx, A.ny, kv, (float)A.diag, A.periodic, mode, bpr);
+    };
+    if (laplace_vec<float>(k) == 4) go(std::integral_constant<int, 4>());
+    else go(std::integral_constant<int, 1>());
   } else {
     throw cuda_error{cudaErrorInvalidValue, "constant-coefficient Laplacian is real"};
   }
