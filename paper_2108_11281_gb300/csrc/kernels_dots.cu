@@ -460,7 +460,9 @@ void launch_multiaxpy(DType t, void *w, const void *V, size_t vstride, int nvec,
 // share would otherwise take longer than its loads.  Per step they stand in place of two
 // reductions of one warp per output (4.7 us each, strided loads), a cleared counter and a
 // per-column Givens kernel (4.7 us, 9 us complex; a 4-byte memset node costs 4 us and the
-// kernel after it 5 us of gap in a replayed graph): k_fgmres_mid takes 3.4 us.
+// kernel after it 5 us of gap in a replayed graph): k_fgmres_mid takes 3.3 us, k_fgmres_tail 8.3
+// (two steps, FP32 data; mostly dependent FP64 instructions, so what earlier steps left is
+// loaded before the sums, and the norm of u_j is added up with the dots: 3.5 and 10 us before).
 namespace {
 
 template <class T> struct fg {
@@ -474,20 +476,28 @@ template <class T> struct fg {
 };
 
 // sums[r * ET + e] (r < nrows, e < ET) = scalar e0 + e of output row r summed over the parts in
-// fixed order; parts are nrows * E scalars apart, rows E.  red: TR * RT sums.
+// fixed order; parts are nrows * E scalars apart, rows E.  With norm (nullable; parts k columns
+// apart) also nsum[c] = column c0 + c of it, c < CB, in the same pass.  red: (TR + 1) * RT sums.
 constexpr int TR = 8;              // rows whose loads are in flight together
 template <class T>
 __device__ void tile_sum(const typename lane_of<T>::A *__restrict__ partial, int nparts, int nrows, int E, int e0,
-                         typename lane_of<T>::A *red, double *sums) {
+                         const typename lane_of<T>::A *__restrict__ norm, int norm_parts, int k, int c0,
+                         typename lane_of<T>::A *red, double *sums, double *nsum) {
   typedef typename lane_of<T>::A A;
-  constexpr int ET = fg<T>::ET, SL = fg<T>::SL;
+  constexpr int ET = fg<T>::ET, SL = fg<T>::SL, CB = fg<T>::CB;
   const int e = threadIdx.x % ET, sl = threadIdx.x / ET;
   const size_t stride = (size_t)nrows * E;
   for (int r0 = 0; r0 < nrows; r0 += TR) {
     const int nr = min(nrows - r0, TR);
-    A a[TR];
+    const bool with_norm = r0 == 0 && norm;
+    A a[TR], an;
+    acc_zero(an);
 #pragma unroll
     for (int r = 0; r < TR; ++r) acc_zero(a[r]);
+    if (with_norm && e < CB && c0 + e < k) {
+#pragma unroll 4
+      for (int p = sl; p < norm_parts; p += SL) acc_add(an, norm[(size_t)p * k + c0 + e]);
+    }
     if (e0 + e < E) {
       const A *src = partial + (size_t)r0 * E + e0 + e;
 #pragma unroll 2
@@ -504,20 +514,23 @@ __device__ void tile_sum(const typename lane_of<T>::A *__restrict__ partial, int
 #pragma unroll
     for (int r = 0; r < TR; ++r)
       if (r < nr) red[(r * SL + sl) * ET + e] = a[r];
+    if (with_norm) red[(nr * SL + sl) * ET + e] = an;
+    const int rows = nr + with_norm;
     __syncthreads();
     // eight threads per sum take the slices q, q + 8, ...; then one adds the eight
-    for (int t = threadIdx.x; t < nr * ET * 8; t += RT) {
+    for (int t = threadIdx.x; t < rows * ET * 8; t += RT) {
       const int q = t & 7, re = t >> 3, r = re / ET, ee = re % ET;
       A v = red[(r * SL + q) * ET + ee];
       for (int s2 = q + 8; s2 < SL; s2 += 8) acc_add(v, red[(r * SL + s2) * ET + ee]);
       red[(r * SL + q) * ET + ee] = v;
     }
     __syncthreads();
-    for (int re = threadIdx.x; re < nr * ET; re += RT) {
+    for (int re = threadIdx.x; re < rows * ET; re += RT) {
       const int r = re / ET, ee = re % ET;
       A v = red[(r * SL) * ET + ee];
       for (int q = 1; q < 8; ++q) acc_add(v, red[(r * SL + q) * ET + ee]);
-      sums[(r0 + r) * ET + ee] = acc_value(v);
+      if (r < nr) sums[(r0 + r) * ET + ee] = acc_value(v);
+      else if (ee < CB) nsum[ee] = acc_value(v);
     }
     __syncthreads();
   }
@@ -533,21 +546,17 @@ __device__ __forceinline__ cdouble shfl(cdouble v, int l) { return {shfl(v.re, l
 }  // namespace
 
 // The tile's sums for step j: dots (rows d_0 .. d_j, then v0.v0 when j = 0, then extra rows)
-// into sums, and n_j into n2[j] (global) and nj[c] (shared).
+// into sums, and n_j into nj[c] (shared) and n2[j] (global).
 template <class T>
 __device__ void fgmres_sums(const typename lane_of<T>::A *partial, int nparts, int nrows,
                             const typename lane_of<T>::A *norm, int norm_parts, int j, int k, int c0, double *n2,
-                            typename lane_of<T>::A *red, double *sums, double *nsum, double *nj) {
+                            typename lane_of<T>::A *red, double *sums, double *nj) {
   constexpr int C = fg<T>::C, ET = fg<T>::ET, CB = fg<T>::CB;
-  typedef typename real_of<T>::type R;
-  // a real tile of ET scalars covers this tile's CB columns (complex: also the next tile's)
-  if (j > 0) tile_sum<R>(norm, norm_parts, 1, k, c0, red, nsum);
-  tile_sum<T>(partial, nparts, nrows, k * C, c0 * C, red, sums);
+  tile_sum<T>(partial, nparts, nrows, k * C, c0 * C, j > 0 ? norm : nullptr, norm_parts, k, c0, red, sums, nj);
   if (threadIdx.x < CB) {
     const int c = threadIdx.x;
-    const double n = j > 0 ? nsum[c] : sums[ET + c * C];
-    nj[c] = n;
-    if (c0 + c < k) n2[(size_t)j * k + c0 + c] = n;
+    if (j == 0) nj[c] = sums[ET + c * C];
+    if (c0 + c < k) n2[(size_t)j * k + c0 + c] = nj[c];
   }
   __syncthreads();
 }
@@ -556,76 +565,77 @@ __device__ void fgmres_sums(const typename lane_of<T>::A *partial, int nparts, i
 template <class T>
 __global__ void __launch_bounds__(RT) k_fgmres_mid(const typename lane_of<T>::A *__restrict__ partial, int nparts,
                                                    int nrows, const typename lane_of<T>::A *__restrict__ norm,
-                                                   int norm_parts, int j, int m, int k, double *__restrict__ n2,
+                                                   int norm_parts, int j, int m, int k, double *n2,
                                                    typename acc_of<T>::type *__restrict__ D, T *__restrict__ coef) {
   typedef typename acc_of<T>::type H;
   constexpr int ET = fg<T>::ET, CB = fg<T>::CB;
-  __shared__ typename lane_of<T>::A red[TR * RT];
-  __shared__ double sums[fg<T>::MAXROWS * ET], nsum[8], nj[8];
+  __shared__ typename lane_of<T>::A red[(TR + 1) * RT];
+  __shared__ double sums[fg<T>::MAXROWS * ET], nj[8];
   const int c0 = blockIdx.x * CB;
-  fgmres_sums<T>(partial, nparts, nrows, norm, norm_parts, j, k, c0, n2, red, sums, nsum, nj);
-  for (int t = threadIdx.x; t < (j + 1) * CB; t += RT) {
-    const int i = t / CB, c = t - i * CB;
-    if (c0 + c >= k) continue;
-    const double n = usable(i == j ? nj[c] : n2[(size_t)i * k + c0 + c]);
-    const H d = at(sums + i * ET, c, H());
-    D[((size_t)j * (m + 1) + i) * k + c0 + c] = d;
-    coef[(size_t)i * k + c0 + c] = cvt<T, H>(rmul(-1.0 / n, d));
-  }
+  // thread (i, c): the norm of u_i is loaded before the sums (at most 32 vectors x 8 columns)
+  const int i = threadIdx.x / CB, c = threadIdx.x - (threadIdx.x / CB) * CB;
+  const bool mine = i <= j && c0 + c < k;
+  double n = mine && i < j ? n2[(size_t)i * k + c0 + c] : 0.0;
+  fgmres_sums<T>(partial, nparts, nrows, norm, norm_parts, j, k, c0, n2, red, sums, nj);
+  if (!mine) return;
+  n = usable(i == j ? nj[c] : n);
+  const H d = at(sums + i * ET, c, H());
+  D[((size_t)j * (m + 1) + i) * k + c0 + c] = d;
+  coef[(size_t)i * k + c0 + c] = cvt<T, H>(rmul(-1.0 / n, d));
 }
 
 // The last step, j = its - 1, and the least-squares problem: y[i * k + c], i < its.
-// One warp per column; lane q keeps column q of G.
+// One warp per column; lane q keeps column q of G, and the norm of u_q.
 template <class T>
 __global__ void __launch_bounds__(RT) k_fgmres_tail(const typename lane_of<T>::A *__restrict__ partial, int nparts,
                                                     int nrows, const typename lane_of<T>::A *__restrict__ norm,
-                                                    int norm_parts, int its, int m, int k, double *__restrict__ n2,
+                                                    int norm_parts, int its, int m, int k, double *n2,
                                                     const typename acc_of<T>::type *__restrict__ D,
                                                     T *__restrict__ y) {
   typedef typename acc_of<T>::type H;
   constexpr int ET = fg<T>::ET, CB = fg<T>::CB, C = fg<T>::C;
-  __shared__ typename lane_of<T>::A red[TR * RT];
-  __shared__ double sums[fg<T>::MAXROWS * ET], nsum[8], nj[8];
-  __shared__ double sn[CB][33], is[CB][33];
+  __shared__ typename lane_of<T>::A red[(TR + 1) * RT];
+  __shared__ double sums[fg<T>::MAXROWS * ET], nj[8];
   extern __shared__ __align__(16) unsigned char tail_smem[];
   const int c0 = blockIdx.x * CB, j = its - 1;
-  fgmres_sums<T>(partial, nparts, nrows, norm, norm_parts, j, k, c0, n2, red, sums, nsum, nj);
   const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (c >= CB || c0 + c >= k) return;
-  H *G = (H *)tail_smem + (size_t)c * (its + 1) * its;      // G[i * its + q]
+  const bool mine = c < CB && c0 + c < k;
   const size_t cg = c0 + c;
-  // norms s_i = sqrt(n_i): zero for a vanished vector, whose 1 / s_i is 1
-  for (int i = lane; i <= its; i += 32) {
-    double n;
-    if (i == its) {
-      n = sums[(nrows - 1) * ET + c * C];                   // |w|^2
-      for (int l = 0; l < its; ++l) {
-        const H d = at(sums + l * ET, c, H());
-        n -= abs2(d) / usable(l == j ? nj[c] : n2[(size_t)l * k + cg]);
-      }
-    } else {
-      n = i == j ? nj[c] : n2[(size_t)i * k + cg];
-    }
-    const double inv = rsqrt(usable(n));
-    is[c][i] = inv;
-    sn[c][i] = n > 0.0 && isfinite(n) ? n * inv : 0.0;
+  H *G = (H *)tail_smem + (size_t)c * (its + 1) * its;      // G[i * its + q], used by warp c < CB
+  // what earlier steps left is loaded before the sums: norms, and the dots d_iq of the columns q < j
+  double n = mine && lane < j ? n2[(size_t)lane * k + cg] : 0.0;
+  if (mine && lane < j)
+    for (int i = 0; i <= lane; ++i) G[i * its + lane] = D[((size_t)lane * (m + 1) + i) * k + cg];
+  fgmres_sums<T>(partial, nparts, nrows, norm, norm_parts, j, k, c0, n2, red, sums, nj);
+  if (!mine) return;
+  // norms s_q = sqrt(n_q): zero for a vanished vector, whose 1 / s_q is 1
+  if (lane == j) n = nj[c];
+  const double is = lane < its ? rsqrt(usable(n)) : 0.0;
+  const double sq = lane < its && n > 0.0 && isfinite(n) ? n * is : 0.0;
+  // n_its = |w|^2 - sum_q |d_q|^2 / n_q
+  const H dl = lane < its ? at(sums + lane * ET, c, H()) : zero<H>();
+  double part = abs2(rmul(is, dl));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+  const double nl = sums[(nrows - 1) * ET + c * C] - part;
+  const double sl = nl > 0.0 && isfinite(nl) ? nl * rsqrt(nl) : 0.0;
+  const double below = __shfl_down_sync(0xffffffffu, sq, 1);   // s_{q+1}, the subdiagonal of column q
+  if (lane == j)
+    for (int i = 0; i < its; ++i) G[i * its + lane] = at(sums + i * ET, c, H());
+  for (int i = 0; i < its; ++i) {
+    const double v = __shfl_sync(0xffffffffu, is, i);
+    if (lane >= i && lane < its) G[i * its + lane] = rmul(v, G[i * its + lane]);
   }
+  if (lane < its) G[(lane + 1) * its + lane] = make<H>(lane == j ? sl : below, 0.0);
   __syncwarp();
-  if (lane < its) {
-    for (int i = 0; i <= lane; ++i) {
-      const H d = lane == j ? at(sums + i * ET, c, H()) : D[((size_t)lane * (m + 1) + i) * k + cg];
-      G[i * its + lane] = rmul(is[c][i], d);
-    }
-    G[(lane + 1) * its + lane] = make<H>(sn[c][lane + 1], 0.0);
-  }
-  __syncwarp();
-  H g = make<H>(sn[c][0], 0.0), gi = zero<H>();             // lane i keeps entry i of the rotated right-hand side
+  const double s0 = __shfl_sync(0xffffffffu, sq, 0);
+  H g = make<H>(s0, 0.0), gi = zero<H>();                   // lane i keeps entry i of the rotated right-hand side
   double inv = 0.0;                                         // and 1 / R_ii
-  bool active = sn[c][0] > 0.0;
+  bool active = s0 > 0.0;
   int J = 0;
   for (int i = 0; i < its && active; ++i) {
     const H a = G[i * its + i];
-    const double b = sn[c][i + 1], r2 = abs2(a) + b * b;
+    const double b = re(G[(i + 1) * its + i]), r2 = abs2(a) + b * b;
     if (!(r2 > 0.0)) break;
     const double ir = rsqrt(r2);
     const H cc = rmul(ir, a);
