@@ -139,63 +139,108 @@ template <int D> struct gen_vec<cfloat, D> { static const int v = D <= 2 ? 2 : 1
     default: throw cuda_error{cudaErrorInvalidValue, "unsupported dofs per site"}; \
   }
 
-// Row-split variant for large site blocks (d >= 8, the small coarse lattices of the
-// Wilson hierarchy): one thread per (row r of a site, CV consecutive columns)
-// accumulates that row over the 5 blocks; block = 32 x CV columns x D rows of one
-// site.  CV = 2 (16-byte loads for complex FP32) halves the coefficient loads per
-// column (Wilson 128^2, level 2, k = 128: apply 22.6 -> 18.8 us, smoother sweep
-// 32.9 -> 26.9 us).  Each column takes the same operations in the same order in
-// either form; the compiler's FMA contraction may differ in the last bit.
-template <class T, int D, int CV>
-__global__ void __launch_bounds__(256) k_stencil_rows(const T *__restrict__ coef, const T *__restrict__ x,
-                                                      const T *__restrict__ b, T *__restrict__ y, int nx, int ny,
-                                                      int k, int mode) {
+// Row-split kernels for large site blocks (d >= 8, the small coarse lattices of the Wilson
+// hierarchy): one thread per (RPT rows of a site, CV consecutive columns); block = 32 x CV
+// columns x D / RPT row groups of one site.  These levels live in L2 and a launch is a few
+// microseconds, so what counts is one round trip to L2: the site's coefficient blocks (one
+// contiguous run) go to shared memory by cp.async while every thread loads its vector entries
+// of all (or, with wide packs, some) of the neighbours into registers.  Beside that FP32 is
+// bound by the load unit: a broadcast of 16 coefficient bytes takes it as long as 32 lanes'
+// 16-byte vector entries, so two rows per thread share the vector entries and CV = 2 halves
+// the coefficient reads per column.  FP64 is bound by its arithmetic and keeps one row.
+// Wilson 128^2, level 2 (32^2 sites, complex FP32), one row per thread and coefficients through
+// the cache before: smoother sweep 16.4 -> 12.3 us at k = 32 and 27.7 -> 16.6 us at k = 128,
+// apply 8.2 -> 6.2 and 19.5 -> 12.3 us (two rows per thread alone: 18.5 us per sweep at both).
+template <class T> constexpr int rows_rpt() { return sizeof(typename real_of<T>::type) == 4 ? 2 : 1; }
+
+__device__ __forceinline__ void copy16_async(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+// `bytes` (a multiple of 16) from 16-byte aligned src to dst, by the block's threads
+__device__ __forceinline__ void block_copy_async(void *dst, const void *src, int bytes, int tid, int threads) {
+  for (int e = tid * 16; e < bytes; e += threads * 16) copy16_async((char *)dst + e, (const char *)src + e);
+}
+
+// acc[r] +- sum over NDIR neighbour blocks of rows r0 + r (blk: [NDIR][D][D] in shared memory)
+// times their x, XB neighbours' entries in flight at a time.  ready(): called after the first
+// loads are issued and before the coefficients are read.
+template <class T, int D, int CV, int RPT, int NDIR, bool SUB, class F>
+__device__ __forceinline__ void rows_accumulate(const T *blk, const T *x, const int nb[NDIR], int r0, int k, int c,
+                                                bool live, Pack<T, CV> acc[RPT], F ready) {
   typedef Pack<T, CV> V;
+  constexpr int WORDS = D * CV * (int)sizeof(T) / 4;                    // registers of one neighbour
+  constexpr int XB = WORDS * NDIR <= 80 ? NDIR : WORDS <= 32 ? 2 : 1;   // neighbours in flight
+  const int kv = k / CV;
+#pragma unroll
+  for (int d0 = 0; d0 < NDIR; d0 += XB) {
+    V xv[XB][D];
+#pragma unroll
+    for (int e = 0; e < XB; ++e)
+      if (d0 + e < NDIR && live) {
+        const V *xs = reinterpret_cast<const V *>(x + (size_t)nb[d0 + e] * D * k + c);
+#pragma unroll
+        for (int q = 0; q < D; ++q) xv[e][q] = xs[(size_t)q * kv];
+      }
+    asm volatile("" ::: "memory");                                      // the loads stay in front
+    if (d0 == 0) ready();
+#pragma unroll
+    for (int e = 0; e < XB; ++e)
+      if (d0 + e < NDIR) {
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+          T row[D];
+          memcpy(row, __builtin_assume_aligned(blk + ((size_t)(d0 + e) * D + r0 + r) * D, 16), sizeof(row));
+#pragma unroll
+          for (int q = 0; q < D; ++q)
+#pragma unroll
+            for (int u = 0; u < CV; ++u)
+              acc[r].v[u] = SUB ? msub(acc[r].v[u], row[q], xv[e][q].v[u]) : madd(acc[r].v[u], row[q], xv[e][q].v[u]);
+        }
+      }
+  }
+}
+
+__device__ __forceinline__ void async_ready() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+}
+
+template <class T, int D, int CV, int RPT>
+__global__ void __launch_bounds__(32 * D / RPT) k_stencil_rows(const T *__restrict__ coef, const T *x, const T *b,
+                                                               T *y, int nx, int ny, int k, int mode) {
+  typedef Pack<T, CV> V;
+  __shared__ __align__(16) unsigned char blk_mem[5 * D * D * sizeof(T)];
+  const T *blk = (const T *)blk_mem;
   const int s = blockIdx.y;
   const int i = s % nx, j = s / nx;
-  const int r = threadIdx.y;
+  const int r0 = threadIdx.y * RPT;
   const int c = (blockIdx.x * 32 + threadIdx.x) * CV;   // k is a multiple of CV
-  if (c >= k) return;
+  const bool live = c < k;
+  block_copy_async(blk_mem, coef + (size_t)s * 5 * D * D, 5 * D * D * (int)sizeof(T), threadIdx.y * 32 + threadIdx.x,
+                   32 * D / RPT);
   int nb[5];
   nb[0] = s;
   nb[1] = j * nx + (i + 1 == nx ? 0 : i + 1);
   nb[2] = j * nx + (i == 0 ? nx - 1 : i - 1);
   nb[3] = (j + 1 == ny ? 0 : j + 1) * nx + i;
   nb[4] = (j == 0 ? ny - 1 : j - 1) * nx + i;
-  const int kv = k / CV;
-  T acc[CV];
+  V acc[RPT];
 #pragma unroll
-  for (int u = 0; u < CV; ++u) acc[u] = zero<T>();
+  for (int r = 0; r < RPT; ++r)
 #pragma unroll
-  for (int dir = 0; dir < 5; ++dir) {
-    T row[D];                                      // row r of the block: 16-byte loads, warp-uniform
-    load_row<T, D>(coef + (((size_t)s * 5 + dir) * D + r) * D, row);
-    if constexpr (CV == 1) {
-      const T *xs = x + (size_t)nb[dir] * D * k + c;
+    for (int u = 0; u < CV; ++u) acc[r].v[u] = zero<T>();
+  rows_accumulate<T, D, CV, RPT, 5, false>(blk, x, nb, r0, k, c, live, acc, async_ready);
+  if (!live) return;
 #pragma unroll
-      for (int q = 0; q < D; ++q) acc[0] = madd(acc[0], row[q], xs[(size_t)q * k]);
-    } else {
-      const V *xs = reinterpret_cast<const V *>(x + (size_t)nb[dir] * D * k + c);
-#pragma unroll
-      for (int q = 0; q < D; ++q) {
-        const V xv = xs[(size_t)q * kv];
-#pragma unroll
-        for (int u = 0; u < CV; ++u) acc[u] = madd(acc[u], row[q], xv.v[u]);
-      }
-    }
-  }
-  const size_t o = ((size_t)s * D + r) * k + c;
-  if constexpr (CV == 1) {
-    y[o] = mode ? b[o] - acc[0] : acc[0];
-  } else {
-    V out;
+  for (int r = 0; r < RPT; ++r) {
+    const size_t o = ((size_t)s * D + r0 + r) * k + c;
+    V out = acc[r];
     if (mode) {
       const V bb = *reinterpret_cast<const V *>(b + o);
 #pragma unroll
-      for (int u = 0; u < CV; ++u) out.v[u] = bb.v[u] - acc[u];
-    } else {
-#pragma unroll
-      for (int u = 0; u < CV; ++u) out.v[u] = acc[u];
+      for (int u = 0; u < CV; ++u) out.v[u] = bb.v[u] - acc[r].v[u];
     }
     *reinterpret_cast<V *>(y + o) = out;
   }
@@ -208,11 +253,12 @@ template <class T, int D>
 static void stencil_go(const StencilView &A, const void *x, const void *b, void *y, int k, int mode, cudaStream_t s) {
   if constexpr (D >= 8) {
     if (A.nx * A.ny <= 65535) {
+      constexpr int RPT = rows_rpt<T>();
       if (rows_cv(k) == 2)
-        k_stencil_rows<T, D, 2><<<dim3((k / 2 + 31) / 32, A.nx * A.ny), dim3(32, D), 0, s>>>(
+        k_stencil_rows<T, D, 2, RPT><<<dim3((k / 2 + 31) / 32, A.nx * A.ny), dim3(32, D / RPT), 0, s>>>(
             (const T *)A.coef, (const T *)x, (const T *)b, (T *)y, A.nx, A.ny, k, mode);
       else
-        k_stencil_rows<T, D, 1><<<dim3((k + 31) / 32, A.nx * A.ny), dim3(32, D), 0, s>>>(
+        k_stencil_rows<T, D, 1, RPT><<<dim3((k + 31) / 32, A.nx * A.ny), dim3(32, D / RPT), 0, s>>>(
             (const T *)A.coef, (const T *)x, (const T *)b, (T *)y, A.nx, A.ny, k, mode);
       return;
     }
@@ -666,68 +712,59 @@ __global__ void __launch_bounds__(128, 8) k_rbgs_half_p(const T *__restrict__ co
   }
 }
 
-// Row-split variant for large site blocks (d >= 8, the coarse levels of the
-// Wilson hierarchy, which are small lattices): one thread per (row r of a site,
-// column c), so a site's block solve is spread over d x 32 threads instead of one
-// thread per column.  Phase 1: res_r = b_r - sum over the 4 neighbour blocks of
-// row r times their x (the 8 row threads of a column share the x loads in L1);
-// phase 2, after the block barrier: x_r = sum_q Dinv[r][q] res_q from shared memory.
-// Block = 32 x CV columns x D rows of one site; grid = (column chunks, sites of the
-// colour).  CV = 2 as in k_stencil_rows.
-template <class T, int D, int CV>
-__global__ void __launch_bounds__(256) k_rbgs_half_rows(const T *__restrict__ coef, const T *__restrict__ dinv,
-                                                        T *__restrict__ x, const T *__restrict__ b, int nx, int ny,
-                                                        int k, int colour, int other_zero) {
+// Row-split half-sweep for large site blocks (see k_stencil_rows).  Phase 1: res_r = b_r - sum
+// over the 4 neighbour blocks of row r times their x; phase 2, after a block barrier:
+// x_r = sum_q Dinv[r][q] res_q from shared memory.  Grid = (column chunks, sites of the colour).
+template <class T, int D, int CV, int RPT>
+__global__ void __launch_bounds__(32 * D / RPT) k_rbgs_half_rows(const T *__restrict__ coef,
+                                                                 const T *__restrict__ dinv, T *x, const T *b, int nx,
+                                                                 int ny, int k, int colour, int other_zero) {
   typedef Pack<T, CV> V;
-  __shared__ T res[D][32 * CV];
+  constexpr int BLK = D * D * (int)sizeof(T);
+  __shared__ __align__(16) unsigned char blk_mem[5 * BLK];   // the four neighbour blocks, then D^-1
+  __shared__ V res[D][32];
   const int hx = nx / 2;
   const int idx = blockIdx.y;                       // site of this colour: row j, position m
   const int j = idx / hx, m = idx - (idx / hx) * hx;
   const int i = 2 * m + ((j + colour) & 1);
   const int s = j * nx + i;
-  const int cl = threadIdx.x, r = threadIdx.y;
+  const int cl = threadIdx.x, r0 = threadIdx.y * RPT, tid = threadIdx.y * 32 + threadIdx.x;
   const int c = (blockIdx.x * 32 + cl) * CV;        // k is a multiple of CV
   const bool live = c < k;
-  const int kv = k / CV;
-  if (live) {
-    const V bb = *reinterpret_cast<const V *>(b + ((size_t)s * D + r) * k + c);
-    T acc[CV];
+  if (!other_zero) block_copy_async(blk_mem, coef + ((size_t)s * 5 + 1) * D * D, 4 * BLK, tid, 32 * D / RPT);
+  block_copy_async(blk_mem + 4 * BLK, dinv + (size_t)s * D * D, BLK, tid, 32 * D / RPT);
+  V acc[RPT];
 #pragma unroll
-    for (int u = 0; u < CV; ++u) acc[u] = bb.v[u];
-    if (!other_zero) {
-      int nb[4];
-      nb[0] = j * nx + (i + 1 == nx ? 0 : i + 1);
-      nb[1] = j * nx + (i == 0 ? nx - 1 : i - 1);
-      nb[2] = (j + 1 == ny ? 0 : j + 1) * nx + i;
-      nb[3] = (j == 0 ? ny - 1 : j - 1) * nx + i;
-#pragma unroll
-      for (int dir = 0; dir < 4; ++dir) {
-        T row[D];                                    // row r of the block: 16-byte loads, warp-uniform
-        load_row<T, D>(coef + (((size_t)s * 5 + dir + 1) * D + r) * D, row);
-        const V *xs = reinterpret_cast<const V *>(x + (size_t)nb[dir] * D * k + c);
-#pragma unroll
-        for (int q = 0; q < D; ++q) {
-          const V xv = xs[(size_t)q * kv];
-#pragma unroll
-          for (int u = 0; u < CV; ++u) acc[u] = msub(acc[u], row[q], xv.v[u]);
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < CV; ++u) res[r][cl * CV + u] = acc[u];
+  for (int r = 0; r < RPT; ++r)
+    if (live) acc[r] = *reinterpret_cast<const V *>(b + ((size_t)s * D + r0 + r) * k + c);
+  if (!other_zero) {
+    int nb[4];
+    nb[0] = j * nx + (i + 1 == nx ? 0 : i + 1);
+    nb[1] = j * nx + (i == 0 ? nx - 1 : i - 1);
+    nb[2] = (j + 1 == ny ? 0 : j + 1) * nx + i;
+    nb[3] = (j == 0 ? ny - 1 : j - 1) * nx + i;
+    rows_accumulate<T, D, CV, RPT, 4, true>((const T *)blk_mem, x, nb, r0, k, c, live, acc, async_ready);
+  } else {
+    async_ready();
   }
+#pragma unroll
+  for (int r = 0; r < RPT; ++r) res[r0 + r][cl] = acc[r];
   __syncthreads();
-  if (live) {
-    T di[D];
-    load_row<T, D>(dinv + ((size_t)s * D + r) * D, di);
-    V out;
+  if (!live) return;
+  V out[RPT];
 #pragma unroll
-    for (int u = 0; u < CV; ++u) out.v[u] = zero<T>();
+  for (int r = 0; r < RPT; ++r) {
+    T row[D];
+    memcpy(row, __builtin_assume_aligned(blk_mem + 4 * BLK + (size_t)(r0 + r) * D * sizeof(T), 16), sizeof(row));
 #pragma unroll
-    for (int q = 0; q < D; ++q)
+    for (int u = 0; u < CV; ++u) out[r].v[u] = zero<T>();
 #pragma unroll
-      for (int u = 0; u < CV; ++u) out.v[u] = madd(out.v[u], di[q], res[q][cl * CV + u]);
-    *reinterpret_cast<V *>(x + ((size_t)s * D + r) * k + c) = out;
+    for (int q = 0; q < D; ++q) {
+      const V rv = res[q][cl];
+#pragma unroll
+      for (int u = 0; u < CV; ++u) out[r].v[u] = madd(out[r].v[u], row[q], rv.v[u]);
+    }
+    *reinterpret_cast<V *>(x + ((size_t)s * D + r0 + r) * k + c) = out[r];
   }
 }
 
@@ -736,11 +773,12 @@ static void rbgs_go(const StencilView &A, void *x, const void *b, int k, int col
                     cudaStream_t s) {
   if constexpr (D >= 8) {
     if ((A.nx / 2) * A.ny <= 65535) {
+      constexpr int RPT = rows_rpt<T>();
       if (rows_cv(k) == 2)
-        k_rbgs_half_rows<T, D, 2><<<dim3((k / 2 + 31) / 32, (A.nx / 2) * A.ny), dim3(32, D), 0, s>>>(
+        k_rbgs_half_rows<T, D, 2, RPT><<<dim3((k / 2 + 31) / 32, (A.nx / 2) * A.ny), dim3(32, D / RPT), 0, s>>>(
             (const T *)A.coef, (const T *)A.dinv, (T *)x, (const T *)b, A.nx, A.ny, k, colour, other_zero);
       else
-        k_rbgs_half_rows<T, D, 1><<<dim3((k + 31) / 32, (A.nx / 2) * A.ny), dim3(32, D), 0, s>>>(
+        k_rbgs_half_rows<T, D, 1, RPT><<<dim3((k + 31) / 32, (A.nx / 2) * A.ny), dim3(32, D / RPT), 0, s>>>(
             (const T *)A.coef, (const T *)A.dinv, (T *)x, (const T *)b, A.nx, A.ny, k, colour, other_zero);
       return;
     }
