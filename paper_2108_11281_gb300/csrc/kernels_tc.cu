@@ -11,7 +11,7 @@
 //            (re, im) of B[j] and row 2j+1 is (-im, re): then
 //            Re y = Ar Br - Ai Bi and Im y = Ar Bi + Ai Br.
 //
-// One CTA of 128 threads owns a 128-row by `ntile`-column tile of Y and a
+// One CTA of 256 threads owns a 128-row by `ntile`-column tile of Y and a
 // slice of the contraction (K) range; its accumulator lives in tensor memory.
 // Per 32-wide K step the CTA stages A[128 x 32] and B^T[ntile x 32] into
 // shared memory in the K-major, no-swizzle core-matrix layout (8 rows x 16 B
@@ -43,7 +43,7 @@ namespace {
 constexpr int TC_M = 128;             // rows per tile (TMEM lanes)
 constexpr int TC_BK = 32;             // K elements per stage (4 MMAs of K = 8)
 constexpr int TC_NT = 128;            // max columns per tile
-constexpr int TC_THREADS = 128;
+constexpr int TC_THREADS = 256;
 constexpr long long TC_WAIT_CYCLES = 2000000000LL;   // ~1 s at 2 GHz
 constexpr long long TC_TEST_WAIT_CYCLES = 2000000LL;  // ~1 ms: the withheld-commit test mode
 
@@ -102,52 +102,92 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   constexpr uint32_t LBO = 128, SBO = (TC_BK / 4) * 128;
 
   // One stage's tiles pass through registers: every thread first issues all its
-  // global loads (A: 8 float4; B^T: up to 8 (column, K quad) pairs of 4 scalars),
-  // and the loads of step t+1 are in flight while the MMAs of step t run.
+  // global loads (A: 4 float4; B^T: up to 4 (column, K quad) pairs of 4 scalars),
+  // and the loads of step t+1 are in flight while the MMAs of step t run.  Where its
+  // elements lie is worked out once; a K step that is whole only adds its offset.
+  // A tile: float4 e4 -> row (e4>>6)*8 + (e4&7), K quad (e4>>3)&7; its core-matrix
+  // offset is exactly 16*e4, so the 16-byte shared stores are dense.
+  // B^T tile: (column c, K quad kq) with c fastest; four K rows per pair.
   constexpr int A_IT = TC_M * TC_BK / 4 / TC_THREADS;
   constexpr int B_IT = TC_NT * (TC_BK / 4) / TC_THREADS;
   float4 ra[A_IT];
   float rb[B_IT][4];
+  const float *pa[A_IT], *pb[B_IT];
+  uint32_t boff[B_IT];
+  bool aok[A_IT], bok[B_IT], bodd[B_IT];
+#pragma unroll
+  for (int it = 0; it < A_IT; ++it) {
+    const int e4 = tid + it * TC_THREADS;
+    const int gi = row0 + (((e4 >> 6) << 3) | (e4 & 7));
+    aok[it] = gi < n;
+    pa[it] = Af + (size_t)(aok[it] ? gi : 0) * lda + 4 * ((e4 >> 3) & 7);
+  }
+#pragma unroll
+  for (int it = 0; it < B_IT; ++it) {
+    const int e = tid + it * TC_THREADS;
+    const int kq = e / ntile, c = e - kq * ntile;
+    bok[it] = kq < TC_BK / 4 && col0 + c < nf;
+    bodd[it] = c & 1;
+    boff[it] = (uint32_t)((((c >> 3) * (TC_BK / 4) + kq) << 7) + ((c & 7) << 4));
+    pb[it] = Bf + (size_t)(bok[it] ? (cplx ? 2 * kq : 4 * kq) : 0) * nf + (bok[it] ? col0 + c : 0);
+  }
   auto load_stage = [&](int t) {
     const int j0 = j_begin + t * TC_BK;
-    // A tile: float4 e4 -> row (e4>>6)*8 + (e4&7), K quad (e4>>3)&7; its core-matrix
-    // offset is exactly 16*e4, so the 16-byte shared stores are dense.
+    if (avec && j0 + TC_BK <= j_end) {
+#pragma unroll
+      for (int it = 0; it < A_IT; ++it)
+        ra[it] = aok[it] ? __ldg((const float4 *)(pa[it] + j0)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      if (!cplx) {
+#pragma unroll
+        for (int it = 0; it < B_IT; ++it) {
+          const float *src = pb[it] + (size_t)j0 * nf;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) rb[it][u] = bok[it] ? __ldg(src + (size_t)u * nf) : 0.f;
+        }
+      } else {
+        // K rows 4 kq .. 4 kq + 3 are (re, im) and (-im, re) of two entries of B
+#pragma unroll
+        for (int it = 0; it < B_IT; ++it) {
+          const float *src = pb[it] + (size_t)(j0 >> 1) * nf;
+          const int other = bodd[it] ? -1 : 1;
+          const float sign = bodd[it] ? 1.f : -1.f;
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            rb[it][2 * u] = bok[it] ? __ldg(src + (size_t)u * nf) : 0.f;
+            rb[it][2 * u + 1] = bok[it] ? sign * __ldg(src + (size_t)u * nf + other) : 0.f;
+          }
+        }
+      }
+      return;
+    }
+    // the last K step of a contraction that 32 does not divide, or rows off 16-byte boundaries
 #pragma unroll
     for (int it = 0; it < A_IT; ++it) {
-      const int e4 = tid + it * TC_THREADS;
-      const int r = ((e4 >> 6) << 3) | (e4 & 7), kq = (e4 >> 3) & 7;
-      const int gi = row0 + r, gj = j0 + 4 * kq;
+      const int gj = j0 + 4 * (((tid + it * TC_THREADS) >> 3) & 7);
+      const float *src = pa[it] + j0;
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (gi < n) {
-        const float *src = Af + (size_t)gi * lda + gj;
-        if (avec && gj + 4 <= j_end) {
-          v = __ldg((const float4 *)src);
-        } else {
-          if (gj + 0 < j_end) v.x = __ldg(src + 0);
-          if (gj + 1 < j_end) v.y = __ldg(src + 1);
-          if (gj + 2 < j_end) v.z = __ldg(src + 2);
-          if (gj + 3 < j_end) v.w = __ldg(src + 3);
-        }
+      if (aok[it]) {
+        if (gj + 0 < j_end) v.x = __ldg(src + 0);
+        if (gj + 1 < j_end) v.y = __ldg(src + 1);
+        if (gj + 2 < j_end) v.z = __ldg(src + 2);
+        if (gj + 3 < j_end) v.w = __ldg(src + 3);
       }
       ra[it] = v;
     }
-    // B^T tile: (column c, K quad kq) with c fastest; four K rows per pair.
 #pragma unroll
     for (int it = 0; it < B_IT; ++it) {
-      const int e = tid + it * TC_THREADS;
-      const int c = e % ntile, kq = e / ntile;
-      const int gc = col0 + c;
+      const int kq = (tid + it * TC_THREADS) / ntile;
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int gj = j0 + 4 * kq + u;
         float x = 0.f;
-        if (e < ntile * (TC_BK / 4) && gj < j_end && gc < nf) {
+        if (bok[it] && gj < j_end) {
           if (!cplx) {
-            x = __ldg(Bf + (size_t)gj * nf + gc);
+            x = __ldg(pb[it] + (size_t)(j0 + u) * nf);
           } else {
-            const float *row = Bf + (size_t)(gj >> 1) * nf;
-            if ((gj & 1) == 0) x = __ldg(row + gc);
-            else x = (gc & 1) ? __ldg(row + gc - 1) : -__ldg(row + gc + 1);
+            const float *row = pb[it] + (size_t)((j0 >> 1) + (u >> 1)) * nf;
+            if ((u & 1) == 0) x = __ldg(row);
+            else x = bodd[it] ? __ldg(row - 1) : -__ldg(row + 1);
           }
         }
         rb[it][u] = x;
@@ -158,13 +198,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 #pragma unroll
     for (int it = 0; it < A_IT; ++it) split_store(Ahi, Alo, (uint32_t)(tid + it * TC_THREADS) * 16, ra[it]);
 #pragma unroll
-    for (int it = 0; it < B_IT; ++it) {
-      const int e = tid + it * TC_THREADS;
-      if (e >= ntile * (TC_BK / 4)) break;
-      const int c = e % ntile, kq = e / ntile;
-      const uint32_t off = (uint32_t)((((c >> 3) * (TC_BK / 4) + kq) << 7) + ((c & 7) << 4));
-      split_store(Bhi, Blo, off, make_float4(rb[it][0], rb[it][1], rb[it][2], rb[it][3]));
-    }
+    for (int it = 0; it < B_IT; ++it)
+      if (tid + it * TC_THREADS < ntile * (TC_BK / 4))
+        split_store(Bhi, Blo, boff[it], make_float4(rb[it][0], rb[it][1], rb[it][2], rb[it][3]));
   };
 
   int issued = 0;      // K steps whose MMAs were committed (uniform over the CTA)
@@ -221,11 +257,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 
   if (!failed) {
     float *Yz = Y + (size_t)blockIdx.z * n * nf;
-    const int r = row0 + warp * 32 + lane;
-    for (int c0 = 0; c0 < ntile; c0 += 16) {
+    // warps w and w + 4 read the tensor-memory lanes 32 (w mod 4) .. + 31, every other 16 columns
+    const int r = row0 + (warp & 3) * 32 + lane;
+    for (int c0 = (warp >> 2) * 16; c0 < ntile; c0 += 32) {
       uint32_t v[16];
       if (issued > 0) {
-        const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
+        const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0;
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
             : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
@@ -263,11 +300,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
   }
 }
 
-// Y = sum of the K-slice partials, added in slice order (deterministic).
-__global__ void k_dense_sum_tc(const float *__restrict__ part, int slices, size_t count, float *__restrict__ Y) {
+// Y = sum of the K-slice partials, added in slice order (deterministic); V: floats per load.
+template <class V>
+__global__ void k_dense_sum_tc(const V *__restrict__ part, int slices, size_t count, V *__restrict__ Y) {
+  constexpr int N = sizeof(V) / 4;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x) {
-    float s = part[i];
-    for (int z = 1; z < slices; ++z) s += part[(size_t)z * count + i];
+    V s = part[i];
+#pragma unroll 8
+    for (int z = 1; z < slices; ++z) {
+      const V p = part[(size_t)z * count + i];
+#pragma unroll
+      for (int u = 0; u < N; ++u) ((float *)&s)[u] += ((const float *)&p)[u];
+    }
     Y[i] = s;
   }
 }
@@ -338,7 +382,10 @@ void launch_dense_apply_tc(DType t, const void *Ainv, const void *B, void *Y, in
                                                   withhold ? TC_TEST_WAIT_CYCLES : TC_WAIT_CYCLES, err);
   if (p.slices > 1) {
     size_t cnt = (size_t)n * p.nf;
-    k_dense_sum_tc<<<grid_for(cnt, 256), 256, 0, s>>>((const float *)part, p.slices, cnt, (float *)Y);
+    if (cnt % 4 == 0)
+      k_dense_sum_tc<float4><<<grid_for(cnt / 4, 128), 128, 0, s>>>((const float4 *)part, p.slices, cnt / 4, (float4 *)Y);
+    else
+      k_dense_sum_tc<float><<<grid_for(cnt, 256), 256, 0, s>>>((const float *)part, p.slices, cnt, (float *)Y);
   }
   MLMC_LAUNCH_CHECK("k_dense_apply_tc");
 }

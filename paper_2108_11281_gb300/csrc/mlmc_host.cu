@@ -1675,18 +1675,22 @@ int mlmc_dense_apply(int complex_data, const void *A, const void *B, void *Y, in
     const DType t = complex_data ? C32 : F32;
     cudaStream_t s = (cudaStream_t)stream;
     g_alloc_stream = s;
-    DevBuf part, err;
-    err.alloc(sizeof(int));
-    check_cuda(cudaMemsetAsync(err.p, 0, sizeof(int), s), "memset err");
-    if (which != MLMC_DENSE_SIMT) {
-      part.alloc(dense_apply_tc_part_bytes(t, n, k));
-      launch_dense_apply_tc(t, A, B, Y, n, k, part.p, part.bytes, err.as<int>(), s, which == MLMC_DENSE_TC_WITHHOLD);
+    // one allocation per call: the error word, then (16 bytes on) the partial products
+    const bool tc = which != MLMC_DENSE_SIMT;
+    const size_t part_bytes = tc ? dense_apply_tc_part_bytes(t, n, k)
+                                 : (size_t)dense_apply_splits(n, k) * n * k * dtype_size(t);
+    DevBuf work;
+    work.alloc(16 + part_bytes);
+    int *err = work.as<int>();
+    void *part = work.as<char>() + 16;
+    if (tc) {
+      check_cuda(cudaMemsetAsync(err, 0, sizeof(int), s), "memset err");
+      launch_dense_apply_tc(t, A, B, Y, n, k, part, part_bytes, err, s, which == MLMC_DENSE_TC_WITHHOLD);
     } else {
-      part.alloc((size_t)dense_apply_splits(n, k) * n * k * dtype_size(t));
-      launch_dense_apply(t, A, B, Y, n, k, part.p, s);
+      launch_dense_apply(t, A, B, Y, n, k, part, s);
     }
     int e = 0;
-    check_cuda(cudaMemcpyAsync(&e, err.p, sizeof(int), cudaMemcpyDeviceToHost, s), "D2H err");
+    if (tc) check_cuda(cudaMemcpyAsync(&e, err, sizeof(int), cudaMemcpyDeviceToHost, s), "D2H err");
     check_cuda(cudaStreamSynchronize(s), "sync");
     if (e == MLMC_ERR_TIMEOUT) fail(MLMC_ERR_TIMEOUT, "a bounded tensor-core wait gave up");
   });
