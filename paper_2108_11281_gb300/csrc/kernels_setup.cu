@@ -653,22 +653,24 @@ void launch_trace(DType t, const void *A, int n, void *out, cudaStream_t s) {
 // Y[i][c] = sum_j Ainv[i][j] B[j][c].
 //
 // FP64 data, and FP32 data with small n: the outputs are dealt out over all SMs.  A warp holds
-// 32 items (R rows x one column each, items in (row group, column) order, so a ragged k wastes
-// no lanes), the eight warps of a block take an eighth of the j range each and meet in shared
-// memory in order.  FP64 issues one warp instruction per 16 clocks and SM, so its loads need no
-// shared-memory tiling; what counts is that every SM has the same share: 256 x 256 x 64
-// columns, 4.2 M FMA = 6.7 us at the measured rate, took 45 us on the 32 blocks of the tiled
-// kernel below and takes 10.9 us (576 x 576 x 21: 61.5 -> 15.5 us).  With FP32 and n < 512 the
-// chain of dependent loads counts, an eighth as long (128 complex x 32: 14 -> 4 us).
-template <class T, int R>
+// IT items (R rows x one column each, items in (row group, column) order, so a ragged k wastes
+// no lanes) times 32 / IT slices of the j range; with the block's eight warps that makes 256 / IT
+// slices, which meet in shared memory in order.  FP64 issues one warp instruction per 16 clocks
+// and SM, so its loads need no shared-memory tiling; what counts is that every SM has the same
+// share: 256 x 256 x 64 columns, 4.2 M FMA = 6.7 us at the measured rate, took 45 us on the 32
+// blocks of the tiled kernel below and takes 10.9 us (576 x 576 x 21: 61.5 -> 15.5 us).  With FP32
+// and n < 512 the chain of dependent loads counts, an eighth as long or less (128 complex x 32:
+// 14 -> 4 us).
+template <class T, int R, int IT>
 __global__ void __launch_bounds__(256) k_dense_spread(const T *__restrict__ A, const T *__restrict__ B,
                                                       T *__restrict__ Y, int n, int k, int chunk, int vec) {
   constexpr int VJ = 16 / (int)sizeof(T);                  // entries of a row per 16-byte load
-  __shared__ T red[8][R][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned t = blockIdx.x * 32u + lane;
+  constexpr int SL = 256 / IT;
+  __shared__ T red[SL][R][IT];
+  const int item = threadIdx.x % IT, slice = threadIdx.x / IT;
+  const unsigned t = blockIdx.x * (unsigned)IT + item;
   const int rg = (int)(t / (unsigned)k), c = (int)(t - (unsigned)rg * k), row0 = rg * R;
-  const int j0 = min(n, warp * chunk), j1 = min(n, j0 + chunk);
+  const int j0 = min(n, slice * chunk), j1 = min(n, j0 + chunk);
   T acc[R];
   const T *a[R];
 #pragma unroll
@@ -702,14 +704,14 @@ __global__ void __launch_bounds__(256) k_dense_spread(const T *__restrict__ A, c
     for (int r = 0; r < R; ++r) acc[r] = madd(acc[r], a[r][j], bv);
   }
 #pragma unroll
-  for (int r = 0; r < R; ++r) red[warp][r][lane] = acc[r];
+  for (int r = 0; r < R; ++r) red[slice][r][item] = acc[r];
   __syncthreads();
-  for (int e = threadIdx.x; e < R * 32; e += 256) {
-    const int r = e >> 5, l = e & 31;
+  for (int e = threadIdx.x; e < R * IT; e += 256) {
+    const int r = e / IT, l = e % IT;
     T s = red[0][r][l];
-#pragma unroll
-    for (int w = 1; w < 8; ++w) s = s + red[w][r][l];
-    const unsigned tt = blockIdx.x * 32u + l;
+#pragma unroll 8
+    for (int w = 1; w < SL; ++w) s = s + red[w][r][l];
+    const unsigned tt = blockIdx.x * (unsigned)IT + l;
     const int i = (int)(tt / (unsigned)k) * R + r;
     if (i < n) Y[(size_t)i * k + tt % (unsigned)k] = s;
   }
@@ -845,27 +847,36 @@ void launch_dense_apply(DType t, const void *Ainv, const void *B, void *Y, int n
   }
   const bool fp64 = t == F64 || t == C64;
   if (fp64 || n * (t == C32 ? 2 : 1) < 512) {
-    // rows per thread: the fewest (blocks on the busiest SM) x rows; more rows where that is
-    // equal, since B is read once per row group
-    int R = 4;
+    // rows per thread and items per warp: the smallest share of the busiest SM, blocks x R x IT;
+    // the larger tile where that is equal (B is read once per row group, and fewer sums meet)
+    int R = 4, IT = 32;
     size_t best = ~(size_t)0;
-    for (int r : {4, 2, 1}) {
-      const size_t blocks = ((size_t)((n + r - 1) / r) * k + 31) / 32, cost = (blocks + 151) / 152 * r;
-      if (cost < best) {
-        best = cost;
-        R = r;
+    for (int it : {32, 16, 8})
+      for (int r : {4, 2, 1}) {
+        const size_t blocks = ((size_t)((n + r - 1) / r) * k + it - 1) / it, cost = (blocks + 151) / 152 * r * it;
+        if (cost < best) {
+          best = cost;
+          R = r;
+          IT = it;
+        }
       }
-    }
-    const unsigned g = (unsigned)(((size_t)((n + R - 1) / R) * k + 31) / 32);
+    const unsigned g = (unsigned)(((size_t)((n + R - 1) / R) * k + IT - 1) / IT);
     MLMC_DISPATCH(t, T, {
       constexpr int VJ = 16 / (int)sizeof(T);
-      const int chunk = ((n + 7) / 8 + VJ - 1) / VJ * VJ, vec = n % VJ == 0 && ((uintptr_t)Ainv & 15) == 0;
-      auto go = [&](auto r) {
-        k_dense_spread<T, decltype(r)::value><<<g, 256, 0, s>>>((const T *)Ainv, (const T *)B, (T *)Y, n, k, chunk, vec);
+      const int slices = 256 / IT, vec = n % VJ == 0 && ((uintptr_t)Ainv & 15) == 0;
+      const int chunk = ((n + slices - 1) / slices + VJ - 1) / VJ * VJ;
+      auto go = [&](auto r, auto it) {
+        k_dense_spread<T, decltype(r)::value, decltype(it)::value><<<g, 256, 0, s>>>((const T *)Ainv, (const T *)B,
+                                                                                    (T *)Y, n, k, chunk, vec);
       };
-      if (R == 4) go(std::integral_constant<int, 4>());
-      else if (R == 2) go(std::integral_constant<int, 2>());
-      else go(std::integral_constant<int, 1>());
+      auto rows = [&](auto it) {
+        if (R == 4) go(std::integral_constant<int, 4>(), it);
+        else if (R == 2) go(std::integral_constant<int, 2>(), it);
+        else go(std::integral_constant<int, 1>(), it);
+      };
+      if (IT == 32) rows(std::integral_constant<int, 32>());
+      else if (IT == 16) rows(std::integral_constant<int, 16>());
+      else rows(std::integral_constant<int, 8>());
     });
     MLMC_LAUNCH_CHECK("k_dense_spread");
     return;
