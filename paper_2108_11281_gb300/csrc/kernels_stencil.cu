@@ -370,10 +370,13 @@ __global__ void __launch_bounds__(256) k_laplace(const T *__restrict__ x, const 
 // on the sites of `colour`.  other_zero = 1: the other colour holds zeros (not read).
 // Colour 1 takes the rows from the last: consecutive half-sweeps alternate direction, so
 // each starts on the rows the previous one wrote last.
+// from_zero = 1: the whole first sweep from x = 0 as one pass over colour 1,
+// x_1 = (b_1 + sum of b_0 / diag) / diag; colour 0 is left unset (see launch_rbgs_first).
 // The grid strides over the units (row, chunk of 256 threads of the row).
 template <class T, int VEC>
 __device__ __forceinline__ void laplace_rbgs_body(T *__restrict__ x, const T *__restrict__ b, int nx, int ny, int kv,
-                                                  T dinv, int periodic, int colour, int other_zero, int j, int t) {
+                                                  T dinv, int periodic, int colour, int other_zero, int from_zero,
+                                                  int j, int t) {
   typedef Pack<T, VEC> V;
   const int i0 = (j + colour) & 1;
   const int hx = (nx - i0 + 1) >> 1;      // sites of this colour in row j (odd nx too)
@@ -386,9 +389,9 @@ __device__ __forceinline__ void laplace_rbgs_body(T *__restrict__ x, const T *__
   if (!other_zero) {
     const Nbrs n = laplace_nbrs(i, j, nx, ny, periodic);
     T sum[VEC];
-    laplace_nbr_sum<T, VEC>(X, n, kv, c, sum);
+    laplace_nbr_sum<T, VEC>(from_zero ? (const V *)b : X, n, kv, c, sum);
 #pragma unroll
-    for (int u = 0; u < VEC; ++u) acc.v[u] = acc.v[u] + sum[u];
+    for (int u = 0; u < VEC; ++u) acc.v[u] = from_zero ? madd(acc.v[u], dinv, sum[u]) : acc.v[u] + sum[u];
   }
 #pragma unroll
   for (int u = 0; u < VEC; ++u) acc.v[u] = acc.v[u] * dinv;
@@ -398,12 +401,12 @@ __device__ __forceinline__ void laplace_rbgs_body(T *__restrict__ x, const T *__
 template <class T, int VEC>
 __global__ void __launch_bounds__(256) k_laplace_rbgs(T *__restrict__ x, const T *__restrict__ b, int nx, int ny,
                                                       int kv, T dinv, int periodic, int colour, int other_zero,
-                                                      int bpr) {
+                                                      int from_zero, int bpr) {
   const int units = bpr * ny;
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
     const int jr = u / bpr;
-    laplace_rbgs_body<T, VEC>(x, b, nx, ny, kv, dinv, periodic, colour, other_zero, colour ? ny - 1 - jr : jr,
-                              (u - jr * bpr) * 256 + threadIdx.x);
+    laplace_rbgs_body<T, VEC>(x, b, nx, ny, kv, dinv, periodic, colour, other_zero, from_zero,
+                              colour ? ny - 1 - jr : jr, (u - jr * bpr) * 256 + threadIdx.x);
   }
 }
 
@@ -559,7 +562,7 @@ static void launch_laplace(const StencilView &A, const void *x, const void *b, v
 }
 
 static void launch_laplace_rbgs(const StencilView &A, void *x, const void *b, int k, int colour, int other_zero,
-                                cudaStream_t s) {
+                                cudaStream_t s, int from_zero = 0) {
   auto go = [&](auto tag, auto vtag) {
     typedef decltype(tag) T;
     constexpr int VEC = decltype(vtag)::value;
@@ -571,7 +574,8 @@ static void launch_laplace_rbgs(const StencilView &A, void *x, const void *b, in
     const unsigned grid = std::is_same<T, double>::value ? resident_grid((size_t)bpr * A.ny, occ)
                                                          : (unsigned)(bpr * A.ny);
     k_laplace_rbgs<T, VEC><<<grid, 256, 0, s>>>(
-        (T *)x, (const T *)b, A.nx, A.ny, kv, (T)(1.0 / A.diag), A.periodic, colour, other_zero, bpr);
+        (T *)x, (const T *)b, A.nx, A.ny, kv, (T)(1.0 / A.diag), A.periodic, colour, other_zero, from_zero,
+        bpr);
   };
   if (A.t == F64) {
     if (laplace_vec<double>(k) == 2) go(double(), std::integral_constant<int, 2>());
@@ -617,9 +621,9 @@ template <int D> struct rbgs_vec<cdouble, D> { static const int v = 1; };
 // grid.y = lattice row j; threads of a row cover (site m of the colour, VEC columns).
 template <class T, int D, int VEC>
 __device__ __forceinline__ void rbgs_half_body(const T *__restrict__ coef, const T *__restrict__ dinv,
-                                               T *__restrict__ x, const T *__restrict__ b, int nx, int ny, int kv,
+                                               T *x, const T *src, const T *b, int nx, int ny, int kv,
                                                int colour, int other_zero, int j, int t) {
-  // j = lattice row; t = (site m of the colour in the row, pack c of VEC columns)
+  // src: where the neighbours' entries are read, x or (launch_rbgs_first) b; j = lattice row; t = (site m of the colour in the row, pack c of VEC columns)
   typedef Pack<T, VEC> V;
   const int hx = nx / 2;
   if (t < hx * kv) {
@@ -644,7 +648,7 @@ __device__ __forceinline__ void rbgs_half_body(const T *__restrict__ coef, const
 #pragma unroll
       for (int dir = 1; dir < 5; ++dir) {
         const T *B = coef + ((size_t)s * 5 + dir) * D * D;
-        const V *xs = (const V *)x + (size_t)nb[dir] * D * kv + c;
+        const V *xs = (const V *)src + (size_t)nb[dir] * D * kv + c;
         V xq[D];
 #pragma unroll
         for (int q = 0; q < D; ++q) xq[q] = xs[(size_t)q * kv];
@@ -679,13 +683,13 @@ __device__ __forceinline__ void rbgs_half_body(const T *__restrict__ coef, const
 
 template <class T, int D, int VEC>
 __global__ void __launch_bounds__(256) k_rbgs_half(const T *__restrict__ coef, const T *__restrict__ dinv,
-                                                   T *__restrict__ x, const T *__restrict__ b, int nx, int ny, int kv,
+                                                   T *x, const T *src, const T *b, int nx, int ny, int kv,
                                                    int colour, int other_zero, int bpr) {
   // resident grid striding over the units (row j, chunk of 256 threads of the row)
   const int units = bpr * ny;
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
     const int j = u / bpr;
-    rbgs_half_body<T, D, VEC>(coef, dinv, x, b, nx, ny, kv, colour, other_zero, j, (u - j * bpr) * 256 + threadIdx.x);
+    rbgs_half_body<T, D, VEC>(coef, dinv, x, src, b, nx, ny, kv, colour, other_zero, j, (u - j * bpr) * 256 + threadIdx.x);
   }
 }
 
@@ -700,7 +704,7 @@ __global__ void __launch_bounds__(256) k_rbgs_half(const T *__restrict__ coef, c
 // 100-104 us with 5-8 blocks of 256 per SM (8-byte packs or spills).
 template <class T, int D, int VEC>
 __global__ void __launch_bounds__(128, 8) k_rbgs_half_p(const T *__restrict__ coef, const T *__restrict__ dinv,
-                                                        T *__restrict__ x, const T *__restrict__ b, int nx, int ny,
+                                                        T *x, const T *src, const T *b, int nx, int ny,
                                                         int kv, int colour, int other_zero, int bpr) {
   // colour 1 walks the rows from the last: consecutive half-sweeps alternate direction,
   // so each starts on the rows the previous one wrote last (still in L2)
@@ -708,7 +712,7 @@ __global__ void __launch_bounds__(128, 8) k_rbgs_half_p(const T *__restrict__ co
   for (int u0 = blockIdx.x; u0 < units; u0 += gridDim.x) {
     const int u = colour ? units - 1 - u0 : u0;
     const int j = u / bpr;
-    rbgs_half_body<T, D, VEC>(coef, dinv, x, b, nx, ny, kv, colour, other_zero, j, (u - j * bpr) * 128 + threadIdx.x);
+    rbgs_half_body<T, D, VEC>(coef, dinv, x, src, b, nx, ny, kv, colour, other_zero, j, (u - j * bpr) * 128 + threadIdx.x);
   }
 }
 
@@ -717,7 +721,8 @@ __global__ void __launch_bounds__(128, 8) k_rbgs_half_p(const T *__restrict__ co
 // x_r = sum_q Dinv[r][q] res_q from shared memory.  Grid = (column chunks, sites of the colour).
 template <class T, int D, int CV, int RPT>
 __global__ void __launch_bounds__(32 * D / RPT) k_rbgs_half_rows(const T *__restrict__ coef,
-                                                                 const T *__restrict__ dinv, T *x, const T *b, int nx,
+                                                                 const T *__restrict__ dinv, T *x, const T *src,
+                                                                 const T *b, int nx,
                                                                  int ny, int k, int colour, int other_zero) {
   typedef Pack<T, CV> V;
   constexpr int BLK = D * D * (int)sizeof(T);
@@ -743,7 +748,7 @@ __global__ void __launch_bounds__(32 * D / RPT) k_rbgs_half_rows(const T *__rest
     nb[1] = j * nx + (i == 0 ? nx - 1 : i - 1);
     nb[2] = (j + 1 == ny ? 0 : j + 1) * nx + i;
     nb[3] = (j == 0 ? ny - 1 : j - 1) * nx + i;
-    rows_accumulate<T, D, CV, RPT, 4, true>((const T *)blk_mem, x, nb, r0, k, c, live, acc, async_ready);
+    rows_accumulate<T, D, CV, RPT, 4, true>((const T *)blk_mem, src, nb, r0, k, c, live, acc, async_ready);
   } else {
     async_ready();
   }
@@ -769,17 +774,17 @@ __global__ void __launch_bounds__(32 * D / RPT) k_rbgs_half_rows(const T *__rest
 }
 
 template <class T, int D>
-static void rbgs_go(const StencilView &A, void *x, const void *b, int k, int colour, int other_zero,
-                    cudaStream_t s) {
+static void rbgs_go(const StencilView &A, const void *coef, void *x, const void *src, const void *b, int k, int colour,
+                    int other_zero, cudaStream_t s) {
   if constexpr (D >= 8) {
     if ((A.nx / 2) * A.ny <= 65535) {
       constexpr int RPT = rows_rpt<T>();
       if (rows_cv(k) == 2)
         k_rbgs_half_rows<T, D, 2, RPT><<<dim3((k / 2 + 31) / 32, (A.nx / 2) * A.ny), dim3(32, D / RPT), 0, s>>>(
-            (const T *)A.coef, (const T *)A.dinv, (T *)x, (const T *)b, A.nx, A.ny, k, colour, other_zero);
+            (const T *)coef, (const T *)A.dinv, (T *)x, (const T *)src, (const T *)b, A.nx, A.ny, k, colour, other_zero);
       else
         k_rbgs_half_rows<T, D, 1, RPT><<<dim3((k + 31) / 32, (A.nx / 2) * A.ny), dim3(32, D / RPT), 0, s>>>(
-            (const T *)A.coef, (const T *)A.dinv, (T *)x, (const T *)b, A.nx, A.ny, k, colour, other_zero);
+            (const T *)coef, (const T *)A.dinv, (T *)x, (const T *)src, (const T *)b, A.nx, A.ny, k, colour, other_zero);
       return;
     }
   }
@@ -790,19 +795,19 @@ static void rbgs_go(const StencilView &A, void *x, const void *b, int k, int col
     {
       const int bpr = ((A.nx / 2) * kv + 127) / 128;
       k_rbgs_half_p<T, D, VW><<<resident_grid(bpr * A.ny, 8), 128, 0, s>>>(
-          (const T *)A.coef, (const T *)A.dinv, (T *)x, (const T *)b, A.nx, A.ny, kv, colour, other_zero, bpr);
+          (const T *)coef, (const T *)A.dinv, (T *)x, (const T *)src, (const T *)b, A.nx, A.ny, kv, colour, other_zero, bpr);
     }
     else {
       const int bpr = ((A.nx / 2) * kv + 255) / 256;
       static const int occ = blocks_per_sm(k_rbgs_half<T, D, VW>, 256, 0);
       k_rbgs_half<T, D, VW><<<resident_grid((size_t)bpr * A.ny, occ), 256, 0, s>>>(
-          (const T *)A.coef, (const T *)A.dinv, (T *)x, (const T *)b, A.nx, A.ny, kv, colour, other_zero, bpr);
+          (const T *)coef, (const T *)A.dinv, (T *)x, (const T *)src, (const T *)b, A.nx, A.ny, kv, colour, other_zero, bpr);
     }
   } else {
     const int bpr = ((A.nx / 2) * k + 255) / 256;
     static const int occ = blocks_per_sm(k_rbgs_half<T, D, 1>, 256, 0);
     k_rbgs_half<T, D, 1><<<resident_grid((size_t)bpr * A.ny, occ), 256, 0, s>>>(
-        (const T *)A.coef, (const T *)A.dinv, (T *)x, (const T *)b, A.nx, A.ny, k, colour, other_zero, bpr);
+        (const T *)coef, (const T *)A.dinv, (T *)x, (const T *)src, (const T *)b, A.nx, A.ny, k, colour, other_zero, bpr);
   }
 }
 
@@ -812,7 +817,7 @@ void launch_rbgs_half(const StencilView &A, void *x, const void *b, int k, int c
     return;
   }
   if (A.taps == 9) throw cuda_error{cudaErrorInvalidValue, "9-point stencils are smoothed in four colours"};
-  MLMC_DISPATCH(A.t, T, MLMC_DDISPATCH(A.d, D, rbgs_go<T, D>(A, x, b, k, colour, 0, s)));
+  MLMC_DISPATCH(A.t, T, MLMC_DDISPATCH(A.d, D, rbgs_go<T, D>(A, A.coef, x, x, b, k, colour, 0, s)));
   MLMC_LAUNCH_CHECK("k_rbgs_half");
 }
 
@@ -830,9 +835,51 @@ void launch_rbgs_sweep(const StencilView &A, void *x, const void *b, int k, int 
   }
   // x_zero: the first half-sweep reads no neighbours and the second none of its own
   // old values, so x needs no initialisation
-  MLMC_DISPATCH(A.t, T, MLMC_DDISPATCH(A.d, D, rbgs_go<T, D>(A, x, b, k, first, x_zero ? 1 : 0, s)));
+  MLMC_DISPATCH(A.t, T, MLMC_DDISPATCH(A.d, D, rbgs_go<T, D>(A, A.coef, x, x, b, k, first, x_zero ? 1 : 0, s)));
   MLMC_LAUNCH_CHECK("k_rbgs_half");
   launch_rbgs_half(A, x, b, k, 1 - first, s);
+}
+
+// ------------------------------------------------------------------ the first sweep from x = 0
+// A red-black sweep from x = 0 sets x_0 = D_0^{-1} b_0 and then x_1 = D_1^{-1} (b_1 - A_10 x_0).  When
+// another sweep follows, it overwrites x_0 without reading it, so only x_1 is wanted, and
+// x_1 = D_1^{-1} (b_1 - (A_10 D_0^{-1}) b_0) is a half-sweep of the same form with b in the place of x
+// and the products A_10 D_0^{-1} (StencilView::first, formed once at setup) in the place of A_10:
+// one launch and 1.5 vector passes instead of two and 2.5.
+void launch_rbgs_first(const StencilView &A, void *x, const void *b, int k, cudaStream_t s) {
+  if (A.const_laplace) {
+    launch_laplace_rbgs(A, x, b, k, 1, 0, s, 1);
+    return;
+  }
+  if (!A.first) throw cuda_error{cudaErrorInvalidValue, "rbgs_first: no products on this level"};
+  MLMC_DISPATCH(A.t, T, MLMC_DDISPATCH(A.d, D, rbgs_go<T, D>(A, A.first, x, b, b, k, 1, 0, s)));
+  MLMC_LAUNCH_CHECK("k_rbgs_half");
+}
+
+// first[s][dir] = A_{s,dir} D_{nb(dir)}^{-1} for the sites s of colour 1, dir = 1 .. 4 (other entries unset)
+template <class T>
+__global__ void k_first_blocks(const T *__restrict__ coef, const T *__restrict__ dinv, T *__restrict__ first, int nx,
+                               int ny, int d) {
+  const unsigned per = 4u * d * d, total = (unsigned)nx * ny / 2 * per;
+  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
+    const unsigned h = t / per, e = t - h * per;
+    const int dir = 1 + (int)(e / (d * d)), r = (int)(e / d) % d, q = (int)e % d;
+    const int j = (int)(h / (nx / 2)), i = 2 * (int)(h % (nx / 2)) + ((j + 1) & 1), s = j * nx + i;
+    const int nb = dir == 1 ? j * nx + (i + 1 == nx ? 0 : i + 1) : dir == 2 ? j * nx + (i == 0 ? nx - 1 : i - 1)
+                 : dir == 3 ? (j + 1 == ny ? 0 : j + 1) * nx + i : (j == 0 ? ny - 1 : j - 1) * nx + i;
+    const T *a = coef + ((size_t)s * 5 + dir) * d * d + r * d, *w = dinv + (size_t)nb * d * d + q;
+    T v = zero<T>();
+    for (int m = 0; m < d; ++m) v = madd(v, a[m], w[(size_t)m * d]);
+    first[((size_t)s * 5 + dir) * d * d + r * d + q] = v;
+  }
+}
+
+void launch_first_blocks(DType t, const void *coef, const void *dinv, void *first, int nx, int ny, int d,
+                         cudaStream_t s) {
+  const size_t total = (size_t)nx * ny / 2 * 4 * d * d;
+  MLMC_DISPATCH(t, T, k_first_blocks<T><<<grid_for(total, 256), 256, 0, s>>>((const T *)coef, (const T *)dinv,
+                                                                             (T *)first, nx, ny, d));
+  MLMC_LAUNCH_CHECK("k_first_blocks");
 }
 
 }  // namespace mlmc

@@ -76,6 +76,7 @@ struct Level {
   int nx = 0, ny = 0, d = 0;
   size_t nsite = 0, n = 0;
   DevBuf coef64, dinv64, coef32, dinv32;   // block stencil and inverse self blocks
+  DevBuf first;                            // A D^-1 of launch_rbgs_first, in the precision of the solves' cycle
   int ax = 0, ay = 0, dc = 0;              // aggregation towards the next level
   DevBuf P64, P32;
   int taps = 5;                            // 5: block stencil; 9: 9-point scalar stencil (bilinear levels >= 2)
@@ -188,6 +189,7 @@ StencilView view(const H_t &h, int l, int lo) {
   v.t = lo ? h.t32 : h.t64;
   v.coef = lo ? L.coef32.p : L.coef64.p;
   v.dinv = lo ? L.dinv32.p : L.dinv64.p;
+  v.first = lo == (h.prm.precision == MLMC_PREC_MIXED_FP32 ? 1 : 0) && L.first.bytes > 16 ? L.first.p : nullptr;
   v.const_laplace = (l == 0 && h.const_laplace) ? 1 : 0;
   v.diag = h.laplace_diag;
   v.periodic = h.periodic;
@@ -468,8 +470,13 @@ void cycle(H_t &h, int lo, int l, const void *b, void *x, int k) {
   const int npost = (l > 0 && h.prm.coarse_smooth > 0) ? h.prm.coarse_smooth : h.prm.smooth_post;
   if (npre < 1) launch_fill_zero(t, x, blk, s);
   for (int it = 0; it < npre; ++it) {
-    launch_rbgs_sweep(A, x, b, k, 0, it == 0, s);
-    h.launches += 2;
+    if (it == 0 && npre > 1 && A.taps == 5 && (A.const_laplace || A.first)) {
+      launch_rbgs_first(A, x, b, k, s);
+      h.launches++;
+    } else {
+      launch_rbgs_sweep(A, x, b, k, 0, it == 0, s);
+      h.launches += 2;
+    }
     h.cost += nnz_of(h, l) * k;
   }
   const ProlongView Pv = pview(h, l, lo);
@@ -957,7 +964,19 @@ void build_levels(H_t &h, const void *V1, const void *const *user_P) {
     h.launches += 5 + 3;
     check_err(h, "coarsest inverse");
   }
-  if (h.prm.precision == MLMC_PREC_MIXED_FP32) {
+  const bool mixed = h.prm.precision == MLMC_PREC_MIXED_FP32;
+  // the products of the first sweep, for levels where a second one follows (FP64 arithmetic; the
+  // mixed form rounds them like the other coefficients)
+  for (int l = 0; l + 1 < h.L; ++l) {
+    Level &Lv = h.lv[l];
+    if (Lv.first.bytes <= 16) continue;
+    DevBuf wide;
+    if (mixed) wide.alloc(Lv.nsite * 5 * Lv.d * Lv.d * es);
+    launch_first_blocks(h.t64, Lv.coef64.p, Lv.dinv64.p, mixed ? wide.p : Lv.first.p, Lv.nx, Lv.ny, Lv.d, h.stream);
+    if (mixed) launch_convert(h.t32, Lv.first.p, h.t64, wide.p, Lv.nsite * 5 * Lv.d * Lv.d, h.stream);
+    h.launches += mixed ? 2 : 1;
+  }
+  if (mixed) {
     for (int l = 0; l < h.L; ++l) {
       Level &Lv = h.lv[l];
       launch_convert(h.t32, Lv.coef32.p, h.t64, Lv.coef64.p, Lv.nsite * Lv.taps * Lv.d * Lv.d, h.stream);
@@ -1227,6 +1246,9 @@ void setup(H_t &h, const mlmc_operator_desc *op, const mlmc_hierarchy_params *p,
       Lv.dc = h.bilinear ? 1 : dc;
       Lv.dinv64.alloc(Lv.nsite * Lv.d * Lv.d * es);
       Lv.P64.alloc(h.bilinear ? 0 : Lv.n * dc * es);      // bilinear P has no stored entries
+      const int npre = l > 0 && p->coarse_smooth > 0 ? p->coarse_smooth : p->smooth_pre;
+      if (!h.bilinear && npre > 1 && !(l == 0 && h.const_laplace))
+        Lv.first.alloc(Lv.nsite * 5 * Lv.d * Lv.d * (mixed ? es32 : es));
       if (mixed) {
         Lv.dinv32.alloc(Lv.nsite * Lv.d * Lv.d * es32);
         Lv.P32.alloc(h.bilinear ? 0 : Lv.n * dc * es32);

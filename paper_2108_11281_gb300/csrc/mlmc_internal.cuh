@@ -157,6 +157,7 @@ struct StencilView {
   DType t;            // element type of coef / dinv
   const void *coef;   // [nsite][5][d][d]
   const void *dinv;   // [nsite][d][d] inverse of the self block (smoother), may be null
+  const void *first;  // [nsite][5][d][d] A_{s,dir} D_nb^{-1} on colour 1 (launch_rbgs_first), may be null
   int const_laplace;  // 1: Example 5.1 operator, applied without reading coef
   double diag;        //    its diagonal 4 + shift
   int periodic;       //    0: Dirichlet
@@ -230,6 +231,10 @@ void launch_rbgs_half(const StencilView &A, void *x, const void *b, int k, int c
 // means x holds zeros on entry (x need not be initialised: the kernels skip it).
 void launch_rbgs_sweep(const StencilView &A, void *x, const void *b, int k, int order, int x_zero,
                        cudaStream_t s);
+// the first red-black sweep from x = 0 when another follows: sets x on colour 1 only
+void launch_rbgs_first(const StencilView &A, void *x, const void *b, int k, cudaStream_t s);
+void launch_first_blocks(DType t, const void *coef, const void *dinv, void *first, int nx, int ny, int d,
+                         cudaStream_t s);
 // rc = P^* r
 void launch_restrict(const ProlongView &P, const void *r, void *rc, int k, cudaStream_t s);
 // x += P ec
