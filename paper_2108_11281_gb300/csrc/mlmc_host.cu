@@ -76,6 +76,7 @@ struct Level {
   int nx = 0, ny = 0, d = 0;
   size_t nsite = 0, n = 0;
   DevBuf coef64, dinv64, coef32, dinv32;   // block stencil and inverse self blocks
+  DevBuf taps9, ra;                        // 9-point levels: [9][site] and R A, likewise
   DevBuf first;                            // A D^-1 of launch_rbgs_first, in the precision of the solves' cycle
   int ax = 0, ay = 0, dc = 0;              // aggregation towards the next level
   DevBuf P64, P32;
@@ -189,7 +190,10 @@ StencilView view(const H_t &h, int l, int lo) {
   v.t = lo ? h.t32 : h.t64;
   v.coef = lo ? L.coef32.p : L.coef64.p;
   v.dinv = lo ? L.dinv32.p : L.dinv64.p;
-  v.first = lo == (h.prm.precision == MLMC_PREC_MIXED_FP32 ? 1 : 0) && L.first.bytes > 16 ? L.first.p : nullptr;
+  const bool solves = lo == (h.prm.precision == MLMC_PREC_MIXED_FP32 ? 1 : 0);   // the solves' cycle
+  v.taps9 = solves ? L.taps9.p : nullptr;
+  v.ra = solves ? L.ra.p : nullptr;
+  v.first = solves && L.first.bytes > 16 ? L.first.p : nullptr;
   v.const_laplace = (l == 0 && h.const_laplace) ? 1 : 0;
   v.diag = h.laplace_diag;
   v.periodic = h.periodic;
@@ -468,8 +472,10 @@ void cycle(H_t &h, int lo, int l, const void *b, void *x, int k) {
   StencilView A = view(h, l, lo);
   const int npre = (l > 0 && h.prm.coarse_smooth > 0) ? h.prm.coarse_smooth : h.prm.smooth_pre;
   const int npost = (l > 0 && h.prm.coarse_smooth > 0) ? h.prm.coarse_smooth : h.prm.smooth_post;
+  // small 9-point levels: everything before the coarse solve is one launch, everything after it another
+  const bool fused9 = npre >= 1 && npost >= 1 && cycle9_ok(A, k);
   if (npre < 1) launch_fill_zero(t, x, blk, s);
-  for (int it = 0; it < npre; ++it) {
+  for (int it = 0; it < npre && !fused9; ++it) {
     if (it == 0 && npre > 1 && A.taps == 5 && (A.const_laplace || A.first)) {
       launch_rbgs_first(A, x, b, k, s);
       h.launches++;
@@ -480,7 +486,11 @@ void cycle(H_t &h, int lo, int l, const void *b, void *x, int k) {
     h.cost += nnz_of(h, l) * k;
   }
   const ProlongView Pv = pview(h, l, lo);
-  if (npre >= 1 && residual_restrict_fused(A, Pv)) {
+  if (fused9) {
+    launch_cycle9_down(A, b, x, cn.b.p, k, npre, s);
+    h.launches++;
+    h.cost += (npre + 1.0) * nnz_of(h, l) * k;
+  } else if (npre >= 1 && residual_restrict_fused(A, Pv)) {
     // the pre-smoothing sweeps end on colour 1, so the residual lives on colour 0 only:
     // residual and restriction in one pass, r never stored
     launch_residual_restrict(A, Pv, x, b, cn.b.p, k, 0, s);
@@ -502,6 +512,12 @@ void cycle(H_t &h, int lo, int l, const void *b, void *x, int k) {
   }
   // the post-smoothing starts with colour 1 and does not read x there, so colour 1 needs no
   // prolongation, unless the fine-level hooks (learned correction, capture) read all of x
+  if (fused9) {
+    launch_cycle9_up(A, b, cn.x.p, x, k, npost, s);
+    h.launches++;
+    h.cost += (double)npost * nnz_of(h, l) * k;
+    return;
+  }
   const bool hooks = l == 0 && lo == 1 && (h.net_on || h.capturing);
   if (npost >= 1 && !hooks && A.taps == 5)
     launch_prolong_add_colour(Pv, cn.x.p, x, k, 0, s);
@@ -1034,6 +1050,27 @@ std::vector<double> galerkin9(const std::vector<double> &Af, int nx, int ny) {
   return Ac;
 }
 
+// R A for bilinear R = P^T as [25][coarse site]: entry (dy + 2) * 5 + dx + 2 multiplies the fine site
+// (2I + 1 + dx, 2J + 1 + dy); entries that leave the grid are zero.
+std::vector<double> restricted9(const std::vector<double> &Af, int nx, int ny) {
+  const int ncx = (nx - 1) / 2, ncy = (ny - 1) / 2;
+  const size_t nc = (size_t)ncx * ncy;
+  std::vector<double> ra(25 * nc, 0.0);
+  auto w1 = [](int a) { return a == 0 ? 1.0 : 0.5; };
+  for (int J = 0; J < ncy; ++J)
+    for (int I = 0; I < ncx; ++I)
+      for (int b = -1; b <= 1; ++b)
+        for (int a = -1; a <= 1; ++a) {
+          const double *ap = &Af[((size_t)(2 * J + 1 + b) * nx + 2 * I + 1 + a) * 9];
+          for (int q = 0; q < 9; ++q) {
+            const int dx = a + kTapDx[q], dy = b + kTapDy[q], ii = 2 * I + 1 + dx, jj = 2 * J + 1 + dy;
+            if (ii < 0 || ii >= nx || jj < 0 || jj >= ny) continue;
+            ra[((size_t)(dy + 2) * 5 + dx + 2) * nc + (size_t)J * ncx + I] += w1(a) * w1(b) * ap[q];
+          }
+        }
+  return ra;
+}
+
 // Levels 2..L by Galerkin coarsening with bilinear P (host, FP64), their smoother
 // diagonals, the coarsest inverse, and the exact term of the hat form,
 // tr(A_L^{-1} R^_L P^_L) = sum_ij (A_L^{-1})_ij M_ji with M = R^_L P^_L obtained by
@@ -1070,7 +1107,27 @@ void build_bilinear(H_t &h, const mlmc_operator_desc *op) {
       }
       check_cuda(cudaMemcpyAsync(C.dinv64.p, dinv.data(), dinv.size() * es, cudaMemcpyHostToDevice, h.stream),
                  "H2D dinv");
-      check_cuda(cudaStreamSynchronize(h.stream), "sync");   // dinv leaves scope
+      // the operator by taps and R A, for the cycle on small levels, in the precision of the solves' cycle
+      std::vector<double> ra, taps;
+      std::vector<float> ra32, taps32;
+      if (C.nsite <= CYCLE9_SITES) {
+        ra = restricted9(A, C.nx, C.ny);
+        taps.resize(A.size());
+        for (size_t s = 0; s < C.nsite; ++s)
+          for (int q = 0; q < 9; ++q) taps[q * C.nsite + s] = A[s * 9 + q];
+        const bool mixed = h.prm.precision == MLMC_PREC_MIXED_FP32;
+        if (mixed) {
+          ra32.assign(ra.begin(), ra.end());
+          taps32.assign(taps.begin(), taps.end());
+        }
+        C.taps9.alloc(taps.size() * (mixed ? sizeof(float) : es));
+        C.ra.alloc(ra.size() * (mixed ? sizeof(float) : es));
+        check_cuda(cudaMemcpyAsync(C.taps9.p, mixed ? (const void *)taps32.data() : taps.data(), C.taps9.bytes,
+                                   cudaMemcpyHostToDevice, h.stream), "H2D taps");
+        check_cuda(cudaMemcpyAsync(C.ra.p, mixed ? (const void *)ra32.data() : ra.data(), C.ra.bytes,
+                                   cudaMemcpyHostToDevice, h.stream), "H2D RA");
+      }
+      check_cuda(cudaStreamSynchronize(h.stream), "sync");   // the host vectors leave scope
     }
     check_cuda(cudaStreamSynchronize(h.stream), "sync");     // A and M are reassigned next
   }

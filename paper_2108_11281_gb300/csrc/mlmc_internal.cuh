@@ -158,6 +158,8 @@ struct StencilView {
   const void *coef;   // [nsite][5][d][d]
   const void *dinv;   // [nsite][d][d] inverse of the self block (smoother), may be null
   const void *first;  // [nsite][5][d][d] A_{s,dir} D_nb^{-1} on colour 1 (launch_rbgs_first), may be null
+  const void *taps9;  // 9-point levels: the operator as [9][nsite], may be null
+  const void *ra;     // 9-point levels: R A as [25][coarse sites], offsets -2 .. 2 in x, then in y
   int const_laplace;  // 1: Example 5.1 operator, applied without reading coef
   double diag;        //    its diagonal 4 + shift
   int periodic;       //    0: Dirichlet
@@ -258,6 +260,12 @@ void launch_jacobi_update(const StencilView &A, void *out, const void *base, con
 void launch_stencil9(const StencilView &A, const void *x, const void *b, void *y, int k, int mode, cudaStream_t s);
 // one 4-colour Gauss-Seidel sweep (order 0: colours 0..3, 1: 3..0); x_zero: x is zeroed first
 void launch_gs9_sweep(const StencilView &A, void *x, const void *b, int k, int order, int x_zero, cudaStream_t s);
+// small 9-point levels, one launch each: x = `sweeps` sweeps from zero and rc = R (b - A x);
+// x += P ec and `sweeps` sweeps in reverse colour order
+constexpr size_t CYCLE9_SITES = 48 * 48;         // the largest such level
+bool cycle9_ok(const StencilView &A, int k);
+void launch_cycle9_down(const StencilView &A, const void *b, void *x, void *rc, int k, int sweeps, cudaStream_t s);
+void launch_cycle9_up(const StencilView &A, const void *b, const void *ec, void *x, int k, int sweeps, cudaStream_t s);
 // rc = P^T r from the fine (2 nxc + 1) x (2 nyc + 1) grid
 void launch_restrict_bilinear(DType t, const void *r, void *rc, int nxc, int nyc, int k, cudaStream_t s);
 // x += P ec on the fine nx x ny grid
