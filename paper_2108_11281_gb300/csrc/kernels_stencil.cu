@@ -91,17 +91,23 @@ __device__ __forceinline__ void stencil_body(const T *__restrict__ coef, const T
   }
 }
 
-// Resident grid striding over the units (row j, chunk of 256 threads of the row): the FP64
-// block applies are bound by the FP64 pipe, which one block per unit leaves idle between
+// Threads per block of the generic kernels.  FP64 is bound by the FP64 pipe, two operations per
+// clock and SM, so what counts is that every SM gets the same number of threads: blocks of 64
+// (the 48^2 x 4 level at 21 columns: smoother half-sweep 7.1 us and apply 11.7 us with 256, whose
+// 96 and 192 blocks load some of 152 SMs twice).
+template <class T> __host__ __device__ constexpr int gen_threads() { return sizeof(typename real_of<T>::type) == 8 ? 64 : 256; }
+
+// Resident grid striding over the units (row j, chunk of one block's threads of the row): the
+// FP64 block applies are bound by the FP64 pipe, which one block per unit leaves idle between
 // blocks.
 template <class T, int D, int VEC>
-__global__ void __launch_bounds__(256) k_stencil(const T *__restrict__ coef, const T *__restrict__ x,
+__global__ void __launch_bounds__(gen_threads<T>()) k_stencil(const T *__restrict__ coef, const T *__restrict__ x,
                                                  const T *__restrict__ b, T *__restrict__ y, int nx, int ny, int kv,
                                                  int mode, int bpr) {
   const int units = bpr * ny;
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
     const int j = u / bpr;
-    stencil_body<T, D, VEC>(coef, x, b, y, nx, ny, kv, mode, j, (u - j * bpr) * 256 + threadIdx.x);
+    stencil_body<T, D, VEC>(coef, x, b, y, nx, ny, kv, mode, j, (u - j * bpr) * gen_threads<T>() + threadIdx.x);
   }
 }
 
@@ -263,7 +269,7 @@ static void stencil_go(const StencilView &A, const void *x, const void *b, void 
       return;
     }
   }
-  constexpr int VW = gen_vec<T, D>::v;
+  constexpr int VW = gen_vec<T, D>::v, TB = gen_threads<T>();
   if (VW > 1 && k % VW == 0) {
     int kv = k / VW;
     if constexpr (std::is_same<T, float>::value && D == 4)
@@ -273,15 +279,15 @@ static void stencil_go(const StencilView &A, const void *x, const void *b, void 
           (const T *)A.coef, (const T *)x, (const T *)b, (T *)y, A.nx, A.ny, kv, mode, bpr, 0);
     }
     else {
-      const int bpr = (A.nx * kv + 255) / 256;
-      static const int occ = blocks_per_sm(k_stencil<T, D, VW>, 256, 0);
-      k_stencil<T, D, VW><<<resident_grid((size_t)bpr * A.ny, occ), 256, 0, s>>>(
+      const int bpr = (A.nx * kv + TB - 1) / TB;
+      static const int occ = blocks_per_sm(k_stencil<T, D, VW>, TB, 0);
+      k_stencil<T, D, VW><<<resident_grid((size_t)bpr * A.ny, occ), TB, 0, s>>>(
           (const T *)A.coef, (const T *)x, (const T *)b, (T *)y, A.nx, A.ny, kv, mode, bpr);
     }
   } else {
-    const int bpr = (A.nx * k + 255) / 256;
-    static const int occ = blocks_per_sm(k_stencil<T, D, 1>, 256, 0);
-    k_stencil<T, D, 1><<<resident_grid((size_t)bpr * A.ny, occ), 256, 0, s>>>(
+    const int bpr = (A.nx * k + TB - 1) / TB;
+    static const int occ = blocks_per_sm(k_stencil<T, D, 1>, TB, 0);
+    k_stencil<T, D, 1><<<resident_grid((size_t)bpr * A.ny, occ), TB, 0, s>>>(
         (const T *)A.coef, (const T *)x, (const T *)b, (T *)y, A.nx, A.ny, k, mode, bpr);
   }
 }
@@ -372,7 +378,7 @@ __global__ void __launch_bounds__(256) k_laplace(const T *__restrict__ x, const 
 // each starts on the rows the previous one wrote last.
 // from_zero = 1: the whole first sweep from x = 0 as one pass over colour 1,
 // x_1 = (b_1 + sum of b_0 / diag) / diag; colour 0 is left unset (see launch_rbgs_first).
-// The grid strides over the units (row, chunk of 256 threads of the row).
+// The grid strides over the units (row, chunk of one block's threads of the row).
 template <class T, int VEC>
 __device__ __forceinline__ void laplace_rbgs_body(T *__restrict__ x, const T *__restrict__ b, int nx, int ny, int kv,
                                                   T dinv, int periodic, int colour, int other_zero, int from_zero,
@@ -399,14 +405,14 @@ __device__ __forceinline__ void laplace_rbgs_body(T *__restrict__ x, const T *__
 }
 
 template <class T, int VEC>
-__global__ void __launch_bounds__(256) k_laplace_rbgs(T *__restrict__ x, const T *__restrict__ b, int nx, int ny,
+__global__ void __launch_bounds__(gen_threads<T>()) k_laplace_rbgs(T *__restrict__ x, const T *__restrict__ b, int nx, int ny,
                                                       int kv, T dinv, int periodic, int colour, int other_zero,
                                                       int from_zero, int bpr) {
   const int units = bpr * ny;
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
     const int jr = u / bpr;
     laplace_rbgs_body<T, VEC>(x, b, nx, ny, kv, dinv, periodic, colour, other_zero, from_zero,
-                              colour ? ny - 1 - jr : jr, (u - jr * bpr) * 256 + threadIdx.x);
+                              colour ? ny - 1 - jr : jr, (u - jr * bpr) * gen_threads<T>() + threadIdx.x);
   }
 }
 
@@ -567,13 +573,14 @@ static void launch_laplace_rbgs(const StencilView &A, void *x, const void *b, in
     typedef decltype(tag) T;
     constexpr int VEC = decltype(vtag)::value;
     int kv = k / VEC;
-    const int bpr = (((A.nx + 1) / 2) * kv + 255) / 256;
-    static const int occ = blocks_per_sm(k_laplace_rbgs<T, VEC>, 256, 0);
+    constexpr int TB = gen_threads<T>();
+    const int bpr = (((A.nx + 1) / 2) * kv + TB - 1) / TB;
+    static const int occ = blocks_per_sm(k_laplace_rbgs<T, VEC>, TB, 0);
     // FP64: a resident grid (FP64-pipe bound); FP32: one block per unit, measured faster
     // there (119 against 124 us per sweep on 1024^2 x 64)
     const unsigned grid = std::is_same<T, double>::value ? resident_grid((size_t)bpr * A.ny, occ)
                                                          : (unsigned)(bpr * A.ny);
-    k_laplace_rbgs<T, VEC><<<grid, 256, 0, s>>>(
+    k_laplace_rbgs<T, VEC><<<grid, TB, 0, s>>>(
         (T *)x, (const T *)b, A.nx, A.ny, kv, (T)(1.0 / A.diag), A.periodic, colour, other_zero, from_zero,
         bpr);
   };
@@ -682,14 +689,15 @@ __device__ __forceinline__ void rbgs_half_body(const T *__restrict__ coef, const
 }
 
 template <class T, int D, int VEC>
-__global__ void __launch_bounds__(256) k_rbgs_half(const T *__restrict__ coef, const T *__restrict__ dinv,
+__global__ void __launch_bounds__(gen_threads<T>()) k_rbgs_half(const T *__restrict__ coef, const T *__restrict__ dinv,
                                                    T *x, const T *src, const T *b, int nx, int ny, int kv,
                                                    int colour, int other_zero, int bpr) {
-  // resident grid striding over the units (row j, chunk of 256 threads of the row)
+  // resident grid striding over the units (row j, chunk of one block's threads of the row)
   const int units = bpr * ny;
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
     const int j = u / bpr;
-    rbgs_half_body<T, D, VEC>(coef, dinv, x, src, b, nx, ny, kv, colour, other_zero, j, (u - j * bpr) * 256 + threadIdx.x);
+    rbgs_half_body<T, D, VEC>(coef, dinv, x, src, b, nx, ny, kv, colour, other_zero, j,
+                              (u - j * bpr) * gen_threads<T>() + threadIdx.x);
   }
 }
 
@@ -788,7 +796,7 @@ static void rbgs_go(const StencilView &A, const void *coef, void *x, const void 
       return;
     }
   }
-  constexpr int VW = rbgs_vec<T, D>::v;
+  constexpr int VW = rbgs_vec<T, D>::v, TB = gen_threads<T>();
   if (VW > 1 && k % VW == 0) {
     int kv = k / VW;
     if constexpr (std::is_same<T, float>::value && D == 4)
@@ -798,15 +806,15 @@ static void rbgs_go(const StencilView &A, const void *coef, void *x, const void 
           (const T *)coef, (const T *)A.dinv, (T *)x, (const T *)src, (const T *)b, A.nx, A.ny, kv, colour, other_zero, bpr);
     }
     else {
-      const int bpr = ((A.nx / 2) * kv + 255) / 256;
-      static const int occ = blocks_per_sm(k_rbgs_half<T, D, VW>, 256, 0);
-      k_rbgs_half<T, D, VW><<<resident_grid((size_t)bpr * A.ny, occ), 256, 0, s>>>(
+      const int bpr = ((A.nx / 2) * kv + TB - 1) / TB;
+      static const int occ = blocks_per_sm(k_rbgs_half<T, D, VW>, TB, 0);
+      k_rbgs_half<T, D, VW><<<resident_grid((size_t)bpr * A.ny, occ), TB, 0, s>>>(
           (const T *)coef, (const T *)A.dinv, (T *)x, (const T *)src, (const T *)b, A.nx, A.ny, kv, colour, other_zero, bpr);
     }
   } else {
-    const int bpr = ((A.nx / 2) * k + 255) / 256;
-    static const int occ = blocks_per_sm(k_rbgs_half<T, D, 1>, 256, 0);
-    k_rbgs_half<T, D, 1><<<resident_grid((size_t)bpr * A.ny, occ), 256, 0, s>>>(
+    const int bpr = ((A.nx / 2) * k + TB - 1) / TB;
+    static const int occ = blocks_per_sm(k_rbgs_half<T, D, 1>, TB, 0);
+    k_rbgs_half<T, D, 1><<<resident_grid((size_t)bpr * A.ny, occ), TB, 0, s>>>(
         (const T *)coef, (const T *)A.dinv, (T *)x, (const T *)src, (const T *)b, A.nx, A.ny, k, colour, other_zero, bpr);
   }
 }
