@@ -193,6 +193,37 @@ __global__ void __launch_bounds__(256) k_prolong_add(const T *__restrict__ P, co
   }
 }
 
+// The same with a site's dofs spread over threads (one thread per site, dof and pack), for
+// levels whose sites and packs alone leave most SMs idle: a thread's d read-modify-writes of x
+// were a serial chain (8 complex dofs on 32^2 sites at k = 32: 6.1 us).
+template <class T, int DC, int VEC>
+__global__ void __launch_bounds__(128) k_prolong_add_dofs(const T *__restrict__ P, const T *__restrict__ ec,
+                                                          T *__restrict__ x, int nx, int ny, int d, int ax, int ay,
+                                                          int kv, int colour) {
+  typedef TPack<T, VEC> V;
+  const int ncx = nx / ax, w = colour < 0 ? nx : nx / 2;
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= (unsigned)w * ny * d * kv) return;
+  const unsigned row = t / (unsigned)kv, ts = row / (unsigned)d;
+  const int c = (int)(t - row * (unsigned)kv), a = (int)(row - ts * (unsigned)d);
+  const int j = (int)(ts / (unsigned)w), m = (int)(ts - (unsigned)j * w);
+  const int i = colour < 0 ? m : 2 * m + ((j + colour) & 1);
+  const int I = (j / ay) * ncx + i / ax, loc = (j % ay) * ax + (i % ax);
+  const V *E = (const V *)ec + (size_t)I * DC * kv + c;
+  const T *Pr = P + ((size_t)I * ax * ay * d + (size_t)loc * d + a) * DC;
+  V *X = (V *)x + ((size_t)(j * nx + i) * d + a) * kv + c;
+  V xv = *X, e[DC];
+#pragma unroll
+  for (int q = 0; q < DC; ++q) e[q] = E[(size_t)q * kv];
+#pragma unroll
+  for (int q = 0; q < DC; ++q) {
+    const T pq = Pr[q];
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) xv.v[u] = madd(xv.v[u], pq, e[q].v[u]);
+  }
+  *X = xv;
+}
+
 template <class T> struct tr_vec { static const int v = 1; };
 template <> struct tr_vec<float> { static const int v = 4; };
 template <> struct tr_vec<double> { static const int v = 2; };
@@ -238,6 +269,16 @@ static void prolong_go(const ProlongView &P, const void *ec, void *x, int k, int
   const int kv = k / vec;
   const size_t sites = colour < 0 ? (size_t)P.nx * P.ny : (size_t)(P.nx / 2) * P.ny;
   const size_t blocks = (sites * kv + 255) / 256;
+  if (P.d > 1 && blocks < 2 * 152) {
+    const unsigned g = (unsigned)((sites * P.d * kv + 127) / 128);
+    if (vec == VW && VW > 1)
+      k_prolong_add_dofs<T, DC, VW><<<g, 128, 0, s>>>((const T *)P.P, (const T *)ec, (T *)x, P.nx, P.ny, P.d, P.ax, P.ay,
+                                                      kv, colour);
+    else
+      k_prolong_add_dofs<T, DC, 1><<<g, 128, 0, s>>>((const T *)P.P, (const T *)ec, (T *)x, P.nx, P.ny, P.d, P.ax, P.ay,
+                                                     kv, colour);
+    return;
+  }
   if (vec == VW && VW > 1) {
     static const int occ = blocks_per_sm(k_prolong_add<T, DC, VW>, 256, 0);
     k_prolong_add<T, DC, VW><<<resident_grid(blocks, occ), 256, 0, s>>>((const T *)P.P, (const T *)ec, (T *)x, P.nx,
