@@ -498,6 +498,89 @@ __global__ void __launch_bounds__(128) k_laplace_residual_restrict(const T *__re
   }
 }
 
+// With few aggregates x packs the colour sites of an aggregate go over RR_SLOTS threads as above, so
+// that a 4 x 4 aggregate's eight are in flight at once (64^2 FP64 level, 64 columns: 9.4 us with
+// one thread per aggregate).  With many, one thread per aggregate needs no sums in shared memory
+// and wins (1024^2 x 64: 94 against 97 us; FP64 192^2 x 21 by 5 us).
+template <class T, int DC, int VEC, int KC>
+__global__ void __launch_bounds__(KC * RR_SLOTS) k_laplace_residual_restrict_slots(const T *__restrict__ x,
+                                                                             const T *__restrict__ b,
+                                                                             const T *__restrict__ P, T *__restrict__ rc,
+                                                                             int nx, int ny, int ax, int ay, int kv,
+                                                                             T diag, int periodic, int colour) {
+  typedef TPack<T, VEC> V;
+  __shared__ V red[RR_SLOTS][DC][KC];
+  const int ncx = nx / ax;
+  const int I = blockIdx.x;
+  const int cc = threadIdx.x, slot = threadIdx.y;
+  const int c = blockIdx.y * KC + cc;
+  const int bi = I % ncx, bj = I / ncx;
+  const V *X = (const V *)x;
+  const V *B = (const V *)b;
+  T acc[DC][VEC];
+#pragma unroll
+  for (int q = 0; q < DC; ++q)
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) acc[q][u] = zero<T>();
+  if (c < kv) {
+    const T *PI = P + (size_t)I * ax * ay * DC;
+    const bool even = ((ax | ay) & 1) == 0;
+    const int hax = ax >> 1, ncol = even ? hax * ay : ax * ay;
+    for (int n = slot; n < ncol; n += RR_SLOTS) {
+      int ii, jj;
+      if (even) {
+        jj = n / hax;
+        ii = 2 * (n - jj * hax) + ((colour + jj) & 1);
+      } else {
+        jj = n / ax;
+        ii = n - jj * ax;
+      }
+      const int i = bi * ax + ii, j = bj * ay + jj;
+      if (((i + j) & 1) != colour) continue;
+      const int s = j * nx + i;
+      const bool on0 = i + 1 < nx || periodic, on1 = i > 0 || periodic;
+      const bool on2 = j + 1 < ny || periodic, on3 = j > 0 || periodic;
+      const int s0 = i + 1 < nx ? s + 1 : j * nx, s1 = i > 0 ? s - 1 : j * nx + nx - 1;
+      const int s2 = j + 1 < ny ? s + nx : i, s3 = j > 0 ? s - nx : (ny - 1) * nx + i;
+      V x0, x1, x2, x3;
+#pragma unroll
+      for (int u = 0; u < VEC; ++u) x0.v[u] = x1.v[u] = x2.v[u] = x3.v[u] = zero<T>();
+      if (on0) x0 = X[(size_t)s0 * kv + c];
+      if (on1) x1 = X[(size_t)s1 * kv + c];
+      if (on2) x2 = X[(size_t)s2 * kv + c];
+      if (on3) x3 = X[(size_t)s3 * kv + c];
+      const V xs = X[(size_t)s * kv + c];
+      const V bb = B[(size_t)s * kv + c];
+      const T *Pr = PI + (size_t)(jj * ax + ii) * DC;
+      T r[VEC];
+#pragma unroll
+      for (int u = 0; u < VEC; ++u) r[u] = (bb.v[u] + ((x0.v[u] + x1.v[u]) + (x2.v[u] + x3.v[u]))) - diag * xs.v[u];
+#pragma unroll
+      for (int q = 0; q < DC; ++q) {
+        const T pq = Pr[q];
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) acc[q][u] = madd(acc[q][u], pq, r[u]);
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < DC; ++q)
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) red[slot][q][cc].v[u] = acc[q][u];
+  __syncthreads();
+  for (int e = slot * KC + cc; e < DC * KC; e += KC * RR_SLOTS) {
+    const int q = e / KC, c2 = e - (e / KC) * KC;
+    const int co = blockIdx.y * KC + c2;
+    if (co >= kv) continue;
+    V o = red[0][q][c2];
+#pragma unroll
+    for (int sl = 1; sl < RR_SLOTS; ++sl)
+#pragma unroll
+      for (int u = 0; u < VEC; ++u) o.v[u] = o.v[u] + red[sl][q][c2].v[u];
+    ((V *)rc)[((size_t)I * DC + q) * kv + co] = o;
+  }
+}
+
 // The same for levels with dc = 8 coarse dofs (the Wilson hierarchy; FP32 data): a block takes one
 // aggregate and 32 columns, a warp a colour site at a time, a lane one column with all its D
 // residual rows and DC sums.  The aggregate's P block and the colour sites' coefficient blocks
@@ -683,6 +766,24 @@ static void laplace_residual_restrict_go(const StencilView &A, const ProlongView
   const int vec = (VW > 1 && k % VW == 0) ? VW : 1;
   const int kv = k / vec;
   const size_t items = (size_t)(P.nx / P.ax) * (P.ny / P.ay) * kv;
+  if (items < (size_t)152 * 128) {
+    // 16 column packs per block, or eight for narrow blocks (and for eight coarse dofs, whose sums
+    // fill the shared memory)
+    auto go = [&](auto vtag, auto ktag) {
+      constexpr int V = decltype(vtag)::value, KC = decltype(ktag)::value;
+      k_laplace_residual_restrict_slots<T, DC, V, KC>
+          <<<dim3((unsigned)(items / kv), (kv + KC - 1) / KC), dim3(KC, RR_SLOTS), 0, s>>>(
+              (const T *)x, (const T *)b, (const T *)P.P, (T *)rc, A.nx, A.ny, P.ax, P.ay, kv, (T)A.diag, A.periodic,
+              colour);
+    };
+    auto width = [&](auto vtag) {
+      if (kv >= 16 && DC <= 4) go(vtag, std::integral_constant<int, 16>());
+      else go(vtag, std::integral_constant<int, 8>());
+    };
+    if (vec == VW && VW > 1) width(std::integral_constant<int, VW>());
+    else width(std::integral_constant<int, 1>());
+    return;
+  }
   const size_t blocks = (items + 127) / 128;
   static const int occ_v = blocks_per_sm(k_laplace_residual_restrict<T, DC, VW>, 128, 0);
   static const int occ_1 = blocks_per_sm(k_laplace_residual_restrict<T, DC, 1>, 128, 0);
