@@ -92,10 +92,11 @@ __device__ __forceinline__ void stencil_body(const T *__restrict__ coef, const T
 }
 
 // Threads per block of the generic kernels.  FP64 is bound by the FP64 pipe, two operations per
-// clock and SM, so what counts is that every SM gets the same number of threads: blocks of 64
+// clock and SM, so what counts is that every SM gets the same number of threads: blocks of 32
 // (the 48^2 x 4 level at 21 columns: smoother half-sweep 7.1 us and apply 11.7 us with 256, whose
-// 96 and 192 blocks load some of 152 SMs twice).
-template <class T> __host__ __device__ constexpr int gen_threads() { return sizeof(typename real_of<T>::type) == 8 ? 64 : 256; }
+// 96 and 192 blocks load some of 152 SMs twice; a 192^2 FP64 solve takes 8.34 ms with 256, 7.97
+// with 64 and 7.77 with 32).
+template <class T> __host__ __device__ constexpr int gen_threads() { return sizeof(typename real_of<T>::type) == 8 ? 32 : 256; }
 
 // Resident grid striding over the units (row j, chunk of one block's threads of the row): the
 // FP64 block applies are bound by the FP64 pipe, which one block per unit leaves idle between
