@@ -1007,7 +1007,7 @@ def main():
     # DRAM bytes per sweep of this kernel version from an ncu capture (None until taken)
     traffic = TRAFFIC.get((w["name"], dom_name))
     if dom_name == "multidot_fp32":
-        label = "k_multidot_partial<float> (inner Arnoldi: 4 basis blocks + w, level 1, k=%d)" % w["block"]
+        label = "k_dots<float> (inner Arnoldi: 4 basis blocks + w, level 1, k=%d)" % w["block"]
     elif w["kind"] == "wilson":
         label = ("k_rbgs_half_rows<cfloat,8> (coarse-level red-black block GS, level 2, d = 8, one sweep = "
                  "2 launches, k=%d; L2-resident working set)" % kcb)

@@ -63,8 +63,8 @@ __global__ void k_add_from_channels(T *x, const float *a, int nsite, int d, int 
 
 // ------------------------------------------------------------------ convolutions
 // out[s][co][c] = epi(sum_{tap, ci} W[co][ci][tap] in[tap_site(s)][ci][c]).  A thread computes
-// PX = 8 consecutive sites of a lattice row for one column and at most 8 output channels: a (row,
-// channel) of its inputs is ten loads for three taps, and a 16-byte shared load of weights
+// PX consecutive sites of a lattice row for one column and at most 8 output channels: with PX = 8 a
+// (row, channel) of its inputs is ten loads for three taps, and a 16-byte shared load of weights
 // (four clocks of the load unit) serves 32 multiply-adds.  Bound by FP32 arithmetic: the 256^2 x
 // 32 network (c0 = 4) takes 14.5 GFLOP, 185 us at the measured 39.2 T FMA/s; 345 us here, 586
 // with one site per thread (five load instructions per 16 multiply-adds), 445 with predicates
@@ -87,11 +87,11 @@ __device__ __forceinline__ void fma_pair(float &a0, float &a1, float x0, float x
 
 enum { EPI_NONE = 0, EPI_RELU = 1, EPI_MASK = 2, EPI_STORE_COMPLEX = 3, EPI_ADD_COMPLEX = 4, EPI_ADD = 5 };
 
-template <int CIN, int COUT, int EPI, bool XIN, int KC>
+template <int CIN, int COUT, int EPI, bool XIN, int KC, int PX>
 __global__ void __launch_bounds__(128, 4) k_conv(const float *__restrict__ in, const float *__restrict__ W, int mirror,
                                                  const float *__restrict__ act, float *__restrict__ out, int nx, int ny,
                                                  int kk, int periodic) {
-  constexpr int PX = 8, CS = XIN ? 2 : 1;                      // sites per thread, channels per load
+  constexpr int CS = XIN ? 2 : 1;                              // channels per load
   constexpr int CB = COUT < 8 ? COUT : 8, HALVES = COUT / CB;  // output channels per thread
   const int k = KC ? KC : kk;
   __shared__ __align__(16) float Ws[9 * CIN * COUT];           // [ty][ci][tx][co]
@@ -405,11 +405,21 @@ static void by_width(int k, F f) {
 template <int CIN, int COUT, int EPI, bool XIN>
 static void conv_go(const float *in, const float *W, int mirror, const float *act, float *out, int nx, int ny, int k,
                     int periodic, cudaStream_t s) {
-  const size_t threads = (size_t)((nx + 7) / 8) * ny * k * (COUT > 8 ? COUT / 8 : 1);
-  by_width(k, [&](auto kc) {
-    k_conv<CIN, COUT, EPI, XIN, decltype(kc)::value><<<resident_grid((threads + 127) / 128, 4), 128, 0, s>>>(
+  auto go = [&](auto px, auto kc) {
+    constexpr int PX = decltype(px)::value;
+    const size_t threads = (size_t)((nx + PX - 1) / PX) * ny * k * (COUT > 8 ? COUT / 8 : 1);
+    k_conv<CIN, COUT, EPI, XIN, decltype(kc)::value, PX><<<resident_grid((threads + 127) / 128, 4), 128, 0, s>>>(
         in, W, mirror, act, out, nx, ny, k, periodic);
-  });
+  };
+  // Sites per thread: eight need the fewest loads, but below some 768 (site, column) pairs per SM
+  // they leave fewer than six warps per SM, each a long serial chain; four or two then give
+  // more, shorter ones (any block width: the offsets' arithmetic hides in the latency).  Network
+  // forward with 8 / 4 / 2 sites: 64^2 x 8 50 / 42.8 / 41.0 us, 96^2 x 8 51 / 46.3 / 47.2, 64^2 x 24
+  // 61 / 53.5 / 56.4, 64^2 x 32 56.6 / 59.1 / 64.9, 128^2 x 8 57.1 / 56.9 / 62.8.
+  const size_t pairs = (size_t)nx * ny * k;
+  if (pairs < (size_t)152 * 384) go(std::integral_constant<int, 2>(), std::integral_constant<int, 0>());
+  else if (pairs < (size_t)152 * 768) go(std::integral_constant<int, 4>(), std::integral_constant<int, 0>());
+  else by_width(k, [&](auto kc) { go(std::integral_constant<int, 8>(), kc); });
   MLMC_LAUNCH_CHECK("k_conv");
 }
 

@@ -334,13 +334,17 @@ __device__ __forceinline__ void laplace_nbr_sum(const Pack<T, VEC> *__restrict__
   for (int u = 0; u < VEC; ++u) sum[u] = (v[0].v[u] + v[1].v[u]) + (v[2].v[u] + v[3].v[u]);
 }
 
-// y = diag x - (sum of the in-grid neighbours) (mode 0) or r = b - that (mode 1),
-// VEC columns per thread with 16-byte loads; grid.y = lattice row, so the +-y
-// neighbours of a block are the rows just touched by the blocks before it (L2
-// hits).  FP32; FP64 data take k_laplace_march.
+// y = diag x - (sum of the in-grid neighbours), r = b - that, or the setup filter's
+// y = diag x + scale (sum of the neighbours); VEC columns per thread with 16-byte loads, rows in
+// order, so the +-y neighbours of a block are the rows just touched by the blocks before it (L2
+// hits).  FP32, and FP64 data of small lattices and narrow blocks; larger ones take
+// k_laplace_march (see laplace_fp64).
+enum { LAP_APPLY = 0, LAP_RESIDUAL = 1, LAP_JACOBI = 2 };
+
 template <class T, int VEC>
 __device__ __forceinline__ void laplace_body(const T *__restrict__ x, const T *__restrict__ b, T *__restrict__ y,
-                                             int nx, int ny, int kv, T diag, int periodic, int mode, int j, int t) {
+                                             int nx, int ny, int kv, T diag, T scale, int periodic, int mode, int j,
+                                             int t) {
   typedef Pack<T, VEC> V;
   if (t >= nx * kv) return;
   const int i = t / kv, c = t - (t / kv) * kv;
@@ -351,10 +355,13 @@ __device__ __forceinline__ void laplace_body(const T *__restrict__ x, const T *_
   T sum[VEC];
   laplace_nbr_sum<T, VEC>(X, n, kv, c, sum);
   V out;
-  if (mode) {
+  if (mode == LAP_RESIDUAL) {
     V bb = ((const V *)b)[(size_t)s * kv + c];
 #pragma unroll
     for (int u = 0; u < VEC; ++u) out.v[u] = (bb.v[u] + sum[u]) - diag * xc.v[u];
+  } else if (mode == LAP_JACOBI) {
+#pragma unroll
+    for (int u = 0; u < VEC; ++u) out.v[u] = diag * xc.v[u] + scale * sum[u];
   } else {
 #pragma unroll
     for (int u = 0; u < VEC; ++u) out.v[u] = diag * xc.v[u] - sum[u];
@@ -365,11 +372,12 @@ __device__ __forceinline__ void laplace_body(const T *__restrict__ x, const T *_
 // Resident grid striding over the units (row j, chunk of 256 threads of the row) in row order.
 template <class T, int VEC>
 __global__ void __launch_bounds__(256) k_laplace(const T *__restrict__ x, const T *__restrict__ b, T *__restrict__ y,
-                                                 int nx, int ny, int kv, T diag, int periodic, int mode, int bpr) {
+                                                 int nx, int ny, int kv, T diag, T scale, int periodic, int mode,
+                                                 int bpr) {
   const int units = bpr * ny;
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
     const int j = u / bpr;
-    laplace_body<T, VEC>(x, b, y, nx, ny, kv, diag, periodic, mode, j, (u - j * bpr) * 256 + threadIdx.x);
+    laplace_body<T, VEC>(x, b, y, nx, ny, kv, diag, scale, periodic, mode, j, (u - j * bpr) * 256 + threadIdx.x);
   }
 }
 
@@ -432,7 +440,6 @@ static int laplace_vec(int k) {
 // The additions are issued as multiply-adds by 1 (same result; 0.63 against 0.53 T/s).
 // 1024^2 x 64: 402 us (3.3 operations per site: 350 us at the measured rate), 531 us with the
 // neighbour sum per site.
-enum { LAP_APPLY = 0, LAP_RESIDUAL = 1, LAP_JACOBI = 2 };
 constexpr int MP = 4;
 
 template <int VEC, int MODE>
@@ -522,10 +529,20 @@ static void laplace_march(const StencilView &A, const void *x, const void *b, vo
                           cudaStream_t s) {
   const int vec = k % 2 == 0 ? 2 : 1, kv = k / vec;
   const size_t strips = (A.nx + MP - 1) / MP;
-  // long walks recompute least (one u per strip column and walk); shorter ones where the grid
-  // would not fill the SMs
-  int JB = 64;
-  while (JB > 2 && strips * ((A.ny + JB - 1) / JB) * kv < (size_t)152 * 512) JB /= 2;
+  // Rows per walk: the smallest time of the busiest SM, blocks x (13 operations per row and 4
+  // before the first, for the strip and pack), with at least four blocks per SM where any walk
+  // allows it; the longer walk where that is equal.  Powers of two alone left 937 blocks on 152
+  // SMs: 768^2 x 13 took 75.8 us.
+  int JB = 2;
+  size_t best = ~(size_t)0;
+  for (int jb = 64; jb >= 2; --jb) {
+    const size_t blocks = (strips * ((A.ny + jb - 1) / jb) * kv + 127) / 128;
+    const size_t cost = (blocks + 151) / 152 * (13 * jb + 4);
+    if (blocks >= 4 * 152 && cost < best) {
+      best = cost;
+      JB = jb;
+    }
+  }
   const size_t threads = strips * ((A.ny + JB - 1) / JB) * kv;
   const unsigned g = (unsigned)((threads + 127) / 128);
   if (vec == 2)
@@ -536,32 +553,45 @@ static void laplace_march(const StencilView &A, const void *x, const void *b, vo
                                                scale, 1.0, A.periodic, JB);
 }
 
+template <class T, int VEC>
+static void laplace_sites(const StencilView &A, const void *x, const void *b, void *y, int k, T diag, T scale, int mode,
+                          cudaStream_t s) {
+  const int kv = k / VEC, bpr = (A.nx * kv + 255) / 256;
+  static const int occ = blocks_per_sm(k_laplace<T, VEC>, 256, 0);
+  k_laplace<T, VEC><<<resident_grid((size_t)bpr * A.ny, occ), 256, 0, s>>>(
+      (const T *)x, (const T *)b, (T *)y, A.nx, A.ny, kv, diag, scale, A.periodic, mode, bpr);
+}
+
+// FP64: strips walked by few threads only pay where the pipe is busy.  Below about 4600 entries
+// per SM a launch is a round trip or two to L2, and a thread per site and pack is shorter
+// (whole calls, site against strip: 64^2 x 2 12.3 / 15.2 us, 256^2 x 5 15.3 / 16.2, 512^2 x 2
+// 16.6 / 17.7, 128^2 x 32 16.9 / 17.0; 192^2 x 21 19.0 / 18.3, 128^2 x 64 21.9 / 20.5).
+template <int MODE>
+static void laplace_fp64(const StencilView &A, const void *x, const void *b, void *y, int k, double diag, double scale,
+                         cudaStream_t s) {
+  if ((size_t)A.nx * A.ny * k >= (size_t)152 * 4608) laplace_march<MODE>(A, x, b, y, k, diag, scale, s);
+  else if (laplace_vec<double>(k) == 2) laplace_sites<double, 2>(A, x, b, y, k, diag, scale, MODE, s);
+  else laplace_sites<double, 1>(A, x, b, y, k, diag, scale, MODE, s);
+}
+
 // One damped-Jacobi sweep of the setup filter for Example 5.1 in one pass (out must not alias x):
 // x - omega D^-1 (A x) with A x = diag x - (sum of the in-grid neighbours), written as
 // (1 - omega) x + (omega / diag) (sum of the neighbours).
 void launch_laplace_jacobi(const StencilView &A, const void *x, void *out, int k, double omega, cudaStream_t s) {
   if (!A.const_laplace || A.t != F64)
     throw cuda_error{cudaErrorInvalidValue, "laplace_jacobi: constant-coefficient Laplacian in FP64 only"};
-  laplace_march<LAP_JACOBI>(A, x, nullptr, out, k, 1.0 - omega, omega / A.diag, s);
+  laplace_fp64<LAP_JACOBI>(A, x, nullptr, out, k, 1.0 - omega, omega / A.diag, s);
   MLMC_LAUNCH_CHECK("k_laplace_march");
 }
 
 static void launch_laplace(const StencilView &A, const void *x, const void *b, void *y, int k, int mode,
                            cudaStream_t s) {
   if (A.t == F64) {
-    if (mode) laplace_march<LAP_RESIDUAL>(A, x, b, y, k, A.diag, 0.0, s);
-    else laplace_march<LAP_APPLY>(A, x, b, y, k, A.diag, 0.0, s);
+    if (mode) laplace_fp64<LAP_RESIDUAL>(A, x, b, y, k, A.diag, 0.0, s);
+    else laplace_fp64<LAP_APPLY>(A, x, b, y, k, A.diag, 0.0, s);
   } else if (A.t == F32) {
-    auto go = [&](auto vtag) {
-      constexpr int VEC = decltype(vtag)::value;
-      int kv = k / VEC;
-      const int bpr = (A.nx * kv + 255) / 256;
-      static const int occ = blocks_per_sm(k_laplace<float, VEC>, 256, 0);
-      k_laplace<float, VEC><<<resident_grid((size_t)bpr * A.ny, occ), 256, 0, s>>>(
-          (const float *)x, (const float *)b, (float *)y, A.nx, A.ny, kv, (float)A.diag, A.periodic, mode, bpr);
-    };
-    if (laplace_vec<float>(k) == 4) go(std::integral_constant<int, 4>());
-    else go(std::integral_constant<int, 1>());
+    if (laplace_vec<float>(k) == 4) laplace_sites<float, 4>(A, x, b, y, k, (float)A.diag, 0.f, mode ? 1 : 0, s);
+    else laplace_sites<float, 1>(A, x, b, y, k, (float)A.diag, 0.f, mode ? 1 : 0, s);
   } else {
     throw cuda_error{cudaErrorInvalidValue, "constant-coefficient Laplacian is real"};
   }
