@@ -707,13 +707,14 @@ bool conv_on_tc(const H_t &h, int nx, int k, int cin, int cout) {
   return want && conv_tc_ok(nx, k, cin, cout);
 }
 
-void conv_forward(H_t &h, int ci, int co, bool relu, const float *in, const float *W, float *out, int k) {
+void conv_forward(H_t &h, int ci, int co, bool relu, const float *in, const float *W, float *out, int k,
+                  bool by_tap = false) {
   const Level &F = h.lv[0];
   const int per = h.periodic || h.complex_op;
   if (conv_on_tc(h, F.nx, k, ci, co))
     launch_conv_tc(in, W, nullptr, out, F.nx, F.ny, k, ci, co, per, 0, relu ? 1 : 0, h.err.as<int>(), h.stream);
   else
-    launch_conv_fwd(ci, co, in, W, out, F.nx, F.ny, k, per, h.stream);
+    launch_conv_fwd(ci, co, in, W, out, F.nx, F.ny, k, per, h.stream, by_tap);
   h.launches++;
 }
 
@@ -749,13 +750,13 @@ void net_hidden(H_t &h, const void *r, int k, bool keep_input) {
   if (keep_input || conv_on_tc(h, F.nx, k, h.net_c0, NET_CH)) {
     launch_to_channels(h.t32, r, h.act0.as<float>(), (int)F.nsite, F.d, k, h.stream);
     h.launches++;
-    conv_forward(h, h.net_c0, NET_CH, true, h.act0.as<float>(), netW1(h), h.act1.as<float>(), k);
+    conv_forward(h, h.net_c0, NET_CH, true, h.act0.as<float>(), netW1(h), h.act1.as<float>(), k, keep_input);
   } else {
     launch_conv_first(h.t32, h.net_c0, r, netW1(h), h.act1.as<float>(), F.nx, F.ny, k, h.periodic || h.complex_op,
                       h.stream);
     h.launches++;
   }
-  conv_forward(h, NET_CH, NET_CH, true, h.act1.as<float>(), netW2(h), h.act2.as<float>(), k);
+  conv_forward(h, NET_CH, NET_CH, true, h.act1.as<float>(), netW2(h), h.act2.as<float>(), k, keep_input);
 }
 
 // e = net(r), or e += net(r)

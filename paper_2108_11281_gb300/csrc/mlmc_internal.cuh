@@ -324,8 +324,9 @@ namespace mlmc {
 // learned correction (kernels_learned.cu)
 void launch_to_channels(DType t, const void *x, float *a, int nsite, int d, int k, cudaStream_t s);
 void launch_add_from_channels(DType t, void *x, const float *a, int nsite, int d, int k, cudaStream_t s);
+// by_tap: layers with a ReLU add up tap by tap (see k_conv)
 void launch_conv_fwd(int ci, int co, const float *in, const float *W, float *out, int nx, int ny, int k,
-                     int periodic, cudaStream_t s);
+                     int periodic, cudaStream_t s, bool by_tap = false);
 void launch_conv_bwd_data(int ci, int co, const float *gout, const float *W, const float *act, float *gin, int nx,
                           int ny, int k, int periodic, cudaStream_t s);
 // the first and last layer reading and writing the vector block itself (real, or complex
