@@ -205,6 +205,17 @@ __global__ void __launch_bounds__(RT) k_dots_reduce(const A *__restrict__ partia
   }
 }
 
+// Columns of a 16-byte pack where every row allows it.
+static int pack_of(DType t, int k) {
+  const int vw = 16 / (int)dtype_size(t);
+  return k % vw ? 1 : vw;
+}
+
+template <class T> constexpr DType type_of() {
+  return std::is_same<T, double>::value ? F64 : std::is_same<T, float>::value ? F32
+       : std::is_same<T, cdouble>::value ? C64 : C32;
+}
+
 int multidot_parts(DType t, size_t rows, int k) {
   // enough row chunks to give every thread a few rows, at most one block per SM; FP64 data two,
   // so that a lane adds up half as many products
@@ -297,29 +308,31 @@ void launch_multidot(DType t, const void *V, size_t vstride, int nvec, const voi
 }
 
 // ------------------------------------------------------------------ multi-AXPY
-// w[r][c] = (INIT ? 0 : w[r][c]) + sign * sum_v V_v[r][c] * h[v * hstride + c] over one pass of
-// nv <= AXPY_GROUP vectors; the coefficients, rounded to the storage precision, sit in shared
-// memory.  norm (optional): per block and column the sum of |w_new|^2 over its rows, for the
-// Arnoldi step, summed per thread in row order (float pairs every 16 rows) and over the
-// block's slots in fixed order; INIT updates (the solution) need none.
-// HBM-bound on large blocks ((nv + 2) passes, nv + 1 with INIT): four FP32 vectors on
-// 1024^2 x 64 take 261 us, 6.18 TB/s (268 us before); on 2.4 MB blocks of 48 columns, whose
-// column groups do not divide 256 threads, 3.7 us (10.3: the norms were summed serially).
+// w[r][c] = (INIT ? 0 : w[r][c]) + sign * sum_v V_v[r][c] * h[v * k + c], v0 <= v < v0 + nv, V_0 = first and
+// V_v = V + v * vstride: one pass over w for all vectors whose coefficients, rounded to the
+// storage precision, fit in 32 KB of shared memory.  norm (optional): per block and column the
+// sum of |w_new|^2 over its rows, for the Arnoldi step, summed per thread in row order (float
+// pairs every 16 rows) and over the block's slots in fixed order; INIT updates (the solution) need none.
+// HBM-bound on large blocks ((nv + 2) passes, nv + 1 with INIT): all vectors in one pass, not
+// eight, since a restarted solve has up to 64 of them.  30 FP64 vectors of 65536 x 64: 223 us
+// (284 in passes of eight, 238 with 256 threads striding over packs), FP32 94 (145, 112);
+// 27 FP64 vectors of 1024 x 8: 10.4 us (30.9, 8.3); 12 FP32 vectors of 262144 x 64: 157 us,
+// 6.0 TB/s (196, 173).  A block has one row of packs per thread where the rows are few: with
+// four, 8 vectors of 1024 x 8 complex FP64 were on four SMs and took 22.6 us, now 8.3.
 template <class T, class H, int VEC, bool INIT>
-__global__ void __launch_bounds__(DT, 2) k_axpy(T *__restrict__ w, VecList<T> V, int nv, const H *__restrict__ h,
-                                                int hstride, double sign, size_t rows, int k,
-                                                typename lane_of<T>::A *__restrict__ norm) {
+__global__ void __launch_bounds__(DT, 2) k_axpy(T *__restrict__ w, const T *__restrict__ first, const T *__restrict__ V,
+                                                size_t vstride, int v0, int nv, const H *__restrict__ h, double sign,
+                                                size_t rows, int k, typename lane_of<T>::A *__restrict__ norm) {
   typedef typename lane_of<T>::S S;
   typedef typename lane_of<T>::A A;
   typedef DPack<T, VEC> P;
+  constexpr int UN = std::is_same<T, cfloat>::value ? 2 : 4;   // vectors in flight (complex FP32 with 4: 5 % slower)
   extern __shared__ __align__(16) unsigned char axpy_smem[];
   __shared__ __align__(16) S red[DT * VEC];
   __shared__ A red2[DT];
   T *hs = (T *)axpy_smem;
-  for (int e = threadIdx.x; e < nv * k; e += DT) {
-    const int v = e / k, c = e - v * k;
-    hs[e] = cvt<T, H>(rmul((typename real_of<H>::type)sign, h[(size_t)v * hstride + c]));
-  }
+  for (int e = threadIdx.x; e < nv * k; e += DT)
+    hs[e] = cvt<T, H>(rmul((typename real_of<H>::type)sign, h[(size_t)v0 * k + e]));
   __syncthreads();
   const int kv = k / VEC, slots = DT / kv;
   const int cv = threadIdx.x % kv, slot = threadIdx.x / kv;
@@ -335,42 +348,47 @@ __global__ void __launch_bounds__(DT, 2) k_axpy(T *__restrict__ w, VecList<T> V,
     sq[u] = 0;
     acc_zero(tot[u]);
   }
-  if (live) {
-    int n = 0;
-    constexpr int U = 2;
-    size_t r = r0 + slot;
-    for (; r < r1; r += (size_t)U * slots) {
-      P a[U];
-      size_t o[U];
+  // rows r, r + slots, ...: U of them
+  auto step = [&](size_t r, auto count) {
+    constexpr int U = decltype(count)::value;
+    P a[U];
+    size_t o[U];
 #pragma unroll
-      for (int q = 0; q < U; ++q) {
-        o[q] = min(r + (size_t)q * slots, r1 - 1) * kv + cv;   // past the end: a row of the chunk, not stored
-        if (INIT) {
+    for (int q = 0; q < U; ++q) {
+      o[q] = (r + (size_t)q * slots) * kv + cv;
+      if (INIT) {
 #pragma unroll
-          for (int u = 0; u < VEC; ++u) a[q].v[u] = zero<T>();
-        } else {
-          a[q] = W[o[q]];
-        }
+        for (int u = 0; u < VEC; ++u) a[q].v[u] = zero<T>();
+      } else {
+        a[q] = W[o[q]];
       }
-#pragma unroll 2
-      for (int v = 0; v < nv; ++v) {
-        const P hh = Hp[v * kv];
-        P x[U];
+    }
+    const T *src = v0 == 0 ? first : V + (size_t)v0 * vstride;
+#pragma unroll UN
+    for (int v = 0; v < nv; ++v) {
+      const P hh = Hp[v * kv];
+      P x[U];
 #pragma unroll
-        for (int q = 0; q < U; ++q) x[q] = ((const P *)V.v[v])[o[q]];
-#pragma unroll
-        for (int q = 0; q < U; ++q)
-#pragma unroll
-          for (int u = 0; u < VEC; ++u) a[q].v[u] = madd(a[q].v[u], x[q].v[u], hh.v[u]);
-      }
+      for (int q = 0; q < U; ++q) x[q] = ((const P *)src)[o[q]];
+      src = V + (size_t)(v0 + v + 1) * vstride;
 #pragma unroll
       for (int q = 0; q < U; ++q)
-        if (r + (size_t)q * slots < r1) {
-          W[o[q]] = a[q];
-          if (!INIT)
 #pragma unroll
-            for (int u = 0; u < VEC; ++u) sq[u] += abs2(a[q].v[u]);
-        }
+        for (int u = 0; u < VEC; ++u) a[q].v[u] = madd(a[q].v[u], x[q].v[u], hh.v[u]);
+    }
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      W[o[q]] = a[q];
+      if (!INIT)
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) sq[u] += abs2(a[q].v[u]);
+    }
+  };
+  if (live) {
+    int n = 0;
+    size_t r = r0 + slot;
+    for (; r + slots < r1; r += 2 * (size_t)slots) {
+      step(r, std::integral_constant<int, 2>());
       if (!INIT && sizeof(S) == 4 && (++n & 7) == 0) {
 #pragma unroll
         for (int u = 0; u < VEC; ++u) {
@@ -379,6 +397,7 @@ __global__ void __launch_bounds__(DT, 2) k_axpy(T *__restrict__ w, VecList<T> V,
         }
       }
     }
+    if (r < r1) step(r, std::integral_constant<int, 1>());
   }
   if (!INIT && norm) {
     S v[VEC];
@@ -395,9 +414,10 @@ __global__ void __launch_bounds__(DT, 2) k_axpy(T *__restrict__ w, VecList<T> V,
 
 static const int AXPY_SMEM = 32 * 1024;
 
-int multiaxpy_norm_parts(size_t rows, int k) {
-  const size_t per = std::max<size_t>(1, (size_t)DT * 4 / std::max(k, 1));
-  return (int)std::min<size_t>(AXPY_PARTS, std::max<size_t>(1, (rows + per - 1) / per));
+// A row of packs per thread, at most two blocks per SM.
+int multiaxpy_norm_parts(DType t, size_t rows, int k) {
+  const size_t slots = std::max(1, DT / std::max(k / pack_of(t, k), 1));
+  return (int)std::min<size_t>(AXPY_PARTS, std::max<size_t>(1, (rows + slots - 1) / slots));
 }
 
 namespace {
@@ -409,22 +429,16 @@ int axpy_all(void *w, const void *v0, const void *V, size_t vstride, int nvec, c
   typedef typename lane_of<T>::A A;
   const bool packed = VW > 1 && packs_ok<T>(k, {w, v0, V}) && vstride % VW == 0;
   if ((packed ? k / VW : k) > DT) throw cuda_error{cudaErrorInvalidValue, "multiaxpy: more column groups than threads"};
-  int group = std::min(DOT_MAXV, AXPY_SMEM / (k * (int)sizeof(T)));
-  if (group < 1) group = 1;
-  const int parts = multiaxpy_norm_parts(rows, k);
+  const int group = std::max(1, AXPY_SMEM / (k * (int)sizeof(T)));
+  const int parts = multiaxpy_norm_parts(type_of<T>(), rows, k);
   int passes = 0;
   for (int i0 = 0; i0 < nvec; i0 += group) {
-    VecList<T> L;
     const int nv = std::min(nvec - i0, group);
-    for (int i = 0; i < DOT_MAXV; ++i) {
-      const int id = i0 + std::min(i, nv - 1);
-      L.v[i] = id == 0 ? (const T *)v0 : (const T *)V + (size_t)id * vstride;
-    }
     const bool first = init && i0 == 0, last = i0 + nv >= nvec;
     const size_t smem = (size_t)nv * k * sizeof(T);
     auto go = [&](auto vec, auto ini) {
       k_axpy<T, H, decltype(vec)::value, decltype(ini)::value><<<parts, DT, smem, s>>>(
-          (T *)w, L, nv, (const H *)h + (size_t)i0 * k, k, sign, rows, k, last ? (A *)norm : nullptr);
+          (T *)w, (const T *)v0, (const T *)V, vstride, i0, nv, (const H *)h, sign, rows, k, last ? (A *)norm : nullptr);
     };
     if (packed && first) go(std::integral_constant<int, VW>(), std::true_type());
     else if (packed) go(std::integral_constant<int, VW>(), std::false_type());
@@ -438,10 +452,13 @@ int axpy_all(void *w, const void *v0, const void *V, size_t vstride, int nvec, c
 
 }  // namespace
 
-void launch_multiaxpy(DType t, void *w, const void *V, size_t vstride, int nvec, const void *h, double sign,
-                      size_t rows, int k, bool init, cudaStream_t s) {
-  if (nvec <= 0) return;
-  MLMC_DISPATCH(t, T, axpy_all<T, typename acc_of<T>::type>(w, V, V, vstride, nvec, h, sign, rows, k, init, nullptr, s));
+int launch_multiaxpy(DType t, void *w, const void *V, size_t vstride, int nvec, const void *h, double sign,
+                     size_t rows, int k, bool init, cudaStream_t s) {
+  int passes = 0;
+  if (nvec <= 0) return passes;
+  MLMC_DISPATCH(t, T, passes = (axpy_all<T, typename acc_of<T>::type>(w, V, V, vstride, nvec, h, sign, rows, k, init,
+                                                                      nullptr, s)));
+  return passes;
 }
 
 // ------------------------------------------------------------------ fixed-length FGMRES, per column
@@ -676,7 +693,7 @@ int launch_fgmres_dots(DType t, const void *b, const void *V, size_t vstride, in
 
 void launch_fgmres_mid(DType t, const void *partials, const void *norm, int j, int m, size_t rows, int k, double *n2,
                        void *D, void *coef, cudaStream_t s) {
-  const int nparts = multidot_parts(t, rows, k), nnorm = multiaxpy_norm_parts(rows, k);
+  const int nparts = multidot_parts(t, rows, k), nnorm = multiaxpy_norm_parts(t, rows, k);
   MLMC_DISPATCH(t, T, {
     typedef typename lane_of<T>::A A;
     typedef typename acc_of<T>::type H;
@@ -689,7 +706,7 @@ void launch_fgmres_mid(DType t, const void *partials, const void *norm, int j, i
 
 void launch_fgmres_tail(DType t, const void *partials, const void *norm, int its, int m, size_t rows, int k,
                         double *n2, const void *D, void *y, cudaStream_t s) {
-  const int nparts = multidot_parts(t, rows, k), nnorm = multiaxpy_norm_parts(rows, k);
+  const int nparts = multidot_parts(t, rows, k), nnorm = multiaxpy_norm_parts(t, rows, k);
   MLMC_DISPATCH(t, T, {
     typedef typename lane_of<T>::A A;
     typedef typename acc_of<T>::type H;

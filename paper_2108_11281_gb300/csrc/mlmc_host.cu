@@ -232,7 +232,7 @@ void alloc_krylov(H_t &h, Krylov &K, DType t, size_t n, int k, int m, bool fixed
   size_t dots = 0, norms = 0;
   for (int kk = 1; kk <= k; ++kk) {
     dots = std::max(dots, (size_t)multidot_parts(t, n, kk) * kk);
-    norms = std::max(norms, (size_t)multiaxpy_norm_parts(n, kk) * kk);
+    norms = std::max(norms, (size_t)multiaxpy_norm_parts(t, n, kk) * kk);
   }
   K.partials.alloc(dots * (m + 2) * as);
   K.H.alloc((size_t)m * (m + 1) * k * as);
@@ -412,13 +412,11 @@ int fgmres(H_t &h, Krylov &K, int l, int lo, const void *b, void *x, int k, doub
       M(Vj(j), Zj(j));
       apply_op(h, l, lo, Zj(j), Vj(j + 1), k);
       multidot(h, K, K.V.p, j + 1, Vj(j + 1), k, Hcol(j));
-      launch_multiaxpy(K.t, Vj(j + 1), K.V.p, blk, j + 1, Hcol(j), -1.0, K.n, k, false, s);
-      h.launches++;
+      h.launches += launch_multiaxpy(K.t, Vj(j + 1), K.V.p, blk, j + 1, Hcol(j), -1.0, K.n, k, false, s);
       if (reorth) {
         multidot(h, K, K.V.p, j + 1, Vj(j + 1), k, K.h2.p);
-        launch_multiaxpy(K.t, Vj(j + 1), K.V.p, blk, j + 1, K.h2.p, -1.0, K.n, k, false, s);
+        h.launches += 1 + launch_multiaxpy(K.t, Vj(j + 1), K.V.p, blk, j + 1, K.h2.p, -1.0, K.n, k, false, s);
         launch_add_acc(K.hc, Hcol(j), K.h2.p, (j + 1) * k, s);
-        h.launches += 2;
       }
       multidot(h, K, Vj(j + 1), 1, Vj(j + 1), k, (char *)Hcol(j) + (size_t)(j + 1) * k * as);
       launch_arnoldi_step(K.hc, K.H.p, K.cs.p, K.sn.p, K.g.p, j, m, k, K.active.as<int>(), K.jdone.as<int>(),
@@ -430,8 +428,7 @@ int fgmres(H_t &h, Krylov &K, int l, int lo, const void *b, void *x, int k, doub
       if (read_nactive(h, K, k) == 0 || its >= maxit) break;
     }
     launch_trisolve(K.hc, K.H.p, K.g.p, K.y.p, K.jdone.as<int>(), m, k, s);
-    launch_multiaxpy(K.t, x, K.Z.p, blk, jlast, K.y.p, 1.0, K.n, k, x_zero, s);
-    h.launches += 2;
+    h.launches += 1 + launch_multiaxpy(K.t, x, K.Z.p, blk, jlast, K.y.p, 1.0, K.n, k, x_zero, s);
     // FP64 true residual: restart, or stop when every column meets tol
     residual_op(h, l, lo, x, b, Vj(0), k);
     r = Vj(0);

@@ -199,8 +199,8 @@ void launch_multidot(DType t, const void *V, size_t vstride, int nvec, const voi
                      int k, void *partials, int nparts, void *out, cudaStream_t s);
 int multidot_parts(DType t, size_t rows, int k);
 // w[i][c] = (init ? 0 : w[i][c]) + sign * sum_v V_v[i][c] * h[v][c], h FP64 (complex FP64)
-void launch_multiaxpy(DType t, void *w, const void *V, size_t vstride, int nvec, const void *h, double sign,
-                      size_t rows, int k, bool init, cudaStream_t s);
+int launch_multiaxpy(DType t, void *w, const void *V, size_t vstride, int nvec, const void *h, double sign,
+                     size_t rows, int k, bool init, cudaStream_t s);   // returns its launches
 
 // The fixed-length FGMRES with an unnormalised basis u_0 = b, u_1, ... (V + i * vstride); each
 // returns its number of launches where that depends on the length.
@@ -218,7 +218,7 @@ int launch_fgmres_axpy(DType t, void *w, const void *b, const void *V, size_t vs
                        size_t rows, int k, void *norm, cudaStream_t s);
 int launch_fgmres_update(DType t, void *x, const void *Z, size_t vstride, int nvec, const void *y, size_t rows, int k,
                          cudaStream_t s);
-int multiaxpy_norm_parts(size_t rows, int k);
+int multiaxpy_norm_parts(DType t, size_t rows, int k);
 
 }  // namespace mlmc
 
