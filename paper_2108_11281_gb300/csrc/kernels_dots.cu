@@ -76,34 +76,59 @@ __device__ __forceinline__ void chunk_of(size_t rows, size_t &r0, size_t &r1) {
   r1 = min(r0 + chunk, rows);
 }
 
-// Sums `val` (one scalar set per thread: NC scalars of columns cv * VEC ...) over the
-// block's slots in fixed order into out[e], e < E = k * C scalars of one output row.
-// red: DT * NC lane values, red2: DT sums.  Ends with the block synchronised.
-template <class T, int NC>
-__device__ void block_sum(const typename lane_of<T>::S *val, typename lane_of<T>::S *red, typename lane_of<T>::A *red2,
-                          int E, int slots, bool live, typename lane_of<T>::A *out) {
+// out[r * E + e] = sum over the block's slots, in fixed order, of the nr <= RB rows of NC scalars per
+// thread in val; e < E = k * C scalars of a row.  The rows are summed together, and the threads that
+// share a scalar meet in steps of at most eight: with a row at a time and one chain over those
+// threads, 511 long for one column, eight FP64 vectors of 1024 x 1 took 174 us (11 now), of
+// 1024 x 8 41 us (14) and of 4096 x 64 20 us (12).  red: RB * DT * NC lane values, red2: DT sums.
+// Ends with the block synchronised.
+template <class T, int NC, int RB>
+__device__ __forceinline__ void block_sums(const typename lane_of<T>::S (*val)[NC], int nr, typename lane_of<T>::S *red,
+                                           typename lane_of<T>::A *red2, int E, int slots, bool live,
+                                           typename lane_of<T>::A *out) {
   typedef typename lane_of<T>::A A;
   const int tid = threadIdx.x;
 #pragma unroll
-  for (int u = 0; u < NC; ++u) red[tid * NC + u] = live ? val[u] : 0;
+  for (int r = 0; r < RB; ++r)
+    if (r < nr) {
+#pragma unroll
+      for (int u = 0; u < NC; ++u) red[(r * DT + tid) * NC + u] = live ? val[r][u] : 0;
+    }
   __syncthreads();
-  // scalar e of the row sits at red[slot * E + e]; G threads share its slots
-  const int G = E < DT ? DT / E : 1;
-  for (int e0 = 0; e0 < E; e0 += DT) {
-    const int e = e0 + tid % min(E, DT), g = tid / min(E, DT);
+  // scalar e of row r sits at red[r * DT * NC + slot * E + e]; G threads share its slots
+  const int items = nr * E;
+  int G = min(DT / items, slots);
+  if (G < 2) {
+    for (int i = tid; i < items; i += DT) {
+      const int r = i / E;
+      const typename lane_of<T>::S *src = red + r * DT * NC + (i - r * E);
+      A a;
+      acc_zero(a);
+      for (int s = 0; s < slots; ++s) acc_add(a, src[s * E]);
+      out[i] = a;
+    }
+  } else {
+    const int g = tid / items, i = tid - g * items, r = i / E;
+    const typename lane_of<T>::S *src = red + r * DT * NC + (i - r * E);
     A a;
     acc_zero(a);
-    if (g < G && e < E)
-      for (int s = g; s < slots; s += G) acc_add(a, red[s * E + e]);
-    if (G > 1) {
+    if (g < G) {
+      for (int s = g; s < slots; s += G) acc_add(a, src[s * E]);
       red2[tid] = a;
+    }
+    while (G > 8) {
+      const int H = G > 64 ? 64 : 8;
       __syncthreads();
-      if (g == 0) {
-        for (int q = 1; q < G; ++q) acc_add(a, red2[q * E + e]);
-        out[e] = a;
+      if (g < H) {
+        for (int q = g + H; q < G; q += H) acc_add(a, red2[q * items + i]);
+        red2[tid] = a;               // read by this thread alone in this step
       }
-    } else if (g == 0 && e < E) {
-      out[e] = a;
+      G = H;
+    }
+    __syncthreads();
+    if (g == 0) {
+      for (int q = 1; q < G; ++q) acc_add(a, red2[q * items + i]);
+      out[i] = a;
     }
   }
   __syncthreads();
@@ -128,7 +153,8 @@ __global__ void __launch_bounds__(DT, 1) k_dots(VecList<T> V, const T *__restric
   constexpr int C = lane_of<T>::C, NC = VEC * C;
   constexpr int R = NV + (EXTRA & 1) + (EXTRA >> 1);
   constexpr int U = NV <= 1 ? 4 : NV <= 3 ? 2 : 1;
-  __shared__ __align__(16) S red[DT * NC];
+  constexpr int RB = R < 4 ? R : 4;                          // rows summed together
+  __shared__ __align__(16) S red[RB * DT * NC];
   __shared__ A red2[DT];
   const int kv = k / VEC, slots = DT / kv;
   const int cv = threadIdx.x % kv, slot = threadIdx.x / kv;
@@ -178,37 +204,42 @@ __global__ void __launch_bounds__(DT, 1) k_dots(VecList<T> V, const T *__restric
   }
   const int E = k * C;
 #pragma unroll
-  for (int r = 0; r < R; ++r)
-    block_sum<T, NC>(acc[r], red, red2, E, slots, live,
-                     partial + ((size_t)blockIdx.x * nrows + row0 + r) * E);
+  for (int r = 0; r < R; r += RB)
+    block_sums<T, NC, RB>(acc + r, R - r < RB ? R - r : RB, red, red2, E, slots, live,
+                          partial + ((size_t)blockIdx.x * nrows + row0 + r) * E);
 }
 
-// out[e] = sum over parts of partial[part][e], e < nrows * k scalars, in fixed order: one
-// block per 32 consecutive scalars (coalesced), 16 warps each taking every 16th part.
+// out[e] = sum over parts of partial[part][e], e < nrows * k scalars, in fixed order: a block per
+// eight consecutive scalars, 64 threads each taking every 64th part, met in steps of eight.
+constexpr int RE = 8, RS = RT / RE;
 template <class A>
 __global__ void __launch_bounds__(RT) k_dots_reduce(const A *__restrict__ partial, int nparts, int entries,
                                                     double *__restrict__ out) {
-  __shared__ A red[RT / 32][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int e = blockIdx.x * 32 + lane;
+  __shared__ A red[RS][RE];
+  const int lane = threadIdx.x % RE, sl = threadIdx.x / RE;
+  const int e = blockIdx.x * RE + lane;
   A a;
   acc_zero(a);
-  if (e < entries) {
-#pragma unroll 4
-    for (int p = warp; p < nparts; p += RT / 32) acc_add(a, partial[(size_t)p * entries + e]);
-  }
-  red[warp][lane] = a;
+  if (e < entries)
+    for (int p = sl; p < nparts; p += RS) acc_add(a, partial[(size_t)p * entries + e]);
+  red[sl][lane] = a;
   __syncthreads();
-  if (warp == 0 && e < entries) {
-    for (int q = 1; q < RT / 32; ++q) acc_add(a, red[q][lane]);
+  if (sl < 8) {
+    for (int q = sl + 8; q < min(nparts, RS); q += 8) acc_add(a, red[q][lane]);
+    red[sl][lane] = a;               // read by this thread alone in this step
+  }
+  __syncthreads();
+  if (sl == 0 && e < entries) {
+    for (int q = 1; q < min(nparts, 8); ++q) acc_add(a, red[q][lane]);
     out[e] = acc_value(a);
   }
 }
 
-// Columns of a 16-byte pack where every row allows it.
+// Columns per pack: 16 bytes, or 8 of an FP32 block (k = 2 mod 4; 4 vectors of 262144 x 62: 84 us,
+// 144 with single columns), where every row allows it.
 static int pack_of(DType t, int k) {
   const int vw = 16 / (int)dtype_size(t);
-  return k % vw ? 1 : vw;
+  return k % vw == 0 ? vw : vw == 4 && k % 2 == 0 ? 2 : 1;
 }
 
 template <class T> constexpr DType type_of() {
@@ -217,24 +248,35 @@ template <class T> constexpr DType type_of() {
 }
 
 int multidot_parts(DType t, size_t rows, int k) {
-  // enough row chunks to give every thread a few rows, at most one block per SM; FP64 data two,
-  // so that a lane adds up half as many products
-  const size_t per = std::max<size_t>(1, (size_t)DT * 8 / std::max(k, 1));
-  const size_t most = dtype_size(dtype_lower(t)) == dtype_size(t) ? DOT_PARTS : 2 * DOT_PARTS;
-  return (int)std::min<size_t>(most, std::max<size_t>(1, (rows + per - 1) / per));
+  // a row of packs per thread where the rows are few, at most one block per SM; FP64 data two, so
+  // that a lane adds up half as many, but whole waves only: a block of k_dots has an SM to itself
+  // (8 vectors of 4096 x 200: 205 blocks 39 us, 304 with block_sums 29)
+  const size_t slots = std::max(1, DT / std::max(k / pack_of(t, k), 1));
+  const size_t p = std::max<size_t>(1, (rows + slots - 1) / slots);
+  const bool fp64 = dtype_lower(t) != t;
+  return fp64 && p >= 2 * DOT_PARTS ? 2 * DOT_PARTS : (int)std::min<size_t>(DOT_PARTS, p);
 }
 
 namespace {
 
-// VEC columns per 16-byte pack where every row and every pointer allows it.
+// The widest pack, of the width pack_of gives or less, that every pointer allows.
 template <class T>
-bool packs_ok(int k, std::initializer_list<const void *> ptrs) {
-  constexpr int VW = 16 / (int)sizeof(T);
-  if (VW == 1) return true;
-  if (k % VW) return false;
+int pack_at(int k, size_t vstride, std::initializer_list<const void *> ptrs) {
+  int vec = pack_of(type_of<T>(), k);
   for (const void *p : ptrs)
-    if ((uintptr_t)p & 15) return false;
-  return true;
+    while (vec > 1 && ((uintptr_t)p % (vec * sizeof(T)) || vstride % vec)) vec /= 2;
+  return vec;
+}
+
+// f(VEC) with the pack as a compile-time width
+template <class T, class F>
+void with_pack(int vec, F &&f) {
+  constexpr int VW = 16 / (int)sizeof(T);
+  if constexpr (VW == 4)
+    if (vec == 4) return f(std::integral_constant<int, 4>());
+  if constexpr (VW >= 2)
+    if (vec == 2) return f(std::integral_constant<int, 2>());
+  f(std::integral_constant<int, 1>());
 }
 
 template <class T, int VEC, int EXTRA>
@@ -266,9 +308,8 @@ void dots_go(const VecList<T> &V, int nv, const T *w, size_t rows, int k, void *
 template <class T>
 int dots_partial(const void *v0, const void *V, size_t vstride, int nvec, const void *w, size_t rows, int k,
                  void *partial, int nparts, int extra, cudaStream_t s) {
-  constexpr int VW = 16 / (int)sizeof(T);
-  const bool packed = VW > 1 && packs_ok<T>(k, {v0, V, w}) && vstride % VW == 0;
-  if ((packed ? k / VW : k) > DT) throw cuda_error{cudaErrorInvalidValue, "multidot: more column groups than threads"};
+  const int pack = pack_at<T>(k, vstride, {v0, V, w});
+  if (k / pack > DT) throw cuda_error{cudaErrorInvalidValue, "multidot: more column groups than threads"};
   const int nrows = nvec + (extra & 1) + (extra >> 1);
   int passes = 0;
   for (int i0 = 0; i0 < nvec; i0 += DOT_MAXV) {
@@ -280,15 +321,13 @@ int dots_partial(const void *v0, const void *V, size_t vstride, int nvec, const 
     }
     // the extra rows ride on the last pass (w.w) or need v0 in it (v0.v0: nvec = 1)
     const int ex = i0 + nv < nvec ? 0 : extra;
-    auto go = [&](auto vec) {
+    with_pack<T>(pack, [&](auto vec) {
       constexpr int VEC = decltype(vec)::value;
       if (ex == 0) dots_go<T, VEC, 0>(L, nv, (const T *)w, rows, k, partial, nparts, i0, nrows, s);
       else if (ex == 1) dots_go<T, VEC, 1>(L, nv, (const T *)w, rows, k, partial, nparts, i0, nrows, s);
       else if (ex == 2) dots_go<T, VEC, 2>(L, nv, (const T *)w, rows, k, partial, nparts, i0, nrows, s);
       else dots_go<T, VEC, 3>(L, nv, (const T *)w, rows, k, partial, nparts, i0, nrows, s);
-    };
-    if (packed) go(std::integral_constant<int, VW>());
-    else go(std::integral_constant<int, 1>());
+    });
     ++passes;
   }
   return passes;
@@ -302,7 +341,7 @@ void launch_multidot(DType t, const void *V, size_t vstride, int nvec, const voi
     typedef typename lane_of<T>::A A;
     dots_partial<T>(V, V, vstride, nvec, w, rows, k, partials, nparts, 0, s);
     const int entries = nvec * k * lane_of<T>::C;
-    k_dots_reduce<A><<<(entries + 31) / 32, RT, 0, s>>>((const A *)partials, nparts, entries, (double *)out);
+    k_dots_reduce<A><<<(entries + RE - 1) / RE, RT, 0, s>>>((const A *)partials, nparts, entries, (double *)out);
     MLMC_LAUNCH_CHECK("k_dots_reduce");
   });
 }
@@ -400,15 +439,15 @@ __global__ void __launch_bounds__(DT, 2) k_axpy(T *__restrict__ w, const T *__re
     if (r < r1) step(r, std::integral_constant<int, 1>());
   }
   if (!INIT && norm) {
-    S v[VEC];
+    S v[1][VEC];
 #pragma unroll
     for (int u = 0; u < VEC; ++u) {
       acc_add(tot[u], sq[u]);
-      if constexpr (sizeof(S) == 4) v[u] = tot[u].h + tot[u].l;   // one rounding to the lane precision
-      else v[u] = tot[u];
+      if constexpr (sizeof(S) == 4) v[0][u] = tot[u].h + tot[u].l;   // one rounding to the lane precision
+      else v[0][u] = tot[u];
     }
     // |w|^2 is real for complex data too: one scalar per column
-    block_sum<typename real_of<T>::type, VEC>(v, red, red2, k, slots, live, norm + (size_t)blockIdx.x * k);
+    block_sums<typename real_of<T>::type, VEC, 1>(v, 1, red, red2, k, slots, live, norm + (size_t)blockIdx.x * k);
   }
 }
 
@@ -425,10 +464,9 @@ namespace {
 template <class T, class H>
 int axpy_all(void *w, const void *v0, const void *V, size_t vstride, int nvec, const void *h, double sign, size_t rows,
              int k, bool init, void *norm, cudaStream_t s) {
-  constexpr int VW = 16 / (int)sizeof(T);
   typedef typename lane_of<T>::A A;
-  const bool packed = VW > 1 && packs_ok<T>(k, {w, v0, V}) && vstride % VW == 0;
-  if ((packed ? k / VW : k) > DT) throw cuda_error{cudaErrorInvalidValue, "multiaxpy: more column groups than threads"};
+  const int pack = pack_at<T>(k, vstride, {w, v0, V});
+  if (k / pack > DT) throw cuda_error{cudaErrorInvalidValue, "multiaxpy: more column groups than threads"};
   const int group = std::max(1, AXPY_SMEM / (k * (int)sizeof(T)));
   const int parts = multiaxpy_norm_parts(type_of<T>(), rows, k);
   int passes = 0;
@@ -436,14 +474,14 @@ int axpy_all(void *w, const void *v0, const void *V, size_t vstride, int nvec, c
     const int nv = std::min(nvec - i0, group);
     const bool first = init && i0 == 0, last = i0 + nv >= nvec;
     const size_t smem = (size_t)nv * k * sizeof(T);
-    auto go = [&](auto vec, auto ini) {
-      k_axpy<T, H, decltype(vec)::value, decltype(ini)::value><<<parts, DT, smem, s>>>(
-          (T *)w, (const T *)v0, (const T *)V, vstride, i0, nv, (const H *)h, sign, rows, k, last ? (A *)norm : nullptr);
-    };
-    if (packed && first) go(std::integral_constant<int, VW>(), std::true_type());
-    else if (packed) go(std::integral_constant<int, VW>(), std::false_type());
-    else if (first) go(std::integral_constant<int, 1>(), std::true_type());
-    else go(std::integral_constant<int, 1>(), std::false_type());
+    with_pack<T>(pack, [&](auto vec) {
+      auto go = [&](auto ini) {
+        k_axpy<T, H, decltype(vec)::value, decltype(ini)::value><<<parts, DT, smem, s>>>(
+            (T *)w, (const T *)v0, (const T *)V, vstride, i0, nv, (const H *)h, sign, rows, k, last ? (A *)norm : nullptr);
+      };
+      if (first) go(std::true_type());
+      else go(std::false_type());
+    });
     MLMC_LAUNCH_CHECK("k_axpy");
     ++passes;
   }

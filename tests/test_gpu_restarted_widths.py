@@ -48,3 +48,21 @@ def test_equal_columns_take_the_same_steps(mlmc, op, reorth):
         r = np.linalg.norm(bn - A @ x.cpu().numpy(), axis=0) / np.linalg.norm(bn, axis=0)
         assert (r <= 1.01 * tol).all(), (k, r.max())
     assert max(its.values()) - min(its.values()) <= 1 and min(its.values()) > 8, its
+
+
+def test_one_column_takes_no_longer_than_a_wide_block(mlmc):
+    """The same 64^2 solve (23 steps or more, so up to 23 basis vectors per reduction) with 1 / 200 of the
+    data: its reductions are shorter chains, not longer ones."""
+    import time
+    best = {}
+    for k in (1, 200):
+        h, A, dt = make(mlmc, "laplace", 64, k)
+        b = torch.randn(A.shape[0], k, dtype=dt, device="cuda", generator=torch.Generator(device="cuda").manual_seed(3))
+        x = torch.empty_like(b)
+        for _ in range(6):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            h.solve(1, b.data_ptr(), x.data_ptr(), k, 1e-10)
+            best[k] = min(best.get(k, 1e9), time.perf_counter() - t)
+        h.close()
+    assert best[1] <= best[200], best
