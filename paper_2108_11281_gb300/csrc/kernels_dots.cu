@@ -6,10 +6,11 @@
 // not allow it) and walks the rows of its block's contiguous chunk, so every load is
 // coalesced and a column's sum stays in one lane until the end of the chunk.
 //
-// FP64 additions run at 1.7 per clock and SM on this GPU (0.53 T/s), FP32 ones at 128: the
-// sums over lanes and blocks of FP32 data are kept as float pairs (a hi + lo sum by the
-// two-sum of Knuth, TAOCP 4.2.2; 48 significant bits, far below the rounding of the FP32
-// lane sums they add up) and become FP64 once per column.  Sums of FP64 data stay FP64.
+// FP64 additions run at 1.7 per clock and SM on this GPU (0.53 T/s), FP32 ones at 128.  A thread
+// adds up its own FP32 products in FP32; a block's lane sums meet as float pairs (a hi + lo sum by
+// the two-sum of Knuth, TAOCP 4.2.2; 48 significant bits, far below the rounding of the FP32 lane
+// sums), or in FP64 where a pair leaves FP32's range, and everything beyond a block is FP64.
+// Sums of FP64 data are FP64 throughout.
 #include <algorithm>
 #include <initializer_list>
 #include <mutex>
@@ -59,9 +60,11 @@ __device__ __forceinline__ double acc_value(double a) { return a; }
 // a += conj(x) * y on scalars
 __device__ __forceinline__ void dot_fma(float a[1], float x, float y) { a[0] += x * y; }
 __device__ __forceinline__ void dot_fma(double a[1], double x, double y) { a[0] += x * y; }
+// complex FP32: the product is formed first, so that the running sum is rounded once per term
+// (262144 x 64: rms error 1.5e-9 of the terms' size, 2.2e-9 with two multiply-adds on the sum)
 __device__ __forceinline__ void dot_fma(float a[2], cfloat x, cfloat y) {
-  a[0] = fma(x.im, y.im, fma(x.re, y.re, a[0]));
-  a[1] = fma(-x.im, y.re, fma(x.re, y.im, a[1]));
+  a[0] += fmaf(x.im, y.im, x.re * y.re);
+  a[1] += fmaf(-x.im, y.re, x.re * y.im);
 }
 __device__ __forceinline__ void dot_fma(double a[2], cdouble x, cdouble y) {
   a[0] = fma(x.im, y.im, fma(x.re, y.re, a[0]));
@@ -84,10 +87,18 @@ __device__ __forceinline__ void chunk_of(size_t rows, size_t &r0, size_t &r1) {
 // Ends with the block synchronised.
 template <class T, int NC, int RB>
 __device__ __forceinline__ void block_sums(const typename lane_of<T>::S (*val)[NC], int nr, typename lane_of<T>::S *red,
-                                           typename lane_of<T>::A *red2, int E, int slots, bool live,
-                                           typename lane_of<T>::A *out) {
+                                           typename lane_of<T>::A *red2, int E, int slots, bool live, double *out) {
   typedef typename lane_of<T>::A A;
   const int tid = threadIdx.x;
+  // the sum as FP64; lane values whose float pair left FP32's range (or are not finite) are added again
+  auto finish = [&](const A &a, const typename lane_of<T>::S *src) {
+    double v = acc_value(a);
+    if (sizeof(typename lane_of<T>::S) == 4 && !isfinite(v)) {
+      v = 0.0;
+      for (int s = 0; s < slots; ++s) v += (double)src[s * E];
+    }
+    return v;
+  };
 #pragma unroll
   for (int r = 0; r < RB; ++r)
     if (r < nr) {
@@ -105,7 +116,7 @@ __device__ __forceinline__ void block_sums(const typename lane_of<T>::S (*val)[N
       A a;
       acc_zero(a);
       for (int s = 0; s < slots; ++s) acc_add(a, src[s * E]);
-      out[i] = a;
+      out[i] = finish(a, src);
     }
   } else {
     const int g = tid / items, i = tid - g * items, r = i / E;
@@ -128,7 +139,7 @@ __device__ __forceinline__ void block_sums(const typename lane_of<T>::S (*val)[N
     __syncthreads();
     if (g == 0) {
       for (int q = 1; q < G; ++q) acc_add(a, red2[q * items + i]);
-      out[i] = a;
+      out[i] = finish(a, src);
     }
   }
   __syncthreads();
@@ -146,7 +157,7 @@ __device__ __forceinline__ void block_sums(const typename lane_of<T>::S (*val)[N
 // threads, 8-byte loads and FP64 block sums); 16384 x 128, L2-resident: 12.4 us (22.6).
 template <class T, int VEC, int NV, int EXTRA>
 __global__ void __launch_bounds__(DT, 1) k_dots(VecList<T> V, const T *__restrict__ w, size_t rows, int k,
-                                                typename lane_of<T>::A *__restrict__ partial, int row0, int nrows) {
+                                                double *__restrict__ partial, int row0, int nrows) {
   typedef typename lane_of<T>::S S;
   typedef typename lane_of<T>::A A;
   typedef DPack<T, VEC> P;
@@ -212,26 +223,24 @@ __global__ void __launch_bounds__(DT, 1) k_dots(VecList<T> V, const T *__restric
 // out[e] = sum over parts of partial[part][e], e < nrows * k scalars, in fixed order: a block per
 // eight consecutive scalars, 64 threads each taking every 64th part, met in steps of eight.
 constexpr int RE = 8, RS = RT / RE;
-template <class A>
-__global__ void __launch_bounds__(RT) k_dots_reduce(const A *__restrict__ partial, int nparts, int entries,
-                                                    double *__restrict__ out) {
-  __shared__ A red[RS][RE];
+static __global__ void __launch_bounds__(RT) k_dots_reduce(const double *__restrict__ partial, int nparts, int entries,
+                                                           double *__restrict__ out) {
+  __shared__ double red[RS][RE];
   const int lane = threadIdx.x % RE, sl = threadIdx.x / RE;
   const int e = blockIdx.x * RE + lane;
-  A a;
-  acc_zero(a);
+  double a = 0.0;
   if (e < entries)
-    for (int p = sl; p < nparts; p += RS) acc_add(a, partial[(size_t)p * entries + e]);
+    for (int p = sl; p < nparts; p += RS) a += partial[(size_t)p * entries + e];
   red[sl][lane] = a;
   __syncthreads();
   if (sl < 8) {
-    for (int q = sl + 8; q < min(nparts, RS); q += 8) acc_add(a, red[q][lane]);
+    for (int q = sl + 8; q < min(nparts, RS); q += 8) a += red[q][lane];
     red[sl][lane] = a;               // read by this thread alone in this step
   }
   __syncthreads();
   if (sl == 0 && e < entries) {
-    for (int q = 1; q < min(nparts, 8); ++q) acc_add(a, red[q][lane]);
-    out[e] = acc_value(a);
+    for (int q = 1; q < min(nparts, 8); ++q) a += red[q][lane];
+    out[e] = a;
   }
 }
 
@@ -248,13 +257,16 @@ template <class T> constexpr DType type_of() {
 }
 
 int multidot_parts(DType t, size_t rows, int k) {
-  // a row of packs per thread where the rows are few, at most one block per SM; FP64 data two, so
-  // that a lane adds up half as many, but whole waves only: a block of k_dots has an SM to itself
-  // (8 vectors of 4096 x 200: 205 blocks 39 us, 304 with block_sums 29)
-  const size_t slots = std::max(1, DT / std::max(k / pack_of(t, k), 1));
+  // a row of packs per thread where the rows are few; FP32 packs of four columns at most one block
+  // per SM, narrower ones and FP64 two, so that a lane adds up half as many, but whole waves only:
+  // a block of k_dots has an SM to itself (8 FP64 vectors of 4096 x 200: 205 blocks 39 us, 304 with
+  // block_sums 29)
+  const int pack = pack_of(t, k);
+  const size_t slots = std::max(1, DT / std::max(k / pack, 1));
   const size_t p = std::max<size_t>(1, (rows + slots - 1) / slots);
-  const bool fp64 = dtype_lower(t) != t;
-  return fp64 && p >= 2 * DOT_PARTS ? 2 * DOT_PARTS : (int)std::min<size_t>(DOT_PARTS, p);
+  if (p <= DOT_PARTS || pack == 4) return (int)std::min<size_t>(DOT_PARTS, p);
+  const bool fp64 = dtype_lower(t) != t;       // no lane sums in FP32 to keep short
+  return fp64 && p < 2 * DOT_PARTS ? DOT_PARTS : 2 * DOT_PARTS;
 }
 
 namespace {
@@ -282,11 +294,10 @@ void with_pack(int vec, F &&f) {
 template <class T, int VEC, int EXTRA>
 void dots_go(const VecList<T> &V, int nv, const T *w, size_t rows, int k, void *partial, int nparts, int row0,
              int nrows, cudaStream_t s) {
-  typedef typename lane_of<T>::A A;
   auto go = [&](auto n) {
     constexpr int NV = decltype(n)::value;
     if constexpr (NV == 1 || EXTRA < 2)           // v0.v0 is asked for with the first vector alone
-      k_dots<T, VEC, NV, EXTRA><<<nparts, DT, 0, s>>>(V, w, rows, k, (A *)partial, row0, nrows);
+      k_dots<T, VEC, NV, EXTRA><<<nparts, DT, 0, s>>>(V, w, rows, k, (double *)partial, row0, nrows);
     else
       throw cuda_error{cudaErrorInvalidValue, "multidot: v0.v0 needs a single vector"};
   };
@@ -338,10 +349,9 @@ int dots_partial(const void *v0, const void *V, size_t vstride, int nvec, const 
 void launch_multidot(DType t, const void *V, size_t vstride, int nvec, const void *w, size_t rows, int k,
                      void *partials, int nparts, void *out, cudaStream_t s) {
   MLMC_DISPATCH(t, T, {
-    typedef typename lane_of<T>::A A;
     dots_partial<T>(V, V, vstride, nvec, w, rows, k, partials, nparts, 0, s);
     const int entries = nvec * k * lane_of<T>::C;
-    k_dots_reduce<A><<<(entries + RE - 1) / RE, RT, 0, s>>>((const A *)partials, nparts, entries, (double *)out);
+    k_dots_reduce<<<(entries + RE - 1) / RE, RT, 0, s>>>((const double *)partials, nparts, entries, (double *)out);
     MLMC_LAUNCH_CHECK("k_dots_reduce");
   });
 }
@@ -361,7 +371,7 @@ void launch_multidot(DType t, const void *V, size_t vstride, int nvec, const voi
 template <class T, class H, int VEC, bool INIT>
 __global__ void __launch_bounds__(DT, 2) k_axpy(T *__restrict__ w, const T *__restrict__ first, const T *__restrict__ V,
                                                 size_t vstride, int v0, int nv, const H *__restrict__ h, double sign,
-                                                size_t rows, int k, typename lane_of<T>::A *__restrict__ norm) {
+                                                size_t rows, int k, double *__restrict__ norm) {
   typedef typename lane_of<T>::S S;
   typedef typename lane_of<T>::A A;
   typedef DPack<T, VEC> P;
@@ -464,7 +474,6 @@ namespace {
 template <class T, class H>
 int axpy_all(void *w, const void *v0, const void *V, size_t vstride, int nvec, const void *h, double sign, size_t rows,
              int k, bool init, void *norm, cudaStream_t s) {
-  typedef typename lane_of<T>::A A;
   const int pack = pack_at<T>(k, vstride, {w, v0, V});
   if (k / pack > DT) throw cuda_error{cudaErrorInvalidValue, "multiaxpy: more column groups than threads"};
   const int group = std::max(1, AXPY_SMEM / (k * (int)sizeof(T)));
@@ -477,7 +486,7 @@ int axpy_all(void *w, const void *v0, const void *V, size_t vstride, int nvec, c
     with_pack<T>(pack, [&](auto vec) {
       auto go = [&](auto ini) {
         k_axpy<T, H, decltype(vec)::value, decltype(ini)::value><<<parts, DT, smem, s>>>(
-            (T *)w, (const T *)v0, (const T *)V, vstride, i0, nv, (const H *)h, sign, rows, k, last ? (A *)norm : nullptr);
+            (T *)w, (const T *)v0, (const T *)V, vstride, i0, nv, (const H *)h, sign, rows, k, last ? (double *)norm : nullptr);
       };
       if (first) go(std::true_type());
       else go(std::false_type());
@@ -511,8 +520,8 @@ int launch_multiaxpy(DType t, void *w, const void *V, size_t vstride, int nvec, 
 // Columns whose right-hand side is zero or not finite, and columns that break down (a zero
 // new vector or a zero pivot), stop there: their later y are zero.
 // Both kernels give a block a few columns and let all its threads add the parts (latency-
-// bound); a tile is 8 (FP32 data) or 4 scalars wide, since the FP64 additions of one block's
-// share would otherwise take longer than its loads.  Per step they stand in place of two
+// bound); a tile is two scalars wide, since the FP64 additions of one block's share would
+// otherwise take longer than its loads.  Per step they stand in place of two
 // reductions of one warp per output (4.7 us each, strided loads), a cleared counter and a
 // per-column Givens kernel (4.7 us, 9 us complex; a 4-byte memset node costs 4 us and the
 // kernel after it 5 us of gap in a replayed graph): k_fgmres_mid takes 3.3 us, k_fgmres_tail 8.3
@@ -521,13 +530,12 @@ int launch_multiaxpy(DType t, void *w, const void *V, size_t vstride, int nvec, 
 namespace {
 
 template <class T> struct fg {
-  typedef typename lane_of<T>::A A;
   typedef typename acc_of<T>::type H;
   static constexpr int C = lane_of<T>::C;
-  static constexpr int ET = sizeof(A) == 8 && sizeof(typename lane_of<T>::S) == 4 ? 8 : 4;   // scalars per tile
-  static constexpr int CB = ET / C;                                                          // columns per tile
-  static constexpr int SL = RT / ET;                                                         // part slices
-  static constexpr int MAXROWS = 34;                                                         // 32 steps, v0.v0, w.w
+  static constexpr int ET = 2;                   // scalars per tile
+  static constexpr int CB = ET / C;              // columns per tile
+  static constexpr int SL = RT / ET;             // part slices
+  static constexpr int MAXROWS = 34;             // 32 steps, v0.v0, w.w
 };
 
 // sums[r * ET + e] (r < nrows, e < ET) = scalar e0 + e of output row r summed over the parts in
@@ -535,35 +543,36 @@ template <class T> struct fg {
 // apart) also nsum[c] = column c0 + c of it, c < CB, in the same pass.  red: (TR + 1) * RT sums.
 constexpr int TR = 8;              // rows whose loads are in flight together
 template <class T>
-__device__ void tile_sum(const typename lane_of<T>::A *__restrict__ partial, int nparts, int nrows, int E, int e0,
-                         const typename lane_of<T>::A *__restrict__ norm, int norm_parts, int k, int c0,
-                         typename lane_of<T>::A *red, double *sums, double *nsum) {
-  typedef typename lane_of<T>::A A;
+__device__ void tile_sum(const double *__restrict__ partial, int nparts, int nrows, int E, int e0,
+                         const double *__restrict__ norm, int norm_parts, int k, int c0, double *red, double *sums,
+                         double *nsum) {
   constexpr int ET = fg<T>::ET, SL = fg<T>::SL, CB = fg<T>::CB;
   const int e = threadIdx.x % ET, sl = threadIdx.x / ET;
   const size_t stride = (size_t)nrows * E;
   for (int r0 = 0; r0 < nrows; r0 += TR) {
     const int nr = min(nrows - r0, TR);
     const bool with_norm = r0 == 0 && norm;
-    A a[TR], an;
-    acc_zero(an);
+    const int used = min(SL, with_norm ? max(nparts, norm_parts) : nparts);   // slices that hold anything
+    double a[TR], an = 0.0;
 #pragma unroll
-    for (int r = 0; r < TR; ++r) acc_zero(a[r]);
-    if (with_norm && e < CB && c0 + e < k) {
-#pragma unroll 4
-      for (int p = sl; p < norm_parts; p += SL) acc_add(an, norm[(size_t)p * k + c0 + e]);
+    for (int r = 0; r < TR; ++r) a[r] = 0.0;
+    if (with_norm && e < CB && c0 + e < k && sl < norm_parts) {
+      an = norm[(size_t)sl * k + c0 + e];
+      for (int p = sl + SL; p < norm_parts; p += SL) an += norm[(size_t)p * k + c0 + e];
     }
-    if (e0 + e < E) {
-      const A *src = partial + (size_t)r0 * E + e0 + e;
-#pragma unroll 2
-      for (int p = sl; p < nparts; p += SL) {
-        A v[TR];
+    if (e0 + e < E && sl < nparts) {
+      const double *src = partial + (size_t)r0 * E + e0 + e;
+#pragma unroll
+      for (int r = 0; r < TR; ++r)
+        if (r < nr) a[r] = src[sl * stride + (size_t)r * E];
+      for (int p = sl + SL; p < nparts; p += SL) {
+        double v[TR];
 #pragma unroll
         for (int r = 0; r < TR; ++r)
           if (r < nr) v[r] = src[p * stride + (size_t)r * E];
 #pragma unroll
         for (int r = 0; r < TR; ++r)
-          if (r < nr) acc_add(a[r], v[r]);
+          if (r < nr) a[r] += v[r];
       }
     }
 #pragma unroll
@@ -572,20 +581,22 @@ __device__ void tile_sum(const typename lane_of<T>::A *__restrict__ partial, int
     if (with_norm) red[(nr * SL + sl) * ET + e] = an;
     const int rows = nr + with_norm;
     __syncthreads();
-    // eight threads per sum take the slices q, q + 8, ...; then one adds the eight
-    for (int t = threadIdx.x; t < rows * ET * 8; t += RT) {
-      const int q = t & 7, re = t >> 3, r = re / ET, ee = re % ET;
-      A v = red[(r * SL + q) * ET + ee];
-      for (int s2 = q + 8; s2 < SL; s2 += 8) acc_add(v, red[(r * SL + s2) * ET + ee]);
+    // 16 threads per sum take the slices q, q + 16, ...; then one adds the 16
+    for (int t = threadIdx.x; t < rows * ET * 16; t += RT) {
+      const int ee = t % ET, q = t / ET % 16, r = t / (ET * 16);
+      double v = red[(r * SL + q) * ET + ee];
+#pragma unroll 4
+      for (int s2 = q + 16; s2 < used; s2 += 16) v += red[(r * SL + s2) * ET + ee];
       red[(r * SL + q) * ET + ee] = v;
     }
     __syncthreads();
     for (int re = threadIdx.x; re < rows * ET; re += RT) {
       const int r = re / ET, ee = re % ET;
-      A v = red[(r * SL) * ET + ee];
-      for (int q = 1; q < 8; ++q) acc_add(v, red[(r * SL + q) * ET + ee]);
-      if (r < nr) sums[(r0 + r) * ET + ee] = acc_value(v);
-      else if (ee < CB) nsum[ee] = acc_value(v);
+      double v = red[(r * SL) * ET + ee];
+#pragma unroll
+      for (int q = 1; q < 16; ++q) v += red[(r * SL + q) * ET + ee];
+      if (r < nr) sums[(r0 + r) * ET + ee] = v;
+      else if (ee < CB) nsum[ee] = v;
     }
     __syncthreads();
   }
@@ -603,9 +614,9 @@ __device__ __forceinline__ cdouble shfl(cdouble v, int l) { return {shfl(v.re, l
 // The tile's sums for step j: dots (rows d_0 .. d_j, then v0.v0 when j = 0, then extra rows)
 // into sums, and n_j into nj[c] (shared) and n2[j] (global).
 template <class T>
-__device__ void fgmres_sums(const typename lane_of<T>::A *partial, int nparts, int nrows,
-                            const typename lane_of<T>::A *norm, int norm_parts, int j, int k, int c0, double *n2,
-                            typename lane_of<T>::A *red, double *sums, double *nj) {
+__device__ void fgmres_sums(const double *partial, int nparts, int nrows,
+                            const double *norm, int norm_parts, int j, int k, int c0, double *n2,
+                            double *red, double *sums, double *nj) {
   constexpr int C = fg<T>::C, ET = fg<T>::ET, CB = fg<T>::CB;
   tile_sum<T>(partial, nparts, nrows, k * C, c0 * C, j > 0 ? norm : nullptr, norm_parts, k, c0, red, sums, nj);
   if (threadIdx.x < CB) {
@@ -618,13 +629,13 @@ __device__ void fgmres_sums(const typename lane_of<T>::A *partial, int nparts, i
 
 // D[(j * (m + 1) + i) * k + c] = d_ij, coef[i * k + c] = -d_ij / n_i for the multi-AXPY of step j.
 template <class T>
-__global__ void __launch_bounds__(RT) k_fgmres_mid(const typename lane_of<T>::A *__restrict__ partial, int nparts,
-                                                   int nrows, const typename lane_of<T>::A *__restrict__ norm,
+__global__ void __launch_bounds__(RT) k_fgmres_mid(const double *__restrict__ partial, int nparts,
+                                                   int nrows, const double *__restrict__ norm,
                                                    int norm_parts, int j, int m, int k, double *n2,
                                                    typename acc_of<T>::type *__restrict__ D, T *__restrict__ coef) {
   typedef typename acc_of<T>::type H;
   constexpr int ET = fg<T>::ET, CB = fg<T>::CB;
-  __shared__ typename lane_of<T>::A red[(TR + 1) * RT];
+  __shared__ double red[(TR + 1) * RT];
   __shared__ double sums[fg<T>::MAXROWS * ET], nj[8];
   const int c0 = blockIdx.x * CB;
   // thread (i, c): the norm of u_i is loaded before the sums (at most 32 vectors x 8 columns)
@@ -642,14 +653,14 @@ __global__ void __launch_bounds__(RT) k_fgmres_mid(const typename lane_of<T>::A 
 // The last step, j = its - 1, and the least-squares problem: y[i * k + c], i < its.
 // One warp per column; lane q keeps column q of G, and the norm of u_q.
 template <class T>
-__global__ void __launch_bounds__(RT) k_fgmres_tail(const typename lane_of<T>::A *__restrict__ partial, int nparts,
-                                                    int nrows, const typename lane_of<T>::A *__restrict__ norm,
+__global__ void __launch_bounds__(RT) k_fgmres_tail(const double *__restrict__ partial, int nparts,
+                                                    int nrows, const double *__restrict__ norm,
                                                     int norm_parts, int its, int m, int k, double *n2,
                                                     const typename acc_of<T>::type *__restrict__ D,
                                                     T *__restrict__ y) {
   typedef typename acc_of<T>::type H;
   constexpr int ET = fg<T>::ET, CB = fg<T>::CB, C = fg<T>::C;
-  __shared__ typename lane_of<T>::A red[(TR + 1) * RT];
+  __shared__ double red[(TR + 1) * RT];
   __shared__ double sums[fg<T>::MAXROWS * ET], nj[8];
   extern __shared__ __align__(16) unsigned char tail_smem[];
   const int c0 = blockIdx.x * CB, j = its - 1;
@@ -733,10 +744,9 @@ void launch_fgmres_mid(DType t, const void *partials, const void *norm, int j, i
                        void *D, void *coef, cudaStream_t s) {
   const int nparts = multidot_parts(t, rows, k), nnorm = multiaxpy_norm_parts(t, rows, k);
   MLMC_DISPATCH(t, T, {
-    typedef typename lane_of<T>::A A;
     typedef typename acc_of<T>::type H;
-    k_fgmres_mid<T><<<(k + fg<T>::CB - 1) / fg<T>::CB, RT, 0, s>>>((const A *)partials, nparts, j + 1 + (j == 0),
-                                                                  (const A *)norm, nnorm, j, m, k, n2, (H *)D,
+    k_fgmres_mid<T><<<(k + fg<T>::CB - 1) / fg<T>::CB, RT, 0, s>>>((const double *)partials, nparts, j + 1 + (j == 0),
+                                                                  (const double *)norm, nnorm, j, m, k, n2, (H *)D,
                                                                   (T *)coef);
   });
   MLMC_LAUNCH_CHECK("k_fgmres_mid");
@@ -746,7 +756,6 @@ void launch_fgmres_tail(DType t, const void *partials, const void *norm, int its
                         double *n2, const void *D, void *y, cudaStream_t s) {
   const int nparts = multidot_parts(t, rows, k), nnorm = multiaxpy_norm_parts(t, rows, k);
   MLMC_DISPATCH(t, T, {
-    typedef typename lane_of<T>::A A;
     typedef typename acc_of<T>::type H;
     auto bytes = [](int n) { return (size_t)fg<T>::CB * (n + 1) * n * sizeof(H); };
     int dev = 0;
@@ -758,7 +767,7 @@ void launch_fgmres_tail(DType t, const void *partials, const void *norm, int its
                  "cudaFuncSetAttribute(k_fgmres_tail)");
     });
     k_fgmres_tail<T><<<(k + fg<T>::CB - 1) / fg<T>::CB, RT, bytes(its), s>>>(
-        (const A *)partials, nparts, its + 1 + (its == 1), (const A *)norm, nnorm, its, m, k, n2, (const H *)D, (T *)y);
+        (const double *)partials, nparts, its + 1 + (its == 1), (const double *)norm, nnorm, its, m, k, n2, (const H *)D, (T *)y);
   });
   MLMC_LAUNCH_CHECK("k_fgmres_tail");
 }

@@ -231,7 +231,7 @@ void alloc_krylov(H_t &h, Krylov &K, DType t, size_t n, int k, int m, bool fixed
   // a solve may be narrower than k; the part counts fall with the width, their products with it grow
   size_t dots = 0, norms = 0;
   for (int kk = 1; kk <= k; ++kk) {
-    dots = std::max(dots, (size_t)multidot_parts(t, n, kk) * kk);
+    dots = std::max(dots, (size_t)std::max(multidot_parts(t, n, kk), multidot_parts(dtype_lower(t), n, kk)) * kk);
     norms = std::max(norms, (size_t)multiaxpy_norm_parts(t, n, kk) * kk);
   }
   K.partials.alloc(dots * (m + 2) * as);
