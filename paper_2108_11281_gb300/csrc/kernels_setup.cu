@@ -660,7 +660,9 @@ void launch_trace(DType t, const void *A, int n, void *out, cudaStream_t s) {
 // share: 256 x 256 x 64 columns, 4.2 M FMA = 6.7 us at the measured rate, took 45 us on the 32
 // blocks of the tiled kernel below and takes 10.9 us (576 x 576 x 21: 61.5 -> 15.5 us).  With FP32
 // and n < 512 the chain of dependent loads counts, an eighth as long or less (128 complex x 32:
-// 14 -> 4 us).
+// 14 -> 4 us).  The slices meet in four chains, and FP32 products of up to eight columns are
+// cut into 32 slices: their rounding is that of a warp per row (256 x 4: 0.8e-7 rms, 1.2e-7 with
+// eight slices in one chain).
 template <class T, int R, int IT>
 __global__ void __launch_bounds__(256) k_dense_spread(const T *__restrict__ A, const T *__restrict__ B,
                                                       T *__restrict__ Y, int n, int k, int chunk, int vec) {
@@ -708,9 +710,12 @@ __global__ void __launch_bounds__(256) k_dense_spread(const T *__restrict__ A, c
   __syncthreads();
   for (int e = threadIdx.x; e < R * IT; e += 256) {
     const int r = e / IT, l = e % IT;
-    T s = red[0][r][l];
-#pragma unroll 8
-    for (int w = 1; w < SL; ++w) s = s + red[w][r][l];
+    T q[4];                          // four short chains: the slices' sum rounds less and waits less
+#pragma unroll
+    for (int u = 0; u < 4; ++u) q[u] = red[u][r][l];
+#pragma unroll
+    for (int w = 4; w < SL; ++w) q[w & 3] = q[w & 3] + red[w][r][l];
+    const T s = (q[0] + q[1]) + (q[2] + q[3]);
     const unsigned tt = blockIdx.x * (unsigned)IT + l;
     const int i = (int)(tt / (unsigned)k) * R + r;
     if (i < n) Y[(size_t)i * k + tt % (unsigned)k] = s;
@@ -772,7 +777,8 @@ __global__ void __launch_bounds__(128) k_dense_apply(const T *__restrict__ A, co
     }
 }
 
-// Up to three columns: one warp
+// Up to three columns, and FP32 with n >= 512 up to eight (1024 x 4: 6.3 us, 20.5 with the tiles
+// above, whose other columns are padding; 2048 x 8 37 and 55 us; complex 512 x 8 12.4 and 16.5): one warp
 // per row of Ainv, the lanes take j = lane, lane + 32, ... for all k columns, then a
 // fixed shuffle tree per column (deterministic).  Reads Ainv once; no padded columns.
 template <class T>
@@ -838,21 +844,29 @@ int dense_apply_splits(int n, int k) {
 
 void launch_dense_apply(DType t, const void *Ainv, const void *B, void *Y, int n, int k, void *part, cudaStream_t s) {
   // one warp per row on up to three columns: with fewer columns than that the rows of the
-  // matrix, not the columns, have to be read by consecutive lanes
-  if (k < 4) {
+  // matrix, not the columns, have to be read by consecutive lanes.  FP32 with n >= 512 on up to
+  // eight: the tiles below pad them to 32
+  const bool fp64 = t == F64 || t == C64, spread = fp64 || n * (t == C32 ? 2 : 1) < 512;
+  if (k < 4 || (k <= 8 && !spread)) {
     const unsigned g = resident_grid(((size_t)n * 32 + 255) / 256, 8);
-    MLMC_DISPATCH(t, T, k_dense_apply_narrow<T, 4><<<g, 256, 0, s>>>((const T *)Ainv, (const T *)B, (T *)Y, n, k));
+    if (k <= 4) {
+      MLMC_DISPATCH(t, T, k_dense_apply_narrow<T, 4><<<g, 256, 0, s>>>((const T *)Ainv, (const T *)B, (T *)Y, n, k));
+    } else if (t == F32) {
+      k_dense_apply_narrow<float, 8><<<g, 256, 0, s>>>((const float *)Ainv, (const float *)B, (float *)Y, n, k);
+    } else {
+      k_dense_apply_narrow<cfloat, 8><<<g, 256, 0, s>>>((const cfloat *)Ainv, (const cfloat *)B, (cfloat *)Y, n, k);
+    }
     MLMC_LAUNCH_CHECK("k_dense_apply_narrow");
     return;
   }
-  const bool fp64 = t == F64 || t == C64;
-  if (fp64 || n * (t == C32 ? 2 : 1) < 512) {
+  if (spread) {
     // rows per thread and items per warp: the smallest share of the busiest SM, blocks x R x IT;
     // the larger tile where that is equal (B is read once per row group, and fewer sums meet)
     int R = 4, IT = 32;
     size_t best = ~(size_t)0;
     for (int it : {32, 16, 8})
       for (int r : {4, 2, 1}) {
+        if (!fp64 && k <= 8 && it > 8) continue;   // FP32: 32 short slices round as little as a warp per row
         const size_t blocks = ((size_t)((n + r - 1) / r) * k + it - 1) / it, cost = (blocks + 151) / 152 * r * it;
         if (cost < best) {
           best = cost;
