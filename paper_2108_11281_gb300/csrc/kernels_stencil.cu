@@ -172,7 +172,7 @@ __device__ __forceinline__ void block_copy_async(void *dst, const void *src, int
 
 // acc[r] +- sum over NDIR neighbour blocks of rows r0 + r (blk: [NDIR][D][D] in shared memory)
 // times their x, XB neighbours' entries in flight at a time.  ready(): called after the first
-// loads are issued and before the coefficients are read.
+// loads are issued and before the coefficients are read.  SUB is the smoother's form (msub4).
 template <class T, int D, int CV, int RPT, int NDIR, bool SUB, class F>
 __device__ __forceinline__ void rows_accumulate(const T *blk, const T *x, const int nb[NDIR], int r0, int k, int c,
                                                 bool live, Pack<T, CV> acc[RPT], F ready) {
@@ -203,7 +203,7 @@ __device__ __forceinline__ void rows_accumulate(const T *blk, const T *x, const 
           for (int q = 0; q < D; ++q)
 #pragma unroll
             for (int u = 0; u < CV; ++u)
-              acc[r].v[u] = SUB ? msub(acc[r].v[u], row[q], xv[e][q].v[u]) : madd(acc[r].v[u], row[q], xv[e][q].v[u]);
+              acc[r].v[u] = SUB ? msub4(acc[r].v[u], row[q], xv[e][q].v[u]) : madd(acc[r].v[u], row[q], xv[e][q].v[u]);
         }
       }
   }
@@ -697,7 +697,7 @@ __device__ __forceinline__ void rbgs_half_body(const T *__restrict__ coef, const
 #pragma unroll
           for (int q = 0; q < D; ++q)
 #pragma unroll
-            for (int u = 0; u < VEC; ++u) res[r][u] = msub(res[r][u], row[q], xq[q].v[u]);
+            for (int u = 0; u < VEC; ++u) res[r][u] = msub4(res[r][u], row[q], xq[q].v[u]);
         }
       }
     }
@@ -713,7 +713,7 @@ __device__ __forceinline__ void rbgs_half_body(const T *__restrict__ coef, const
 #pragma unroll
       for (int q = 0; q < D; ++q)
 #pragma unroll
-        for (int u = 0; u < VEC; ++u) out.v[u] = madd(out.v[u], row[q], res[q][u]);
+        for (int u = 0; u < VEC; ++u) out.v[u] = madd4(out.v[u], row[q], res[q][u]);
       X[o + (size_t)r * kv] = out;
     }
   }
@@ -806,7 +806,7 @@ __global__ void __launch_bounds__(32 * D / RPT) k_rbgs_half_rows(const T *__rest
     for (int q = 0; q < D; ++q) {
       const V rv = res[q][cl];
 #pragma unroll
-      for (int u = 0; u < CV; ++u) out[r].v[u] = madd(out[r].v[u], row[q], rv.v[u]);
+      for (int u = 0; u < CV; ++u) out[r].v[u] = madd4(out[r].v[u], row[q], rv.v[u]);
     }
     *reinterpret_cast<V *>(x + ((size_t)s * D + r0 + r) * k + c) = out[r];
   }

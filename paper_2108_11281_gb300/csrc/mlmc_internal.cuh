@@ -70,10 +70,14 @@ __host__ __device__ inline float rmul(float s, float a) { return s * a; }
 __host__ __device__ inline cdouble rmul(double s, cdouble a) { return {s * a.re, s * a.im}; }
 __host__ __device__ inline cfloat rmul(float s, cfloat a) { return {s * a.re, s * a.im}; }
 
-// acc + a * b and acc - a * b.  Complex: four multiply-adds; acc + (a * b) as written above is
+// acc + a * b and acc - a * b.  Complex FP64: four multiply-adds; acc + (a * b) as written above is
 // a product, a multiply-add and an addition per component, six instructions (the compiler keeps
 // the order of the sum), which FP64 kernels pay in full (8 x 8 complex FP64 blocks on 32^2 x 128:
-// 475 us so, 285 us with four, at 168 M FMA = 268 us of the measured rate).
+// 475 us so, 285 us with four, at 168 M FMA = 268 us of the measured rate).  Four multiply-adds round
+// the sum twice per term (40 terms: rms 3.0e-16 of the result against 2.2e-16).  Complex FP32 forms
+// the product first: its kernels wait for memory, and a product with the operator, the update of
+// a solution and the dense products keep their digits (an inner solve of the Wilson operator stagnates
+// at a residual of 3.4e-7, at 4.4e-7 with four multiply-adds; 128^2 estimate 70.5 against 69.2 ms).
 __host__ __device__ inline double madd(double c, double a, double b) { return c + a * b; }
 __host__ __device__ inline float madd(float c, float a, float b) { return c + a * b; }
 __host__ __device__ inline double msub(double c, double a, double b) { return c - a * b; }
@@ -85,9 +89,20 @@ __host__ __device__ inline cdouble msub(cdouble c, cdouble a, cdouble b) {
   return {fma(a.im, b.im, fma(-a.re, b.re, c.re)), fma(-a.im, b.re, fma(-a.re, b.im, c.im))};
 }
 __host__ __device__ inline cfloat madd(cfloat c, cfloat a, cfloat b) {
-  return {fmaf(-a.im, b.im, fmaf(a.re, b.re, c.re)), fmaf(a.im, b.re, fmaf(a.re, b.im, c.im))};
+  return {c.re + fmaf(-a.im, b.im, a.re * b.re), c.im + fmaf(a.im, b.re, a.re * b.im)};
 }
 __host__ __device__ inline cfloat msub(cfloat c, cfloat a, cfloat b) {
+  return {c.re - fmaf(-a.im, b.im, a.re * b.re), c.im - fmaf(a.im, b.re, a.re * b.im)};
+}
+// The same in four multiply-adds for complex FP32 too: for the smoothers, whose result the flexible
+// FGMRES takes as it is, so that its rounding does not reach the solution (all kernels with the
+// product first: 128^2 Wilson estimate 72.1 ms).
+template <class T> __host__ __device__ inline T madd4(T c, T a, T b) { return madd(c, a, b); }
+template <class T> __host__ __device__ inline T msub4(T c, T a, T b) { return msub(c, a, b); }
+template <> __host__ __device__ inline cfloat madd4(cfloat c, cfloat a, cfloat b) {
+  return {fmaf(-a.im, b.im, fmaf(a.re, b.re, c.re)), fmaf(a.im, b.re, fmaf(a.re, b.im, c.im))};
+}
+template <> __host__ __device__ inline cfloat msub4(cfloat c, cfloat a, cfloat b) {
   return {fmaf(a.im, b.im, fmaf(-a.re, b.re, c.re)), fmaf(-a.im, b.re, fmaf(-a.re, b.im, c.im))};
 }
 
