@@ -152,12 +152,14 @@ __device__ __forceinline__ void block_sums(const typename lane_of<T>::S (*val)[N
 // then (EXTRA & 2) v0.v0 and (EXTRA & 1) w.w in the following rows: quantities of the same
 // read of the data that would otherwise need passes of their own.
 // HBM-bound on large blocks: 16 warps per SM with about eight 16-byte loads in flight per
-// thread; one block per SM, so only 152 partial sums per column are left to add.  Four FP32
+// thread; one block per SM, so only 152 partial sums per column are left to add (complex FP32,
+// whose 304 blocks keep the lane sums short, two per SM: 8 vectors of 4096 x 200 24.7 -> 20.7 us,
+// 30 of 4096 x 64 49 -> 41).  Four FP32
 // vectors of 1024^2 x 64 with the reduction: 209 us, 6.41 TB/s (250 us with 608 blocks of 256
 // threads, 8-byte loads and FP64 block sums); 16384 x 128, L2-resident: 12.4 us (22.6).
 template <class T, int VEC, int NV, int EXTRA>
-__global__ void __launch_bounds__(DT, 1) k_dots(VecList<T> V, const T *__restrict__ w, size_t rows, int k,
-                                                double *__restrict__ partial, int row0, int nrows) {
+__global__ void __launch_bounds__(DT, std::is_same<T, cfloat>::value ? 2 : 1)
+    k_dots(VecList<T> V, const T *__restrict__ w, size_t rows, int k, double *__restrict__ partial, int row0, int nrows) {
   typedef typename lane_of<T>::S S;
   typedef typename lane_of<T>::A A;
   typedef DPack<T, VEC> P;
@@ -259,7 +261,7 @@ template <class T> constexpr DType type_of() {
 int multidot_parts(DType t, size_t rows, int k) {
   // a row of packs per thread where the rows are few; FP32 packs of four columns at most one block
   // per SM, narrower ones and FP64 two, so that a lane adds up half as many, but whole waves only:
-  // a block of k_dots has an SM to itself (8 FP64 vectors of 4096 x 200: 205 blocks 39 us, 304 with
+  // a block of k_dots has an SM to itself or half of one (8 FP64 vectors of 4096 x 200: 205 blocks 39 us, 304 with
   // block_sums 29)
   const int pack = pack_of(t, k);
   const size_t slots = std::max(1, DT / std::max(k / pack, 1));
