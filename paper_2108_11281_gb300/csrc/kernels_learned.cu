@@ -370,28 +370,26 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_conv_bwd_weight(const float *
     }
 }
 
-// grad[w] = scale * sum over parts of partial[part][w]: a block takes 32 weights (coalesced),
-// its eight warps every eighth part as float pairs (hi + lo, two-sum), added in warp order.
+// grad[w] = scale * sum over parts of partial[part][w] in FP64: a block takes eight weights (one
+// sector per part), 32 threads each adding every 32nd part (up to 1216 parts of a narrow layer; with 32
+// weights per block their FP64 additions would take one SM 12 us), met in fixed order.
 __global__ void __launch_bounds__(256) k_weight_reduce(const float *partial, int nparts, int nw, float *grad,
                                                        float scale) {
-  __shared__ float2 red[8][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = blockIdx.x * 32 + lane;
-  float h = 0.f, l = 0.f;
+  __shared__ double red[32][8];
+  const int lane = threadIdx.x & 7, sl = threadIdx.x >> 3, w = blockIdx.x * 8 + lane;
+  double a = 0.0;
   if (w < nw) {
 #pragma unroll 4
-    for (int b = warp; b < nparts; b += 8) {
-      const float x = partial[(size_t)b * nw + w], s = h + x, t = s - h;
-      l += (h - (s - t)) + (x - t);
-      h = s;
-    }
+    for (int p = sl; p < nparts; p += 32) a += (double)partial[(size_t)p * nw + w];
   }
-  red[warp][lane] = make_float2(h, l);
+  red[sl][lane] = a;
   __syncthreads();
-  if (warp == 0 && w < nw) {
-    double s = 0.0;
-    for (int q = 0; q < 8; ++q) s += (double)red[q][lane].x + (double)red[q][lane].y;
-    grad[w] = (float)(s * scale);
+  if (sl < 4) {
+    for (int q = sl + 4; q < 32; q += 4) a += red[q][lane];
+    red[sl][lane] = a;               // read by this thread alone in this step
   }
+  __syncthreads();
+  if (sl == 0 && w < nw) grad[w] = (float)(((a + red[1][lane]) + (red[2][lane] + red[3][lane])) * scale);
 }
 
 // ------------------------------------------------------------------ Adam
@@ -527,7 +525,7 @@ void launch_conv_bwd_weight(int ci, int co, const float *in, const float *gout, 
 }
 
 void launch_weight_reduce(const float *partial, int nparts, int nw, float *grad, float scale, cudaStream_t s) {
-  k_weight_reduce<<<(nw + 31) / 32, 256, 0, s>>>(partial, nparts, nw, grad, scale);
+  k_weight_reduce<<<(nw + 7) / 8, 256, 0, s>>>(partial, nparts, nw, grad, scale);
   MLMC_LAUNCH_CHECK("k_weight_reduce");
 }
 
