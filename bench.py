@@ -990,14 +990,16 @@ def main():
         if "bytes" in v and "gbs" in v and "flops" not in v and v["bytes"] < 100e6:
             v["bound"] = "l2"
             v["l2_frac"] = v["gbs"] * 1e9 / l2bw
-    # the FP64 fine-level apply: 4 FP64 operations per element (3 additions, 1 FMA)
+    # the FP64 fine-level apply: with the neighbour sums shared along the lattice diagonal an element
+    # takes two additions and one FMA, all issued as FMAs: the FP64 time floor.  The strips of four
+    # columns (0.7 M entries and more) do 13 operations per four elements, a thread per site 4 each.
     if w["kind"] == "laplace" and w.get("transfer") != "bilinear":
         st = kern["stencil_fp64"]
-        ops = 4.0 * w["nx"] * w["ny"] * w["block"]
+        entries = float(w["nx"]) * w["ny"] * w["block"]
+        ops = (13.0 / 4.0 if entries >= 152 * 4608 else 4.0) * entries
         st["fp64_ops_per_s"] = ops / (st["ms"] * 1e-3)
         st["alu_frac_of_measured_fma_rate"] = st["fp64_ops_per_s"] / fma64
-        # 3 additions and 1 FMA per element at the measured rates: the FP64 ALU time floor
-        floor_s = w["nx"] * w["ny"] * w["block"] * (3.0 / add64 + 1.0 / fma64)
+        floor_s = 3.0 * entries / fma64
         st["alu_floor_ms"] = floor_s * 1e3
         st["alu_frac"] = floor_s * 1e3 / st["ms"]
     # dominant kernel of the timed step (largest share of the step's ncu launch list): the

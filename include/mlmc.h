@@ -266,8 +266,8 @@ int mlmc_nominal_sample_cost(const mlmc_hierarchy *h, int level, int form, doubl
  * (the x_j^* y_j products of the difference samples, Remark 4.3), in FP64:
  * double (complex = 0) or interleaved complex double (complex = 1) inputs; out
  * is device memory of k doubles or k complex doubles.  Summation order is
- * fixed (per-column partial sums over 608 row chunks, then a fixed tree).
- * Allocates and frees its scratch (608 x k partial sums) on every call; k <= 256. */
+ * fixed (per-column partial sums over at most 304 row chunks, then a fixed tree).
+ * Allocates and frees its scratch (one partial sum per chunk and column) on every call; k <= 256. */
 int mlmc_column_dots(int complex_data, const void *x, const void *y, int n, int k, void *out, void *stream);
 
 /* mlmc_column_dots without any allocation (the paper has no counterpart).  It
@@ -277,8 +277,8 @@ int mlmc_column_dots(int complex_data, const void *x, const void *y, int n, int 
  * that must not pay an allocator's synchronisation or its failure modes in the
  * middle of a run.  Same arguments and result as mlmc_column_dots, and like it
  * the call returns once `out` has been written.  Its scratch is a fixed array
- * of 2,490,368 bytes inside the library (608 row chunks x 256 columns x 16
- * bytes), present on every GPU that loads the library until the process
+ * of 2,490,368 bytes inside the library (room for 608 row chunks x 256 columns x
+ * 16 bytes; a call uses at most 304 chunks), present on every GPU that loads the library until the process
  * exits; k > 256 is rejected with MLMC_ERR_INVALID_ARG.  The first call on a
  * device (and the first after its context was replaced, e.g. by
  * cudaDeviceReset) looks up the array's device address with

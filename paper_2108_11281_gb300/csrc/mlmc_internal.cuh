@@ -209,7 +209,7 @@ void launch_scale_cols(DType t, void *y, const void *x, const void *alpha, int a
                        size_t rows, int k, cudaStream_t s);
 // out[v][c] = sum_i conj(V_v[i][c]) * w[i][c], v < nvec, FP64 (complex FP64), fixed order
 // (kernels_dots.cu).  partials: nparts * nvec * k FP64 (complex FP64) entries, nparts =
-// multidot_parts(t, rows, k) <= 608.
+// multidot_parts(t, rows, k) <= 304.
 void launch_multidot(DType t, const void *V, size_t vstride, int nvec, const void *w, size_t rows,
                      int k, void *partials, int nparts, void *out, cudaStream_t s);
 int multidot_parts(DType t, size_t rows, int k);

@@ -16,9 +16,9 @@
 
 namespace {
 
-// Largest scratch the entry point may need: 608 row chunks x 256 columns x
-// one complex double.  2,490,368 bytes, held by every GPU that loads the
-// library until the process exits.
+// The scratch, of the documented size: 608 row chunks x 256 columns x one
+// complex double (a call uses at most 304 chunks).  2,490,368 bytes, held by
+// every GPU that loads the library until the process exits.
 constexpr size_t kMaxParts = 608;
 constexpr size_t kMaxColumns = 256;
 constexpr size_t kScratchBytes = kMaxParts * kMaxColumns * 16;
