@@ -155,7 +155,7 @@ __device__ __forceinline__ void block_sums(const typename lane_of<T>::S (*val)[N
 // thread; one block per SM, so only 152 partial sums per column are left to add (complex FP32,
 // whose 304 blocks keep the lane sums short, two per SM: 8 vectors of 4096 x 200 24.7 -> 20.7 us,
 // 30 of 4096 x 64 49 -> 41).  Four FP32
-// vectors of 1024^2 x 64 with the reduction: 209 us, 6.41 TB/s (250 us with 608 blocks of 256
+// vectors of 1024^2 x 64 with the reduction: 210 us, 6.37 TB/s (250 us with 608 blocks of 256
 // threads, 8-byte loads and FP64 block sums); 16384 x 128, L2-resident: 12.4 us (22.6).
 template <class T, int VEC, int NV, int EXTRA>
 __global__ void __launch_bounds__(DT, std::is_same<T, cfloat>::value ? 2 : 1)
@@ -531,9 +531,11 @@ int launch_multiaxpy(DType t, void *w, const void *V, size_t vstride, int nvec, 
 // otherwise take longer than its loads.  Per step they stand in place of two
 // reductions of one warp per output (4.7 us each, strided loads), a cleared counter and a
 // per-column Givens kernel (4.7 us, 9 us complex; a 4-byte memset node costs 4 us and the
-// kernel after it 5 us of gap in a replayed graph): k_fgmres_mid takes 3.3 us, k_fgmres_tail 8.3
-// (two steps, FP32 data; mostly dependent FP64 instructions, so what earlier steps left is
-// loaded before the sums, and the norm of u_j is added up with the dots: 3.5 and 10 us before).
+// kernel after it 5 us of gap in a replayed graph).  Two steps, 64 columns, 152 parts: k_fgmres_mid
+// 3.3 us and k_fgmres_tail 6.7 (FP32), 4.3 and 8.3 (complex FP32, 304 parts), 4.2 and 7.6 (FP64);
+// mostly dependent FP64 instructions, so what earlier steps left is loaded before the sums, and
+// the norm of u_j is added up with the dots.  Tiles of eight scalars with float-pair parts took
+// 3.8 and 8.6 us (FP32).
 namespace {
 
 template <class T> struct fg {

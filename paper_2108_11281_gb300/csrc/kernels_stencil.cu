@@ -157,7 +157,8 @@ template <int D> struct gen_vec<cfloat, D> { static const int v = D <= 2 ? 2 : 1
 // the coefficient reads per column.  FP64 is bound by its arithmetic and keeps one row.
 // Wilson 128^2, level 2 (32^2 sites, complex FP32), one row per thread and coefficients through
 // the cache before: smoother sweep 16.4 -> 12.3 us at k = 32 and 27.7 -> 16.6 us at k = 128,
-// apply 8.2 -> 6.2 and 19.5 -> 12.3 us (two rows per thread alone: 18.5 us per sweep at both).
+// apply 8.2 -> 6.2 and 19.5 -> 14.4 us, 12.3 with the smoother's madd4 (two rows per thread alone:
+// 18.5 us per sweep at both).
 template <class T> constexpr int rows_rpt() { return sizeof(typename real_of<T>::type) == 4 ? 2 : 1; }
 
 __device__ __forceinline__ void copy16_async(void *dst, const void *src) {
