@@ -765,19 +765,22 @@ static void laplace_residual_restrict_go(const StencilView &A, const ProlongView
   constexpr int VW = tr_vec<T>::v;
   const int vec = (VW > 1 && k % VW == 0) ? VW : 1;
   const int kv = k / vec;
-  const size_t items = (size_t)(P.nx / P.ax) * (P.ny / P.ay) * kv;
-  if (items < (size_t)152 * 128) {
-    // 16 column packs per block, or eight for narrow blocks (and for eight coarse dofs, whose sums
-    // fill the shared memory)
+  const size_t aggs = (size_t)(P.nx / P.ax) * (P.ny / P.ay), items = aggs * kv;
+  // 16 column packs per block, or eight for narrow blocks (and for eight coarse dofs, whose sums
+  // fill the shared memory).  Lanes without a pack take their share of the FP64 pipe too, so they
+  // count: 512^2 at one column, 16384 aggregates of one pack, takes 42 us in slots and 12.5 with
+  // a thread per aggregate (FP64, eight coarse dofs; two columns 80 and 14.5).
+  const int kc = kv >= 16 && DC <= 4 ? 16 : 8;
+  if (aggs * ((kv + kc - 1) / kc * kc) < (size_t)152 * 128) {
     auto go = [&](auto vtag, auto ktag) {
       constexpr int V = decltype(vtag)::value, KC = decltype(ktag)::value;
       k_laplace_residual_restrict_slots<T, DC, V, KC>
-          <<<dim3((unsigned)(items / kv), (kv + KC - 1) / KC), dim3(KC, RR_SLOTS), 0, s>>>(
+          <<<dim3((unsigned)aggs, (kv + KC - 1) / KC), dim3(KC, RR_SLOTS), 0, s>>>(
               (const T *)x, (const T *)b, (const T *)P.P, (T *)rc, A.nx, A.ny, P.ax, P.ay, kv, (T)A.diag, A.periodic,
               colour);
     };
     auto width = [&](auto vtag) {
-      if (kv >= 16 && DC <= 4) go(vtag, std::integral_constant<int, 16>());
+      if (kc == 16) go(vtag, std::integral_constant<int, 16>());
       else go(vtag, std::integral_constant<int, 8>());
     };
     if (vec == VW && VW > 1) width(std::integral_constant<int, VW>());
