@@ -269,7 +269,10 @@ static void prolong_go(const ProlongView &P, const void *ec, void *x, int k, int
   const int kv = k / vec;
   const size_t sites = colour < 0 ? (size_t)P.nx * P.ny : (size_t)(P.nx / 2) * P.ny;
   const size_t blocks = (sites * kv + 255) / 256;
-  if (P.d > 1 && blocks < 2 * 152) {
+  // FP32 gains up to about 200 blocks (8 complex dofs on 32^2 sites: 100 columns 8.4 us both ways, 128, 256
+  // blocks, 8.4 with a thread per site and 10.4 over dofs); FP64, whose pipe counts, further (128
+  // columns of 8 real dofs: 20.7 and 18.5)
+  if (P.d > 1 && blocks < (sizeof(typename real_of<T>::type) == 8 ? 2 * 152 : 152 * 3 / 2)) {
     const unsigned g = (unsigned)((sites * P.d * kv + 127) / 128);
     if (vec == VW && VW > 1)
       k_prolong_add_dofs<T, DC, VW><<<g, 128, 0, s>>>((const T *)P.P, (const T *)ec, (T *)x, P.nx, P.ny, P.d, P.ax, P.ay,
