@@ -161,6 +161,26 @@ template <int D> struct gen_vec<cfloat, D> { static const int v = D <= 2 ? 2 : 1
 // 18.5 us per sweep at both).
 template <class T> constexpr int rows_rpt() { return sizeof(typename real_of<T>::type) == 4 ? 2 : 1; }
 
+// Real FP64 with more blocks than SMs reads the coefficients through the cache instead (STAGED
+// false): its arithmetic fills the FP64 pipe only with other blocks beside a block that waits, and
+// with all neighbours' entries in registers two fit on an SM.  128^2 x 8 sites, FP64: apply 317 us
+// staged and 285 through the cache at k = 32, 1228 and 1119 at k = 128, smoother sweep 1183 and 1097;
+// 32^2 x 8: apply 25.8 and 22.5 at k = 32; 24^2 x 8: sweep 18.3 and 16.6.  Fewer blocks wait for one
+// round trip to L2: 8^2 x 8 at k = 64 9.2 and 10.3, sweep of 16^2 x 8 at k = 21 12.5 and 14.4.
+template <class T> static bool rows_staged(size_t blocks) { return !std::is_same<T, double>::value || blocks <= 152; }
+// go(CV, STAGED) with both as compile-time constants
+template <class T, class F> static void rows_dispatch(int k, int sites, F &&go) {
+  const int cv = (k % 2 == 0 && k >= 64) ? 2 : 1;        // two columns per thread on blocks of at least 64 even columns
+  const dim3 grid((k / cv + 31) / 32, sites);
+  auto with_cv = [&](auto c) {
+    if constexpr (std::is_same<T, double>::value)
+      if (!rows_staged<T>((size_t)grid.x * grid.y)) return go(c, std::false_type(), grid);
+    go(c, std::true_type(), grid);
+  };
+  if (cv == 2) with_cv(std::integral_constant<int, 2>());
+  else with_cv(std::integral_constant<int, 1>());
+}
+
 __device__ __forceinline__ void copy16_async(void *dst, const void *src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
                : "memory");
@@ -171,15 +191,15 @@ __device__ __forceinline__ void block_copy_async(void *dst, const void *src, int
   for (int e = tid * 16; e < bytes; e += threads * 16) copy16_async((char *)dst + e, (const char *)src + e);
 }
 
-// acc[r] +- sum over NDIR neighbour blocks of rows r0 + r (blk: [NDIR][D][D] in shared memory)
-// times their x, XB neighbours' entries in flight at a time.  ready(): called after the first
-// loads are issued and before the coefficients are read.  SUB is the smoother's form (msub4).
-template <class T, int D, int CV, int RPT, int NDIR, bool SUB, class F>
+// acc[r] +- sum over NDIR neighbour blocks of rows r0 + r (blk: [NDIR][D][D], STAGED in shared
+// memory) times their x, XB neighbours' entries in flight at a time.  ready(): STAGED, called after
+// the first loads are issued and before the coefficients are read.  SUB is the smoother's form (msub4).
+template <class T, int D, int CV, int RPT, int NDIR, bool SUB, bool STAGED, class F>
 __device__ __forceinline__ void rows_accumulate(const T *blk, const T *x, const int nb[NDIR], int r0, int k, int c,
                                                 bool live, Pack<T, CV> acc[RPT], F ready) {
   typedef Pack<T, CV> V;
   constexpr int WORDS = D * CV * (int)sizeof(T) / 4;                    // registers of one neighbour
-  constexpr int XB = WORDS * NDIR <= 80 ? NDIR : WORDS <= 32 ? 2 : 1;   // neighbours in flight
+  constexpr int XB = !STAGED ? 1 : WORDS * NDIR <= 80 ? NDIR : WORDS <= 32 ? 2 : 1;   // neighbours in flight
   const int kv = k / CV;
 #pragma unroll
   for (int d0 = 0; d0 < NDIR; d0 += XB) {
@@ -191,15 +211,19 @@ __device__ __forceinline__ void rows_accumulate(const T *blk, const T *x, const 
 #pragma unroll
         for (int q = 0; q < D; ++q) xv[e][q] = xs[(size_t)q * kv];
       }
-    asm volatile("" ::: "memory");                                      // the loads stay in front
-    if (d0 == 0) ready();
+    if constexpr (STAGED) {
+      asm volatile("" ::: "memory");                                    // the loads stay in front
+      if (d0 == 0) ready();
+    }
 #pragma unroll
     for (int e = 0; e < XB; ++e)
       if (d0 + e < NDIR) {
 #pragma unroll
         for (int r = 0; r < RPT; ++r) {
           T row[D];
-          memcpy(row, __builtin_assume_aligned(blk + ((size_t)(d0 + e) * D + r0 + r) * D, 16), sizeof(row));
+          const T *src = blk + ((size_t)(d0 + e) * D + r0 + r) * D;
+          if constexpr (STAGED) memcpy(row, __builtin_assume_aligned(src, 16), sizeof(row));
+          else load_row<T, D>(src, row);
 #pragma unroll
           for (int q = 0; q < D; ++q)
 #pragma unroll
@@ -215,19 +239,20 @@ __device__ __forceinline__ void async_ready() {
   __syncthreads();
 }
 
-template <class T, int D, int CV, int RPT>
+template <class T, int D, int CV, int RPT, bool STAGED>
 __global__ void __launch_bounds__(32 * D / RPT) k_stencil_rows(const T *__restrict__ coef, const T *x, const T *b,
                                                                T *y, int nx, int ny, int k, int mode) {
   typedef Pack<T, CV> V;
-  __shared__ __align__(16) unsigned char blk_mem[5 * D * D * sizeof(T)];
-  const T *blk = (const T *)blk_mem;
+  __shared__ __align__(16) unsigned char blk_mem[STAGED ? 5 * D * D * sizeof(T) : 16];
   const int s = blockIdx.y;
+  const T *blk = STAGED ? (const T *)blk_mem : coef + (size_t)s * 5 * D * D;
   const int i = s % nx, j = s / nx;
   const int r0 = threadIdx.y * RPT;
   const int c = (blockIdx.x * 32 + threadIdx.x) * CV;   // k is a multiple of CV
   const bool live = c < k;
-  block_copy_async(blk_mem, coef + (size_t)s * 5 * D * D, 5 * D * D * (int)sizeof(T), threadIdx.y * 32 + threadIdx.x,
-                   32 * D / RPT);
+  if constexpr (STAGED)
+    block_copy_async(blk_mem, coef + (size_t)s * 5 * D * D, 5 * D * D * (int)sizeof(T), threadIdx.y * 32 + threadIdx.x,
+                     32 * D / RPT);
   int nb[5];
   nb[0] = s;
   nb[1] = j * nx + (i + 1 == nx ? 0 : i + 1);
@@ -239,7 +264,7 @@ __global__ void __launch_bounds__(32 * D / RPT) k_stencil_rows(const T *__restri
   for (int r = 0; r < RPT; ++r)
 #pragma unroll
     for (int u = 0; u < CV; ++u) acc[r].v[u] = zero<T>();
-  rows_accumulate<T, D, CV, RPT, 5, false>(blk, x, nb, r0, k, c, live, acc, async_ready);
+  rows_accumulate<T, D, CV, RPT, 5, false, STAGED>(blk, x, nb, r0, k, c, live, acc, async_ready);
   if (!live) return;
 #pragma unroll
   for (int r = 0; r < RPT; ++r) {
@@ -254,20 +279,15 @@ __global__ void __launch_bounds__(32 * D / RPT) k_stencil_rows(const T *__restri
   }
 }
 
-// two columns per thread on blocks of at least 64 even columns
-inline int rows_cv(int k) { return (k % 2 == 0 && k >= 64) ? 2 : 1; }
-
 template <class T, int D>
 static void stencil_go(const StencilView &A, const void *x, const void *b, void *y, int k, int mode, cudaStream_t s) {
   if constexpr (D >= 8) {
     if (A.nx * A.ny <= 65535) {
       constexpr int RPT = rows_rpt<T>();
-      if (rows_cv(k) == 2)
-        k_stencil_rows<T, D, 2, RPT><<<dim3((k / 2 + 31) / 32, A.nx * A.ny), dim3(32, D / RPT), 0, s>>>(
+      rows_dispatch<T>(k, A.nx * A.ny, [&](auto cv, auto staged, dim3 grid) {
+        k_stencil_rows<T, D, decltype(cv)::value, RPT, decltype(staged)::value><<<grid, dim3(32, D / RPT), 0, s>>>(
             (const T *)A.coef, (const T *)x, (const T *)b, (T *)y, A.nx, A.ny, k, mode);
-      else
-        k_stencil_rows<T, D, 1, RPT><<<dim3((k + 31) / 32, A.nx * A.ny), dim3(32, D / RPT), 0, s>>>(
-            (const T *)A.coef, (const T *)x, (const T *)b, (T *)y, A.nx, A.ny, k, mode);
+      });
       return;
     }
   }
@@ -759,14 +779,14 @@ __global__ void __launch_bounds__(128, 8) k_rbgs_half_p(const T *__restrict__ co
 // Row-split half-sweep for large site blocks (see k_stencil_rows).  Phase 1: res_r = b_r - sum
 // over the 4 neighbour blocks of row r times their x; phase 2, after a block barrier:
 // x_r = sum_q Dinv[r][q] res_q from shared memory.  Grid = (column chunks, sites of the colour).
-template <class T, int D, int CV, int RPT>
+template <class T, int D, int CV, int RPT, bool STAGED>
 __global__ void __launch_bounds__(32 * D / RPT) k_rbgs_half_rows(const T *__restrict__ coef,
                                                                  const T *__restrict__ dinv, T *x, const T *src,
                                                                  const T *b, int nx,
                                                                  int ny, int k, int colour, int other_zero) {
   typedef Pack<T, CV> V;
   constexpr int BLK = D * D * (int)sizeof(T);
-  __shared__ __align__(16) unsigned char blk_mem[5 * BLK];   // the four neighbour blocks, then D^-1
+  __shared__ __align__(16) unsigned char blk_mem[STAGED ? 5 * BLK : 16];   // the four neighbour blocks, then D^-1
   __shared__ V res[D][32];
   const int hx = nx / 2;
   const int idx = blockIdx.y;                       // site of this colour: row j, position m
@@ -776,8 +796,11 @@ __global__ void __launch_bounds__(32 * D / RPT) k_rbgs_half_rows(const T *__rest
   const int cl = threadIdx.x, r0 = threadIdx.y * RPT, tid = threadIdx.y * 32 + threadIdx.x;
   const int c = (blockIdx.x * 32 + cl) * CV;        // k is a multiple of CV
   const bool live = c < k;
-  if (!other_zero) block_copy_async(blk_mem, coef + ((size_t)s * 5 + 1) * D * D, 4 * BLK, tid, 32 * D / RPT);
-  block_copy_async(blk_mem + 4 * BLK, dinv + (size_t)s * D * D, BLK, tid, 32 * D / RPT);
+  const T *blk = STAGED ? (const T *)blk_mem : coef + ((size_t)s * 5 + 1) * D * D;
+  if constexpr (STAGED) {
+    if (!other_zero) block_copy_async(blk_mem, coef + ((size_t)s * 5 + 1) * D * D, 4 * BLK, tid, 32 * D / RPT);
+    block_copy_async(blk_mem + 4 * BLK, dinv + (size_t)s * D * D, BLK, tid, 32 * D / RPT);
+  }
   V acc[RPT];
 #pragma unroll
   for (int r = 0; r < RPT; ++r)
@@ -788,8 +811,8 @@ __global__ void __launch_bounds__(32 * D / RPT) k_rbgs_half_rows(const T *__rest
     nb[1] = j * nx + (i == 0 ? nx - 1 : i - 1);
     nb[2] = (j + 1 == ny ? 0 : j + 1) * nx + i;
     nb[3] = (j == 0 ? ny - 1 : j - 1) * nx + i;
-    rows_accumulate<T, D, CV, RPT, 4, true>((const T *)blk_mem, src, nb, r0, k, c, live, acc, async_ready);
-  } else {
+    rows_accumulate<T, D, CV, RPT, 4, true, STAGED>(blk, src, nb, r0, k, c, live, acc, async_ready);
+  } else if constexpr (STAGED) {
     async_ready();
   }
 #pragma unroll
@@ -800,7 +823,10 @@ __global__ void __launch_bounds__(32 * D / RPT) k_rbgs_half_rows(const T *__rest
 #pragma unroll
   for (int r = 0; r < RPT; ++r) {
     T row[D];
-    memcpy(row, __builtin_assume_aligned(blk_mem + 4 * BLK + (size_t)(r0 + r) * D * sizeof(T), 16), sizeof(row));
+    if constexpr (STAGED)
+      memcpy(row, __builtin_assume_aligned(blk_mem + 4 * BLK + (size_t)(r0 + r) * D * sizeof(T), 16), sizeof(row));
+    else
+      load_row<T, D>(dinv + ((size_t)s * D + r0 + r) * D, row);
 #pragma unroll
     for (int u = 0; u < CV; ++u) out[r].v[u] = zero<T>();
 #pragma unroll
@@ -819,12 +845,10 @@ static void rbgs_go(const StencilView &A, const void *coef, void *x, const void 
   if constexpr (D >= 8) {
     if ((A.nx / 2) * A.ny <= 65535) {
       constexpr int RPT = rows_rpt<T>();
-      if (rows_cv(k) == 2)
-        k_rbgs_half_rows<T, D, 2, RPT><<<dim3((k / 2 + 31) / 32, (A.nx / 2) * A.ny), dim3(32, D / RPT), 0, s>>>(
+      rows_dispatch<T>(k, (A.nx / 2) * A.ny, [&](auto cv, auto staged, dim3 grid) {
+        k_rbgs_half_rows<T, D, decltype(cv)::value, RPT, decltype(staged)::value><<<grid, dim3(32, D / RPT), 0, s>>>(
             (const T *)coef, (const T *)A.dinv, (T *)x, (const T *)src, (const T *)b, A.nx, A.ny, k, colour, other_zero);
-      else
-        k_rbgs_half_rows<T, D, 1, RPT><<<dim3((k + 31) / 32, (A.nx / 2) * A.ny), dim3(32, D / RPT), 0, s>>>(
-            (const T *)coef, (const T *)A.dinv, (T *)x, (const T *)src, (const T *)b, A.nx, A.ny, k, colour, other_zero);
+      });
       return;
     }
   }
