@@ -95,20 +95,24 @@ __device__ __forceinline__ void stencil_body(const T *__restrict__ coef, const T
 // clock and SM, so what counts is that every SM gets the same number of threads: blocks of 32
 // (the 48^2 x 4 level at 21 columns: smoother half-sweep 7.1 us and apply 11.7 us with 256, whose
 // 96 and 192 blocks load some of 152 SMs twice; a 192^2 FP64 solve takes 8.34 ms with 256, 7.97
-// with 64 and 7.77 with 32).
-template <class T> __host__ __device__ constexpr int gen_threads() { return sizeof(typename real_of<T>::type) == 8 ? 32 : 256; }
+// with 64 and 7.77 with 32).  One dof per site has so little arithmetic that the loads count, and 32
+// blocks of 32 threads are half of what an SM holds: 128 (128^2 x 1 at 32 columns, apply: 10.3 us
+// with 32, 8.4 with 128; 128^2 x 2 8.4 and 8.4).
+template <class T, int D> __host__ __device__ constexpr int gen_threads() {
+  return sizeof(typename real_of<T>::type) == 8 ? (D == 1 ? 128 : 32) : 256;
+}
 
 // Resident grid striding over the units (row j, chunk of one block's threads of the row): the
 // FP64 block applies are bound by the FP64 pipe, which one block per unit leaves idle between
 // blocks.
 template <class T, int D, int VEC>
-__global__ void __launch_bounds__(gen_threads<T>()) k_stencil(const T *__restrict__ coef, const T *__restrict__ x,
+__global__ void __launch_bounds__(gen_threads<T, D>()) k_stencil(const T *__restrict__ coef, const T *__restrict__ x,
                                                  const T *__restrict__ b, T *__restrict__ y, int nx, int ny, int kv,
                                                  int mode, int bpr) {
   const int units = bpr * ny;
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
     const int j = u / bpr;
-    stencil_body<T, D, VEC>(coef, x, b, y, nx, ny, kv, mode, j, (u - j * bpr) * gen_threads<T>() + threadIdx.x);
+    stencil_body<T, D, VEC>(coef, x, b, y, nx, ny, kv, mode, j, (u - j * bpr) * gen_threads<T, D>() + threadIdx.x);
   }
 }
 
@@ -291,7 +295,7 @@ static void stencil_go(const StencilView &A, const void *x, const void *b, void 
       return;
     }
   }
-  constexpr int VW = gen_vec<T, D>::v, TB = gen_threads<T>();
+  constexpr int VW = gen_vec<T, D>::v, TB = gen_threads<T, D>();
   if (VW > 1 && k % VW == 0) {
     int kv = k / VW;
     if constexpr (std::is_same<T, float>::value && D == 4)
@@ -362,10 +366,9 @@ __device__ __forceinline__ void laplace_nbr_sum(const Pack<T, VEC> *__restrict__
 // k_laplace_march (see laplace_fp64).
 enum { LAP_APPLY = 0, LAP_RESIDUAL = 1, LAP_JACOBI = 2 };
 
-template <class T, int VEC>
+template <class T, int VEC, int MODE>
 __device__ __forceinline__ void laplace_body(const T *__restrict__ x, const T *__restrict__ b, T *__restrict__ y,
-                                             int nx, int ny, int kv, T diag, T scale, int periodic, int mode, int j,
-                                             int t) {
+                                             int nx, int ny, int kv, T diag, T scale, int periodic, int j, int t) {
   typedef Pack<T, VEC> V;
   if (t >= nx * kv) return;
   const int i = t / kv, c = t - (t / kv) * kv;
@@ -376,11 +379,11 @@ __device__ __forceinline__ void laplace_body(const T *__restrict__ x, const T *_
   T sum[VEC];
   laplace_nbr_sum<T, VEC>(X, n, kv, c, sum);
   V out;
-  if (mode == LAP_RESIDUAL) {
+  if (MODE == LAP_RESIDUAL) {
     V bb = ((const V *)b)[(size_t)s * kv + c];
 #pragma unroll
     for (int u = 0; u < VEC; ++u) out.v[u] = (bb.v[u] + sum[u]) - diag * xc.v[u];
-  } else if (mode == LAP_JACOBI) {
+  } else if (MODE == LAP_JACOBI) {
 #pragma unroll
     for (int u = 0; u < VEC; ++u) out.v[u] = diag * xc.v[u] + scale * sum[u];
   } else {
@@ -391,28 +394,32 @@ __device__ __forceinline__ void laplace_body(const T *__restrict__ x, const T *_
 }
 
 // Resident grid striding over the units (row j, chunk of 256 threads of the row) in row order.
-template <class T, int VEC>
+template <class T, int VEC, int MODE>
 __global__ void __launch_bounds__(256) k_laplace(const T *__restrict__ x, const T *__restrict__ b, T *__restrict__ y,
-                                                 int nx, int ny, int kv, T diag, T scale, int periodic, int mode,
-                                                 int bpr) {
+                                                 int nx, int ny, int kv, T diag, T scale, int periodic, int bpr) {
   const int units = bpr * ny;
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
     const int j = u / bpr;
-    laplace_body<T, VEC>(x, b, y, nx, ny, kv, diag, scale, periodic, mode, j, (u - j * bpr) * 256 + threadIdx.x);
+    laplace_body<T, VEC, MODE>(x, b, y, nx, ny, kv, diag, scale, periodic, j, (u - j * bpr) * 256 + threadIdx.x);
   }
 }
+
+// Threads per block of the half-sweep below.  FP64: small blocks for an even share per SM, but not so
+// small that 32 of them, the most an SM holds, leave it half empty (512^2 at 21 columns: sweep 67.8 us
+// with 32, 65.7 with 64; 192^2 at 5: 12.3 and 10.0).  FROM_ZERO is a compile-time flag: as an argument
+// it cost the FP64 pipe a multiply-add per entry (512^2 at 21 columns: 78.0 us).
+template <class T> __host__ __device__ constexpr int lap_threads() { return sizeof(T) == 8 ? 64 : 256; }
 
 // Red-black Gauss-Seidel half-sweep for Example 5.1: x_s = (b_s + sum of neighbours) / diag
 // on the sites of `colour`.  other_zero = 1: the other colour holds zeros (not read).
 // Colour 1 takes the rows from the last: consecutive half-sweeps alternate direction, so
 // each starts on the rows the previous one wrote last.
-// from_zero = 1: the whole first sweep from x = 0 as one pass over colour 1,
+// FROM_ZERO: the whole first sweep from x = 0 as one pass over colour 1,
 // x_1 = (b_1 + sum of b_0 / diag) / diag; colour 0 is left unset (see launch_rbgs_first).
 // The grid strides over the units (row, chunk of one block's threads of the row).
-template <class T, int VEC>
+template <class T, int VEC, bool FROM_ZERO>
 __device__ __forceinline__ void laplace_rbgs_body(T *__restrict__ x, const T *__restrict__ b, int nx, int ny, int kv,
-                                                  T dinv, int periodic, int colour, int other_zero, int from_zero,
-                                                  int j, int t) {
+                                                  T dinv, int periodic, int colour, int other_zero, int j, int t) {
   typedef Pack<T, VEC> V;
   const int i0 = (j + colour) & 1;
   const int hx = (nx - i0 + 1) >> 1;      // sites of this colour in row j (odd nx too)
@@ -425,24 +432,24 @@ __device__ __forceinline__ void laplace_rbgs_body(T *__restrict__ x, const T *__
   if (!other_zero) {
     const Nbrs n = laplace_nbrs(i, j, nx, ny, periodic);
     T sum[VEC];
-    laplace_nbr_sum<T, VEC>(from_zero ? (const V *)b : X, n, kv, c, sum);
+    laplace_nbr_sum<T, VEC>(FROM_ZERO ? (const V *)b : X, n, kv, c, sum);
 #pragma unroll
-    for (int u = 0; u < VEC; ++u) acc.v[u] = from_zero ? madd(acc.v[u], dinv, sum[u]) : acc.v[u] + sum[u];
+    for (int u = 0; u < VEC; ++u) acc.v[u] = FROM_ZERO ? madd(acc.v[u], dinv, sum[u]) : acc.v[u] + sum[u];
   }
 #pragma unroll
   for (int u = 0; u < VEC; ++u) acc.v[u] = acc.v[u] * dinv;
   X[(size_t)s * kv + c] = acc;
 }
 
-template <class T, int VEC>
-__global__ void __launch_bounds__(gen_threads<T>()) k_laplace_rbgs(T *__restrict__ x, const T *__restrict__ b, int nx, int ny,
-                                                      int kv, T dinv, int periodic, int colour, int other_zero,
-                                                      int from_zero, int bpr) {
+template <class T, int VEC, bool FROM_ZERO>
+__global__ void __launch_bounds__(lap_threads<T>()) k_laplace_rbgs(T *__restrict__ x, const T *__restrict__ b, int nx,
+                                                                   int ny, int kv, T dinv, int periodic, int colour,
+                                                                   int other_zero, int bpr) {
   const int units = bpr * ny;
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
     const int jr = u / bpr;
-    laplace_rbgs_body<T, VEC>(x, b, nx, ny, kv, dinv, periodic, colour, other_zero, from_zero,
-                              colour ? ny - 1 - jr : jr, (u - jr * bpr) * gen_threads<T>() + threadIdx.x);
+    laplace_rbgs_body<T, VEC, FROM_ZERO>(x, b, nx, ny, kv, dinv, periodic, colour, other_zero,
+                                         colour ? ny - 1 - jr : jr, (u - jr * bpr) * lap_threads<T>() + threadIdx.x);
   }
 }
 
@@ -574,13 +581,13 @@ static void laplace_march(const StencilView &A, const void *x, const void *b, vo
                                                scale, 1.0, A.periodic, JB);
 }
 
-template <class T, int VEC>
-static void laplace_sites(const StencilView &A, const void *x, const void *b, void *y, int k, T diag, T scale, int mode,
+template <class T, int VEC, int MODE>
+static void laplace_sites(const StencilView &A, const void *x, const void *b, void *y, int k, T diag, T scale,
                           cudaStream_t s) {
   const int kv = k / VEC, bpr = (A.nx * kv + 255) / 256;
-  static const int occ = blocks_per_sm(k_laplace<T, VEC>, 256, 0);
-  k_laplace<T, VEC><<<resident_grid((size_t)bpr * A.ny, occ), 256, 0, s>>>(
-      (const T *)x, (const T *)b, (T *)y, A.nx, A.ny, kv, diag, scale, A.periodic, mode, bpr);
+  static const int occ = blocks_per_sm(k_laplace<T, VEC, MODE>, 256, 0);
+  k_laplace<T, VEC, MODE><<<resident_grid((size_t)bpr * A.ny, occ), 256, 0, s>>>(
+      (const T *)x, (const T *)b, (T *)y, A.nx, A.ny, kv, diag, scale, A.periodic, bpr);
 }
 
 // FP64: strips walked by few threads only pay where the pipe is busy.  Below about 4600 entries
@@ -591,8 +598,8 @@ template <int MODE>
 static void laplace_fp64(const StencilView &A, const void *x, const void *b, void *y, int k, double diag, double scale,
                          cudaStream_t s) {
   if ((size_t)A.nx * A.ny * k >= (size_t)152 * 4608) laplace_march<MODE>(A, x, b, y, k, diag, scale, s);
-  else if (laplace_vec<double>(k) == 2) laplace_sites<double, 2>(A, x, b, y, k, diag, scale, MODE, s);
-  else laplace_sites<double, 1>(A, x, b, y, k, diag, scale, MODE, s);
+  else if (laplace_vec<double>(k) == 2) laplace_sites<double, 2, MODE>(A, x, b, y, k, diag, scale, s);
+  else laplace_sites<double, 1, MODE>(A, x, b, y, k, diag, scale, s);
 }
 
 // One damped-Jacobi sweep of the setup filter for Example 5.1 in one pass (out must not alias x):
@@ -611,8 +618,13 @@ static void launch_laplace(const StencilView &A, const void *x, const void *b, v
     if (mode) laplace_fp64<LAP_RESIDUAL>(A, x, b, y, k, A.diag, 0.0, s);
     else laplace_fp64<LAP_APPLY>(A, x, b, y, k, A.diag, 0.0, s);
   } else if (A.t == F32) {
-    if (laplace_vec<float>(k) == 4) laplace_sites<float, 4>(A, x, b, y, k, (float)A.diag, 0.f, mode ? 1 : 0, s);
-    else laplace_sites<float, 1>(A, x, b, y, k, (float)A.diag, 0.f, mode ? 1 : 0, s);
+    auto go = [&](auto vec) {
+      constexpr int VEC = decltype(vec)::value;
+      if (mode) laplace_sites<float, VEC, LAP_RESIDUAL>(A, x, b, y, k, (float)A.diag, 0.f, s);
+      else laplace_sites<float, VEC, LAP_APPLY>(A, x, b, y, k, (float)A.diag, 0.f, s);
+    };
+    if (laplace_vec<float>(k) == 4) go(std::integral_constant<int, 4>());
+    else go(std::integral_constant<int, 1>());
   } else {
     throw cuda_error{cudaErrorInvalidValue, "constant-coefficient Laplacian is real"};
   }
@@ -620,21 +632,24 @@ static void launch_laplace(const StencilView &A, const void *x, const void *b, v
 }
 
 static void launch_laplace_rbgs(const StencilView &A, void *x, const void *b, int k, int colour, int other_zero,
-                                cudaStream_t s, int from_zero = 0) {
-  auto go = [&](auto tag, auto vtag) {
+                                cudaStream_t s, bool from_zero = false) {
+  auto launch = [&](auto tag, auto vtag, auto ztag) {
     typedef decltype(tag) T;
-    constexpr int VEC = decltype(vtag)::value;
+    constexpr int VEC = decltype(vtag)::value, TB = lap_threads<T>();
+    constexpr bool FROM_ZERO = decltype(ztag)::value;
     int kv = k / VEC;
-    constexpr int TB = gen_threads<T>();
     const int bpr = (((A.nx + 1) / 2) * kv + TB - 1) / TB;
-    static const int occ = blocks_per_sm(k_laplace_rbgs<T, VEC>, TB, 0);
+    static const int occ = blocks_per_sm(k_laplace_rbgs<T, VEC, FROM_ZERO>, TB, 0);
     // FP64: a resident grid (FP64-pipe bound); FP32: one block per unit, measured faster
     // there (119 against 124 us per sweep on 1024^2 x 64)
     const unsigned grid = std::is_same<T, double>::value ? resident_grid((size_t)bpr * A.ny, occ)
                                                          : (unsigned)(bpr * A.ny);
-    k_laplace_rbgs<T, VEC><<<grid, TB, 0, s>>>(
-        (T *)x, (const T *)b, A.nx, A.ny, kv, (T)(1.0 / A.diag), A.periodic, colour, other_zero, from_zero,
-        bpr);
+    k_laplace_rbgs<T, VEC, FROM_ZERO><<<grid, TB, 0, s>>>((T *)x, (const T *)b, A.nx, A.ny, kv, (T)(1.0 / A.diag),
+                                                          A.periodic, colour, other_zero, bpr);
+  };
+  auto go = [&](auto tag, auto vtag) {
+    if (from_zero) launch(tag, vtag, std::true_type());
+    else launch(tag, vtag, std::false_type());
   };
   if (A.t == F64) {
     if (laplace_vec<double>(k) == 2) go(double(), std::integral_constant<int, 2>());
@@ -741,7 +756,7 @@ __device__ __forceinline__ void rbgs_half_body(const T *__restrict__ coef, const
 }
 
 template <class T, int D, int VEC>
-__global__ void __launch_bounds__(gen_threads<T>()) k_rbgs_half(const T *__restrict__ coef, const T *__restrict__ dinv,
+__global__ void __launch_bounds__(gen_threads<T, D>()) k_rbgs_half(const T *__restrict__ coef, const T *__restrict__ dinv,
                                                    T *x, const T *src, const T *b, int nx, int ny, int kv,
                                                    int colour, int other_zero, int bpr) {
   // resident grid striding over the units (row j, chunk of one block's threads of the row)
@@ -749,7 +764,7 @@ __global__ void __launch_bounds__(gen_threads<T>()) k_rbgs_half(const T *__restr
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
     const int j = u / bpr;
     rbgs_half_body<T, D, VEC>(coef, dinv, x, src, b, nx, ny, kv, colour, other_zero, j,
-                              (u - j * bpr) * gen_threads<T>() + threadIdx.x);
+                              (u - j * bpr) * gen_threads<T, D>() + threadIdx.x);
   }
 }
 
@@ -852,7 +867,7 @@ static void rbgs_go(const StencilView &A, const void *coef, void *x, const void 
       return;
     }
   }
-  constexpr int VW = rbgs_vec<T, D>::v, TB = gen_threads<T>();
+  constexpr int VW = rbgs_vec<T, D>::v, TB = gen_threads<T, D>();
   if (VW > 1 && k % VW == 0) {
     int kv = k / VW;
     if constexpr (std::is_same<T, float>::value && D == 4)
@@ -912,7 +927,7 @@ void launch_rbgs_sweep(const StencilView &A, void *x, const void *b, int k, int 
 // one launch and 1.5 vector passes instead of two and 2.5.
 void launch_rbgs_first(const StencilView &A, void *x, const void *b, int k, cudaStream_t s) {
   if (A.const_laplace) {
-    launch_laplace_rbgs(A, x, b, k, 1, 0, s, 1);
+    launch_laplace_rbgs(A, x, b, k, 1, 0, s, true);
     return;
   }
   if (!A.first) throw cuda_error{cudaErrorInvalidValue, "rbgs_first: no products on this level"};
