@@ -264,10 +264,13 @@ int multidot_parts(DType t, size_t rows, int k) {
   // a block of k_dots has an SM to itself or half of one (8 FP64 vectors of 4096 x 200: 205 blocks 39 us, 304 with
   // block_sums 29)
   const int pack = pack_of(t, k);
-  const size_t slots = std::max(1, DT / std::max(k / pack, 1));
-  const size_t p = std::max<size_t>(1, (rows + slots - 1) / slots);
-  if (p <= DOT_PARTS || pack == 4) return (int)std::min<size_t>(DOT_PARTS, p);
   const bool fp64 = dtype_lower(t) != t;       // no lane sums in FP32 to keep short
+  const size_t packs = std::max(k / pack, 1), slots = std::max<size_t>(1, DT / packs);
+  const size_t p = std::max<size_t>(1, (rows + slots - 1) / slots);
+  // FP64 that would stay on less than half of the SMs: 64 packs per block, whose arithmetic otherwise
+  // takes longer than the loads
+  if (fp64 && p <= 64) return (int)std::min<size_t>(DOT_PARTS, (rows + std::max<size_t>(1, 64 / packs) - 1) / std::max<size_t>(1, 64 / packs));
+  if (p <= DOT_PARTS || pack == 4) return (int)std::min<size_t>(DOT_PARTS, p);
   return fp64 && p < 2 * DOT_PARTS ? DOT_PARTS : 2 * DOT_PARTS;
 }
 
@@ -465,9 +468,10 @@ __global__ void __launch_bounds__(DT, 2) k_axpy(T *__restrict__ w, const T *__re
 
 static const int AXPY_SMEM = 32 * 1024;
 
-// A row of packs per thread, at most two blocks per SM.
+// A row of packs per thread, at most two blocks per SM.  FP64: 64 packs per block where the rows are
+// few, since a block's FP64 arithmetic takes its SM longer than the loads.
 int multiaxpy_norm_parts(DType t, size_t rows, int k) {
-  const size_t slots = std::max(1, DT / std::max(k / pack_of(t, k), 1));
+  const size_t packs = std::max(k / pack_of(t, k), 1), slots = std::max<size_t>(1, (dtype_lower(t) != t ? 64 : DT) / packs);
   return (int)std::min<size_t>(AXPY_PARTS, std::max<size_t>(1, (rows + slots - 1) / slots));
 }
 
