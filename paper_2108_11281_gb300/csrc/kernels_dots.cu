@@ -267,9 +267,13 @@ int multidot_parts(DType t, size_t rows, int k) {
   const bool fp64 = dtype_lower(t) != t;       // no lane sums in FP32 to keep short
   const size_t packs = std::max(k / pack, 1), slots = std::max<size_t>(1, DT / packs);
   const size_t p = std::max<size_t>(1, (rows + slots - 1) / slots);
-  // FP64 that would stay on less than half of the SMs: 64 packs per block, whose arithmetic otherwise
-  // takes longer than the loads
-  if (fp64 && p <= 64) return (int)std::min<size_t>(DOT_PARTS, (rows + std::max<size_t>(1, 64 / packs) - 1) / std::max<size_t>(1, 64 / packs));
+  // complex FP64 that would stay on less than half of the SMs: 64 packs per block, whose arithmetic
+  // otherwise takes longer than the loads (four vectors of 128 x 8: 12.4 -> 10.4 us; real ones lose 1 us
+  // to the longer second stage where it is not that)
+  if (t == C64 && p <= 64) {
+    const size_t few = std::max<size_t>(1, 64 / packs);
+    return (int)std::min<size_t>(DOT_PARTS, (rows + few - 1) / few);
+  }
   if (p <= DOT_PARTS || pack == 4) return (int)std::min<size_t>(DOT_PARTS, p);
   return fp64 && p < 2 * DOT_PARTS ? DOT_PARTS : 2 * DOT_PARTS;
 }
@@ -469,7 +473,8 @@ __global__ void __launch_bounds__(DT, 2) k_axpy(T *__restrict__ w, const T *__re
 static const int AXPY_SMEM = 32 * 1024;
 
 // A row of packs per thread, at most two blocks per SM.  FP64: 64 packs per block where the rows are
-// few, since a block's FP64 arithmetic takes its SM longer than the loads.
+// few, since a block's FP64 arithmetic takes its SM longer than the loads (four vectors of 1024 x 32:
+// 7.2 us with 512 packs per block, 4.5 now).
 int multiaxpy_norm_parts(DType t, size_t rows, int k) {
   const size_t packs = std::max(k / pack_of(t, k), 1), slots = std::max<size_t>(1, (dtype_lower(t) != t ? 64 : DT) / packs);
   return (int)std::min<size_t>(AXPY_PARTS, std::max<size_t>(1, (rows + slots - 1) / slots));
