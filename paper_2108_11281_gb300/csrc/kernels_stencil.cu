@@ -407,7 +407,8 @@ __global__ void __launch_bounds__(256) k_laplace(const T *__restrict__ x, const 
 // Threads per block of the half-sweep below.  FP64: small blocks for an even share per SM, but not so
 // small that 32 of them, the most an SM holds, leave it half empty (512^2 at 21 columns: sweep 67.8 us
 // with 32, 65.7 with 64; 192^2 at 5: 12.3 and 10.0).  FROM_ZERO is a compile-time flag: as an argument
-// it cost the FP64 pipe a multiply-add per entry (512^2 at 21 columns: 78.0 us).
+// it cost the FP64 pipe a multiply-add per entry (512^2 at 21 columns: 78.0 us).  The register bound
+// keeps 2048 threads on an SM: the FP32 form takes 34 without it (1024^2 x 64: 135 us, 126 with).
 template <class T> __host__ __device__ constexpr int lap_threads() { return sizeof(T) == 8 ? 64 : 256; }
 
 // Red-black Gauss-Seidel half-sweep for Example 5.1: x_s = (b_s + sum of neighbours) / diag
@@ -442,9 +443,9 @@ __device__ __forceinline__ void laplace_rbgs_body(T *__restrict__ x, const T *__
 }
 
 template <class T, int VEC, bool FROM_ZERO>
-__global__ void __launch_bounds__(lap_threads<T>()) k_laplace_rbgs(T *__restrict__ x, const T *__restrict__ b, int nx,
-                                                                   int ny, int kv, T dinv, int periodic, int colour,
-                                                                   int other_zero, int bpr) {
+__global__ void __launch_bounds__(lap_threads<T>(), 2048 / lap_threads<T>())
+    k_laplace_rbgs(T *__restrict__ x, const T *__restrict__ b, int nx, int ny, int kv, T dinv, int periodic, int colour,
+                   int other_zero, int bpr) {
   const int units = bpr * ny;
   for (int u = blockIdx.x; u < units; u += gridDim.x) {
     const int jr = u / bpr;
